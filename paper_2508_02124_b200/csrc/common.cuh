@@ -63,8 +63,47 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
                   void* dK, void* dV, float* dM, void* ws, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------
+// launches that overlap the tail of the kernel before them (programmatic dependent launch)
+// ---------------------------------------------------------------------------------------------
+// A kernel launched this way may become resident while the previous kernel of the stream still runs. Every such kernel
+// calls pdl_enter() with ALL its global pointers before its first access to global memory: it returns once the previous
+// kernel has completed and its writes are visible, and lets the next kernel in. What is saved is the launch latency and
+// the drain between dependent kernels, about 1 us each, which is what the short kernels of a decoding step are made of.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cluster > 1) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// ---------------------------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------------------------
+// Waits for the previous kernel, then lets the next one start. The pointers pass through an empty asm statement behind the
+// wait, so that no load through them (a read-only load of a const __restrict__ parameter is free to move) comes before it.
+template <typename... Ts>
+__device__ __forceinline__ void pdl_enter(Ts&... ptrs) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    auto pin = [](auto& p) { asm volatile("" : "+l"(p) :: "memory"); };
+    (pin(ptrs), ...);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void store_as(float* p, float x) { *p = x; }

@@ -1,362 +1,415 @@
 // Decoding step (Sec. 3.2 for a single query at the end of the sequence; Alg. 1 with the per-key mask M in R^N, the
 // configuration of the paper's decode benchmark): every (batch, query head) keeps the w cached keys with the largest
 // dynamic weight delta (ties to the lower index; all N keys if N <= w) and attends to them with delta as the bias.
-// HBM / L2-bound: the delta row is scanned to select, then only the selected K and V rows are read.
+// HBM / L2-bound: the delta row is read once to select, then only the selected K and V rows are read.
 //
 // Kernels
-//   decode_row_select_kernel   rows of up to 32768 keys: radix select over the 64-bit keys (delta bits << 32 | ~index) for
-//                          the threshold T with exactly min(w, N) keys >= T, one CTA per row on a shared-memory copy of the
-//                          row (a decoding step at these lengths is bound by dependent launches, not by their work)
-//   decode_hist_kernel x3, decode_thr_kernel   longer rows: the same three histogram passes spread over CTAs of 8192 keys
-//                          (per-row global histograms) and the final pick
-//   decode_index_kernel    optional: the selected indices in ascending order
-//   decode_attn_kernel     per (batch, head, split of <= 2048 keys): selected keys of the split are compacted into shared
-//                          memory; each warp then takes four of them per round (8 bytes of the K / V row per lane),
-//                          online softmax per warp, warps combined in shared memory -> partial (m, l, o). The CTA that
-//                          finishes a row last (a ticket counter, no waiting) combines the row's partials -> o, log-sum-exp
+//   decode_select_kernel   one cluster of CTAs per (batch, head) row: exact selection and the kept indices in ascending order
+//   decode_attn_kernel     per (batch, head, split of the kept list): every warp gathers a batch of K and V rows with all its
+//                          loads in flight, softmax per batch, warps combined in shared memory -> partial (m, l, o). The CTA
+//                          that finishes a row last (a ticket counter, no waiting) combines the row's partials -> o, lse
+//   decode_list_attn_kernel, decode_step_combine_kernel   the same for a kept set that is carried from step to step
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace dma {
 namespace {
 
-constexpr int kSplitKeys = 2048;
+namespace cg = cooperative_groups;
+
 constexpr int kAttnThreads = 256;
+constexpr int kMinSplit = 128, kMaxSplit = 512;     // kept keys per CTA of decode_attn_kernel
 
 __device__ __forceinline__ unsigned long long key_of(float dl, int j) {
     return ((unsigned long long)__float_as_uint(dl) << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
 }
 
-// Radix select of the min(w, N)-th largest key of every (batch, head) row, spread over many CTAs. Three histogram
-// passes over the delta bit patterns, bits [30:20], [19:9], [8:0] (delta > 0: the sign bit is clear and the pattern orders
-// like the value; exponent plus three mantissa bits spread a row over enough bins that shared-memory adds rarely
-// collide). Pass p: every CTA first re-derives the prefix chosen by the passes before it from their global histograms
-// (pick_bin: a 2048-bin suffix scan, identical in every CTA), then histograms the next bits of its 8192-key slice of the
-// row for the keys that match the prefix and adds the non-zero bins to the row's global histogram. A last kernel picks
-// the final bin and, only if several keys tie at the threshold delta and not all of them are wanted, walks the row in
-// index order for the cut. state[bh] = {prefix bits, keys still wanted inside the prefix}.
-struct SelState { uint32_t prefix; int need; };
+// Selection of a row's `keep` best keys by the delta bit patterns (delta > 0: the sign bit is clear and the pattern orders
+// like the value), then an ordered compaction of the keys above the threshold and of the first (lowest-index) keys at it.
+// The first histogram divides the row's own range [min, max] into 2048 bins, so that a bin near the threshold holds a few
+// dozen keys: those are gathered and ranked against each other. (Bins of fixed bit fields put a row into a few dozen bins in
+// all; a warp's shared-memory adds then collide and three passes over the row are needed.) Only a row with more than
+// kCandidates keys in the threshold's bin takes further passes, over the bin's own range.
+// What bounds it is a chain of barriers and sweeps, not the row's bytes (read once), so the sweeps run on registers: a thread
+// holds kKeys keys, key t of lane i of a warp at 32 t + i of the warp's contiguous part, which is both coalesced and in index
+// order for the compaction. Rows of up to kCtaKeys keys take one CTA; longer ones a cluster, whose CTAs read each other's
+// histograms (one cluster barrier per pass, a histogram buffer per pass); rows beyond eight CTAs' registers are read again in
+// every sweep (kKeys = 0), and their first range comes from a sample: a threshold in one of its end bins starts over with the
+// true range. Measured, kept list written (before: threshold only, and a scan of the delta row in the attention kernel):
+// 32 rows of 16384 keys 8.1 us (7.1), 256 rows of 65536 73 us (83 in four launches), 32 rows of 65536 13.9 us, where a
+// cluster of two takes 16.8 and one CTA that reads the row again 52. A cluster is slow to start (1024 keys: 3.8 us on one CTA,
+// 7.1 on two, 34 on eight), hence only where the registers demand it.
+constexpr int kSelectThreads = 1024, kSelectWarps = kSelectThreads / 32;
+constexpr int kSelectMaxCluster = 8;
+constexpr int kCandidates = 256;
+constexpr int kCtaKeys = 32 * kSelectThreads;
+constexpr int kStateHeader = 8;               // int32 words before the kept indices in a row of an incremental state
 
-// hist: 2048 counters of one pass; returns through `st` the bin holding the need-th largest key (scanning from the top
-// bin) and the rank wanted inside it. Called by every thread of a CTA of 256 threads.
-__device__ __forceinline__ void pick_bin(const int* __restrict__ hist, int shift, SelState& st, int* s_scan, SelState* s_out) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int c[8], sum = 0;
-#pragma unroll
-    for (int t = 0; t < 8; ++t) { c[t] = __ldcg(&hist[2047 - (8 * tid + t)]); sum += c[t]; }       // descending bin order
-    int incl = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    int before = 0;
-    for (int wq = 0; wq < warp; ++wq) before += s_scan[wq];
-    int excl = before + incl - sum;                       // keys in bins above this thread's first bin
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (excl < st.need && st.need <= excl + c[t]) {
-            s_out->prefix = st.prefix | ((uint32_t)(2047 - (8 * tid + t)) << shift);
-            s_out->need = st.need - excl;
-        }
-        excl += c[t];
-    }
-    __syncthreads();
-    st = *s_out;
-    __syncthreads();
-}
+struct alignas(16) SelectShared {
+    int hist[4][2048];                        // this CTA's histogram of each pass
+    unsigned long long cand[kCandidates];     // keys of this CTA in the threshold's bin ...
+    unsigned long long all[kCandidates];      // ... and of the whole row
+    int scan[kSelectWarps];
+    uint32_t warp_min[kSelectWarps], warp_max[kSelectWarps];
+    int warp_gt[kSelectWarps], warp_eq[kSelectWarps];
+    uint32_t umin, umax;                      // of this CTA's slice
+    int gt, eq;                               // keys above / at the threshold in this CTA's slice
+    int ncand;
+    uint32_t prefix;
+    int need, count, bin;
+};
 
-constexpr int kSliceKeys = 8192;
-
-// one histogram pass (pass = 0, 1, 2) of one 8192-key slice of one row; ghist [3][BH][2048] zeroed before pass 0
-__device__ __forceinline__ void hist_slice(const float* __restrict__ delta, int64_t ld, int N, int w, int pass, int* __restrict__ ghist,
-                                           int BH, int bh, int slice, int* hist, int* s_scan, SelState* s_out_p) {
-    SelState& s_out = *s_out_p;
-    const int tid = threadIdx.x;
-    const float* dl = delta + (size_t)bh * ld;
-    const int shifts[3] = {20, 9, 0}, widths[3] = {11, 11, 9};
-    SelState st{0u, w};
-    for (int q = 0; q < pass; ++q) pick_bin(ghist + ((size_t)q * BH + bh) * 2048, shifts[q], st, s_scan, &s_out);
-    for (int t = tid; t < 2048; t += 256) hist[t] = 0;
-    __syncthreads();
-    const int shift = shifts[pass], nb = 1 << widths[pass];
-    const uint32_t himask = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + widths[pass]));
-    const int j0 = slice * kSliceKeys, j1 = min(N, j0 + kSliceKeys);
-    for (int base = j0; base < j1; base += 4 * 256) {
-        uint32_t u[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int j = base + t * 256 + tid;
-            u[t] = j < j1 ? __float_as_uint(dl[j]) : 0xFFFFFFFFu;              // never matches: deltas have the sign bit clear
-        }
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-            if (u[t] != 0xFFFFFFFFu && (u[t] & himask) == st.prefix) atomicAdd(&hist[(u[t] >> shift) & (nb - 1)], 1);
-    }
-    __syncthreads();
-    int* g = ghist + ((size_t)pass * BH + bh) * 2048;
-    for (int t = tid; t < 2048; t += 256)
-        if (hist[t]) atomicAdd(&g[t], hist[t]);
-    __syncthreads();                               // the shared histogram is reused by the caller's next slice
-}
-
-__global__ void __launch_bounds__(256) decode_hist_kernel(const float* __restrict__ delta, int64_t ld, int N, int w, int pass,
-                                                          int* __restrict__ ghist, int BH) {
-    __shared__ int hist[2048];
-    __shared__ int s_scan[8];
-    __shared__ SelState s_out;
-    if (N <= w) return;
-    hist_slice(delta, ld, N, w, pass, ghist, BH, blockIdx.y, blockIdx.x, hist, s_scan, &s_out);
-}
-
-// one CTA per row: final pick; thr = (delta bits << 32) | ~index cut
-__device__ __forceinline__ void thr_row(const float* __restrict__ delta, int64_t ld, int N, int w, const int* __restrict__ ghist, int BH,
-                                        unsigned long long* __restrict__ thr, int bh, int* s_scan, SelState* s_out_p, int* s_warp,
-                                        int* s_found_p) {
-    SelState& s_out = *s_out_p;
-    int& s_found = *s_found_p;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (N <= w) {
-        if (tid == 0) thr[bh] = 0ull;          // every key qualifies
+// list: row bh's kept indices go to list + bh * list_stride. tickets (may be NULL): one counter per row, zeroed here.
+// kState: list points at the rows of an incremental state; count and weakest kept key go to the header before it.
+template <int kKeys, bool kState>
+__global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_select_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep, int slice,
+                                                                       int* __restrict__ list, int64_t list_stride, int* __restrict__ tickets) {
+    extern __shared__ __align__(16) uint8_t select_smem[];
+    SelectShared& S = *reinterpret_cast<SelectShared*>(select_smem);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int bh = blockIdx.x / nrank, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int j0 = rank * slice, n = max(0, min(slice, N - j0));
+    // this warp's part of the slice: [i0, i1), `seg` (a multiple of 32) keys per warp
+    const int seg = kKeys ? 32 * kKeys : (slice + kSelectThreads - 1) / kSelectThreads * 32;
+    const int i0 = warp * seg, i1 = min(n, i0 + seg), sweeps = seg / 32;
+    for (int t = tid; t < (int)sizeof(S.hist) / 4; t += kSelectThreads) (&S.hist[0][0])[t] = 0;
+    if (tid == 0) S.ncand = 0;
+    pdl_enter(delta, list, tickets);
+    int* out = list + (size_t)bh * list_stride;
+    if (tickets && rank == 0 && tid == 0) tickets[bh] = 0;
+    if (!kState && keep >= N) {                // every key is kept
+        for (int i = tid; i < n; i += kSelectThreads) out[j0 + i] = j0 + i;
         return;
     }
-    const float* dl = delta + (size_t)bh * ld;
-    const int shifts[3] = {20, 9, 0};
-    SelState st{0u, w};
-    const int* g2 = ghist + ((size_t)2 * BH + bh) * 2048;
-    for (int q = 0; q < 3; ++q) pick_bin(ghist + ((size_t)q * BH + bh) * 2048, shifts[q], st, s_scan, &s_out);
-    // st.prefix = delta bits of the threshold; st.need of the keys with exactly that delta are kept, lowest index first
-    const uint32_t dstar = st.prefix;
-    const int equal = __ldcg(&g2[dstar & 511]);
-    if (st.need >= equal) {                    // every key with this delta is wanted: no cut inside the group
-        if (tid == 0) thr[bh] = (unsigned long long)dstar << 32;
-        return;
-    }
-    if (tid == 0) s_found = -1;
-    int seen = 0;
-    for (int base = 0; base < N; base += 256) {
-        const int j = base + tid;
-        const bool eq = j < N && __float_as_uint(dl[j]) == dstar;
-        const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-        if (lane == 0) s_warp[warp] = __popc(bal);
-        __syncthreads();
-        int before = 0, total = 0;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(delta + (size_t)bh * ld) + j0 + i0 + lane;
+    // Keys beyond the row read as 0xFFFFFFFF, which no pass counts (the sign bit of the others is masked: delta > 0, and a
+    // row that breaks this still yields `keep` distinct indices).
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    auto fetch = [&](int t) { return i0 + 32 * t + lane < i1 ? src[32 * t] & 0x7FFFFFFFu : kNone; };
+    uint32_t key[kKeys ? kKeys : 1];
+    if constexpr (kKeys > 0) {
 #pragma unroll
-        for (int wq = 0; wq < 8; ++wq) {
-            const int c = s_warp[wq];
-            before += wq < warp ? c : 0;
-            total += c;
-        }
-        const int rank = seen + before + __popc(bal & ((1u << lane) - 1));      // 0-based rank among the equal keys
-        if (eq && rank == st.need - 1) s_found = j;
-        seen += total;
-        __syncthreads();
-        if (seen >= st.need) break;
+        for (int t = 0; t < kKeys; ++t) key[t] = fetch(t);
     }
-    __syncthreads();
-    if (tid == 0) thr[bh] = key_of(__uint_as_float(dstar), s_found);
-}
-
-__global__ void __launch_bounds__(256) decode_thr_kernel(const float* __restrict__ delta, int64_t ld, int N, int w,
-                                                         const int* __restrict__ ghist, int BH, unsigned long long* __restrict__ thr) {
-    __shared__ int s_scan[8];
-    __shared__ SelState s_out;
-    __shared__ int s_warp[8], s_found;
-    thr_row(delta, ld, N, w, ghist, BH, thr, blockIdx.x, s_scan, &s_out, s_warp, &s_found);
-}
-
-// The whole selection of a row by ONE CTA, for rows that fit in shared memory (N <= kRowSelectMax): the row is loaded
-// once, the three histogram passes and the final pick run on the shared copy with CTA-wide barriers only. A decoding step
-// at these lengths is bound by dependent launches and global round trips, not by the work: this replaces a memset and
-// four launches by one. Also zeroes the row's combine ticket.
-constexpr int kRowSelectMax = 32768;
-constexpr int kRowSelectThreads = 1024;
-
-__global__ void __launch_bounds__(kRowSelectThreads) decode_row_select_kernel(const float* __restrict__ delta, int64_t ld, int N, int w,
-                                                                              unsigned long long* __restrict__ thr, int* __restrict__ tickets) {
-    extern __shared__ uint32_t row[];                  // the row's delta bit patterns
-    __shared__ int hist[2048];
-    __shared__ int s_scan[32];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_need, s_equal, s_found, s_warp[32];
-    const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) tickets[bh] = 0;
-    if (N <= w) {
-        if (tid == 0) thr[bh] = 0ull;                  // every key qualifies
-        return;
-    }
-    const float* dl = delta + (size_t)bh * ld;
-    for (int j = tid; j < N; j += kRowSelectThreads) row[j] = __float_as_uint(dl[j]);
-    uint32_t prefix = 0u;
-    int need = w;
-    const int shifts[3] = {20, 9, 0}, widths[3] = {11, 11, 9};
-    for (int pass = 0; pass < 3; ++pass) {
-        for (int t = tid; t < 2048; t += kRowSelectThreads) hist[t] = 0;
-        __syncthreads();                               // (also: the row is complete before the first pass reads it)
-        const int shift = shifts[pass], nb = 1 << widths[pass];
-        const uint32_t himask = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + widths[pass]));
-        for (int j = tid; j < N; j += kRowSelectThreads) {
-            const uint32_t u = row[j];
-            if ((u & himask) == prefix) atomicAdd(&hist[(u >> shift) & (nb - 1)], 1);
+    auto sweep = [&](auto&& f) {               // f(t, key) for the warp's keys, in index order
+        if constexpr (kKeys > 0) {
+#pragma unroll
+            for (int t = 0; t < kKeys; ++t) f(t, key[t]);
+        } else {
+#pragma unroll 8
+            for (int t = 0; t < sweeps; ++t) f(t, fetch(t));
         }
+    };
+    // the range of the row's keys (`part`: of the first four of every lane only)
+    auto range = [&](bool part, uint32_t& umin, uint32_t& umax) {
+        umin = 0x7FFFFFFFu;
+        umax = 0u;
+        auto take = [&](int, uint32_t u) { if (u != kNone) { umin = min(umin, u); umax = max(umax, u); } };
+        if (part) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) take(t, fetch(t));
+        } else {
+            sweep(take);
+        }
+        umin = __reduce_min_sync(0xffffffffu, umin);
+        umax = __reduce_max_sync(0xffffffffu, umax);
+        if (lane == 0) { S.warp_min[warp] = umin; S.warp_max[warp] = umax; }
         __syncthreads();
-        // the bin holding the need-th largest key, scanning from the top bin: two bins per thread, descending order
-        const int c0 = hist[2047 - 2 * tid], c1 = hist[2046 - 2 * tid], sum = c0 + c1;
+        umin = __reduce_min_sync(0xffffffffu, S.warp_min[lane]);
+        umax = __reduce_max_sync(0xffffffffu, S.warp_max[lane]);
+        if (nrank > 1) {
+            if (tid == 0) { S.umin = umin; S.umax = umax; }
+            cluster.sync();
+            for (int q = 0; q < nrank; ++q) {
+                umin = min(umin, *cluster.map_shared_rank(&S.umin, q));
+                umax = max(umax, *cluster.map_shared_rank(&S.umax, q));
+            }
+            cluster.sync();                    // (the words may be written again)
+        }
+    };
+    bool sampled = kKeys == 0 && sweeps > 16;
+    uint32_t lo, umax;
+    range(sampled, lo, umax);                  // (its barrier: the histograms are zero)
+    int shift = max(0, 21 - __clz((int)(umax - lo))), need = keep, cgt = 0, ceq = 0;
+    bool counted = false;
+    uint32_t nbins = 2048u;
+    for (int pass = 0;; ++pass) {
+        // the keys in [lo, lo + nbins << shift) into nbins bins; all others, and kNone, have a bin number beyond (shift <= 20),
+        // or fall into the end bins after a sample
+        int* hist = S.hist[pass];
+        if (sampled) {
+            sweep([&](int, uint32_t u) { if (u != kNone) atomicAdd(&hist[u < lo ? 0u : min((u - lo) >> shift, 2047u)], 1); });
+        } else {
+            sweep([&](int, uint32_t u) {
+                const uint32_t bin = (u - lo) >> shift;
+                if (bin < nbins) atomicAdd(&hist[bin], 1);
+            });
+        }
+        // the bin holding the need-th largest key: two bins per thread in descending order
+        int c0 = 0, c1 = 0;
+        const int top = 2046 - 2 * tid;
+        if (nrank > 1) {
+            cluster.sync();
+            for (int q = 0; q < nrank; ++q) {
+                const int2 v = *reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, q) + top);
+                c0 += v.y;
+                c1 += v.x;
+            }
+        } else {
+            __syncthreads();
+            const int2 v = *reinterpret_cast<const int2*>(hist + top);
+            c0 = v.y;
+            c1 = v.x;
+        }
+        const int sum = c0 + c1;
         int incl = sum;
+#pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
         }
-        if (lane == 31) s_scan[warp] = incl;
+        if (lane == 31) S.scan[warp] = incl;
         __syncthreads();
-        int before = 0;
-        for (int wq = 0; wq < warp; ++wq) before += s_scan[wq];
-        int excl = before + incl - sum;                // keys in bins above this thread's first bin
-        if (excl < need && need <= excl + c0) { s_prefix = prefix | ((uint32_t)(2047 - 2 * tid) << shift); s_need = need - excl; s_equal = c0; }
-        excl += c0;
-        if (excl < need && need <= excl + c1) { s_prefix = prefix | ((uint32_t)(2046 - 2 * tid) << shift); s_need = need - excl; s_equal = c1; }
-        __syncthreads();
-        prefix = s_prefix;
-        need = s_need;
-        __syncthreads();
-    }
-    // prefix = delta bits of the threshold; `need` of the keys with exactly that delta are kept, lowest index first
-    const int equal = s_equal;
-    if (need >= equal) {                               // every key with this delta is wanted: no cut inside the group
-        if (tid == 0) thr[bh] = (unsigned long long)prefix << 32;
-        return;
-    }
-    if (tid == 0) s_found = -1;
-    int seen = 0;
-    for (int base = 0; base < N; base += kRowSelectThreads) {
-        const int j = base + tid;
-        const bool eq = j < N && row[j] == prefix;
-        const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-        if (lane == 0) s_warp[warp] = __popc(bal);
-        __syncthreads();
-        int bef = 0, total = 0;
-        for (int wq = 0; wq < 32; ++wq) {
-            const int c = s_warp[wq];
-            bef += wq < warp ? c : 0;
-            total += c;
+        const int before = __reduce_add_sync(0xffffffffu, lane < warp ? S.scan[lane] : 0);
+        const int excl = before + incl - sum;  // keys in bins above this thread's first bin
+        const bool in0 = excl < need && need <= excl + c0, in1 = excl + c0 < need && need <= excl + sum;
+        if (in0 || in1) {
+            S.bin = in0 ? top + 1 : top;
+            S.need = need - excl - (in0 ? 0 : c0);
+            S.count = in0 ? c0 : c1;
         }
-        const int rank = seen + bef + __popc(bal & ((1u << lane) - 1));          // 0-based rank among the equal keys
-        if (eq && rank == need - 1) s_found = j;
-        seen += total;
         __syncthreads();
-        if (seen >= need) break;
+        const int bin = S.bin, count = S.count;
+        if (sampled) {
+            sampled = false;
+            if (bin == 0 || bin == 2047) {     // beyond the sample's range (its ends included): once more with the true one
+                range(false, lo, umax);
+                shift = max(0, 21 - __clz((int)(umax - lo)));
+                continue;
+            }
+        }
+        lo += (uint32_t)bin << shift;
+        need = S.need;
+        if (shift == 0) break;                 // one pattern left: `need` keys with exactly this delta are kept
+        if (count <= kCandidates) {
+            // rank the bin's keys against each other; the keys above the bin are counted in the same sweep
+            const uint32_t size = 1u << shift;
+            sweep([&](int t, uint32_t u) {
+                cgt += u - lo >= size && u > lo && u != kNone;
+                if (u - lo < size) S.cand[atomicAdd(&S.ncand, 1)] = key_of(__uint_as_float(u), j0 + i0 + 32 * t + lane);
+            });
+            cgt = __reduce_add_sync(0xffffffffu, cgt);
+            if (lane == 0) { S.warp_gt[warp] = cgt; S.warp_eq[warp] = 0; }
+            const unsigned long long* cand = S.cand;
+            if (nrank > 1) {
+                cluster.sync();
+                int at = 0;
+                for (int q = 0; q < nrank; ++q) {
+                    const int nq = *cluster.map_shared_rank(&S.ncand, q);
+                    if (tid < nq) S.all[at + tid] = cluster.map_shared_rank(S.cand, q)[tid];
+                    at += nq;
+                }
+                cand = S.all;
+            }
+            __syncthreads();
+            if (tid < count) {
+                const unsigned long long k = cand[tid];
+                int rank_k = 0, above = 0;
+                for (int i = 0; i < count; ++i) {
+                    const unsigned long long x = cand[i];
+                    rank_k += x > k;
+                    above += (uint32_t)(x >> 32) > (uint32_t)(k >> 32);
+                }
+                if (rank_k == need - 1) { S.prefix = (uint32_t)(k >> 32); S.need = need - above; }
+            }
+            __syncthreads();
+            lo = S.prefix;
+            need = S.need;
+            if (tid < S.ncand) {               // this CTA's candidates join their warps' counts
+                const unsigned long long k = S.cand[tid];
+                const uint32_t u = (uint32_t)(k >> 32);
+                const int owner = (int)(0xFFFFFFFFu - (uint32_t)k - (uint32_t)j0) / seg;
+                if (u > lo) atomicAdd(&S.warp_gt[owner], 1);
+                else if (u == lo) atomicAdd(&S.warp_eq[owner], 1);
+            }
+            counted = true;
+            break;
+        }
+        nbins = 1u << min(11, shift);          // the next pass covers this bin and nothing above it
+        shift = max(0, shift - 11);
+        __syncthreads();                       // everyone has read the pass's result
+    }
+    const uint32_t prefix = lo;
+    // prefix: delta bits of the threshold; `need` of the keys with exactly that delta are kept, lowest index first. Every
+    // warp counts its part and writes from the position its lower-index neighbours leave it.
+    if (!counted) {
+        sweep([&](int, uint32_t u) { cgt += u > prefix && u != kNone; ceq += u == prefix; });
+        cgt = __reduce_add_sync(0xffffffffu, cgt);
+        ceq = __reduce_add_sync(0xffffffffu, ceq);
+        if (lane == 0) { S.warp_gt[warp] = cgt; S.warp_eq[warp] = ceq; }
     }
     __syncthreads();
-    if (tid == 0) thr[bh] = key_of(__uint_as_float(prefix), s_found);
-}
-
-__global__ void __launch_bounds__(256) decode_index_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep,
-                                                           const unsigned long long* __restrict__ thr, int32_t* __restrict__ idx,
-                                                           int64_t idx_stride) {
-    __shared__ int wsum[2][8];
-    const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float* dl = delta + (size_t)bh * ld;
-    const unsigned long long T = thr[bh];
-    int n = 0, buf = 0;
-    for (int base = 0; base < N; base += 256, buf ^= 1) {
-        const int j = base + tid;
-        const bool sel = j < N && key_of(dl[j], j) >= T;
-        const uint32_t bal = __ballot_sync(0xffffffffu, sel);
-        if (lane == 0) wsum[buf][warp] = __popc(bal);
-        __syncthreads();
-        int before = 0, total = 0;
-#pragma unroll
-        for (int wq = 0; wq < 8; ++wq) {
-            const int c = wsum[buf][wq];
-            before += wq < warp ? c : 0;
-            total += c;
-        }
-        const int pos = n + before + __popc(bal & ((1u << lane) - 1));
-        if (sel && pos < keep) idx[(size_t)bh * idx_stride + pos] = j;
-        n += total;
+    cgt = S.warp_gt[warp];
+    ceq = S.warp_eq[warp];
+    int gtb = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_gt[lane] : 0);
+    int eqb = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_eq[lane] : 0);
+    if (nrank > 1) {
+        if (warp == kSelectWarps - 1 && lane == 0) { S.gt = gtb + cgt; S.eq = eqb + ceq; }
+        cluster.sync();
+        for (int q = 0; q < rank; ++q) { gtb += *cluster.map_shared_rank(&S.gt, q); eqb += *cluster.map_shared_rank(&S.eq, q); }
     }
+    const uint32_t below = (1u << lane) - 1u;
+    if (ceq == 0) {                            // (all but a few warps)
+        gtb += min(need, eqb);
+        sweep([&](int t, uint32_t u) {
+            const bool g = u > prefix && u != kNone;
+            const uint32_t bg = __ballot_sync(0xffffffffu, g);
+            if (g) out[gtb + __popc(bg & below)] = j0 + i0 + 32 * t + lane;
+            gtb += __popc(bg);
+        });
+    } else {
+        sweep([&](int t, uint32_t u) {
+            const bool g = u > prefix && u != kNone, e = u == prefix;
+            const uint32_t bg = __ballot_sync(0xffffffffu, g), be = __ballot_sync(0xffffffffu, e);
+            const int j = j0 + i0 + 32 * t + lane, erank = eqb + __popc(be & below), pos = gtb + __popc(bg & below) + min(need, erank);
+            if (g || (e && erank < need)) out[pos] = j;
+            if (kState && e && erank == need - 1) {      // the weakest kept key: lowest delta, highest index
+                int* hdr = out - kStateHeader;
+                const unsigned long long k = key_of(__uint_as_float(u), j);
+                hdr[0] = keep;
+                hdr[1] = pos;
+                hdr[2] = (int)(uint32_t)k;
+                hdr[3] = (int)(uint32_t)(k >> 32);
+            }
+            gtb += __popc(bg);
+            eqb += __popc(be);
+        });
+    }
+    if (nrank > 1) cluster.sync();             // no CTA leaves while another may still read its shared memory
 }
 
-__device__ __forceinline__ void load4(const float* p, float (&v)[4]) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-}
-__device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4]) {
-    const uint2 a = *reinterpret_cast<const uint2*>(p);
-    v[0] = __uint_as_float(a.x << 16); v[1] = __uint_as_float(a.x & 0xffff0000u);
-    v[2] = __uint_as_float(a.y << 16); v[3] = __uint_as_float(a.y & 0xffff0000u);
-}
+// 16 bytes of a K, V or q row, widened to fp32
+template <typename T> struct Wide;
+template <> struct Wide<float> {
+    static constexpr int kN = 4;
+    static __device__ __forceinline__ void get(const uint4& a, float (&v)[4]) {
+        v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y); v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
+    }
+};
+template <> struct Wide<__nv_bfloat16> {
+    static constexpr int kN = 8;
+    static __device__ __forceinline__ void get(const uint4& a, float (&v)[8]) {
+        const uint32_t u[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[2 * i] = __uint_as_float(u[i] << 16);
+            v[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u);
+        }
+    }
+};
 
-// partial [bh][split][D + 2]: o (unnormalised, relative to m), m (log2 domain), l
-// The attention part shared by the two decoding kernels: `list` (shared memory) holds `count` key indices of this CTA.
-// Each warp takes four of them per round (8 bytes of the K / V row per lane), online softmax per warp, then the warps are
-// combined in shared memory and the CTA's partial (o relative to m, m in the log2 domain, l) is written.
+// Sum over the LPR lanes of a row group of eight per-lane partials: after three levels in which a lane keeps half of its
+// values and hands the other half to its partner, lane `sub` holds the sum of value bitrev(sub & 7). 7 + log2(LPR / 8)
+// shuffles for eight rows.
+template <int LPR>
+__device__ __forceinline__ float reduce8(float (&p)[8], int sub) {
+#pragma unroll
+    for (int m = 1, keep = 4; m < 8; m <<= 1, keep >>= 1) {
+        const bool up = (sub & m) != 0;
+#pragma unroll
+        for (int q = 0; q < keep; ++q) {
+            const float stay = up ? p[q + keep] : p[q], give = up ? p[q] : p[q + keep];
+            p[q] = stay + __shfl_xor_sync(0xffffffffu, give, m);
+        }
+    }
+#pragma unroll
+    for (int m = 8; m < LPR; m <<= 1) p[0] += __shfl_xor_sync(0xffffffffu, p[0], m);
+    return p[0];
+}
+__device__ __forceinline__ int bitrev3(int x) { return ((x & 1) << 2) | (x & 2) | ((x >> 2) & 1); }
+
+// The attention part shared by the two decoding kernels: `list` (shared memory) holds `count` key indices of this CTA;
+// partial [D + 2]: o (unnormalised, relative to m), m (log2 domain), l.
+// A step's attention is a gather of 2 * D * sizeof(T) bytes per kept key, bound by how many of those bytes are in flight, so
+// a warp takes batches of eight 16-byte K loads AND eight V loads per lane (bf16, D = 128: 16 keys, 8 KB per warp) issued
+// back to back, and spends few instructions per key: one transposing reduction and one exponential per lane for the whole
+// batch. Measured against the form before (8 bytes per lane, four keys in flight, five shuffles and two exponentials in every
+// lane per key): 256 rows of 4096 kept keys in 65536 (537 MB of rows) 254 -> 99 us, 5.4 TB/s; 32 rows of 2048 in 16384,
+// 21 -> 8 us; a step with a carried state 12.2 -> 7 us.
 template <typename T, int D>
 __device__ __forceinline__ void decode_attend(const int* list, int count, const T* __restrict__ q, const T* __restrict__ K,
                                               const T* __restrict__ V, const float* __restrict__ dl, float* __restrict__ out,
                                               int bh, int b, int hk, float scale_log2, int64_t ks_b, int64_t ks_l, int64_t ks_h,
                                               int64_t vs_b, int64_t vs_l, int64_t vs_h) {
-    constexpr int LPK = D / 4;                 // lanes per key row (4 channels per lane)
-    constexpr int KPW = 32 / LPK;              // keys per warp instruction
-    __shared__ float s_part[8][D + 2];
+    constexpr int CPL = Wide<T>::kN;           // channels per lane
+    constexpr int LPR = D / CPL;               // lanes per key row
+    constexpr int RPI = 32 / LPR;              // key rows per warp instruction
+    constexpr int kBatch = 8 * RPI;            // keys a warp takes at a time
+    __shared__ __align__(16) float s_part[8][D + 4];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // each warp: KPW keys per instruction (LPK lanes per key, 4 channels per lane), four such groups per round
-    const int sub = lane % LPK, grp = lane / LPK;
-    float qv[4];
-    load4(q + (size_t)bh * D + sub * 4, qv);
-    float m = -INFINITY, l = 0.0f, o[4] = {0.f, 0.f, 0.f, 0.f};
-    const T* Kb = K + b * ks_b + hk * ks_h + sub * 4;
-    const T* Vb = V + b * vs_b + hk * vs_h + sub * 4;
-    constexpr int kInFlight = 4;               // key rows whose K and V loads are in flight together, per lane group (8 was slower)
-    for (int base = warp * KPW * kInFlight; base < count; base += 8 * KPW * kInFlight) {
-        int jj[kInFlight];
-        float kv[kInFlight][4], vv[kInFlight][4], bias[kInFlight];
+    const int sub = lane % LPR, grp = lane / LPR;
+    float qv[CPL];
+    Wide<T>::get(*reinterpret_cast<const uint4*>(q + (size_t)bh * D + sub * CPL), qv);
+    float m = -INFINITY, l = 0.0f, o[CPL];
 #pragma unroll
-        for (int u = 0; u < kInFlight; ++u) {
-            const int e = base + u * KPW + grp;
-            jj[u] = e < count ? list[e] : -1;
-            if (jj[u] >= 0) {
-                load4(Kb + (int64_t)jj[u] * ks_l, kv[u]);
-                load4(Vb + (int64_t)jj[u] * vs_l, vv[u]);
-                bias[u] = dl[jj[u]];
-            } else {
+    for (int c = 0; c < CPL; ++c) o[c] = 0.0f;
+    const T* Kb = K + b * ks_b + hk * ks_h + sub * CPL;
+    const T* Vb = V + b * vs_b + hk * vs_h + sub * CPL;
+    const int mine = bitrev3(sub & 7) * RPI + grp;                 // the key of the batch whose score ends up in this lane
+    for (int base = warp * kBatch; base < count; base += 8 * kBatch) {
+        uint4 kr[8], vr[8];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) { kv[u][c] = 0.0f; vv[u][c] = 0.0f; }
-                bias[u] = 0.0f;
-            }
+        for (int u = 0; u < 8; ++u) {                              // (entries beyond the list repeat its last key)
+            const int64_t j = list[min(base + u * RPI + grp, count - 1)];
+            kr[u] = __ldg(reinterpret_cast<const uint4*>(Kb + j * ks_l));
+            vr[u] = __ldg(reinterpret_cast<const uint4*>(Vb + j * vs_l));
         }
+        const bool real = base + mine < count;
+        const float bias = dl[list[min(base + mine, count - 1)]];
+        float p[8];
 #pragma unroll
-        for (int u = 0; u < kInFlight; ++u) {
-            float s = qv[0] * kv[u][0] + qv[1] * kv[u][1] + qv[2] * kv[u][2] + qv[3] * kv[u][3];
+        for (int u = 0; u < 8; ++u) {
+            float kv[CPL], a = 0.0f;
+            Wide<T>::get(kr[u], kv);
 #pragma unroll
-            for (int mm = 1; mm < LPK; mm <<= 1) s += __shfl_xor_sync(0xffffffffu, s, mm);
-            const float x = jj[u] >= 0 ? fmaf(s, scale_log2, bias[u] * 1.4426950408889634f) : -INFINITY;
-            const float m_new = fmaxf(m, x);
-            const float f = m_new == -INFINITY ? 1.0f : exp2f(m - m_new);
-            const float p = m_new == -INFINITY ? 0.0f : exp2f(x - m_new);
-            l = l * f + p;
+            for (int c = 0; c < CPL; ++c) a = fmaf(qv[c], kv[c], a);
+            p[u] = a;
+        }
+        const float s = reduce8<LPR>(p, sub);
+        const float x = real ? fmaf(s, scale_log2, bias * 1.4426950408889634f) : -INFINITY;
+        float mx = x;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) o[c] = o[c] * f + p * vv[u][c];
-            m = m_new;
+        for (int mm = 1; mm < 32; mm <<= 1)
+            if (mm < 8 || mm >= LPR) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, mm));
+        const float m_new = fmaxf(m, mx), m_use = m_new == -INFINITY ? 0.0f : m_new;
+        const float f = exp2f(m - m_use), w = exp2f(x - m_use);
+        m = m_new;
+        l = l * f + (sub < 8 ? w : 0.0f);                          // (lanes 8 and up of a row group repeat the first eight)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) o[c] *= f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float wu = __shfl_sync(0xffffffffu, w, grp * LPR + bitrev3(u));
+            float vv[CPL];
+            Wide<T>::get(vr[u], vv);
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) o[c] = fmaf(wu, vv[c], o[c]);
         }
     }
-    // the KPW key groups of a warp hold different keys: merge them, then the warps, in shared memory
+    // the row groups of a warp share m: plain sums; then the warps are combined in shared memory
 #pragma unroll
-    for (int mm = LPK; mm < 32; mm <<= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, mm), l2 = __shfl_xor_sync(0xffffffffu, l, mm);
-        float o2[4];
+    for (int mm = LPR; mm < 32; mm <<= 1)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) o2[c] = __shfl_xor_sync(0xffffffffu, o[c], mm);
-        const float mn = fmaxf(m, m2);
-        const float f1 = mn == -INFINITY ? 1.0f : exp2f(m - mn), f2 = mn == -INFINITY ? 1.0f : exp2f(m2 - mn);
-        l = l * f1 + l2 * f2;
+        for (int c = 0; c < CPL; ++c) o[c] += __shfl_xor_sync(0xffffffffu, o[c], mm);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) o[c] = o[c] * f1 + o2[c] * f2;
-        m = mn;
-    }
+    for (int mm = 1; mm < 32; mm <<= 1) l += __shfl_xor_sync(0xffffffffu, l, mm);
     if (grp == 0) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) s_part[warp][sub * 4 + c] = o[c];
+        for (int c = 0; c < CPL; c += 4) *reinterpret_cast<float4*>(&s_part[warp][sub * CPL + c]) = make_float4(o[c], o[c + 1], o[c + 2], o[c + 3]);
         if (sub == 0) { s_part[warp][D] = m; s_part[warp][D + 1] = l; }
     }
     __syncthreads();
@@ -369,7 +422,7 @@ __device__ __forceinline__ void decode_attend(const int* list, int count, const 
 #pragma unroll
         for (int wq = 0; wq < 8; ++wq) {
             const float mw = s_part[wq][D];
-            const float f = (mw == -INFINITY || mx == -INFINITY) ? 0.0f : exp2f(mw - mx);
+            const float f = mw == -INFINITY ? 0.0f : exp2f(mw - mx);
             acc += s_part[wq][c] * f;                 // c == D + 1 is l
         }
         out[c] = acc;
@@ -437,52 +490,23 @@ __device__ __forceinline__ bool last_of_row(int* ticket, int nsplit) {
     return s_last != 0;
 }
 
+// One CTA per (row, split of `per_split` entries of the row's kept list).
 template <typename T, int D>
-__global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
-                                                                   const float* __restrict__ delta, int64_t ld,
-                                                                   const unsigned long long* __restrict__ thr, float* __restrict__ partial,
-                                                                   int N, int Hq, int G, float scale_log2, int nsplit,
-                                                                   int64_t ks_b, int64_t ks_l, int64_t ks_h, int64_t vs_b, int64_t vs_l,
-                                                                   int64_t vs_h, int* __restrict__ tickets, T* __restrict__ o,
-                                                                   float* __restrict__ lse) {
-    __shared__ int list[kSplitKeys];
-    __shared__ int s_count, wsum[2][8];
+__global__ void __launch_bounds__(kAttnThreads, 2) decode_attn_kernel(const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
+                                                                      const float* __restrict__ delta, int64_t ld,
+                                                                      const int* __restrict__ kept, int64_t kept_stride, float* __restrict__ partial,
+                                                                      int keep, int per_split, int Hq, int G, float scale_log2, int nsplit,
+                                                                      int64_t ks_b, int64_t ks_l, int64_t ks_h, int64_t vs_b, int64_t vs_l,
+                                                                      int64_t vs_h, int* __restrict__ tickets, T* __restrict__ o,
+                                                                      float* __restrict__ lse) {
+    __shared__ int list[kMaxSplit];
     const int split = blockIdx.x, bh = blockIdx.y, b = bh / Hq, h = bh % Hq, hk = h / G;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float* dl = delta + (size_t)bh * ld;
-    const unsigned long long Tkey = thr[bh];
-    const int j_begin = split * kSplitKeys, j_end = min(N, j_begin + kSplitKeys);
-    // ordered compaction of the split's selected keys
-    int n = 0, buf = 0;
-    float dpre[kSplitKeys / kAttnThreads];          // the split's deltas of this thread, all loads in flight together
-#pragma unroll
-    for (int t = 0; t < kSplitKeys / kAttnThreads; ++t) {
-        const int j = j_begin + t * kAttnThreads + tid;
-        dpre[t] = j < j_end ? dl[j] : 0.0f;
-    }
-#pragma unroll
-    for (int t = 0; t < kSplitKeys / kAttnThreads; ++t, buf ^= 1) {
-        const int base = j_begin + t * kAttnThreads;
-        if (base >= j_end) break;
-        const int j = base + tid;
-        const bool sel = j < j_end && key_of(dpre[t], j) >= Tkey;
-        const uint32_t bal = __ballot_sync(0xffffffffu, sel);
-        if (lane == 0) wsum[buf][warp] = __popc(bal);
-        __syncthreads();
-        int before = 0, total = 0;
-#pragma unroll
-        for (int wq = 0; wq < 8; ++wq) {
-            const int c = wsum[buf][wq];
-            before += wq < warp ? c : 0;
-            total += c;
-        }
-        if (sel) list[n + before + __popc(bal & ((1u << lane) - 1))] = j;
-        n += total;
-    }
-    if (tid == 0) s_count = n;
+    const int e0 = split * per_split, count = min(per_split, keep - e0);
+    pdl_enter(q, K, V, delta, kept, partial, tickets, o, lse);
+    for (int e = threadIdx.x; e < count; e += kAttnThreads) list[e] = kept[(size_t)bh * kept_stride + e0 + e];
     __syncthreads();
-    decode_attend<T, D>(list, s_count, q, K, V, dl, partial + ((size_t)bh * nsplit + split) * (D + 2), bh, b, hk, scale_log2, ks_b, ks_l,
-                        ks_h, vs_b, vs_l, vs_h);
+    decode_attend<T, D>(list, count, q, K, V, delta + (size_t)bh * ld, partial + ((size_t)bh * nsplit + split) * (D + 2), bh, b, hk, scale_log2,
+                        ks_b, ks_l, ks_h, vs_b, vs_l, vs_h);
     if (last_of_row(tickets + bh, nsplit)) combine_row<T, D>(partial, o, lse, nsplit, bh);
 }
 
@@ -493,7 +517,6 @@ __global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(const T* __re
 //         [4..7] unused
 //   int32 [8 .. 8 + w)       the kept key indices, in no particular order
 // A step costs O(w), whatever the number of cached keys: no scan of the delta row.
-constexpr int kStateHeader = 8;
 constexpr int kListSplit = 128;            // kept keys per CTA of the list attention kernel (256: 4 us slower per step at w = 2048)
 
 __device__ __forceinline__ int state_stride(int w_cap) { return kStateHeader + ((w_cap + 3) & ~3); }
@@ -534,15 +557,6 @@ __device__ __forceinline__ void store_weakest(int* hdr, const int* kept, int cou
     }
 }
 
-// after decode_index_kernel has written the kept indices of the first N keys: count and weakest key
-__global__ void __launch_bounds__(256) decode_state_init_kernel(const float* __restrict__ delta, int64_t ld, int keep, int w_cap,
-                                                                int* __restrict__ state) {
-    const int bh = blockIdx.x;
-    int* hdr = state + (size_t)bh * state_stride(w_cap);
-    if (threadIdx.x == 0) hdr[0] = keep;
-    store_weakest(hdr, hdr + kStateHeader, keep, delta + (size_t)bh * ld, -1, 0);
-}
-
 // brings a row's state up to date with the appended key N - 1 (every thread of the CTA takes part)
 __device__ __forceinline__ void decode_state_update(const float* __restrict__ delta, int64_t ld, int N, int w_cap,
                                                     int* __restrict__ state, int bh) {
@@ -570,7 +584,7 @@ __device__ __forceinline__ void decode_state_update(const float* __restrict__ de
 // attention over the row's kept list as it is AFTER the appended key N - 1 is taken into account (the stored state still
 // describes the first N - 1 keys; decode_state_update_kernel brings it up to date afterwards)
 template <typename T, int D>
-__global__ void __launch_bounds__(kAttnThreads) decode_list_attn_kernel(const T* __restrict__ q, const T* __restrict__ K,
+__global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const T* __restrict__ q, const T* __restrict__ K,
                                                                         const T* __restrict__ V, const float* __restrict__ delta,
                                                                         int64_t ld, const int* __restrict__ state, int w_cap,
                                                                         float* __restrict__ partial, int N, int Hq, int G,
@@ -579,6 +593,7 @@ __global__ void __launch_bounds__(kAttnThreads) decode_list_attn_kernel(const T*
     __shared__ int list[kListSplit];
     const int split = blockIdx.x, bh = blockIdx.y, b = bh / Hq, h = bh % Hq, hk = h / G;
     const int tid = threadIdx.x;
+    pdl_enter(q, K, V, delta, state, partial);
     const float* dl = delta + (size_t)bh * ld;
     const int* hdr = state + (size_t)bh * state_stride(w_cap);
     const int* kept = hdr + kStateHeader;
@@ -603,6 +618,7 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
                                                                     int N, int w_cap, int* __restrict__ state) {
     __shared__ float s_m[8], s_l[8], s_o[8][D];
     const int bh = blockIdx.x, c = threadIdx.x % D, g = threadIdx.x / D;     // group g takes the splits s = g, g + 8, ...
+    pdl_enter(partial, o, lse, delta, state);
     const float* p = partial + (size_t)bh * nsplit * (D + 2);
     float mx = -INFINITY;
     for (int s = g; s < nsplit; s += 8) mx = fmaxf(mx, p[(size_t)s * (D + 2) + D]);
@@ -637,42 +653,48 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
 
 
 
+// Splits of a row's kept list: few enough that all CTAs are resident at once (two per SM), which matters when a step is
+// short, but no longer than kMaxSplit keys, so that a large batch still comes in waves that balance.
+int split_keys(const Prob& P) {
+    const int64_t bh = (int64_t)P.B * P.Hq;
+    int per = kMinSplit;
+    while (per < kMaxSplit && bh * ((P.w + per - 1) / per) > 2 * 148) per += kMinSplit;
+    return per;
+}
+
 template <typename T, int D>
 int launch_typed(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, void* o, float* lse,
-                 const unsigned long long* thr, int* tickets, float* partial, int nsplit, cudaStream_t st) {
-    decode_attn_kernel<T, D><<<dim3(nsplit, P.B * P.Hq), kAttnThreads, 0, st>>>(
-        (const T*)q, (const T*)K, (const T*)V, delta, ld, thr, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, nsplit, P.ks[0],
-        P.ks[1], P.ks[2], P.vs[0], P.vs[1], P.vs[2], tickets, (T*)o, lse);
+                 const int* kept, int64_t kept_stride, int* tickets, float* partial, cudaStream_t st) {
+    const int per = split_keys(P), nsplit = (P.w + per - 1) / per;
+    if (launch_overlapped(decode_attn_kernel<T, D>, dim3(nsplit, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
+                          delta, ld, kept, kept_stride, partial, P.w, per, P.Hq, P.G, P.scale * 1.4426950408889634f, nsplit, P.ks[0], P.ks[1],
+                          P.ks[2], P.vs[0], P.vs[1], P.vs[2], tickets, (T*)o, lse) != cudaSuccess)
+        return DMA_ERR_CUDA;
     count_launch();
     return check_launch();
 }
 
 }  // namespace
 
-static int decode_splits(const Prob& P) { return (P.L + kSplitKeys - 1) / kSplitKeys; }
-
-static size_t decode_hist_bytes(const Prob& P) { return (size_t)3 * P.B * P.Hq * 2048 * sizeof(int); }
-
 static int list_splits(const Prob& P) { return (P.w_cap + kListSplit - 1) / kListSplit; }
 
-// header | thresholds | tickets | histograms | partials of the larger of the two attention kernels' split counts
+// header | tickets | kept lists | partials of the larger of the two attention kernels' split counts
 struct DecodeWs {
-    unsigned long long* thr;
     int* tickets;
-    int* ghist;
+    int* kept;
     float* partial;
     size_t bytes;
 };
 static DecodeWs decode_ws(const Prob& P, void* ws) {
     const size_t bh = (size_t)P.B * P.Hq;
-    const size_t splits = (size_t)(decode_splits(P) > list_splits(P) ? decode_splits(P) : list_splits(P));
+    const int per = split_keys(P), ns = (P.w + per - 1) / per;
+    const size_t splits = (size_t)(ns > list_splits(P) ? ns : list_splits(P));
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     DecodeWs w;
     size_t off = kWsHeaderBytes;
     char* base = (char*)ws;
-    w.thr = reinterpret_cast<unsigned long long*>(base + off); off += up(bh * sizeof(unsigned long long));
     w.tickets = reinterpret_cast<int*>(base + off); off += up(bh * sizeof(int));
-    w.ghist = reinterpret_cast<int*>(base + off); off += decode_hist_bytes(P);
+    w.kept = reinterpret_cast<int*>(base + off); off += up(bh * P.w * sizeof(int));
     w.partial = reinterpret_cast<float*>(base + off); off += bh * splits * (P.d + 2) * sizeof(float);
     w.bytes = off;
     return w;
@@ -687,72 +709,57 @@ size_t decode_state_bytes(const Prob& P) {
     return (size_t)P.B * P.Hq * (kStateHeader + ((P.w_cap + 3) & ~3)) * sizeof(int);
 }
 
-// The selection (threshold key per row, tickets zeroed): rows that fit in shared memory are selected by one CTA each in one
-// launch; longer rows by the histogram passes spread over CTAs of 8192 keys (a memset and four launches).
-static int launch_select(const Prob& P, const float* delta, int64_t ld, const DecodeWs& W, cudaStream_t st) {
-    const int BH = P.B * P.Hq, nslices = (P.L + kSliceKeys - 1) / kSliceKeys;
-    if (P.L <= kRowSelectMax) {
-        const size_t smem = (size_t)P.L * sizeof(uint32_t);
-        if (cudaFuncSetAttribute(decode_row_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRowSelectMax * sizeof(uint32_t))) != cudaSuccess)
-            return DMA_ERR_CUDA;
-        decode_row_select_kernel<<<(unsigned)BH, kRowSelectThreads, smem, st>>>(delta, ld, P.L, P.w, W.thr, W.tickets);
-        count_launch();
-        return check_launch();
-    }
-    // tickets and histograms are adjacent: one memset
-    const size_t zero_bytes = (size_t)((char*)W.ghist - (char*)W.tickets) + (P.w < P.L ? decode_hist_bytes(P) : 0);
-    if (cudaMemsetAsync(W.tickets, 0, zero_bytes, st) != cudaSuccess) return DMA_ERR_CUDA;
-    if (P.w < P.L) {
-        const dim3 grid(nslices, (unsigned)BH);
-        for (int pass = 0; pass < 3; ++pass)
-            decode_hist_kernel<<<grid, 256, 0, st>>>(delta, ld, P.L, P.w, pass, W.ghist, BH);
-        count_launch(3);
-    }
-    decode_thr_kernel<<<(unsigned)BH, 256, 0, st>>>(delta, ld, P.L, P.w, W.ghist, BH, W.thr);
+// The selection: kept indices of every row, ascending, to list (rows list_stride entries apart). `state`: list points into
+// an incremental state, whose row headers are written too.
+static int launch_select(const Prob& P, const float* delta, int64_t ld, int* list, int64_t list_stride, int* tickets, bool state, cudaStream_t st) {
+    int nrank = 1;
+    // the fewest CTAs whose registers hold a row; a row that needs a cluster gets more while all rows still run at once
+    while (nrank < kSelectMaxCluster && ((int64_t)nrank * kCtaKeys < P.L || (nrank > 1 && 2ll * nrank * P.B * P.Hq <= 148))) nrank *= 2;
+    const int slice = ((P.L + nrank - 1) / nrank + 31) / 32 * 32;
+    auto pick = [&](auto st_tag) {
+        constexpr bool kState = decltype(st_tag)::value;
+        return slice <= 4 * kSelectThreads ? decode_select_kernel<4, kState> : slice <= 16 * kSelectThreads ? decode_select_kernel<16, kState>
+               : slice <= kCtaKeys ? decode_select_kernel<32, kState> : decode_select_kernel<0, kState>;
+    };
+    auto kern = state ? pick(std::true_type{}) : pick(std::false_type{});
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelectShared)) != cudaSuccess) return DMA_ERR_CUDA;
+    if (launch_overlapped(kern, dim3((unsigned)(P.B * P.Hq) * nrank), dim3(kSelectThreads), sizeof(SelectShared), st, nrank, delta, ld, P.L, P.w,
+                          slice, list, list_stride, tickets) != cudaSuccess)
+        return DMA_ERR_CUDA;
     count_launch();
     return check_launch();
 }
 
 int launch_decode(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, void* o, float* lse,
                   int32_t* sel_idx, void* ws, cudaStream_t st) {
-    const size_t bh = (size_t)P.B * P.Hq;
     const DecodeWs W = decode_ws(P, ws);
-    int rc = launch_select(P, delta, ld, W, st);
+    int* kept = sel_idx ? sel_idx : W.kept;              // the caller's index output is the list the attention kernel reads
+    int rc = launch_select(P, delta, ld, kept, P.w, W.tickets, false, st);
     if (rc) return rc;
-    if (sel_idx) {
-        decode_index_kernel<<<(unsigned)bh, 256, 0, st>>>(delta, ld, P.L, P.w, W.thr, sel_idx, P.w);
-        count_launch();
-    }
-    const int ns = decode_splits(P);
     if (P.dtype == DMA_BF16)
-        return P.d == 128 ? launch_typed<__nv_bfloat16, 128>(P, q, K, V, delta, ld, o, lse, W.thr, W.tickets, W.partial, ns, st)
-                          : launch_typed<__nv_bfloat16, 64>(P, q, K, V, delta, ld, o, lse, W.thr, W.tickets, W.partial, ns, st);
-    return P.d == 128 ? launch_typed<float, 128>(P, q, K, V, delta, ld, o, lse, W.thr, W.tickets, W.partial, ns, st)
-                      : launch_typed<float, 64>(P, q, K, V, delta, ld, o, lse, W.thr, W.tickets, W.partial, ns, st);
+        return P.d == 128 ? launch_typed<__nv_bfloat16, 128>(P, q, K, V, delta, ld, o, lse, kept, P.w, W.tickets, W.partial, st)
+                          : launch_typed<__nv_bfloat16, 64>(P, q, K, V, delta, ld, o, lse, kept, P.w, W.tickets, W.partial, st);
+    return P.d == 128 ? launch_typed<float, 128>(P, q, K, V, delta, ld, o, lse, kept, P.w, W.tickets, W.partial, st)
+                      : launch_typed<float, 64>(P, q, K, V, delta, ld, o, lse, kept, P.w, W.tickets, W.partial, st);
 }
 
-// Builds the incremental state from the first N = P.L cached keys: the selection, the kept indices into the state's
-// lists, then count and weakest key.
+// Builds the incremental state from the first N = P.L cached keys: the selection writes lists and headers in place.
 int launch_decode_state_init(const Prob& P, const float* delta, int64_t ld, int* state, void* ws, cudaStream_t st) {
-    const size_t bh = (size_t)P.B * P.Hq;
-    const DecodeWs W = decode_ws(P, ws);
-    int rc = launch_select(P, delta, ld, W, st);
-    if (rc) return rc;
+    (void)ws;
     const int stride = kStateHeader + ((P.w_cap + 3) & ~3);
-    decode_index_kernel<<<(unsigned)bh, 256, 0, st>>>(delta, ld, P.L, P.w, W.thr, state + kStateHeader, stride);
-    decode_state_init_kernel<<<(unsigned)bh, 256, 0, st>>>(delta, ld, P.w, P.w_cap, state);
-    count_launch(2);
-    return check_launch();
+    return launch_select(P, delta, ld, state + kStateHeader, stride, nullptr, true, st);
 }
 
 template <typename T, int D>
 static int launch_step_typed(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, int* state,
                              void* o, float* lse, float* partial, cudaStream_t st) {
     const int ns = list_splits(P);
-    decode_list_attn_kernel<T, D><<<dim3(ns, P.B * P.Hq), kAttnThreads, 0, st>>>(
-        (const T*)q, (const T*)K, (const T*)V, delta, ld, state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns,
-        P.ks[0], P.ks[1], P.ks[2], P.vs[0], P.vs[1], P.vs[2]);
-    decode_step_combine_kernel<T, D><<<P.B * P.Hq, 8 * D, 0, st>>>(partial, (T*)o, lse, ns, delta, ld, P.L, P.w_cap, state);
+    if (launch_overlapped(decode_list_attn_kernel<T, D>, dim3(ns, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
+                          delta, ld, (const int*)state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns, P.ks[0], P.ks[1],
+                          P.ks[2], P.vs[0], P.vs[1], P.vs[2]) != cudaSuccess ||
+        launch_overlapped(decode_step_combine_kernel<T, D>, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
+                          ld, P.L, P.w_cap, state) != cudaSuccess)
+        return DMA_ERR_CUDA;
     count_launch(2);
     return check_launch();
 }

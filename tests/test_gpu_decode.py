@@ -64,3 +64,27 @@ def test_ties_go_to_the_lower_index():
 def test_long_cache_config5_shapes():
     # the paper's decode setting on the long-context shapes: 65 536 cached keys, w = 4096, 32 / 8 heads
     run_case(wl.CONFIGS["5"], cap_extra=128)
+
+
+@pytest.mark.parametrize("N,w", [(1, 1), (33, 7), (4096, 512), (4097, 4096), (16384, 2048), (16385, 1), (32768, 8192), (32769, 100),
+                                 (65537, 4096), (262144, 1000), (262177, 20000)])
+@pytest.mark.parametrize("kind", ["random", "tied", "few", "ramp", "outlier"])
+def test_selection_at_the_edges_of_the_register_and_cluster_sizes(N, w, kind):
+    """The kept indices (ascending) against a stable sort, at the row lengths where the selection kernel changes shape, for rows
+    whose threshold takes one pass, several passes over ever narrower ranges (few distinct values, one value far above the
+    others) or a cut among equal keys."""
+    g = torch.Generator().manual_seed(N + w)
+    BH = 3
+    z = torch.randn(1, BH, N, generator=g)
+    delta = {"random": lambda: torch.exp(torch.nn.functional.softplus(z)), "tied": lambda: torch.full((1, BH, N), 1.5),
+             "few": lambda: 1.0 + torch.randint(0, 4, (1, BH, N), generator=g) / 7.0,
+             "ramp": lambda: torch.exp(3.0 * torch.arange(N) / N).expand(1, BH, N).contiguous(),
+             "outlier": lambda: torch.where(torch.rand(1, BH, N, generator=g) < 2.0 / N, 1e38, 1.0 + 1e-3 * torch.rand(1, BH, N, generator=g))}[kind]()
+    p = dma.problem(1, BH, 1, N, 64, w)
+    K = torch.randn(1, N, 1, 64, generator=g).bfloat16().cuda()
+    q = torch.zeros(1, BH, 64, dtype=torch.bfloat16, device="cuda")
+    _, _, idx = dma.dma_decode(p, q, K, K, delta.cuda(), want_idx=True)
+    want = torch.sort(torch.sort(delta, dim=-1, descending=True, stable=True)[1][..., :min(w, N)], dim=-1)[0]
+    assert torch.equal(idx.cpu().long(), want)
+    state = dma.dma_decode_state_init(p, delta.cuda(), dma.dma_decode_state(p, "cuda"))
+    assert dma.decode_state_sets(state, w) == [r.tolist() for r in want[0]]
