@@ -462,3 +462,19 @@ def test_compact_backward_full_size_sampled(key):
     inp = wl.make_inputs(case)
     ref = Samples(case, inp)
     ref.check(gpu_run(case, inp, stored=ref.stored, flags=dma.DMA_FLAG_COMPACT_KV), "compact ")
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,d,w", [(1, 1, 1, 7, 64, 3), (1, 2, 1, 9, 128, 9), (1, 3, 1, 64, 64, 20), (1, 1, 1, 65, 128, 1),
+                                            (1, 2, 2, 129, 64, 200), (8, 20, 20, 33, 64, 10), (8, 20, 10, 40, 128, 40), (4, 16, 2, 97, 64, 31)])
+def test_cuda_core_kernels_at_the_edges_of_their_tiles(B, Hq, Hkv, L, d, w):
+    """fp32, 8-row CTAs (small grids) and 32-row CTAs: lengths around the warps' rows and the 64-row streamed tiles; causal against
+    the oracle, and every gradient the same bits from run to run."""
+    case = wl.small(C1, B=B, Hq=Hq, Hkv=Hkv, L=L, d=d, w=w, seed=L + d, name="edge")
+    inp = wl.make_inputs(case)
+    dl, e, bmp = oracle_mask(case, inp)
+    ref = oracle_all(case, inp, dl, e)
+    st = stored_forward(case, ref["O"], ref["lse"])
+    got = gpu_run(case, inp, stored=st)
+    compare(case, got, ref)
+    again = gpu_run(case, inp, stored=st)
+    assert all(torch.equal(got[k], again[k]) for k in ("O", "lse", "dQ", "dK", "dV", "dM"))
