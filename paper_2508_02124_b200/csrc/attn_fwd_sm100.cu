@@ -48,6 +48,9 @@ struct SharedStorage {
     // unswizzled K-major core matrices (row r, element e at (r/8) 256 + (e/8) 128 + (r%8) 16 + (e%8) 2 bytes). The
     // product adds bias / scale to the score, -BIG for keys that expired before the tile's rows, and -BIG from row
     // expiry[j_k] on for the up to 13 keys j_k that expire inside the tile's rows (t_k(r) = 1 from that row on).
+    // Token-compacted mode: the A rows are constant and elements 8-15 of every row zero, so the same 16 KB hold, in blocks of
+    // 2 KB (128 rows x 16 bytes): ones | B of stage 0, tile 0 | stage 0, tile 1 | stage 1, tile 0 | stage 1, tile 1 | zeros
+    // (the descriptors' second core matrix is the block of zeros), and the stager runs a whole slice ahead of the S products.
     alignas(128) uint8_t aext[2][4096];
     alignas(128) uint8_t bext[2][4096];
     alignas(16) int len[kStages][128];        // expiry[j] (0 beyond L): row i keeps key j iff j <= i < expiry[j]
@@ -426,14 +429,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // vectors, and the mask of 32-column chunks that hold a key expiring or entering inside the tile's rows (only
             // those need the per-element test). Two dependent levels of global loads, each issued a tile ahead.
             constexpr uint32_t kOne = 0x3F80u, kNegBig = 0xF14Au;     // bf16 1.0 and about -1e30
+            uint8_t* ext = &S.aext[0][0];
             for (int r = lane; r < 128; r += 32) {
-#pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    uint8_t* arow = S.aext[w] + (r >> 3) * 256 + (r & 7) * 16;
-                    *reinterpret_cast<uint4*>(arow) = make_uint4(kOne | (kOne << 16), kOne, 0u, 0u);
-                    *reinterpret_cast<uint4*>(arow + 128) = make_uint4(0u, 0u, 0u, 0u);
-                    *reinterpret_cast<uint4*>(S.bext[w] + (r >> 3) * 256 + (r & 7) * 16 + 128) = make_uint4(0u, 0u, 0u, 0u);
-                }
+                *reinterpret_cast<uint4*>(ext + r * 16) = make_uint4(kOne | (kOne << 16), kOne, 0u, 0u);
+                *reinterpret_cast<uint4*>(ext + 5 * 2048 + r * 16) = make_uint4(0u, 0u, 0u, 0u);
             }
             const int* list = P.cidx + ((size_t)bh * npairs + lpair) * P.ccap;
             auto vals = [&](const int (&jv)[4], float (&bv)[4], int (&ev)[4]) {
@@ -489,10 +488,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         }
                     }
                 }
-                // the vectors of this stage were last read by the softmax groups before they released P of tile
-                // it - kStages (hence before its P V); the B rows were last read by the S products of tile it - 1
+                // what this stage holds was last read by the softmax groups before they released P of slice it - kStages,
+                // hence before its P V, and by that slice's S products, which were issued before that P V
                 if (it >= kStages) ok = mbar_wait_warp(&S.v_empty[st], ((it / kStages) - 1) & 1, abort_flag);
-                if (ok && it >= 1) ok = mbar_wait_warp(&S.k_empty[(it - 1) % kStages], ((it - 1) / kStages) & 1, abort_flag);
                 if (!ok) break;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -501,7 +499,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     S.len[st][c] = ev[t];
 #pragma unroll
                     for (int w = 0; w < 2; ++w)
-                        *reinterpret_cast<uint4*>(S.bext[w] + (c >> 3) * 256 + (c & 7) * 16) =
+                        *reinterpret_cast<uint4*>(ext + (1 + st * 2 + w) * 2048 + c * 16) =
                             make_uint4(b0[w][t], b0[w][t] == kNegBig ? 0u : b1[t], 0u, 0u);
                     jv[t] = jn[t]; bv[t] = bn[t]; ev[t] = en[t]; jn[t] = jnn[t];
                 }
@@ -691,6 +689,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const uint64_t dQ0 = smem_desc_sw128(smem_u32(S.q[0]), 16, 1024), dK0 = smem_desc_sw128(smem_u32(S.k[0]), 16, 1024);
             const uint64_t dV0 = smem_desc_sw128(smem_u32(S.v[0]), kTileBytes / 2, 1024);
             const uint64_t dA0 = smem_desc_plain(smem_u32(S.aext[0]), 128, 256), dB0 = smem_desc_plain(smem_u32(S.bext[0]), 128, 256);
+            // token-compacted mode: the second core matrix of every operand is the block of zeros, five blocks behind the ones
+            const uint64_t dOnes = smem_desc_plain(smem_u32(S.aext[0]), 5 * 2048, 128);
+            const uint64_t dRows = smem_desc_plain(smem_u32(S.aext[0]) + 2048, 4 * 2048, 128);      // stage 0, tile 0
+            constexpr uint64_t kNextBlock = (uint64_t)(2048 >> 4) - ((uint64_t)(2048 >> 4) << 16);  // one block on, one less to the zeros
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             const int n_iters_u = __shfl_sync(0xffffffffu, n_iters, 0);
             // MMA-block skipping (the finer granularity inside an active tile): the stager marks the 16-key blocks of the key
@@ -709,7 +711,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         const uint32_t off = ((kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32) >> 4;
                         mma_ss(d_tmem, dq + off, dk + off, idesc_s, kk > 0);
                     }
-                    mma_ss(d_tmem, dA0 + (uint64_t)(w * (4096 >> 4)), dB0 + (uint64_t)(w * (4096 >> 4)), idesc_s, 1u);
+                    if constexpr (kCompact) mma_ss(d_tmem, dOnes, dRows + kNextBlock * (uint64_t)(st * 2 + w), idesc_s, 1u);
+                    else mma_ss(d_tmem, dA0 + (uint64_t)(w * (4096 >> 4)), dB0 + (uint64_t)(w * (4096 >> 4)), idesc_s, 1u);
                     tc_commit(&S.s_full[w]);
                 }
                 __syncwarp();
@@ -717,6 +720,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 // costs hundreds of cycles while the MMAs stream their operands, and the S products are on the critical path)
                 if constexpr (kBlockSkip) live[w] = *reinterpret_cast<volatile uint32_t*>(&S.fast[st][w]) >> 8;     // (every lane reads the same word; first used at the P V issue)
             };
+            const uint32_t both = (1u << 30) | (has1 ? (1u << 31) : 0u);     // token-compacted mode: every slice serves both tiles
             int n_p[2] = {0, 0};
             bool ok = mbar_wait_warp(&S.q_full, 0, abort_flag);
             if (ok && n_iters_u > 0) {
@@ -727,15 +731,21 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     const uint32_t e0 = __shfl_sync(0xffffffffu, S.sched[0], 0);
 #pragma unroll
                     for (int w = 0; w < 2; ++w)
-                        if (use_bit(e0, w)) issue_s(w, 0);
+                        if (ok && use_bit(e0, w)) {
+                            // token-compacted mode: the second tile starts half a slice after the first. Started together, the
+                            // two softmax groups stay in step: they contend for the issue slots and then wait for the MMAs
+                            // together (L = 16384, w = 2048: 694 -> 680 us; 700 before the stager ran ahead)
+                            if (kCompact && w == 1) ok = mbar_wait_warp(&S.p_half[0], 0, abort_flag);
+                            if (ok) issue_s(w, 0);
+                        }
                     if (elect_one()) tc_commit(&S.k_empty[0]);
                     __syncwarp();
                 }
             }
             for (int it = 0; it < n_iters_u && ok; ++it) {
                 const int st = it % kStages, nst = (it + 1) % kStages;
-                const uint32_t entry = __shfl_sync(0xffffffffu, S.sched[it], 0);
-                const uint32_t next = it + 1 < n_iters_u ? __shfl_sync(0xffffffffu, S.sched[it + 1], 0) : 0u;
+                const uint32_t entry = kCompact ? both : __shfl_sync(0xffffffffu, S.sched[it], 0);
+                const uint32_t next = it + 1 >= n_iters_u ? 0u : kCompact ? both : __shfl_sync(0xffffffffu, S.sched[it + 1], 0);
                 ok = mbar_wait_warp(&S.v_full[st], (it / kStages) & 1, abort_flag);
                 if constexpr (kCompact) fence_proxy_async();     // the gathered tiles were written through the generic proxy
                 bool k_ready = false;
