@@ -94,7 +94,9 @@ struct BwdParams {
     float* dKacc;               // fp32 [B, L, Hkv, 128] accumulators (several query heads add into one KV head's rows)
     float* dVacc;
     int64_t acc_slot;           // 0: the group's heads add into one accumulator with atomics; else: elements between the
-                                // per-head slots [G][B, L, Hkv, 128], written with plain stores and summed in head order afterwards
+                                // slots [slot][B, L, Hkv, d] (one per query head of the group, or per split of the group in tile
+                                // mode), written with plain stores and summed in slot order afterwards
+    int nsplit;                 // tile mode: CTAs that share a KV head's query heads, G / nsplit each (1: dK, dV are written directly)
     int64_t ks_b, ks_l, ks_h, vs_b, vs_l, vs_h;
 };
 
@@ -122,16 +124,18 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     constexpr bool kDouble = kD == 64;               // P^T / dS^T in two buffers used in turn (see the file header)
     extern __shared__ uint8_t smem_raw[];
     SharedStorage& S = *reinterpret_cast<SharedStorage*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // warp-uniform to the compiler: role branches stay uniform
-    // tile mode: blockIdx.x = (batch, KV head); token-compacted mode: (batch, query head), whose group index is fixed
+    // tile mode: blockIdx.x = (batch, KV head, split of its query heads); token-compacted mode: (batch, query head), whose group index is fixed
     // CTAs start in the order of lin: heads of one scheduling group (P.sched_group of them) innermost, then key tiles (key
     // tile 0 has the most query tiles: heaviest first), then the groups
     const int lin = blockIdx.y * gridDim.x + blockIdx.x, per_group = P.sched_group * (int)gridDim.y;
     const int bx = (lin / per_group) * P.sched_group + (lin % per_group) % P.sched_group;
-    const int b = bx / (kCompact ? P.Hq : P.Hkv);
+    const int nsplit = kCompact ? 1 : P.nsplit, sp = kCompact ? 0 : bx % nsplit;
+    const int b = kCompact ? bx / P.Hq : bx / (nsplit * P.Hkv);
     const int hq_c = bx % P.Hq;                        // token-compacted mode only
-    const int hk = kCompact ? hq_c / P.G : bx % P.Hkv;
+    const int hk = kCompact ? hq_c / P.G : bx / nsplit % P.Hkv;
     const int kt = (lin % per_group) / P.sched_group;
     const int j0 = kt * 128;
     const int* my_perm = kCompact ? P.perm + ((size_t)bx * P.Tc + kt) * 128 : nullptr;
@@ -200,7 +204,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 }
             }
         } else {
-        for (int g = 0; g < P.G; ++g) {
+        const int gper = P.G / nsplit;                     // this CTA's query heads of the group
+        for (int g = sp * gper; g < (sp + 1) * gper; ++g) {
             const int bh = b * P.Hq + hk * P.G + g;
             for (int base = kt; base < P.Tr; base += 32) {
                 const int qt = base + lane;
@@ -348,8 +353,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             tc_fence_after();
             __nv_bfloat16* dk = P.dK + b * P.ks_b + (int64_t)j * P.ks_l + hk * P.ks_h;
             __nv_bfloat16* dv = P.dV + b * P.vs_b + (int64_t)j * P.vs_l + hk * P.vs_h;
-            const size_t arow = ((size_t)(b * P.L + min(j, P.L - 1)) * P.Hkv + hk) * kD +      // accumulator row (compact mode)
-                                (kCompact ? (size_t)(hq_c % P.G) * (size_t)P.acc_slot : 0);
+            const size_t arow = ((size_t)(b * P.L + min(j, P.L - 1)) * P.Hkv + hk) * kD +      // accumulator row
+                                (size_t)(kCompact ? hq_c % P.G : sp) * (size_t)P.acc_slot;
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
                 const float mul = which == 0 ? P.scale : 1.0f;
@@ -380,6 +385,14 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                     red_add_v4(acc + c * 32 + u, __uint_as_float(o[u]), __uint_as_float(o[u + 1]), __uint_as_float(o[u + 2]),
                                                __uint_as_float(o[u + 3]));
                             }
+                        }
+                    } else if (nsplit > 1) {
+                        // this split's part of the group sum (unscaled; zeros where it had nothing to add), to its own slot
+                        if (j < P.L) {
+#pragma unroll
+                            for (int u = 0; u < 32; u += 4)
+                                *reinterpret_cast<float4*>(acc + c * 32 + u) = make_float4(__uint_as_float(o[u]), __uint_as_float(o[u + 1]),
+                                                                                          __uint_as_float(o[u + 2]), __uint_as_float(o[u + 3]));
                         }
                     } else if (j < P.L) {
 #pragma unroll
@@ -611,66 +624,117 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     if (tid == 0 && S.abort_flag) atomicExch(P.status, (int32_t)DMA_ERR_DEVICE_TIMEOUT);
 }
 
-// D_i = dO_i . O_i  (Alg. 2): kLanes = d / 8 lanes per (b, h, i), 16-byte loads (a row of 128 bf16 is 16 x 16 bytes)
+// What the backward needs before its main kernel, in one launch: D_i = dO_i . O_i (Alg. 2; kLanes = d / 8 lanes per (b, h, i),
+// 16-byte loads) and zeros in the accumulators that are added to. HBM-bound (at L = 16384 with 32 / 8 heads of 128 channels
+// 268 MB read, 405 MB written); the CTAs' parts of the zeros are as large as their parts of the rows, so that loads and
+// stores are in flight together, and a short problem has one launch instead of four.
+struct PrepareParams {
+    const __nv_bfloat16* O;
+    const __nv_bfloat16* dO;
+    float* Dv;
+    int B, L, Hq;
+    int64_t os_b, os_l, os_h;
+    float* zero[3];             // accumulator of dQ, dM, accumulators of dK and dV: 16-byte aligned
+    int64_t zero_n[3];          // floats
+    int64_t zero_part[3];       // 16-byte chunks per CTA
+    int32_t* status;            // the workspace header
+};
+constexpr int kPrepareRows = 4;     // rows per lane group
+
 template <int kLanes>
-__global__ void rowdot_bf16_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
-                                   float* __restrict__ Dv, int B, int L, int Hq, int64_t os_b, int64_t os_l, int64_t os_h) {
-    const long row = (long)blockIdx.x * (blockDim.x / kLanes) + threadIdx.x / kLanes;
-    const int sub = threadIdx.x % kLanes;
-    float s = 0.0f;
-    if (row < (long)B * Hq * L) {
-        const int i = row % L, h = (row / L) % Hq, b = row / ((long)L * Hq);
-        const int64_t off = b * os_b + (int64_t)i * os_l + h * os_h + sub * 8;
-        const uint4 a = *reinterpret_cast<const uint4*>(O + off), g = *reinterpret_cast<const uint4*>(dO + off);
-        const uint32_t au[4] = {a.x, a.y, a.z, a.w}, gu[4] = {g.x, g.y, g.z, g.w};
+__global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepareParams P) {
+    pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x < kWsHeaderBytes / 4) P.status[threadIdx.x] = 0;
+    const int sub = threadIdx.x % kLanes, per_cta = 256 / kLanes;
+    const uint32_t rows = (uint32_t)P.B * P.Hq * P.L, r0 = blockIdx.x * per_cta * kPrepareRows + threadIdx.x / kLanes;
+    uint4 a[kPrepareRows], g[kPrepareRows];
+#pragma unroll
+    for (int n = 0; n < kPrepareRows; ++n) {
+        const uint32_t row = min(r0 + n * per_cta, rows - 1), bh = row / (uint32_t)P.L;
+        const int i = (int)(row - bh * P.L), h = (int)(bh % (uint32_t)P.Hq), b = (int)(bh / (uint32_t)P.Hq);
+        const int64_t off = b * P.os_b + (int64_t)i * P.os_l + h * P.os_h + sub * 8;
+        a[n] = *reinterpret_cast<const uint4*>(P.O + off);
+        g[n] = *reinterpret_cast<const uint4*>(P.dO + off);
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        const int64_t n4 = P.zero_n[z] >> 2, e0 = P.zero_part[z] * blockIdx.x, e1 = min(n4, e0 + P.zero_part[z]);
+        float4* dst = reinterpret_cast<float4*>(P.zero[z]);
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) dst[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (blockIdx.x == 0 && threadIdx.x < (P.zero_n[z] & 3)) P.zero[z][4 * n4 + threadIdx.x] = 0.0f;
+    }
+#pragma unroll
+    for (int n = 0; n < kPrepareRows; ++n) {
+        const uint32_t au[4] = {a[n].x, a[n].y, a[n].z, a[n].w}, gu[4] = {g[n].x, g[n].y, g[n].z, g[n].w};
+        float s = 0.0f;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             s = fmaf(__uint_as_float(au[t] << 16), __uint_as_float(gu[t] << 16), s);
             s = fmaf(__uint_as_float(au[t] & 0xffff0000u), __uint_as_float(gu[t] & 0xffff0000u), s);
         }
+        for (int m = kLanes / 2; m; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        const uint32_t row = r0 + n * per_cta;
+        if (sub == 0 && row < rows) P.Dv[row] = s;
     }
-    for (int m = kLanes / 2; m; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-    if (sub == 0 && row < (long)B * Hq * L) Dv[row] = s;
 }
 
-// fp32 accumulator [B, L, Hq, d] (unscaled dS K sums) -> softmax scale applied -> bf16 dQ in the caller's layout; 8 elements per thread.
-// nslots > 1: the accumulator is nslots copies, slot_stride elements apart, added here in slot order (a fixed order: the
-// result is then the same bits from run to run).
-__global__ void dq_convert_bf16_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dQ, size_t n8, int L, int Hq,
-                                       int64_t qs_b, int64_t qs_l, int64_t qs_h, float scale, int d, int nslots = 1, int64_t slot_stride = 0) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n8) return;
-    const size_t e = t * 8;
-    const int c = e % d, h = (e / d) % Hq, i = (e / ((size_t)d * Hq)) % L, b = e / ((size_t)d * Hq * L);
+// After the main kernel, in one launch (HBM-bound): the first q_blocks CTAs turn the blocked fp32 dQ accumulator (see
+// BwdParams::dQacc) into bf16 dQ in the caller's layout, softmax scale applied; the others the fp32 dK, dV accumulators
+// [B, L, Hkv, d] where the main kernel did not write dK, dV itself.
+//   dQ: one CTA per (batch, head, 16-row block, or two of them at d = 64); a thread takes two neighbouring channels (they share
+//   their chunk position) and four rows: two 16-byte loads, four 4-byte stores that the lanes of a warp, consecutive channel
+//   pairs, make whole 128-byte lines of.
+//   dK, dV: 8 elements per thread. nslots > 1: the accumulator is nslots copies, slot_stride elements apart, added in slot
+//   order (a fixed order: the result is then the same bits from run to run).
+struct FinishParams {
+    const float* dQacc;
+    const float* acc[2];        // of dK, dV
+    __nv_bfloat16* dQ;
+    __nv_bfloat16* out[2];
+    int q_blocks, kv_blocks;    // CTAs of dQ, of each of dK and dV
+    int L, Hq, Hkv, Lblk, d, nslots;
+    int64_t nkv;                // elements of dK
+    uint32_t q_rows16;          // 16-row blocks of dQ in all
+    int64_t qs[3], st[2][3];
+    float scale;
+};
+
+__global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
+    pdl_enter();
+    if ((int)blockIdx.x < P.q_blocks) {
+        const int per = P.d * 2, t = threadIdx.x % per;                    // threads per 16-row block
+        const uint32_t blk = blockIdx.x * (256 / per) + threadIdx.x / per;
+        if (blk >= P.q_rows16) return;
+        const int bh = (int)(blk / (uint32_t)P.Lblk), rb = (int)(blk - (uint32_t)bh * P.Lblk), h = bh % P.Hq, b = bh / P.Hq;
+        const int pairs = P.d >> 1, c = 2 * (t % pairs), q = t / pairs;    // channel pair, quad of rows
+        const int cc = c & 31;
+        const float* src = P.dQacc + (size_t)blk * P.d * 16 + (c >> 5) * 512 + cc * 16 + ((q ^ ((cc >> 1) & 3)) << 2);
+        const float4 x = *reinterpret_cast<const float4*>(src), y = *reinterpret_cast<const float4*>(src + 16);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+        __nv_bfloat16* out = P.dQ + b * P.qs[0] + h * P.qs[2] + c;
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+            const int i = rb * 16 + 4 * q + rr;
+            if (i < P.L) *reinterpret_cast<uint32_t*>(out + (int64_t)i * P.qs[1]) = ptx::pack_bf16(xs[rr] * P.scale, ys[rr] * P.scale);
+        }
+        return;
+    }
+    const int blk = (int)blockIdx.x - P.q_blocks, which = blk / P.kv_blocks;
+    const int64_t e = ((int64_t)(blk % P.kv_blocks) * 256 + threadIdx.x) * 8;
+    if (e >= P.nkv) return;
+    const float* acc = P.acc[which];
+    const uint32_t row = (uint32_t)(e >> (P.d == 128 ? 7 : 6)), bl = row / (uint32_t)P.Hkv;
+    const int c = (int)(e & (P.d - 1)), h = (int)(row - bl * P.Hkv), b = (int)(bl / (uint32_t)P.L), i = (int)(bl - (uint32_t)b * P.L);
     float4 a = *reinterpret_cast<const float4*>(acc + e), bb = *reinterpret_cast<const float4*>(acc + e + 4);
-    for (int sl = 1; sl < nslots; ++sl) {
-        const float4 a2 = *reinterpret_cast<const float4*>(acc + (size_t)sl * slot_stride + e), b2 = *reinterpret_cast<const float4*>(acc + (size_t)sl * slot_stride + e + 4);
+    for (int sl = 1; sl < P.nslots; ++sl) {
+        const float4 a2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e), b2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e + 4);
         a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w; bb.x += b2.x; bb.y += b2.y; bb.z += b2.z; bb.w += b2.w;
     }
+    const float scale = which == 0 ? P.scale : 1.0f;
     uint4 o;
     o.x = ptx::pack_bf16(a.x * scale, a.y * scale); o.y = ptx::pack_bf16(a.z * scale, a.w * scale);
     o.z = ptx::pack_bf16(bb.x * scale, bb.y * scale); o.w = ptx::pack_bf16(bb.z * scale, bb.w * scale);
-    *reinterpret_cast<uint4*>(dQ + b * qs_b + (int64_t)i * qs_l + h * qs_h + c) = o;
-}
-
-// blocked fp32 dQ accumulator (see BwdParams::dQacc) -> softmax scale applied -> bf16 dQ in the caller's layout. One CTA per
-// (batch, head, 16-row block); a thread takes two neighbouring channels (they share their chunk position) and four rows:
-// two 16-byte loads, four 4-byte stores that the lanes of a warp, consecutive channel pairs, make whole 128-byte lines of.
-__global__ void __launch_bounds__(256) dq_unblock_bf16_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dQ, int L, int Hq,
-                                                              int Lblk, int64_t qs_b, int64_t qs_l, int64_t qs_h, float scale, int d) {
-    const int t = threadIdx.x, rb = blockIdx.x % Lblk, bh = blockIdx.x / Lblk, h = bh % Hq, b = bh / Hq;
-    const int pairs = d >> 1, p = t % pairs, q = t / pairs;            // channel pair, quad of rows
-    if (q >= 4) return;
-    const int c = 2 * p, cc = c & 31;
-    const float* src = acc + ((size_t)bh * Lblk + rb) * (size_t)d * 16 + (c >> 5) * 512 + cc * 16 + ((q ^ ((cc >> 1) & 3)) << 2);
-    const float4 x = *reinterpret_cast<const float4*>(src), y = *reinterpret_cast<const float4*>(src + 16);
-    const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
-    __nv_bfloat16* out = dQ + b * qs_b + h * qs_h + c;
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-        const int i = rb * 16 + 4 * q + rr;
-        if (i < L) *reinterpret_cast<uint32_t*>(out + (int64_t)i * qs_l) = ptx::pack_bf16(xs[rr] * scale, ys[rr] * scale);
-    }
+    *reinterpret_cast<uint4*>(P.out[which] + b * P.st[which][0] + (int64_t)i * P.st[which][1] + h * P.st[which][2] + c) = o;
 }
 
 }  // namespace
@@ -688,6 +752,7 @@ __global__ void __launch_bounds__(1024) lifetime_perm_kernel(const int32_t* __re
     __shared__ int offs[64];                 // next free position of each class
     __shared__ int cnt[32][64];              // per warp and class: keys in this chunk, then their start position
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_enter(expiry, perm);
     const int32_t* e = expiry + (size_t)blockIdx.x * L;
     int* out = perm + (size_t)blockIdx.x * Tc * 128;
     const int band = max(2048, (L + 61) / 62);
@@ -732,11 +797,30 @@ static size_t bwd_rows64(const Prob& P) { return ((((size_t)P.B * P.Hq * P.L) + 
 static size_t bwd_acc_floats(const Prob& P) { return (size_t)P.B * P.Hq * P.Tr * 128 * P.d; }     // rows padded to whole query tiles
 static size_t bwd_perm_ints(const Prob& P) { return (((size_t)P.B * P.Hq * P.Tc * 128) + 63) / 64 * 64; }
 
+// Tile mode: a CTA owns a key tile of one KV head and walks all its query heads. Where that leaves fewer than two CTAs per SM,
+// the group's heads are dealt out to several CTAs, whose parts of dK and dV go to slots of their own: the serial walk of the
+// heaviest CTA (2 G L / 128 steps) is what a short sequence waits for. Two batch entries of 1000 rows, 16 / 4 heads, d = 64:
+// main kernel 68.7 -> 37.5 us with four CTAs per KV head. A divisor of G, so that every (key, query head) keeps one writer of dM.
+int tc_bwd_splits(const Prob& P) {
+    if (P.flags & DMA_FLAG_COMPACT_KV) return 1;
+    if (P.bwd_split) return P.bwd_split;
+    const int64_t ctas = (int64_t)P.B * P.Hkv * P.Tc;
+    int n = 1;
+    while (n < P.G && ctas * n < 2 * 148) {
+        do ++n; while (P.G % n);
+    }
+    return n;
+}
+// copies of the dK, dV accumulators (0: the main kernel writes dK, dV itself)
+static size_t bwd_slots(const Prob& P) {
+    if (P.flags & DMA_FLAG_COMPACT_KV) return (P.flags & DMA_FLAG_DETERMINISTIC) ? (size_t)P.G : 1;
+    return tc_bwd_splits(P) > 1 ? (size_t)tc_bwd_splits(P) : 0;
+}
+
 size_t tc_bwd_ws_bytes(const Prob& P) {
     size_t n = kWsHeaderBytes + (bwd_rows64(P) + bwd_acc_floats(P)) * sizeof(float);
-    const size_t slots = (P.flags & DMA_FLAG_DETERMINISTIC) ? (size_t)P.G : 1;      // per-head dK / dV accumulators
-    if (P.flags & DMA_FLAG_COMPACT_KV) n += bwd_perm_ints(P) * sizeof(int) + 2 * slots * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
-    return n;
+    if (P.flags & DMA_FLAG_COMPACT_KV) n += bwd_perm_ints(P) * sizeof(int);
+    return n + 2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
 }
 
 int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,
@@ -745,12 +829,13 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     const bool compact = (P.flags & DMA_FLAG_COMPACT_KV) != 0;
     if (!P.causal && !compact) return DMA_ERR_UNSUPPORTED;
     if ((size_t)P.G * P.Tr * 2 > (size_t)kMaxSteps || P.G > 16 || P.Tr > 1024) return DMA_ERR_UNSUPPORTED;
-    const size_t rows = (size_t)P.B * P.Hq * P.L, nq = rows * P.d, nkv = (size_t)P.B * P.L * P.Hkv * P.d;
+    const size_t rows = (size_t)P.B * P.Hq * P.L, nkv = (size_t)P.B * P.L * P.Hkv * P.d;
     float* Dv = reinterpret_cast<float*>((char*)ws + kWsHeaderBytes);
     float* acc = Dv + bwd_rows64(P);
     int* perm = reinterpret_cast<int*>(acc + bwd_acc_floats(P));
-    const size_t slots = (compact && (P.flags & DMA_FLAG_DETERMINISTIC)) ? (size_t)P.G : 1;
-    float* accK = reinterpret_cast<float*>(perm + bwd_perm_ints(P));
+    const size_t slots = bwd_slots(P);
+    const int nsplit = tc_bwd_splits(P);
+    float* accK = reinterpret_cast<float*>(perm + (compact ? bwd_perm_ints(P) : 0));
     float* accV = accK + slots * nkv;
     CUtensorMap tmQ, tmK, tmV, tmG;
     int rc;
@@ -758,17 +843,19 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     if ((rc = make_tmap_bf16(&tmG, dO, P.B, P.L, P.Hq, P.d, P.os, 64))) return rc;
     if ((rc = make_tmap_bf16(&tmK, K, P.B, P.L, P.Hkv, P.d, P.ks, 128))) return rc;
     if ((rc = make_tmap_bf16(&tmV, V, P.B, P.L, P.Hkv, P.d, P.vs, 128))) return rc;
-    if (P.d == 128)
-        rowdot_bf16_kernel<16><<<(unsigned)((rows + 15) / 16), 256, 0, st>>>((const __nv_bfloat16*)O, (const __nv_bfloat16*)dO, Dv, P.B, P.L, P.Hq,
-                                                                            P.os[0], P.os[1], P.os[2]);
-    else
-        rowdot_bf16_kernel<8><<<(unsigned)((rows + 31) / 32), 256, 0, st>>>((const __nv_bfloat16*)O, (const __nv_bfloat16*)dO, Dv, P.B, P.L, P.Hq,
-                                                                           P.os[0], P.os[1], P.os[2]);
-    if (cudaMemsetAsync(acc, 0, bwd_acc_floats(P) * sizeof(float), st) != cudaSuccess) return DMA_ERR_CUDA;
-    if (cudaMemsetAsync(dM, 0, rows * sizeof(float), st) != cudaSuccess) return DMA_ERR_CUDA;   // two partial sums are added per key
+    PrepareParams pp;
+    pp.O = (const __nv_bfloat16*)O; pp.dO = (const __nv_bfloat16*)dO; pp.Dv = Dv; pp.B = P.B; pp.L = P.L; pp.Hq = P.Hq;
+    pp.os_b = P.os[0]; pp.os_l = P.os[1]; pp.os_h = P.os[2];
+    pp.status = (int32_t*)ws;
+    pp.zero[0] = acc; pp.zero_n[0] = (int64_t)bwd_acc_floats(P);
+    pp.zero[1] = dM; pp.zero_n[1] = (int64_t)rows;                                       // two partial sums are added per key
+    pp.zero[2] = accK; pp.zero_n[2] = compact ? (int64_t)(2 * slots * nkv) : 0;
+    const int per_cta = 256 / (P.d / 8) * kPrepareRows;
+    const unsigned prep_ctas = (unsigned)((rows + per_cta - 1) / per_cta);
+    for (int z = 0; z < 3; ++z) pp.zero_part[z] = ((pp.zero_n[z] >> 2) + prep_ctas - 1) / prep_ctas;
+    launch_overlapped(P.d == 128 ? bwd_prepare_kernel<16> : bwd_prepare_kernel<8>, dim3(prep_ctas), dim3(256), 0, st, 1, pp);
     if (compact) {
-        if (cudaMemsetAsync(accK, 0, 2 * slots * nkv * sizeof(float), st) != cudaSuccess) return DMA_ERR_CUDA;
-        lifetime_perm_kernel<<<P.B * P.Hq, 1024, 0, st>>>(expiry, perm, P.L, P.Tc, P.causal);
+        launch_overlapped(lifetime_perm_kernel, dim3(P.B * P.Hq), dim3(1024), 0, st, 1, expiry, perm, P.L, P.Tc, P.causal);
         count_launch();
     }
     BwdParams bp;
@@ -782,10 +869,10 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
         // stay in L2 while they are in use. About 160 MB of such rows per group was the best of the orders measured at
         // L = 16384 with 32 / 8 heads (two KV heads per group: 1.3 % faster in a long run than all eight at once; one
         // KV head per group starts the heaviest CTAs of the last group too late).
-        const int gx = compact ? P.B * P.Hq : P.B * P.Hkv;
+        const int gx = compact ? P.B * P.Hq : P.B * P.Hkv * nsplit;
         int sg = gx;
         {
-            const double per_entry = (double)(compact ? 1 : P.G) * P.L * P.d * 8;     // token-compacted mode: an entry is one query head
+            const double per_entry = (double)(compact ? 1 : P.G / nsplit) * P.L * P.d * 8;     // token-compacted mode: an entry is one query head
             // (token-compacted mode, eight heads at L = 16384: 1.69 ms against 1.74 with four and 1.82 with sixteen, once the
             //  CTAs walk backwards; with the forward walk four at a time was the best, 1.77 against 1.88)
             int want = (int)(160.0 * 1024 * 1024 / per_entry);
@@ -797,25 +884,22 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     bp.scale = P.scale; bp.scale_log2 = P.scale * 1.4426950408889634f; bp.inv_scale = 1.0f / P.scale;
     bp.ks_b = P.ks[0]; bp.ks_l = P.ks[1]; bp.ks_h = P.ks[2]; bp.vs_b = P.vs[0]; bp.vs_l = P.vs[1]; bp.vs_h = P.vs[2];
     bp.perm = perm; bp.expiry_all = expiry; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
-    bp.dKacc = accK; bp.dVacc = accV; bp.acc_slot = slots > 1 ? (int64_t)nkv : 0;
+    bp.dKacc = accK; bp.dVacc = accV; bp.acc_slot = slots > 1 ? (int64_t)nkv : 0; bp.nsplit = nsplit;
     const size_t smem = sizeof(SharedStorage) + 1024;
+    auto kern = compact ? (P.d == 128 ? bwd_kernel<true, 128> : bwd_kernel<true, 64>) : (P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     timing_mark(1, false, st);
-    if (compact) {
-        auto kern = P.d == 128 ? bwd_kernel<true, 128> : bwd_kernel<true, 64>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-        kern<<<dim3(P.B * P.Hq, P.Tc), kThreads, smem, st>>>(tmQ, tmK, tmV, tmG, bp);
-        timing_mark(1, true, st);
-        const int nb = (int)((nkv / 8 + 255) / 256);
-        dq_convert_bf16_kernel<<<nb, 256, 0, st>>>(accK, (__nv_bfloat16*)dK, nkv / 8, P.L, P.Hkv, P.ks[0], P.ks[1], P.ks[2], P.scale, P.d, (int)slots, (int64_t)nkv);
-        dq_convert_bf16_kernel<<<nb, 256, 0, st>>>(accV, (__nv_bfloat16*)dV, nkv / 8, P.L, P.Hkv, P.vs[0], P.vs[1], P.vs[2], 1.0f, P.d, (int)slots, (int64_t)nkv);
-        count_launch(2);
-    } else {
-        auto kern = P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-        kern<<<dim3(P.B * P.Hkv, P.Tc), kThreads, smem, st>>>(tmQ, tmK, tmV, tmG, bp);
-        timing_mark(1, true, st);
-    }
-    dq_unblock_bf16_kernel<<<(unsigned)((size_t)P.B * P.Hq * P.Tr * 8), 256, 0, st>>>(acc, (__nv_bfloat16*)dQ, P.L, P.Hq, P.Tr * 8, P.qs[0], P.qs[1], P.qs[2], P.scale, P.d);
+    launch_overlapped(kern, dim3(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc), dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
+    timing_mark(1, true, st);
+    FinishParams f;
+    f.dQacc = acc; f.acc[0] = accK; f.acc[1] = accV; f.dQ = (__nv_bfloat16*)dQ; f.out[0] = (__nv_bfloat16*)dK; f.out[1] = (__nv_bfloat16*)dV;
+    f.L = P.L; f.Hq = P.Hq; f.Hkv = P.Hkv; f.Lblk = P.Tr * 8; f.d = P.d; f.nslots = (int)slots; f.nkv = (int64_t)nkv;
+    f.q_rows16 = (uint32_t)((size_t)P.B * P.Hq * P.Tr * 8);
+    f.q_blocks = (int)(((size_t)f.q_rows16 * P.d * 2 + 255) / 256);
+    f.kv_blocks = (int)((nkv / 8 + 255) / 256);
+    for (int t = 0; t < 3; ++t) { f.qs[t] = P.qs[t]; f.st[0][t] = P.ks[t]; f.st[1][t] = P.vs[t]; }
+    f.scale = P.scale;
+    launch_overlapped(bwd_finish_kernel, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
     count_launch(3);
     return check_launch();
 }

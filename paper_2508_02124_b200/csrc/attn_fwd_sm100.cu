@@ -115,6 +115,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     constexpr uint32_t kLoadBytes = kHalves * (kTileBytes / 2);
     extern __shared__ uint8_t smem_raw[];
     SharedStorage& S = *reinterpret_cast<SharedStorage*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // warp-uniform to the compiler: role branches stay uniform
     const int bh = blockIdx.x, b = bh / P.Hq, h = bh % P.Hq, hk = h / P.G;
@@ -153,7 +154,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         int n = 0;
         if constexpr (kCompact) {
             // every 128-key slice of the gathered list, used by both query tiles
-            n = min((P.ccnt[(size_t)bh * npairs + lpair] + 127) / 128, kMaxSched);
+            const int listed = P.ccnt[(size_t)bh * npairs + lpair];
+            if (listed > P.ccap && lane == 0) atomicExch(P.status, (int32_t)DMA_ERR_MASK_OVERFLOW);
+            n = min((min(listed, P.ccap) + 127) / 128, kMaxSched);
             for (int t = lane; t < n; t += 32) S.sched[t] = (uint32_t)t | (1u << 30) | (has1 ? (1u << 31) : 0u);
         } else {
             const int kt_last = min(has1 ? qt1 : qt0, P.Tc - 1);
@@ -874,6 +877,7 @@ __global__ void __launch_bounds__(256) compact_lists_kernel(const int32_t* __res
     __shared__ int wcount[2][8];
     const int list = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bh = list / npairs, pair = list % npairs, i0 = q_off + pair * 256;
+    pdl_enter(expiry, cidx, ccnt, status);
     if (!causal && pair != 0) return;                    // non-causal: the head's one list is that of its first pair
     const int32_t* e = expiry + (size_t)bh * L;
     int* out = cidx + (size_t)list * cap;
@@ -913,12 +917,12 @@ __global__ void __launch_bounds__(256) compact_lists_kernel(const int32_t* __res
         p1 += __popc(b1);
         p2 += __popc(b2);
     }
-    int n = n1 + n2;
-    // more kept keys than the list holds (a mask that keeps more than w keys in some row): reported, not truncated silently
-    if (n > cap && tid == 0) atomicExch(status, (int32_t)DMA_ERR_MASK_OVERFLOW);
-    n = min(n, cap);
+    // more kept keys than the list holds (a mask that keeps more than w keys in some row): the count says so and the forward
+    // kernel reports it. (This is the stage's first kernel: it clears the workspace header.)
+    if (list == 0 && tid < kWsHeaderBytes / 4) status[tid] = 0;
+    if (tid == 0) ccnt[list] = n1 + n2;
+    const int n = min(n1 + n2, cap);
     for (int t = n + tid; t < ((n + 127) / 128) * 128 && t < cap; t += 256) out[t] = -1;
-    if (tid == 0) ccnt[list] = n;
 }
 
 static int compact_cap(const Prob& P) { return ((P.w + 256 + 127) / 128) * 128; }
@@ -957,7 +961,7 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         const size_t nl = (size_t)P.B * P.Hq * npairs;
         int* ccnt = reinterpret_cast<int*>((char*)ws + kWsHeaderBytes);
         int* cidx = reinterpret_cast<int*>((char*)ws + kWsHeaderBytes + ((nl * sizeof(int) + 255) / 256) * 256);
-        compact_lists_kernel<<<(unsigned)nl, 256, 0, st>>>(expiry, cidx, ccnt, P.L, npairs, compact_cap(P), P.causal, P.q_off, (int32_t*)ws);
+        launch_overlapped(compact_lists_kernel, dim3((unsigned)nl), dim3(256), 0, st, 1, expiry, cidx, ccnt, P.L, npairs, compact_cap(P), P.causal, P.q_off, (int32_t*)ws);
         count_launch();
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);
     }
@@ -977,7 +981,7 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
     dim3 grid(P.B * P.Hq, npairs);
     timing_mark(0, false, st);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-    kern<<<grid, kThreads, smem, st>>>(tmQ, tmK, tmV, fp);
+    launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, fp);
     timing_mark(0, true, st);
     count_launch();
     return check_launch();

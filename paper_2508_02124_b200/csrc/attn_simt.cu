@@ -48,16 +48,27 @@ __device__ __forceinline__ void dots(const float* own, const float* tile, int la
     for (int a = 0; a < kOwn; ++a) s[a][0] = s[a][1] = 0.0f;
     const float* y0 = tile + lane * LD;
     const float* y1 = y0 + 32 * LD;
-#pragma unroll 4
-    for (int c = 0; c < D; c += 4) {
-        const float4 u = *reinterpret_cast<const float4*>(y0 + c), v = *reinterpret_cast<const float4*>(y1 + c);
+#pragma unroll 1
+    for (int c0 = 0; c0 < D; c0 += 32) {       // partial sums of 32 channels: shorter chains lose less
+        float p[kOwn][2];
+#pragma unroll
+        for (int a = 0; a < kOwn; ++a) p[a][0] = p[a][1] = 0.0f;
+#pragma unroll
+        for (int c = c0; c < c0 + 32; c += 4) {
+            const float4 u = *reinterpret_cast<const float4*>(y0 + c), v = *reinterpret_cast<const float4*>(y1 + c);
+#pragma unroll
+            for (int a = 0; a < kOwn; ++a) {
+                const float4 x = *reinterpret_cast<const float4*>(own + a * D + c);
+                p[a][0] = fmaf(x.x, u.x, p[a][0]); p[a][1] = fmaf(x.x, v.x, p[a][1]);
+                p[a][0] = fmaf(x.y, u.y, p[a][0]); p[a][1] = fmaf(x.y, v.y, p[a][1]);
+                p[a][0] = fmaf(x.z, u.z, p[a][0]); p[a][1] = fmaf(x.z, v.z, p[a][1]);
+                p[a][0] = fmaf(x.w, u.w, p[a][0]); p[a][1] = fmaf(x.w, v.w, p[a][1]);
+            }
+        }
 #pragma unroll
         for (int a = 0; a < kOwn; ++a) {
-            const float4 x = *reinterpret_cast<const float4*>(own + a * D + c);
-            s[a][0] = fmaf(x.x, u.x, s[a][0]); s[a][1] = fmaf(x.x, v.x, s[a][1]);
-            s[a][0] = fmaf(x.y, u.y, s[a][0]); s[a][1] = fmaf(x.y, v.y, s[a][1]);
-            s[a][0] = fmaf(x.z, u.z, s[a][0]); s[a][1] = fmaf(x.z, v.z, s[a][1]);
-            s[a][0] = fmaf(x.w, u.w, s[a][0]); s[a][1] = fmaf(x.w, v.w, s[a][1]);
+            s[a][0] += p[a][0];
+            s[a][1] += p[a][1];
         }
     }
 }
@@ -139,6 +150,7 @@ __global__ void __launch_bounds__(32 * NW) simt_fwd_kernel(const T* __restrict__
     const int i0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * BM, L = P.L;       // first row inside the chunk (longest walks first)
     const int ia0 = P.q_off + i0;                // its position in the sequence
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_enter(Q, K, V, bias, expiry, bitmap, O, lse);
     const T* q = Q + b * P.qs[0] + h * P.qs[2];
     const T* k = K + b * P.ks[0] + hk * P.ks[2];
     const T* v = V + b * P.vs[0] + hk * P.vs[2];
@@ -189,7 +201,7 @@ __global__ void __launch_bounds__(32 * NW) simt_fwd_kernel(const T* __restrict__
 #pragma unroll
             for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             const float m_new = fmaxf(m[a], mx), m_use = m_new == -INFINITY ? 0.0f : m_new;
-            const float alpha = __expf(m[a] - m_use), p0 = __expf(s[a][0] - m_use), p1 = __expf(s[a][1] - m_use);
+            const float alpha = expf(m[a] - m_use), p0 = expf(s[a][0] - m_use), p1 = expf(s[a][1] - m_use);
             m[a] = m_new;
             l[a] = l[a] * alpha + (p0 + p1);     // this lane's part of the row sum
             wts[a * kTile + lane] = p0;
@@ -218,6 +230,7 @@ template <typename T>
 __global__ void rowdot_kernel(const T* __restrict__ O, const T* __restrict__ dO, float* __restrict__ Dv, Prob P) {
     const long row = (long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x % 32;
+    pdl_enter(O, dO, Dv);
     if (row >= (long)P.B * P.Hq * P.L) return;
     const int i = row % P.L, h = (row / P.L) % P.Hq, b = row / ((long)P.L * P.Hq);
     const T* o = O + b * P.os[0] + (int64_t)i * P.os[1] + h * P.os[2];
@@ -242,6 +255,7 @@ __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__
     float* sY = sA + 2 * BM * D;                 // two buffers of Q, dO (or K, V) tiles, [kTile][LD] each
     float* sP = sY + 4 * kTile * LD;             // [NW][2][kOwn][kTile]
     const int b = blockIdx.z, L = P.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_enter(Q, K, V, dO, lse, Dv, bias, expiry, bitmap, dQ, dK, dV, dM);
     float* wts = sP + warp * 2 * kOwn * kTile;
     const float* own1 = sA + warp * kOwn * D;
     const float* own2 = own1 + BM * D;
@@ -297,7 +311,7 @@ __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__
                     for (int t = 0; t < 2; ++t) {
                         const int i = i0 + lane + 32 * t;
                         const bool ok = (j <= i || !P.causal) && i < ej[a] && i < L;
-                        const float p = ok ? __expf(s[a][t] * P.scale + bj[a] - li[t]) : 0.0f;
+                        const float p = ok ? expf(s[a][t] * P.scale + bj[a] - li[t]) : 0.0f;
                         const float ds = p * (dp[a][t] - di[t]);
                         wts[a * kTile + lane + 32 * t] = p;
                         wts[(kOwn + a) * kTile + lane + 32 * t] = ds;
@@ -370,7 +384,7 @@ __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__
                 for (int t = 0; t < 2; ++t) {
                     const int j = j0 + lane + 32 * t;
                     const bool ok = (j <= i || !P.causal) && i < ej[t] && i < L;
-                    const float p = ok ? __expf(s[a][t] * P.scale + bj[t] - li[a]) : 0.0f;
+                    const float p = ok ? expf(s[a][t] * P.scale + bj[t] - li[a]) : 0.0f;
                     wts[a * kTile + lane + 32 * t] = p * (dp[a][t] - di[a]);
                 }
             }
@@ -396,8 +410,8 @@ int fwd_t(const Prob& P, const void* Q, const void* K, const void* V, const floa
     // a chunk of query rows that does not start on a bitmap row boundary (or comes without a bitmap) visits every key tile
     int use_bitmap = bitmap && !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0 && P.q_off % kTile == 0;
     timing_mark(0, false, st);
-    kern<<<dim3((P.Lq + kOwn * NW - 1) / (kOwn * NW), P.Hq, P.B), 32 * NW, smem, st>>>((const T*)Q, (const T*)K, (const T*)V, bias, expiry,
-                                                                                     bitmap, (T*)O, lse, P, use_bitmap);
+    launch_overlapped(kern, dim3((P.Lq + kOwn * NW - 1) / (kOwn * NW), P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K, (const T*)V,
+                      bias, expiry, bitmap, (T*)O, lse, P, use_bitmap);
     timing_mark(0, true, st);
     count_launch();
     return check_launch();
@@ -412,11 +426,11 @@ int bwd_t(const Prob& P, const void* Q, const void* K, const void* V, const void
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     const size_t rows = (size_t)P.B * P.Hq * P.L;
     float* Dv = reinterpret_cast<float*>((char*)ws + kWsHeaderBytes);
-    rowdot_kernel<T><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>((const T*)O, (const T*)dO, Dv, P);
+    launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P);
     int use_bitmap = !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0;
     timing_mark(1, false, st);
-    kern<<<dim3((P.L + kOwn * NW - 1) / (kOwn * NW), P.Hkv + P.Hq, P.B), 32 * NW, smem, st>>>(
-        (const T*)Q, (const T*)K, (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap);
+    launch_overlapped(kern, dim3((P.L + kOwn * NW - 1) / (kOwn * NW), P.Hkv + P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
+                      (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap);
     timing_mark(1, true, st);
     count_launch(2);
     return check_launch();

@@ -19,6 +19,7 @@ struct Prob {
     int dtype, flags;
     int causal;            // 1: key j visible to rows i >= j; 0: to every row (the key's first row is 0 instead of j)
     int bm, bn, Tr, Tc, Wd;   // bitmap tile sizes, tile counts, uint32 words per bitmap row
+    int bwd_split;            // CTAs that share a KV head in the tile-mode backward (0: tc_bwd_splits chooses)
     int Lq, q_off;            // forward over a chunk of query rows: Q, O, lse hold the rows q_off .. q_off + Lq - 1 (Lq = L, q_off = 0: all)
     float scale;
     int64_t qs[3], ks[3], vs[3], os[3];   // batch, seq, head strides in elements
@@ -58,6 +59,11 @@ size_t tc_fwd_ws_bytes(const Prob& P);
 int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
                   const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st);
 size_t tc_bwd_ws_bytes(const Prob& P);
+int tc_bwd_splits(const Prob& P);
+// dma_attn_bwd on a part of a problem: with the split of the whole one, so that the parts' results are the whole's
+int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* K, const void* V, const void* O, const void* dO,
+                  const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ, void* dK, void* dV,
+                  float* dM, void* ws, size_t ws_bytes, cudaStream_t st);
 int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,
                   const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ,
                   void* dK, void* dV, float* dM, void* ws, cudaStream_t st);
@@ -65,10 +71,13 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
 // ---------------------------------------------------------------------------------------------
 // launches that overlap the tail of the kernel before them (programmatic dependent launch)
 // ---------------------------------------------------------------------------------------------
-// A kernel launched this way may become resident while the previous kernel of the stream still runs. Every such kernel
-// calls pdl_enter() with ALL its global pointers before its first access to global memory: it returns once the previous
-// kernel has completed and its writes are visible, and lets the next kernel in. What is saved is the launch latency and
-// the drain between dependent kernels, about 1 us each, which is what the short kernels of a decoding step are made of.
+// A kernel launched this way may become resident once every CTA of the previous kernel of the stream has left the chip or is
+// about to, instead of after that kernel's completion has been reported. Every such kernel calls pdl_enter() with ALL its
+// global pointers before its first access to global memory: it returns once the previous kernel has completed and its writes
+// are visible. What is saved is the launch latency between dependent kernels, about 1 to 2 us each, which short kernels are
+// made of: step of 2 x 1000 rows, d = 64: 112 -> 103 us, prefill of 4096 keys 123 -> 107 us. (Letting the next kernel in early,
+// with griddepcontrol.launch_dependents at the top, was slower everywhere: its waiting CTAs take the places that the running
+// kernel's CTAs leave unevenly, 218 -> 239 us for 2048 rows of a 16384-key prefill, 2998 -> 3071 us for its training step.)
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -94,14 +103,13 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 b
 // ---------------------------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------------------------
-// Waits for the previous kernel, then lets the next one start. The pointers pass through an empty asm statement behind the
+// Waits for the previous kernel. The pointers pass through an empty asm statement behind the
 // wait, so that no load through them (a read-only load of a const __restrict__ parameter is free to move) comes before it.
 template <typename... Ts>
 __device__ __forceinline__ void pdl_enter(Ts&... ptrs) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     auto pin = [](auto& p) { asm volatile("" : "+l"(p) :: "memory"); };
     (pin(ptrs), ...);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 __device__ __forceinline__ float to_f32(float x) { return x; }

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? 2 : 1) delta_kernel(cons
     const int hk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = lane % LPR, grp = lane / LPR;
+    pdl_enter(V, W, A, delta);
     const int ntiles = (L - j_off + kRows - 1) / kRows;        // keys [j_off, L) of a row of ld entries
     const T* Vb = V + b * vs_b + hk * vs_h + sub * 8;
     auto request = [&](int tile, Raw (&raw)[kPass]) {
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V
     int mine = 0;                         // the head (within a batch) this lane ends up with: sub, bit-reversed
 #pragma unroll
     for (int m = 1, t = LPR >> 1; m < LPR; m <<= 1, t >>= 1) mine |= (sub & m) ? t : 0;
+    pdl_enter(V, W, A, delta);
     for (int i = tid; i < HqP * C; i += 256) sW[i] = i < Hq * C ? W[i] : 0.0f;
     __syncthreads();
     for (int r0 = 0; r0 < kFullRows; r0 += kPass) {
@@ -300,14 +302,22 @@ __device__ __forceinline__ unsigned long long sort_key(float dl, int j) {
     return ((unsigned long long)__float_as_uint(dl) << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
 }
 
+// this CTA's share of zeros (a later kernel of the stage ORs bits into the bitmap)
+__device__ __forceinline__ void zero_share(uint32_t* p, int64_t n) {
+    const int64_t cta = (int64_t)blockIdx.y * gridDim.x + blockIdx.x, ctas = (int64_t)gridDim.x * gridDim.y;
+    for (int64_t i = n * cta / ctas + threadIdx.x; i < n * (cta + 1) / ctas; i += blockDim.x) p[i] = 0u;
+}
+
 // Chunks are written in DESCENDING order, padding keys (beyond L) carry their index and sort below every real key, and
 // the kernel also emits the eight lowest levels of the rank tree (node sizes 256 ... 2, see below) by splitting the sorted
 // chunk on one index bit per level.
 __global__ void __launch_bounds__(kChunk) chunk_sort_kernel(const float* __restrict__ delta,
                                                             unsigned long long* __restrict__ sorted, int L, int nchunk,
-                                                            uint2* __restrict__ lev, int m) {
+                                                            uint2* __restrict__ lev, int m, uint32_t* __restrict__ bitmap, int64_t bitmap_words) {
     __shared__ unsigned long long s[2][kChunk];
     const int bh = blockIdx.y, c = blockIdx.x, t = threadIdx.x, j = c * kChunk + t;
+    pdl_enter(delta, sorted, lev, bitmap);
+    zero_share(bitmap, bitmap_words);
     // padding sorts below every real key (delta > 0) and keeps its index in the low word
     unsigned long long v = j < L ? sort_key(delta[(size_t)bh * L + j], j) : (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
     // bitonic network, ascending; thread t holds position t. Partners less than 32 apart exchange by shuffle, the six
@@ -419,6 +429,7 @@ __global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const unsigne
                                                                    unsigned long long* __restrict__ dst,
                                                                    uint2* __restrict__ lev, int Lc, int m) {
     extern __shared__ __align__(16) unsigned long long sk[];         // two buffers of kBlockKeys keys
+    pdl_enter(src, dst, lev);
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
     const int base = blockIdx.x * kBlockKeys, nreal = min(kBlockKeys, Lc - base);
     const size_t Wl = (size_t)Lc / 32;
@@ -463,6 +474,7 @@ __global__ void __launch_bounds__(kMergeThreads) tree_merge_kernel(const unsigne
                                                                    uint2* __restrict__ lev_l, int Lc, int R, int m) {
     __shared__ __align__(16) unsigned long long sA[kMergeOut], sB[kMergeOut];
     __shared__ int s_a0;
+    pdl_enter(src, dst, lev_l);
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int o0 = blockIdx.x * kMergeOut;                       // first output position of this CTA within the head
     const int base = o0 & ~(2 * R - 1), t0 = o0 - base;
@@ -518,6 +530,7 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
                                                           int32_t* __restrict__ expiry, int L, int Lc, int w, int m,
                                                           const int32_t* __restrict__ cu, int nseq) {
     const int r = blockIdx.x * 256 + threadIdx.x, bh = blockIdx.y;
+    pdl_enter(sorted, lev, expiry, cu);
     if (r >= L) return;                                          // ranks from L on are padding
     const int j = (int)(0xFFFFFFFFu - (uint32_t)sorted[(size_t)bh * Lc + r]);
     const size_t W = (size_t)Lc / 32;
@@ -567,8 +580,10 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
     expiry[(size_t)bh * L + j] = e;
 }
 
-__global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v) {
+__global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v, uint32_t* bitmap, int64_t bitmap_words) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_enter(p, bitmap);
+    zero_share(bitmap, bitmap_words);
     if (i < n) p[i] = v;
 }
 
@@ -579,6 +594,7 @@ __global__ void __launch_bounds__(128) bitmap_kernel(const int32_t* __restrict__
                                                      int L, int bm, int bn, int Tr, int Wd, int causal) {
     extern __shared__ int diff[];                 // [Tr + 1]
     const int kt = blockIdx.x, bh = blockIdx.y, t = threadIdx.x;
+    pdl_enter(expiry, bitmap);
     for (int i = t; i <= Tr; i += blockDim.x) diff[i] = 0;
     __syncthreads();
     const int jend = min(L, (kt + 1) * bn);
@@ -642,8 +658,8 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
         if (bytes > 200 * 1024) return DMA_ERR_UNSUPPORTED;
         if (cudaFuncSetAttribute(delta_full_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
             return DMA_ERR_CUDA;
-        delta_full_kernel<T, D><<<dim3((j_end - j_begin + kFullRows - 1) / kFullRows, P.B), 256, bytes, st>>>(
-            (const T*)V, W, A, bias, j_end, P.Hq, P.Hkv, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+        launch_overlapped(delta_full_kernel<T, D>, dim3((j_end - j_begin + kFullRows - 1) / kFullRows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A,
+                          bias, j_end, P.Hq, P.Hkv, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
         count_launch();
         return check_launch();
     }
@@ -655,7 +671,7 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     dim3 grid(per_pair, P.Hkv, P.B);
     size_t smem = (size_t)P.G * (D + 2 * 128) * sizeof(float);
     if (smem > 48 * 1024) return DMA_ERR_UNSUPPORTED;
-    delta_kernel<T, D><<<grid, 256, smem, st>>>((const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+    launch_overlapped(delta_kernel<T, D>, grid, dim3(256), smem, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
     count_launch();
     return check_launch();
 }
@@ -697,9 +713,10 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
 
     const int BH = P.B * P.Hq;
     const int nchunk = (P.L + kChunk - 1) / kChunk;
+    const int64_t bitmap_words = (int64_t)BH * P.Tr * P.Wd;        // zeroed by the kernel after the deltas
     if (P.w >= P.L && !cu) {   // every visible key is kept
         size_t n = (size_t)BH * P.L;
-        fill_i32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(expiry, n, P.L);
+        launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, bitmap_words);
         count_launch();
     } else {
         // rank tree: sorted chunks and the low levels, one merge pass per further level, then one walk per key
@@ -708,30 +725,28 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
         auto* buf0 = reinterpret_cast<unsigned long long*>((char*)ws + kWsHeaderBytes);
         auto* buf1 = buf0 + keys;
         uint2* lev = reinterpret_cast<uint2*>(buf1 + keys);
-        chunk_sort_kernel<<<dim3(nchunk, BH), kChunk, 0, st>>>(bias, buf0, P.L, nchunk, lev, m);
+        launch_overlapped(chunk_sort_kernel, dim3(nchunk, BH), dim3(kChunk), 0, st, 1, bias, buf0, P.L, nchunk, lev, m, bitmap, bitmap_words);
         int launches = 2;
         if (Lc > kChunk) {
-            tree_block_kernel<<<dim3((Lc + kBlockKeys - 1) / kBlockKeys, BH), kBlockThreads, kBlockSmem, st>>>(buf0, buf1, lev, Lc, m);
+            launch_overlapped(tree_block_kernel, dim3((Lc + kBlockKeys - 1) / kBlockKeys, BH), dim3(kBlockThreads), kBlockSmem, st, 1, buf0, buf1, lev, Lc, m);
             std::swap(buf0, buf1);
             ++launches;
         }
         int l = m - 13;                                          // level of the nodes of 2 * kBlockKeys keys
         for (int R = kBlockKeys; R < Lc; R *= 2, --l, ++launches) {
-            tree_merge_kernel<<<dim3((Lc + kMergeOut - 1) / kMergeOut, BH), kMergeThreads, 0, st>>>(buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
+            launch_overlapped(tree_merge_kernel, dim3((Lc + kMergeOut - 1) / kMergeOut, BH), dim3(kMergeThreads), 0, st, 1, buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
             std::swap(buf0, buf1);
         }
         const dim3 grid((P.L + 255) / 256, BH);
-        if (cu) expiry_tree_kernel<1><<<grid, 256, 0, st>>>(buf0, lev, expiry, P.L, Lc, P.w, m, cu, nseq);
-        else if (P.causal) expiry_tree_kernel<0><<<grid, 256, 0, st>>>(buf0, lev, expiry, P.L, Lc, P.w, m, nullptr, 0);
-        else expiry_tree_kernel<2><<<grid, 256, 0, st>>>(buf0, lev, expiry, P.L, Lc, P.w, m, nullptr, 0);
+        launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev, expiry,
+                          P.L, Lc, P.w, m, cu, nseq);
         count_launch(launches);
     }
     if ((rc = check_launch())) return rc;
 
-    if (cudaMemsetAsync(bitmap, 0, (size_t)BH * P.Tr * P.Wd * sizeof(uint32_t), st) != cudaSuccess) return DMA_ERR_CUDA;
     size_t smem = (size_t)(P.Tr + 1) * sizeof(int);
     if (smem > 48 * 1024) return DMA_ERR_UNSUPPORTED;
-    bitmap_kernel<<<dim3(P.Tc, BH), 128, smem, st>>>(expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
+    launch_overlapped(bitmap_kernel, dim3(P.Tc, BH), dim3(128), smem, st, 1, expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
     count_launch();
     return check_launch();
 }

@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(kThreads) mask_bwd_kernel(const T* __restrict_
     const int hk = blockIdx.y, b = blockIdx.z, j0 = blockIdx.x * kRows;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = lane % LPR, grp = lane / LPR;
+    pdl_enter(V, W, A, delta, dM, dV, partial);
     float* sGD = sAcc + 8 * G * (D + 1);             // [G][kRows]: dM * delta of the CTA's keys, fetched in one batch
     for (int i = tid; i < G * D; i += kThreads) sW[i] = W[(size_t)hk * G * D + i];
     for (int i = tid; i < G * kRows; i += kThreads) {
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(kThreads) mask_bwd_kernel(const T* __restrict_
         const int j = j0 + warp * RPW + n * 8 * RPW + grp;
         const float z = myDz[pr];
         const float gd = sGD[g * kRows + (j - j0)];
-        const float e = __expf(-fabsf(z));                       // in (0, 1]
+        const float e = expf(-fabsf(z));                       // in (0, 1]
         const float sp = fmaxf(z, 0.0f) + log1pf(e);
         const float sig = (z >= 0.0f ? 1.0f : e) / (1.0f + e);
         myDz[pr] = gd * A[hk * G + g] * sig;
@@ -171,6 +172,7 @@ __global__ void __launch_bounds__((D == 128 ? 4 : 8) * (D + 1)) mask_bwd_reduce_
                                                                      float* __restrict__ dA, int B, int Hkv, int G, int nblk) {
     constexpr int kGroups = D == 128 ? 4 : 8;      // kGroups * (D + 1) threads <= 1024
     __shared__ float part[kGroups][D + 1];
+    pdl_enter(partial, dW, dA);
     const int h = blockIdx.x, hk = h / G, g = h % G;
     const int c = threadIdx.x % (D + 1), grp = threadIdx.x / (D + 1);
     float s = 0.0f;
@@ -213,6 +215,7 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
     const int b = blockIdx.y, j0 = blockIdx.x * R;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int C8 = C / 8, D8 = D / 8;
+    pdl_enter(V, W, A, delta, dM, dV, partial);
 
     for (int i = tid; i < R * C8; i += kFullThreads) {
         const int row = i / C8, ch = i % C8, j = j0 + row;
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
             const size_t at = ((size_t)b * Hq + h) * L + j;
             const float gd = dM[at] * delta[at];
             const float z = sZ[i];
-            const float e = __expf(-fabsf(z));
+            const float e = expf(-fabsf(z));
             gs = gd * (fmaxf(z, 0.0f) + log1pf(e));
             dz = gd * A[h] * ((z >= 0.0f ? 1.0f : e) / (1.0f + e));
         }
@@ -349,6 +352,7 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
 __global__ void __launch_bounds__(512) mask_bwd_full_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dW,
                                                                    float* __restrict__ dA, int n, int Hq, int C) {
     __shared__ float part[4][128];
+    pdl_enter(partial, dW, dA);
     const int h = blockIdx.y, c = blockIdx.x * 128 + (threadIdx.x & 127), grp = threadIdx.x >> 7;
     float s = 0.0f;
     if (c <= C)
@@ -387,9 +391,9 @@ static int launch_typed(const Prob& P, const void* V, const float* W, const floa
     const int nblk = (P.L + kRows - 1) / kRows;
     const size_t smem = (size_t)P.G * (D + 8 * (D + 1) + 3 * kRows) * sizeof(float);
     if (cudaFuncSetAttribute(mask_bwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-    mask_bwd_kernel<T, D><<<dim3(nblk, P.Hkv, P.B), kThreads, smem, st>>>((const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
+    launch_overlapped(mask_bwd_kernel<T, D>, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
                                                                             P.G, P.vs[0], P.vs[1], P.vs[2]);
-    mask_bwd_reduce_kernel<D><<<P.Hq, (D == 128 ? 4 : 8) * (D + 1), 0, st>>>((const float*)ws, dW, dA, P.B, P.Hkv, P.G, nblk);
+    launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(P.Hq), dim3((D == 128 ? 4 : 8) * (D + 1)), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G, nblk);
     count_launch(2);
     return check_launch();
 }
@@ -402,9 +406,9 @@ static int launch_full(const Prob& P, const void* V, const float* W, const float
     const size_t smem = ((size_t)R * C + (size_t)R * HqP + (size_t)P.Hq * R) * sizeof(float);
     if (cudaFuncSetAttribute(mask_bwd_full_kernel<T, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return DMA_ERR_CUDA;
-    mask_bwd_full_kernel<T, RW><<<dim3(nblk, P.B), kFullThreads, smem, st>>>((const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
+    launch_overlapped(mask_bwd_full_kernel<T, RW>, dim3(nblk, P.B), dim3(kFullThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
                                                                           P.Hkv, P.d, P.vs[0], P.vs[1], P.vs[2]);
-    mask_bwd_full_reduce_kernel<<<dim3((C + 1 + 127) / 128, P.Hq), 512, 0, st>>>((const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
+    launch_overlapped(mask_bwd_full_reduce_kernel, dim3((C + 1 + 127) / 128, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
     count_launch(2);
     return check_launch();
 }

@@ -184,6 +184,9 @@ int dma_step_host(const dma_problem_t* p, int backward, const void* hQ, const vo
 
     dma_problem_t sub = *p;
     sub.B = GB; sub.Hq = nqh; sub.Hkv = nkh;
+    Prob whole;
+    if ((rc = resolve(p, &whole))) return cleanup(rc);
+    const int split = tc_bwd_splits(whole);          // (of the whole problem: the groups' gradients are then those of one call on it)
     const int64_t qs[3] = {(int64_t)L * p->Hq * d, (int64_t)p->Hq * d, d}, ks[3] = {(int64_t)L * p->Hkv * d, (int64_t)p->Hkv * d, d};
     for (int i = 0; i < 3; ++i) { sub.q_stride[i] = sub.o_stride[i] = qs[i]; sub.k_stride[i] = sub.v_stride[i] = ks[i]; }
     const size_t f_ws = Lo.f_ws - (size_t)NG * kWsHeaderBytes, b_ws = Lo.b_ws - (size_t)NG * kWsHeaderBytes;
@@ -210,7 +213,7 @@ int dma_step_host(const dma_problem_t* p, int backward, const void* hQ, const vo
             char* wsb = a + Lo.ws_bwd + (size_t)g * kWsHeaderBytes;
             float* dM = (float*)(a + Lo.dM) + (size_t)g * Lo.gh;
             if (!ok || !wait(st, e[kdO])) return cleanup(DMA_ERR_CUDA);
-            if ((rc = dma_attn_bwd(&sub, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, a + Lo.O + G.q * esz,
+            if ((rc = attn_bwd_part(&sub, split, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, a + Lo.O + G.q * esz,
                                    a + Lo.dO + G.q * esz, lse, bias, expiry, bitmap, a + Lo.dQ + G.q * esz, a + Lo.dK + G.k * esz,
                                    a + Lo.dV + G.k * esz, dM, wsb, b_ws, st))) return cleanup(rc);
             ok = rec(e[kG], st) && wait(s_out, e[kG]) &&

@@ -478,3 +478,18 @@ def test_cuda_core_kernels_at_the_edges_of_their_tiles(B, Hq, Hkv, L, d, w):
     compare(case, got, ref)
     again = gpu_run(case, inp, stored=st)
     assert all(torch.equal(got[k], again[k]) for k in ("O", "lse", "dQ", "dK", "dV", "dM"))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,d", [(1, 6, 1, 300, 128), (1, 6, 1, 129, 64), (2, 8, 2, 640, 64), (1, 4, 4, 200, 128), (1, 12, 2, 1100, 128)])
+def test_tile_backward_with_the_group_dealt_out_to_several_ctas(B, Hq, Hkv, L, d):
+    """Short sequences: a KV head's query heads go to several CTAs (2, 3, 4 or 6 of them, or one), whose dK / dV parts are summed from
+    slots: against the oracle, and dK, dV, dM the same bits from run to run."""
+    case = wl.small(C2, B=B, Hq=Hq, Hkv=Hkv, L=L, d=d, w=L // 3, backward=True, seed=L + Hq, name="split")
+    inp = wl.make_inputs(case)
+    dl, e, bmp = oracle_mask(case, inp)
+    ref = oracle_all(case, inp, dl, e)
+    st = stored_forward(case, ref["O"], ref["lse"])
+    got = gpu_run(case, inp, stored=st, flags=dma.DMA_FLAG_TILE_PATH)
+    compare(case, got, ref)
+    again = gpu_run(case, inp, stored=st, flags=dma.DMA_FLAG_TILE_PATH)
+    assert all(torch.equal(got[k], again[k]) for k in ("dK", "dV", "dM"))
