@@ -868,61 +868,156 @@ int make_tmap_bf16(CUtensorMap* m, const void* base, int B, int L, int H, int d,
 // At most w + 256 keys qualify. The list is in two parts, each ascending: first the keys that ALL 256 rows keep
 // (j <= i0 and expiry[j] >= i0 + 256), then the keys that enter or expire inside the pair's rows. The forward kernel
 // needs no order among the columns, and this one leaves the keys that need the per-element test (a few hundred per pair)
-// in the last slices instead of a few in every slice. One CTA of 256 threads per list; every warp owns a contiguous
-// eighth of the candidate keys, counts its keys of either part in a first pass and writes them from its start positions
-// (the sums of the earlier warps' counts) in a second one: one barrier. Padded with -1 to the next multiple of 128.
-__global__ void __launch_bounds__(256) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
-                                                            int* __restrict__ ccnt, int L, int npairs, int cap, int causal,
-                                                            int q_off, int32_t* __restrict__ status) {
-    __shared__ int wcount[2][8];
-    const int list = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bh = list / npairs, pair = list % npairs, i0 = q_off + pair * 256;
+// in the last slices instead of a few in every slice.
+// A CTA makes the lists of `group` consecutive pairs of one head. Every list on its own would read all keys before its rows, in
+// two passes (count, write), which at 65536 keys was 781 us, an eighth of the prefill. With group > 1 the CTA first collects the
+// keys that some row of the group keeps (at most the list's capacity and the group's rows: shared memory), and its lists are
+// made from those: the head is read once per 256 group rows. group = 1: the lists are made straight from the head.
+// Every warp owns a contiguous part of what it reads, 128 keys at a time (16-byte loads where rows are 16-byte aligned), and
+// writes from the sum of the earlier parts' counts. Padded with -1 to the next multiple of 128.
+constexpr int kListThreads = 256, kListWarps = 8;
+
+template <bool kVec>
+__global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
+                                                                     int* __restrict__ ccnt, int L, int npairs, int cap, int causal,
+                                                                     int q_off, int32_t* __restrict__ status, int group, int ccap) {
+    extern __shared__ int2 cand[];                       // group > 1: (key, expiry) of the keys some row of the group keeps
+    __shared__ int wcount[2][kListWarps];
+    const int ngroups = (npairs + group - 1) / group;
+    const int bh = blockIdx.x / ngroups, pair0 = blockIdx.x % ngroups * group;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t below = (1u << lane) - 1u;
     pdl_enter(expiry, cidx, ccnt, status);
-    if (!causal && pair != 0) return;                    // non-causal: the head's one list is that of its first pair
+    if (blockIdx.x == 0 && tid < kWsHeaderBytes / 4) status[tid] = 0;       // the stage's first kernel: it clears the workspace header
+    if (!causal && pair0 != 0) return;                   // non-causal: the head's one list is that of its first pair
     const int32_t* e = expiry + (size_t)bh * L;
-    int* out = cidx + (size_t)list * cap;
-    const int jend = causal ? min(L, i0 + 256) : L;     // non-causal: key j is kept by the rows i < expiry[j], whatever j
-    const int seg = (((jend + 7) / 8 + 31) / 32) * 32, j0 = warp * seg, j1 = min(jend, j0 + seg);
+    const int pairs = causal ? min(group, npairs - pair0) : 1;
+    const int lo = q_off + pair0 * 256, jend = causal ? min(L, lo + pairs * 256) : L;
+    // four keys of the head per lane, from base on: (key, expiry), expiry 0 (never kept) beyond `end`
+    auto load4 = [&](int base, int end, int (&j)[4], int (&ej)[4]) {
+        if (kVec && base + 128 <= end) {
+            const int4 v = *reinterpret_cast<const int4*>(e + base + 4 * lane);
+            ej[0] = v.x; ej[1] = v.y; ej[2] = v.z; ej[3] = v.w;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) j[u] = base + 4 * lane + u;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                j[u] = base + 32 * u + lane;
+                ej[u] = j[u] < end ? e[j[u]] : 0;
+            }
+        }
+    };
+    int ncand = jend;
+    bool over = false;
+    if (group > 1) {
+        const int seg = ((jend + kListWarps - 1) / kListWarps + 127) / 128 * 128, j0 = warp * seg, j1 = min(jend, j0 + seg);
+        int c = 0;
+#pragma unroll 4
+        for (int base = j0; base < j1; base += 128) {
+            int j[4], ej[4];
+            load4(base, j1, j, ej);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c += ej[u] > max(lo, causal ? j[u] : 0);
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) wcount[0][warp] = c;
+        __syncthreads();
+        int at = 0, all = 0;
+#pragma unroll
+        for (int q = 0; q < kListWarps; ++q) {
+            at += q < warp ? wcount[0][q] : 0;
+            all += wcount[0][q];
+        }
+#pragma unroll 2
+        for (int base = j0; base < j1; base += 128) {
+            int j[4], ej[4];
+            load4(base, j1, j, ej);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = ej[u] > max(lo, causal ? j[u] : 0);
+                const uint32_t bal = __ballot_sync(0xffffffffu, in);
+                const int p = at + __popc(bal & below);
+                if (in && p < ccap) cand[p] = make_int2(j[u], ej[u]);
+                at += __popc(bal);
+            }
+        }
+        over = all > ccap;                               // then the group's first row alone keeps more than a list holds
+        ncand = min(all, ccap);
+        __syncthreads();
+    }
+    // the lists: kListWarps / group warps per pair
+    const int per = kListWarps / group, part = warp % per, pair = pair0 + warp / per;
+    const bool exists = warp / per < pairs;
+    const int i0 = q_off + pair * 256, list = bh * npairs + pair;
+    const int end = group > 1 ? ncand : causal ? min(L, i0 + 256) : L;
+    const int seg = ((end + per - 1) / per + 127) / 128 * 128, k0 = part * seg, k1 = exists ? min(end, k0 + seg) : 0;
+    auto fetch = [&](int base, int (&j)[4], int (&ej)[4]) {
+        if (group > 1) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = base + 32 * u + lane;
+                const int2 v = k < k1 ? cand[k] : make_int2(0, 0);
+                j[u] = v.x;
+                ej[u] = v.y;
+            }
+        } else {
+            load4(base, k1, j, ej);
+        }
+    };
     // 0: not in the list, 1: kept by every row of the pair, 2: kept by some
-    auto kind = [&](int j) {
-        if (j >= j1) return 0;
-        const int ej = e[j], first = causal ? j : 0;
-        if (ej <= max(i0, first)) return 0;
+    auto kind = [&](int j, int ej) {
+        const int first = causal ? j : 0;
+        if (ej <= max(i0, first) || first > i0 + 255) return 0;
         return (first <= i0 && ej >= i0 + 256) ? 1 : 2;
     };
     int c1 = 0, c2 = 0;
-    for (int base = j0; base < j1; base += 32) {
-        const int k = kind(base + lane);
-        c1 += __popc(__ballot_sync(0xffffffffu, k == 1));
-        c2 += __popc(__ballot_sync(0xffffffffu, k == 2));
+#pragma unroll 4
+    for (int base = k0; base < k1; base += 128) {
+        int j[4], ej[4];
+        fetch(base, j, ej);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = kind(j[u], ej[u]);
+            c1 += k == 1;
+            c2 += k == 2;
+        }
     }
+    c1 = __reduce_add_sync(0xffffffffu, c1);
+    c2 = __reduce_add_sync(0xffffffffu, c2);
+    if (group > 1) __syncthreads();                      // wcount was read above
     if (lane == 0) { wcount[0][warp] = c1; wcount[1][warp] = c2; }
     __syncthreads();
+    if (!exists) return;
     int p1 = 0, p2 = 0, n1 = 0, n2 = 0;
-#pragma unroll
-    for (int wq = 0; wq < 8; ++wq) {
-        const int a = wcount[0][wq], bq = wcount[1][wq];
-        p1 += wq < warp ? a : 0;
-        p2 += wq < warp ? bq : 0;
+    for (int q = 0; q < per; ++q) {
+        const int a = wcount[0][warp - part + q], b = wcount[1][warp - part + q];
+        p1 += q < part ? a : 0;
+        p2 += q < part ? b : 0;
         n1 += a;
-        n2 += bq;
+        n2 += b;
     }
     p2 += n1;                                            // the second part starts behind the first
-    for (int base = j0; base < j1; base += 32) {
-        const int j = base + lane, k = kind(j);
-        const uint32_t b1 = __ballot_sync(0xffffffffu, k == 1), b2 = __ballot_sync(0xffffffffu, k == 2);
-        const uint32_t below = (1u << lane) - 1;
-        const int at = k == 1 ? p1 + __popc(b1 & below) : p2 + __popc(b2 & below);
-        if (k != 0 && at < cap) out[at] = j;
-        p1 += __popc(b1);
-        p2 += __popc(b2);
+    int* out = cidx + (size_t)list * cap;
+#pragma unroll 2
+    for (int base = k0; base < k1; base += 128) {
+        int j[4], ej[4];
+        fetch(base, j, ej);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = kind(j[u], ej[u]);
+            const uint32_t b1 = __ballot_sync(0xffffffffu, k == 1), b2 = __ballot_sync(0xffffffffu, k == 2);
+            const int at = k == 1 ? p1 + __popc(b1 & below) : p2 + __popc(b2 & below);
+            if (k != 0 && at < cap) out[at] = j[u];
+            p1 += __popc(b1);
+            p2 += __popc(b2);
+        }
     }
     // more kept keys than the list holds (a mask that keeps more than w keys in some row): the count says so and the forward
-    // kernel reports it. (This is the stage's first kernel: it clears the workspace header.)
-    if (list == 0 && tid < kWsHeaderBytes / 4) status[tid] = 0;
-    if (tid == 0) ccnt[list] = n1 + n2;
-    const int n = min(n1 + n2, cap);
-    for (int t = n + tid; t < ((n + 127) / 128) * 128 && t < cap; t += 256) out[t] = -1;
+    // kernel reports it
+    const int n = min(n1 + n2, cap), fill = over ? cap : (n + 127) / 128 * 128;
+    for (int t = n + part * 32 + lane; t < fill && t < cap; t += per * 32) out[t] = -1;
+    if (part == 0 && lane == 0) ccnt[list] = over ? cap + 1 : n1 + n2;
 }
 
 static int compact_cap(const Prob& P) { return ((P.w + 256 + 127) / 128) * 128; }
@@ -961,7 +1056,17 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         const size_t nl = (size_t)P.B * P.Hq * npairs;
         int* ccnt = reinterpret_cast<int*>((char*)ws + kWsHeaderBytes);
         int* cidx = reinterpret_cast<int*>((char*)ws + kWsHeaderBytes + ((nl * sizeof(int) + 255) / 256) * 256);
-        launch_overlapped(compact_lists_kernel, dim3((unsigned)nl), dim3(256), 0, st, 1, expiry, cidx, ccnt, P.L, npairs, compact_cap(P), P.causal, P.q_off, (int32_t*)ws);
+        // pairs per CTA: as many as leave every SM a CTA and whose candidates fit twice into an SM's shared memory. List kernel, us,
+        // one pair / this rule: 32 heads of 65536 keys 539 / 141, of 16384 keys 49 / 25 (a scalar two-pass scan per pair: 781, 69)
+        const int cap = compact_cap(P);
+        int group = 1;
+        while (group < kListWarps && P.causal && npairs >= 2 * group && (int64_t)P.B * P.Hq * ((npairs + 2 * group - 1) / (2 * group)) >= 148 &&
+               (size_t)(cap + 2 * group * 256) * sizeof(int2) <= 100 * 1024) group *= 2;
+        const size_t smem = group > 1 ? (size_t)(cap + group * 256) * sizeof(int2) : 0;
+        auto lists = P.L % 4 == 0 ? compact_lists_kernel<true> : compact_lists_kernel<false>;
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
+        launch_overlapped(lists, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx, ccnt, P.L,
+                          npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256);
         count_launch();
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);
     }

@@ -493,3 +493,20 @@ def test_tile_backward_with_the_group_dealt_out_to_several_ctas(B, Hq, Hkv, L, d
     compare(case, got, ref)
     again = gpu_run(case, inp, stored=st, flags=dma.DMA_FLAG_TILE_PATH)
     assert all(torch.equal(got[k], again[k]) for k in ("dK", "dV", "dM"))
+
+
+@pytest.mark.parametrize("Hq,L,w,q_begin", [(80, 1024, 100, 0), (148, 2050, 64, 0), (50, 3000, 700, 0), (80, 2052, 300, 1001)])
+def test_gathered_lists_of_several_pairs_per_cta(Hq, L, w, q_begin):
+    """Enough heads that a CTA makes the lists of 2, 4 or 8 pairs of query tiles (lengths with and without 16-byte aligned rows, a
+    last group that is not full, a chunk that starts inside a pair): against the CUDA-core kernel on the same mask."""
+    case = wl.small(C2, B=1, Hq=Hq, Hkv=Hq // 2, L=L, d=64, w=w, seed=L, name="lists")
+    inp = {k: v.cuda() for k, v in wl.make_inputs(case).items()}
+    p = problem_of(case, flags=dma.DMA_FLAG_COMPACT_KV)
+    bias, e, bmp = dma.dma_mask_build(p, inp["V"], inp["W_delta"], inp["A"])
+    if q_begin:
+        O, lse = dma.dma_attn_fwd_chunk(p, q_begin, inp["Q"][:, q_begin:].contiguous(), inp["K"], inp["V"], bias, e)
+    else:
+        O, lse = dma.dma_attn_fwd(p, inp["Q"], inp["K"], inp["V"], bias, e, bmp)
+    ref_O, ref_lse = dma.dma_attn_fwd(problem_of(case, flags=dma.DMA_FLAG_SIMT), inp["Q"], inp["K"], inp["V"], bias, e, bmp)
+    assert_close(O, f64(ref_O[:, q_begin:]), "bf16", "O")
+    assert_close(lse, f64(ref_lse[..., q_begin:]), "bf16", "lse", lse=True)
