@@ -2,15 +2,17 @@
 // Eq. delta_calc differentiated, the top-w selection held fixed):
 //   z = v . W_h, sp = softplus(z), delta = exp(A_h sp)   (delta is taken from the forward's bias output)
 //   g = dM delta;  dA_h = sum g sp;  dz = g A_h sigmoid(z);  dW_h = sum dz v;  dV[j, kv head] += sum_h dz W_h
-// HBM-bound: V and dV rows are read once, dV written once. One CTA owns 64 consecutive keys of one (batch, KV head)
-// and all G query heads of the group; dW / dA partial sums go to the workspace and a second kernel adds them in a
-// fixed order (no floating-point atomics: the result does not depend on the launch schedule).
+// HBM-bound: V and dV rows are read once, dV written once. A CTA walks keys of one (batch, KV head) with all G query heads of
+// the group; its dW / dA sums go to the workspace and a second kernel adds them in a fixed order (no floating-point atomics:
+// the result does not depend on the launch schedule).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace dma {
 namespace {
 
-constexpr int kRows = 64;      // keys per CTA
+constexpr int kRows = 8;       // keys per warp and unit
 constexpr int kThreads = 256;
 
 __device__ __forceinline__ void load8f(const float* p, float (&v)[8]) {
@@ -39,121 +41,233 @@ __device__ __forceinline__ void store8f(__nv_bfloat16* p, const float (&v)[8]) {
     *reinterpret_cast<uint4*>(p) = o;
 }
 
-// A group of D/8 lanes owns a key row (8 channels per lane); each thread keeps its rows of V and of the dV update in
-// registers while the query heads of the group are walked, so V is read exactly once.
-// partial [blocks][G][D + 1]: per CTA the sums over its keys of dz v (D values) and of g sp (1 value).
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) mask_bwd_kernel(const T* __restrict__ V, const float* __restrict__ W,
+// A warp takes units of eight consecutive keys of its (batch, KV head) pair, grid-stride; a group of D/8 lanes owns a row (8
+// channels per lane). Nothing is shared between warps until the end, so there is no barrier in the loop: the next unit's value
+// rows and dM, delta are requested before the current unit is worked on, z of four heads at a time goes through a transposing
+// butterfly, softplus / sigmoid are evaluated once per (row, head) pair by one lane of the row's group, and the sums dW, dA stay
+// in registers over all units (kG = G heads; kG = 0, any other G: in the warp's part of shared memory). Two CTAs per SM in all,
+// one partial sum per CTA: at L = 16384, 32 / 8 heads, d = 128 (105 MB) 64 -> 28.9 us and the sum of the partials 13.4 -> 4.1
+// us, against CTAs of 64 keys that each staged, synchronised and wrote partials.
+// partial [CTAs of the pair][G][D + 1]: the sums over the CTA's keys of dz v (D values) and of g sp (1 value).
+template <typename T> struct Row8;
+template <> struct Row8<__nv_bfloat16> {
+    uint4 a;
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { a = *reinterpret_cast<const uint4*>(p); }
+    __device__ __forceinline__ void clear() { a = make_uint4(0u, 0u, 0u, 0u); }
+    __device__ __forceinline__ void get(float (&v)[8]) const {
+        const uint32_t u[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { v[2 * i] = __uint_as_float(u[i] << 16); v[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
+    }
+};
+template <> struct Row8<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float* p) { a = *reinterpret_cast<const float4*>(p); b = *reinterpret_cast<const float4*>(p + 4); }
+    __device__ __forceinline__ void clear() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
+};
+
+template <typename T, int D, int kG>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) mask_bwd_kernel(const T* __restrict__ V, const float* __restrict__ W,
                                                             const float* __restrict__ A, const float* __restrict__ delta,
                                                             const float* __restrict__ dM, T* __restrict__ dV,
-                                                            float* __restrict__ partial, int L, int Hq, int G,
+                                                            float* __restrict__ partial, int L, int Hq, int G_,
                                                             int64_t vs_b, int64_t vs_l, int64_t vs_h) {
     constexpr int LPR = D / 8;                       // lanes per row
-    constexpr int RPW = 32 / LPR;                    // rows per warp and pass
-    constexpr int NR = kRows / (8 * RPW);            // rows per thread
+    constexpr int RPW = 32 / LPR;                    // rows per warp instruction
+    constexpr int NR = kRows / RPW;                  // rows per thread and unit
+    const int G = kG ? kG : G_;
+    constexpr int kPairs = kG ? (NR * kG + LPR - 1) / LPR : 1;      // (row, head) pairs per lane whose dM, delta are requested ahead
     extern __shared__ float smem[];
     float* sW = smem;                                // [G][D]
     float* sAcc = smem + G * D;                      // [8 warps][G][D + 1]
-    const int hk = blockIdx.y, b = blockIdx.z, j0 = blockIdx.x * kRows;
+    const int hk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = lane % LPR, grp = lane / LPR;
+    float* myZ = sAcc + 8 * G * (D + 1) + (warp * RPW + grp) * 2 * NR * G;      // z, then dz, of the group's (row, head) pairs
+    float* myGs = myZ + NR * G;                      // dM delta softplus(z)
+    float* wAcc = sAcc + (size_t)warp * G * (D + 1);
     pdl_enter(V, W, A, delta, dM, dV, partial);
-    float* sGD = sAcc + 8 * G * (D + 1);             // [G][kRows]: dM * delta of the CTA's keys, fetched in one batch
     for (int i = tid; i < G * D; i += kThreads) sW[i] = W[(size_t)hk * G * D + i];
-    for (int i = tid; i < G * kRows; i += kThreads) {
-        const int g = i / kRows, j = j0 + i % kRows;
-        const size_t at = ((size_t)b * Hq + hk * G + g) * L + j;
-        sGD[i] = j < L ? dM[at] * delta[at] : 0.0f;
-    }
+    if (kG == 0)
+        for (int i = lane; i < G * (D + 1); i += 32) wAcc[i] = 0.0f;
     __syncthreads();
-
-    float v[NR][8], upd[NR][8];
-#pragma unroll
-    for (int n = 0; n < NR; ++n) {
-        const int j = j0 + warp * RPW + n * 8 * RPW + grp;
-        if (j < L) {
-            load8f(V + b * vs_b + (int64_t)j * vs_l + hk * vs_h + sub * 8, v[n]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) v[n][c] = 0.0f;
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) upd[n][c] = 0.0f;
-    }
-    // z of every (row, head) pair of the lane group, then softplus / sigmoid ONCE per pair (the LPR lanes of a group would
-    // all repeat the same forty instructions): lane `sub` takes the pairs sub, sub + LPR, ... and leaves dz and
-    // dM delta softplus(z) in shared memory for the whole group
-    float* sDz = sGD + G * kRows;                     // [8 warps][RPW][NR * G]
-    float* sGs = sDz + 8 * RPW * NR * G;              // same shape
-    float* myDz = sDz + (warp * RPW + grp) * NR * G;
-    float* myGs = sGs + (warp * RPW + grp) * NR * G;
-    for (int g = 0; g < G; ++g) {
-        float w[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) w[c] = sW[g * D + sub * 8 + c];
+    const T* Vb = V + b * vs_b + hk * vs_h + sub * 8;
+    T* dVb = dV + b * vs_b + hk * vs_h + sub * 8;
+    const size_t head0 = ((size_t)b * Hq + hk * G) * L;
+    const int units = (L + kRows - 1) / kRows, stride = gridDim.x * 8;
+    auto request = [&](int u, Row8<T> (&v)[NR], float (&gd)[kPairs]) {
 #pragma unroll
         for (int n = 0; n < NR; ++n) {
-            float z = 0.0f;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) z = fmaf(v[n][c], w[c], z);
-#pragma unroll
-            for (int m = 1; m < LPR; m <<= 1) z += __shfl_xor_sync(0xffffffffu, z, m);
-            if (sub == 0) myDz[n * G + g] = z;
+            const int j = u * kRows + n * RPW + grp;
+            if (u < units && j < L) v[n].load(Vb + (int64_t)j * vs_l);
+            else v[n].clear();
         }
-    }
-    __syncwarp();
-    for (int pr = sub; pr < NR * G; pr += LPR) {
-        const int n = pr / G, g = pr % G;
-        const int j = j0 + warp * RPW + n * 8 * RPW + grp;
-        const float z = myDz[pr];
-        const float gd = sGD[g * kRows + (j - j0)];
-        const float e = expf(-fabsf(z));                       // in (0, 1]
-        const float sp = fmaxf(z, 0.0f) + log1pf(e);
-        const float sig = (z >= 0.0f ? 1.0f : e) / (1.0f + e);
-        myDz[pr] = gd * A[hk * G + g] * sig;
-        myGs[pr] = gd * sp;
-    }
-    __syncwarp();
-    for (int g = 0; g < G; ++g) {
-        float w[8], pw[8], pa = 0.0f;
+        if constexpr (kG > 0) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) { w[c] = sW[g * D + sub * 8 + c]; pw[c] = 0.0f; }
-#pragma unroll
-        for (int n = 0; n < NR; ++n) {
-            const float dz = myDz[n * G + g];
-            if (sub == 0) pa += myGs[n * G + g];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                pw[c] = fmaf(dz, v[n][c], pw[c]);
-                upd[n][c] = fmaf(dz, w[c], upd[n][c]);
+            for (int q = 0; q < kPairs; ++q) {
+                const int pr = sub + q * LPR, j = u * kRows + pr / kG * RPW + grp;
+                const bool in = pr < NR * kG && u < units && j < L;
+                const size_t at = head0 + (size_t)(pr % kG) * L + j;
+                gd[q] = in ? dM[at] * delta[at] : 0.0f;
             }
         }
-        // lanes with the same channel slice (the RPW row groups of the warp) are added by shuffles, then each warp
-        // leaves its sums in its own shared-memory slice; the slices are added in warp order below
+    };
+    float pw[kG ? kG : 1][8], ga[kPairs];
 #pragma unroll
-        for (int m = LPR; m < 32; m <<= 1) {
+    for (int g = 0; g < (kG ? kG : 1); ++g)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) pw[c] += __shfl_xor_sync(0xffffffffu, pw[c], m);
-            pa += __shfl_xor_sync(0xffffffffu, pa, m);
+        for (int c = 0; c < 8; ++c) pw[g][c] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kPairs; ++q) ga[q] = 0.0f;
+    Row8<T> cur[NR], nxt[NR];
+    float gd[kPairs], gdn[kPairs];
+    int u = blockIdx.x * 8 + warp;
+    request(u, cur, gd);
+    for (; u < units; u += stride) {
+        Row8<T> old[NR];                             // the dV rows to be updated
+#pragma unroll
+        for (int n = 0; n < NR; ++n) {
+            const int j = u * kRows + n * RPW + grp;
+            if (j < L) old[n].load(dVb + (int64_t)j * vs_l);
         }
-        if (grp == 0) {
-            float* dst = sAcc + ((size_t)warp * G + g) * (D + 1);
+        request(u + stride, nxt, gdn);
+        // z of the unit's (row, head) pairs: heads in blocks of 4 (then 2, then 1)
+        auto block = [&](int g0, auto nb_tag) {
+            constexpr int NB = decltype(nb_tag)::value;
+            float w[NB][8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) dst[sub * 8 + c] = pw[c];
-            if (sub == 0) dst[D] = pa;
+            for (int q = 0; q < NB; ++q) load8f(sW + (g0 + q) * D + sub * 8, w[q]);
+#pragma unroll
+            for (int n = 0; n < NR; ++n) {
+                float v[8], p[NB];
+                cur[n].get(v);
+#pragma unroll
+                for (int q = 0; q < NB; ++q) {
+                    p[q] = 0.0f;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) p[q] = fmaf(v[c], w[q][c], p[q]);
+                }
+#pragma unroll
+                for (int m = 1, keep = NB >> 1; m < LPR; m <<= 1, keep >>= 1) {      // a lane keeps half of its heads per level, then plain sums
+                    if (keep >= 1) {
+                        const bool up = (sub & m) != 0;
+#pragma unroll
+                        for (int q = 0; q < NB / 2; ++q) {
+                            if (q < keep) {
+                                const float stay = up ? p[q + keep] : p[q], give = up ? p[q] : p[q + keep];
+                                p[q] = stay + __shfl_xor_sync(0xffffffffu, give, m);
+                            }
+                        }
+                    } else {
+                        p[0] += __shfl_xor_sync(0xffffffffu, p[0], m);
+                    }
+                }
+                int mine = 0;                        // the head of the block this lane ends up with
+#pragma unroll
+                for (int m = 1, t = NB >> 1; m < NB; m <<= 1, t >>= 1) mine |= (sub & m) ? t : 0;
+                if (sub < NB) myZ[n * G + g0 + mine] = p[0];
+            }
+        };
+        int g0 = 0;
+        for (; g0 + 4 <= G; g0 += 4) block(g0, std::integral_constant<int, 4>{});
+        if (g0 + 2 <= G) { block(g0, std::integral_constant<int, 2>{}); g0 += 2; }
+        if (g0 < G) block(g0, std::integral_constant<int, 1>{});
+        __syncwarp();
+        auto pair_of = [&](int pr, float gdv) {      // dz to the row group's scratch; returns g softplus(z)
+            const float z = myZ[pr], e = expf(-fabsf(z));            // e in (0, 1]
+            myZ[pr] = gdv * A[hk * G + pr % G] * ((z >= 0.0f ? 1.0f : e) / (1.0f + e));
+            return gdv * (fmaxf(z, 0.0f) + log1pf(e));
+        };
+        if constexpr (kG > 0) {
+#pragma unroll
+            for (int q = 0; q < kPairs; ++q)
+                if (sub + q * LPR < NR * kG) ga[q] += pair_of(sub + q * LPR, gd[q]);       // (LPR is a multiple of kG: always head sub % kG)
+        } else {
+            for (int pr = sub; pr < NR * G; pr += LPR) {
+                const int j = u * kRows + pr / G * RPW + grp;
+                const size_t at = head0 + (size_t)(pr % G) * L + j;
+                myGs[pr] = pair_of(pr, j < L ? dM[at] * delta[at] : 0.0f);
+            }
         }
+        __syncwarp();
+        float upd[NR][8];
+#pragma unroll
+        for (int n = 0; n < NR; ++n)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) upd[n][c] = 0.0f;
+        auto head = [&](int g, float (&pg)[8]) {
+            float w[8];
+            load8f(sW + g * D + sub * 8, w);
+#pragma unroll
+            for (int n = 0; n < NR; ++n) {
+                const float dz = myZ[n * G + g];
+                float v[8];
+                cur[n].get(v);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    pg[c] = fmaf(dz, v[c], pg[c]);
+                    upd[n][c] = fmaf(dz, w[c], upd[n][c]);
+                }
+            }
+        };
+        if constexpr (kG > 0) {
+#pragma unroll
+            for (int g = 0; g < kG; ++g) head(g, pw[g]);
+        } else {
+            for (int g = 0; g < G; ++g) {
+                float pg[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, pa = 0.0f;
+                head(g, pg);
+                if (sub == 0)
+                    for (int n = 0; n < NR; ++n) pa += myGs[n * G + g];
+#pragma unroll
+                for (int m = LPR; m < 32; m <<= 1) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) pg[c] += __shfl_xor_sync(0xffffffffu, pg[c], m);
+                    pa += __shfl_xor_sync(0xffffffffu, pa, m);
+                }
+                if (grp == 0) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) wAcc[g * (D + 1) + sub * 8 + c] += pg[c];
+                    if (sub == 0) wAcc[g * (D + 1) + D] += pa;
+                }
+            }
+        }
+#pragma unroll
+        for (int n = 0; n < NR; ++n) {
+            const int j = u * kRows + n * RPW + grp;
+            if (j < L) {
+                float o[8];
+                old[n].get(o);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) o[c] += upd[n][c];
+                store8f(dVb + (int64_t)j * vs_l, o);
+            }
+        }
+        __syncwarp();                                // the scratch may be written again
+#pragma unroll
+        for (int n = 0; n < NR; ++n) cur[n] = nxt[n];
+#pragma unroll
+        for (int q = 0; q < kPairs; ++q) gd[q] = gdn[q];
     }
+    if constexpr (kG > 0) {
+        float pa = 0.0f;
 #pragma unroll
-    for (int n = 0; n < NR; ++n) {
-        const int j = j0 + warp * RPW + n * 8 * RPW + grp;
-        if (j < L) {
-            T* p = dV + b * vs_b + (int64_t)j * vs_l + hk * vs_h + sub * 8;
-            float cur[8];
-            load8f(p, cur);
+        for (int q = 0; q < kPairs; ++q) pa += ga[q];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) cur[c] += upd[n][c];
-            store8f(p, cur);
+        for (int m = kG; m < 32; m <<= 1) pa += __shfl_xor_sync(0xffffffffu, pa, m);      // lanes of the same head: equal sub % kG
+#pragma unroll
+        for (int g = 0; g < kG; ++g) {
+#pragma unroll
+            for (int m = LPR; m < 32; m <<= 1)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) pw[g][c] += __shfl_xor_sync(0xffffffffu, pw[g][c], m);
+            if (grp == 0) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) wAcc[g * (D + 1) + sub * 8 + c] = pw[g][c];
+            }
         }
+        if (lane < kG) wAcc[lane * (D + 1) + D] = pa;
     }
     __syncthreads();
     const size_t blk = ((size_t)b * gridDim.y + hk) * gridDim.x + blockIdx.x;
@@ -373,6 +487,12 @@ static int full_rows(const Prob& P) {
     return 0;
 }
 
+// CTAs of a (batch, KV head) pair: two per SM in all, eight units of eight keys per CTA and turn
+int ctas_per_pair(const Prob& P) {
+    const int pairs = P.B * P.Hkv, want = (2 * 148 + pairs - 1) / pairs, most = (P.L + 8 * kRows - 1) / (8 * kRows);
+    return want < most ? want : most;
+}
+
 }  // namespace
 
 size_t mask_bwd_ws_bytes(const Prob& P) {
@@ -381,18 +501,18 @@ size_t mask_bwd_ws_bytes(const Prob& P) {
         if (R == 0) return 0;
         return (size_t)P.B * ((P.L + R - 1) / R) * P.Hq * ((size_t)P.Hkv * P.d + 1) * sizeof(float);
     }
-    const size_t nblk = (size_t)(P.L + kRows - 1) / kRows;
-    return (size_t)P.B * P.Hkv * nblk * P.G * (P.d + 1) * sizeof(float);
+    return (size_t)P.B * P.Hkv * ctas_per_pair(P) * P.G * (P.d + 1) * sizeof(float);
 }
 
 template <typename T, int D>
 static int launch_typed(const Prob& P, const void* V, const float* W, const float* A, const float* delta, const float* dM,
                         void* dV, float* dW, float* dA, void* ws, cudaStream_t st) {
-    const int nblk = (P.L + kRows - 1) / kRows;
-    const size_t smem = (size_t)P.G * (D + 8 * (D + 1) + 3 * kRows) * sizeof(float);
-    if (cudaFuncSetAttribute(mask_bwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-    launch_overlapped(mask_bwd_kernel<T, D>, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
-                                                                            P.G, P.vs[0], P.vs[1], P.vs[2]);
+    const int nblk = ctas_per_pair(P);
+    const size_t smem = (size_t)P.G * (D + 8 * (D + 1) + 8 * 2 * kRows) * sizeof(float);
+    auto kern = P.G == 1 ? mask_bwd_kernel<T, D, 1> : P.G == 2 ? mask_bwd_kernel<T, D, 2> : P.G == 4 ? mask_bwd_kernel<T, D, 4> : mask_bwd_kernel<T, D, 0>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
+    launch_overlapped(kern, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
+                      P.G, P.vs[0], P.vs[1], P.vs[2]);
     launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(P.Hq), dim3((D == 128 ? 4 : 8) * (D + 1)), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G, nblk);
     count_launch(2);
     return check_launch();

@@ -67,3 +67,12 @@ def test_argument_checks():
     with pytest.raises(dma.DmaError) as e:
         dma.dma_mask_bwd(p, V, W, A, bias, dM, V.clone(), ws=tiny)
     assert e.value.status == -5
+
+
+@pytest.mark.parametrize("G", [1, 2, 3, 4, 6])
+@pytest.mark.parametrize("L,d,dtype", [(1, 64, "bf16"), (7, 128, "bf16"), (9, 64, "fp32"), (2500, 128, "bf16"), (6001, 64, "bf16")])
+def test_group_sizes_and_ragged_units(G, L, d, dtype):
+    """Every way of holding the group's sums (registers for 1, 2, 4 heads, shared memory otherwise), units of eight keys that are
+    not full, and warps that take several units."""
+    run_case(wl.small(wl.CONFIGS["2"], name="mask-bwd-units", backward=True, B=1, Hq=2 * G, Hkv=2, L=L, d=d, w=max(1, L // 4), dtype=dtype, seed=L + G),
+             seed=13)
