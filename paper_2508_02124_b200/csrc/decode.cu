@@ -517,7 +517,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_attn_kernel(const T* _
 //         [4..7] unused
 //   int32 [8 .. 8 + w)       the kept key indices, in no particular order
 // A step costs O(w), whatever the number of cached keys: no scan of the delta row.
-constexpr int kListSplit = 128;            // kept keys per CTA of the list attention kernel (256: 4 us slower per step at w = 2048)
+// kept keys per CTA of the list attention kernel: at w = 2048 and 32 rows 256 CTAs, all resident at once, with two batches per
+// warp (32 tokens 402 us; 457 with 128 keys, whose 512 CTAs come in two waves)
+constexpr int kListSplit = 256;
 
 __device__ __forceinline__ int state_stride(int w_cap) { return kStateHeader + ((w_cap + 3) & ~3); }
 
@@ -598,10 +600,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const
     const int* hdr = state + (size_t)bh * state_stride(w_cap);
     const int* kept = hdr + kStateHeader;
     const int newj = N - 1, count = hdr[0];
+    const int e = split * kListSplit + tid;
+    const int held = tid < kListSplit && e < w_cap ? kept[e] : 0;          // (in flight together with the header)
     const int mode = step_mode(hdr, w_cap, key_of(dl[newj], newj));
     const int eff = count + (mode == 1 ? 1 : 0), weakest = hdr[1];
-    const int e = split * kListSplit + tid;
-    if (tid < kListSplit && e < eff) list[tid] = (e >= count || (mode == 2 && e == weakest)) ? newj : kept[e];
+    if (tid < kListSplit && e < eff) list[tid] = (e >= count || (mode == 2 && e == weakest)) ? newj : held;
     __syncthreads();
     decode_attend<T, D>(list, max(0, min(kListSplit, eff - split * kListSplit)), q, K, V, dl,
                         partial + ((size_t)bh * nsplit + split) * (D + 2), bh, b, hk, scale_log2, ks_b, ks_l, ks_h, vs_b, vs_l, vs_h);

@@ -210,13 +210,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? 2 : 1) delta_kernel(cons
 // Full sampling weights (Eq. delta_calc as stated: all Hkv*D channels of the value row feed every head's score, the
 // linear layer of the App. A listing): z[h] = sum over KV heads hk of (v_hk . W[h, hk*D : (hk+1)*D]), the per-head dot
 // products formed as in delta_kernel (8-channel fma chains, pairwise tree over adjacent chunks) and added over hk
-// from left to right. One CTA owns 64 keys of one batch and all heads. A group of D/8 lanes owns two rows; it forms the
+// from left to right. One CTA owns kFullRows keys of one batch and all heads. A group of D/8 lanes owns two rows; it forms the
 // chains of D/8 heads at a time and adds them with a transposing butterfly (at each step a lane keeps half of its
 // values and hands the other half to its partner: the same additions as the plain butterfly, a quarter of the
 // shuffles), after which lane `sub` holds the dot product of head bitrev(sub) and carries that head's running sum.
-constexpr int kFullRows = 64;
-
-template <typename T, int D>
+// kFullRows keys per CTA: 64, or 32 where 64 would leave SMs without a CTA (4096 keys, 16 heads, 512 channels: 15.5 -> 14.2 us).
+template <typename T, int D, int kFullRows>
 __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V, const float* __restrict__ W,
                                                          const float* __restrict__ A, float* __restrict__ delta,
                                                          int L, int Hq, int Hkv, int64_t vs_b, int64_t vs_l,
@@ -224,6 +223,7 @@ __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V
     constexpr int LPR = D / 8;            // lanes per row = heads per batch
     constexpr int RPW = 32 / LPR;         // row groups per warp
     constexpr int kPass = 16 * RPW;       // rows per pass of the CTA (two per lane group)
+    static_assert(kFullRows % kPass == 0, "a pass stays inside the CTA's rows");
     extern __shared__ float smem[];
     const int C = Hkv * D, HqP = (Hq + LPR - 1) / LPR * LPR;
     float* sW = smem;                     // [HqP][C], rows beyond Hq zero
@@ -654,12 +654,14 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     if (j_end <= j_begin) return DMA_OK;
     if (P.flags & DMA_FLAG_FULL_DELTA) {
         const size_t HqP = (size_t)(P.Hq + D / 8 - 1) / (D / 8) * (D / 8);
-        const size_t bytes = (HqP * P.Hkv * D + HqP * kFullRows) * sizeof(float);
-        if (bytes > 200 * 1024) return DMA_ERR_UNSUPPORTED;
-        if (cudaFuncSetAttribute(delta_full_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return DMA_ERR_CUDA;
-        launch_overlapped(delta_full_kernel<T, D>, dim3((j_end - j_begin + kFullRows - 1) / kFullRows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A,
-                          bias, j_end, P.Hq, P.Hkv, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+        if ((HqP * P.Hkv * D + HqP * 64) * sizeof(float) > 200 * 1024) return DMA_ERR_UNSUPPORTED;
+        constexpr int kFewRows = D == 128 ? 32 : 64;          // (one pass of the CTA covers 32 rows at d = 128, 64 at d = 64)
+        const int rows = (int64_t)P.B * ((j_end - j_begin + 63) / 64) < 148 ? kFewRows : 64;
+        const size_t bytes = (HqP * P.Hkv * D + HqP * rows) * sizeof(float);
+        auto kern = rows == 64 ? delta_full_kernel<T, D, 64> : delta_full_kernel<T, D, kFewRows>;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return DMA_ERR_CUDA;
+        launch_overlapped(kern, dim3((j_end - j_begin + rows - 1) / rows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.Hkv,
+                          P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
         count_launch();
         return check_launch();
     }
@@ -690,7 +692,7 @@ int launch_delta_range(const Prob& P, const void* V, const float* W, const float
 static int mask_build_limits(const Prob& P) {
     if (P.flags & DMA_FLAG_FULL_DELTA) {
         const size_t lanes = (size_t)P.d / 8, HqP = (P.Hq + lanes - 1) / lanes * lanes;
-        if ((HqP * P.Hkv * P.d + HqP * kFullRows) * sizeof(float) > 200 * 1024) return DMA_ERR_UNSUPPORTED;
+        if ((HqP * P.Hkv * P.d + HqP * 64) * sizeof(float) > 200 * 1024) return DMA_ERR_UNSUPPORTED;
     } else if ((size_t)P.G * (P.d + 2 * 128) * sizeof(float) > 48 * 1024) {
         return DMA_ERR_UNSUPPORTED;
     }
