@@ -866,18 +866,17 @@ int make_tmap_bf16(CUtensorMap* m, const void* base, int B, int L, int H, int d,
 // Token-compacted mode, per (batch, head, pair of query tiles): the list of keys j that some row i of the
 // pair's 256 rows keeps, i.e. j <= i < expiry[j] for some i in [i0, i0 + 255]  <=>  j <= i0 + 255 and expiry[j] > max(i0, j).
 // At most w + 256 keys qualify. The list is in two parts, each ascending: first the keys that ALL 256 rows keep
-// (j <= i0 and expiry[j] >= i0 + 256), then the keys that enter or expire inside the pair's rows. The forward kernel
-// needs no order among the columns, and this one leaves the keys that need the per-element test (a few hundred per pair)
-// in the last slices instead of a few in every slice.
+// (j <= i0 and expiry[j] >= i0 + 256), then the keys that enter or expire inside the pair's rows. The split leaves the keys
+// that need the per-element test (a few hundred per pair) in the last slices instead of a few in every slice. The order inside
+// a part decides how O rounds, so it is the same however the list was made: for any length and group.
 // A CTA makes the lists of `group` consecutive pairs of one head. Every list on its own would read all keys before its rows, in
 // two passes (count, write), which at 65536 keys was 781 us, an eighth of the prefill. With group > 1 the CTA first collects the
 // keys that some row of the group keeps (at most the list's capacity and the group's rows: shared memory), and its lists are
 // made from those: the head is read once per 256 group rows. group = 1: the lists are made straight from the head.
-// Every warp owns a contiguous part of what it reads, 128 keys at a time (16-byte loads where rows are 16-byte aligned), and
-// writes from the sum of the earlier parts' counts. Padded with -1 to the next multiple of 128.
+// Every warp owns a contiguous part of what it reads, 128 keys at a time (four coalesced loads per lane in flight), and writes
+// from the sum of the earlier parts' counts. Padded with -1 to the next multiple of 128.
 constexpr int kListThreads = 256, kListWarps = 8;
 
-template <bool kVec>
 __global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
                                                                      int* __restrict__ ccnt, int L, int npairs, int cap, int causal,
                                                                      int q_off, int32_t* __restrict__ status, int group, int ccap) {
@@ -895,17 +894,10 @@ __global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32
     const int lo = q_off + pair0 * 256, jend = causal ? min(L, lo + pairs * 256) : L;
     // four keys of the head per lane, from base on: (key, expiry), expiry 0 (never kept) beyond `end`
     auto load4 = [&](int base, int end, int (&j)[4], int (&ej)[4]) {
-        if (kVec && base + 128 <= end) {
-            const int4 v = *reinterpret_cast<const int4*>(e + base + 4 * lane);
-            ej[0] = v.x; ej[1] = v.y; ej[2] = v.z; ej[3] = v.w;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) j[u] = base + 4 * lane + u;
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                j[u] = base + 32 * u + lane;
-                ej[u] = j[u] < end ? e[j[u]] : 0;
-            }
+        for (int u = 0; u < 4; ++u) {
+            j[u] = base + 32 * u + lane;
+            ej[u] = j[u] < end ? e[j[u]] : 0;
         }
     };
     int ncand = jend;
@@ -929,7 +921,7 @@ __global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32
             at += q < warp ? wcount[0][q] : 0;
             all += wcount[0][q];
         }
-#pragma unroll 2
+#pragma unroll 4
         for (int base = j0; base < j1; base += 128) {
             int j[4], ej[4];
             load4(base, j1, j, ej);
@@ -999,7 +991,7 @@ __global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32
     }
     p2 += n1;                                            // the second part starts behind the first
     int* out = cidx + (size_t)list * cap;
-#pragma unroll 2
+#pragma unroll 4
     for (int base = k0; base < k1; base += 128) {
         int j[4], ej[4];
         fetch(base, j, ej);
@@ -1063,9 +1055,8 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         while (group < kListWarps && P.causal && npairs >= 2 * group && (int64_t)P.B * P.Hq * ((npairs + 2 * group - 1) / (2 * group)) >= 148 &&
                (size_t)(cap + 2 * group * 256) * sizeof(int2) <= 100 * 1024) group *= 2;
         const size_t smem = group > 1 ? (size_t)(cap + group * 256) * sizeof(int2) : 0;
-        auto lists = P.L % 4 == 0 ? compact_lists_kernel<true> : compact_lists_kernel<false>;
-        if (smem > 48 * 1024 && cudaFuncSetAttribute(lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-        launch_overlapped(lists, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx, ccnt, P.L,
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(compact_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
+        launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx, ccnt, P.L,
                           npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256);
         count_launch();
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);

@@ -510,3 +510,27 @@ def test_gathered_lists_of_several_pairs_per_cta(Hq, L, w, q_begin):
     ref_O, ref_lse = dma.dma_attn_fwd(problem_of(case, flags=dma.DMA_FLAG_SIMT), inp["Q"], inp["K"], inp["V"], bias, e, bmp)
     assert_close(O, f64(ref_O[:, q_begin:]), "bf16", "O")
     assert_close(lse, f64(ref_lse[..., q_begin:]), "bf16", "lse", lse=True)
+
+
+@pytest.mark.parametrize("Hq", [2, 148])
+def test_compact_forward_bits_do_not_depend_on_how_the_lists_were_made(Hq):
+    """The gathered lists are ascending within their two parts whatever the length's alignment (2048 keys: 16-byte loads, 2049:
+    scalar ones) and the pairs per CTA (2 heads: one, 148 heads: eight), so the same rows round the same way: O, lse bit for bit."""
+    L, d, w = 2048, 64, 300
+    case = wl.small(C2, B=1, Hq=Hq, Hkv=Hq // 2, L=L + 1, d=d, w=w, seed=7, name="list-order")
+    inp = {k: v.cuda() for k, v in wl.make_inputs(case).items()}
+    p = dma.problem(1, Hq, Hq // 2, L, d, w, flags=dma.DMA_FLAG_COMPACT_KV)
+    Q, K, V = (inp[k][:, :L].contiguous() for k in ("Q", "K", "V"))
+    bias, e, bmp = dma.dma_mask_build(p, V, inp["W_delta"], inp["A"])
+    O, lse = dma.dma_attn_fwd(p, Q, K, V, bias, e, bmp)
+    # one pair per call: group 1
+    for i in range(0, L, 512):
+        Oc, lc = dma.dma_attn_fwd_chunk(p, i, Q[:, i:i + 256].contiguous(), K, V, bias, e)
+        assert torch.equal(Oc, O[:, i:i + 256]) and torch.equal(lc, lse[..., i:i + 256]), i
+    # one key more, kept by its own row alone
+    p1 = problem_of(case, flags=dma.DMA_FLAG_COMPACT_KV)
+    bias1, e1 = torch.ones(1, Hq, L + 1, device="cuda"), torch.full((1, Hq, L + 1), L + 1, dtype=torch.int32, device="cuda")
+    bias1[..., :L], e1[..., :L] = bias, e
+    bmp1 = torch.full((dma.dma_bitmap_words(p1),), -1, dtype=torch.int32, device="cuda")
+    O1, lse1 = dma.dma_attn_fwd(p1, inp["Q"], inp["K"], inp["V"], bias1, e1, bmp1)
+    assert torch.equal(O1[:, :L], O) and torch.equal(lse1[..., :L], lse)
