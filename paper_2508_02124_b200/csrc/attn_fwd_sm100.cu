@@ -876,6 +876,7 @@ int make_tmap_bf16(CUtensorMap* m, const void* base, int B, int L, int H, int d,
 // Every warp owns a contiguous part of what it reads, 128 keys at a time (four coalesced loads per lane in flight), and writes
 // from the sum of the earlier parts' counts. Padded with -1 to the next multiple of 128.
 constexpr int kListThreads = 256, kListWarps = 8;
+constexpr int kListSmem = 100 * 1024;       // the most dynamic shared memory a CTA takes: two fit on an SM
 
 __global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
                                                                      int* __restrict__ ccnt, int L, int npairs, int cap, int causal,
@@ -1053,11 +1054,13 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         const int cap = compact_cap(P);
         int group = 1;
         while (group < kListWarps && P.causal && npairs >= 2 * group && (int64_t)P.B * P.Hq * ((npairs + 2 * group - 1) / (2 * group)) >= 148 &&
-               (size_t)(cap + 2 * group * 256) * sizeof(int2) <= 100 * 1024) group *= 2;
+               (size_t)(cap + 2 * group * 256) * sizeof(int2) <= (size_t)kListSmem) group *= 2;
         const size_t smem = group > 1 ? (size_t)(cap + group * 256) * sizeof(int2) : 0;
-        if (smem > 48 * 1024 && cudaFuncSetAttribute(compact_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-        launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx, ccnt, P.L,
-                          npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256);
+        // (the limit is state of the function, which other threads' calls share: always the same value)
+        if (smem && cudaFuncSetAttribute(compact_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kListSmem) != cudaSuccess) return DMA_ERR_CUDA;
+        if (launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx,
+                              ccnt, P.L, npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256) != cudaSuccess)
+            return DMA_ERR_CUDA;       // the forward kernel must not run on lists that nobody wrote
         count_launch();
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);
     }

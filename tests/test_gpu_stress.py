@@ -146,3 +146,66 @@ def test_two_host_threads_on_two_streams():
     for t in threads:
         t.join()
     assert not errors, errors[:5]
+
+
+# 148 heads, 2048 rows: the lists of eight pairs of query tiles per CTA, (roundup(w + 256, 128) + 2048) * 8 bytes of shared memory
+LIST_SHAPES = {3800: 48 * 1024, 4096: 50 * 1024, 8192: 82 * 1024}
+
+
+def lists_of_eight_pairs(w, seed=0):
+    """The forward of 2048 rows with window w, on 148 heads together (eight pairs per CTA) and on each of four heads alone
+    (one pair per CTA, no dynamic shared memory): a function that runs the former, and what it has to give."""
+    H, rows, d, L = 148, 2048, 64, max(4096, w + 256)
+    g = torch.Generator(DEV).manual_seed(seed)
+    Q, K, V = (torch.randn(1, n, H, d, generator=g, device=DEV).to(torch.bfloat16) for n in (rows, L, L))
+    W, A = torch.randn(H, d, generator=g, device=DEV) / 8, torch.rand(H, generator=g, device=DEV) + 0.5
+    p, one = dma.problem(1, H, H, L, d, w), dma.problem(1, 1, 1, L, d, w)
+    bias, e, _ = dma.dma_mask_build(p, V, W, A)
+    heads = [0, 51, 52, 147]
+    pick = lambda t, h: t[:, :, h:h + 1].contiguous()                                                   # noqa: E731
+    ref = [dma.dma_attn_fwd_chunk(one, L - rows, *(pick(t, h) for t in (Q, K, V)), bias[:, h:h + 1].contiguous(), e[:, h:h + 1].contiguous())
+           for h in heads]
+    torch.cuda.synchronize()
+
+    def run():
+        O, lse = dma.dma_attn_fwd_chunk(p, L - rows, Q, K, V, bias, e)
+        torch.cuda.current_stream().synchronize()
+        return all(torch.equal(O[:, :, h:h + 1], r[0]) and torch.equal(lse[:, h:h + 1], r[1]) for h, r in zip(heads, ref))
+
+    return run
+
+
+def test_list_kernel_shared_memory_sizes_from_two_threads():
+    """Two threads whose list kernels take 50 and 82 KB of shared memory: the opt-in above 48 KB is state of the kernel that both
+    share, so a call may not lower it to its own size."""
+    import threading
+    runs = [lists_of_eight_pairs(w, seed=w) for w in (4096, 8192)]
+    bad = []
+
+    def worker(run):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                bad.extend(i for i in range(40) if not run())
+        except Exception as ex:
+            bad.append(repr(ex))
+
+    threads = [threading.Thread(target=worker, args=(r,)) for r in runs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad[:5]
+
+
+@pytest.mark.parametrize("w", sorted(LIST_SHAPES))
+def test_list_kernel_shared_memory_size_in_a_fresh_process(w):
+    """The first call of a process, at sizes on both sides of the 48 KB that need no opt-in (static shared memory counts too:
+    exactly 48 KB of dynamic shared memory does need it)."""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    assert (((w + 256 + 127) // 128) * 128 + 2048) * 8 == LIST_SHAPES[w]
+    code = f"import sys; sys.path[:0] = [{here!r}, {os.path.dirname(here)!r}]; import test_gpu_stress as t; assert t.lists_of_eight_pairs({w})()"
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
