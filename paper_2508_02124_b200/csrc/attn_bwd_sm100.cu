@@ -853,10 +853,9 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     const int per_cta = 256 / (P.d / 8) * kPrepareRows;
     const unsigned prep_ctas = (unsigned)((rows + per_cta - 1) / per_cta);
     for (int z = 0; z < 3; ++z) pp.zero_part[z] = ((pp.zero_n[z] >> 2) + prep_ctas - 1) / prep_ctas;
-    launch_overlapped(P.d == 128 ? bwd_prepare_kernel<16> : bwd_prepare_kernel<8>, dim3(prep_ctas), dim3(256), 0, st, 1, pp);
+    if ((rc = launch_overlapped(P.d == 128 ? bwd_prepare_kernel<16> : bwd_prepare_kernel<8>, dim3(prep_ctas), dim3(256), 0, st, 1, pp))) return rc;
     if (compact) {
-        launch_overlapped(lifetime_perm_kernel, dim3(P.B * P.Hq), dim3(1024), 0, st, 1, expiry, perm, P.L, P.Tc, P.causal);
-        count_launch();
+        if ((rc = launch_overlapped(lifetime_perm_kernel, dim3(P.B * P.Hq), dim3(1024), 0, st, 1, expiry, perm, P.L, P.Tc, P.causal))) return rc;
     }
     BwdParams bp;
     bp.lse = lse; bp.Dv = Dv; bp.bias = bias; bp.expiry = expiry; bp.bitmap = bitmap; bp.dQacc = acc; bp.Lblk = P.Tr * 8;
@@ -889,8 +888,9 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     auto kern = compact ? (P.d == 128 ? bwd_kernel<true, 128> : bwd_kernel<true, 64>) : (P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     timing_mark(1, false, st);
-    launch_overlapped(kern, dim3(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc), dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
+    rc = launch_overlapped(kern, dim3(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc), dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
     timing_mark(1, true, st);
+    if (rc) return rc;
     FinishParams f;
     f.dQacc = acc; f.acc[0] = accK; f.acc[1] = accV; f.dQ = (__nv_bfloat16*)dQ; f.out[0] = (__nv_bfloat16*)dK; f.out[1] = (__nv_bfloat16*)dV;
     f.L = P.L; f.Hq = P.Hq; f.Hkv = P.Hkv; f.Lblk = P.Tr * 8; f.d = P.d; f.nslots = (int)slots; f.nkv = (int64_t)nkv;
@@ -899,9 +899,7 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     f.kv_blocks = (int)((nkv / 8 + 255) / 256);
     for (int t = 0; t < 3; ++t) { f.qs[t] = P.qs[t]; f.st[0][t] = P.ks[t]; f.st[1][t] = P.vs[t]; }
     f.scale = P.scale;
-    launch_overlapped(bwd_finish_kernel, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
-    count_launch(3);
-    return check_launch();
+    return launch_overlapped(bwd_finish_kernel, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
 }
 
 }  // namespace dma

@@ -1058,10 +1058,9 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         const size_t smem = group > 1 ? (size_t)(cap + group * 256) * sizeof(int2) : 0;
         // (the limit is state of the function, which other threads' calls share: always the same value)
         if (smem && cudaFuncSetAttribute(compact_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kListSmem) != cudaSuccess) return DMA_ERR_CUDA;
-        if (launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1, expiry, cidx,
-                              ccnt, P.L, npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256) != cudaSuccess)
-            return DMA_ERR_CUDA;       // the forward kernel must not run on lists that nobody wrote
-        count_launch();
+        if ((rc = launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1,
+                                    expiry, cidx, ccnt, P.L, npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256)))
+            return rc;                 // the forward kernel must not run on lists that nobody wrote
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);
     }
     fp.Kg = (const __nv_bfloat16*)K; fp.Vg = (const __nv_bfloat16*)V;
@@ -1080,10 +1079,9 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
     dim3 grid(P.B * P.Hq, npairs);
     timing_mark(0, false, st);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-    launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, fp);
+    rc = launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, fp);
     timing_mark(0, true, st);
-    count_launch();
-    return check_launch();
+    return rc;
 }
 
 }  // namespace dma

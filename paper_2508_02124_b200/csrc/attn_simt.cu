@@ -410,11 +410,10 @@ int fwd_t(const Prob& P, const void* Q, const void* K, const void* V, const floa
     // a chunk of query rows that does not start on a bitmap row boundary (or comes without a bitmap) visits every key tile
     int use_bitmap = bitmap && !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0 && P.q_off % kTile == 0;
     timing_mark(0, false, st);
-    launch_overlapped(kern, dim3((P.Lq + kOwn * NW - 1) / (kOwn * NW), P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K, (const T*)V,
-                      bias, expiry, bitmap, (T*)O, lse, P, use_bitmap);
+    const int rc = launch_overlapped(kern, dim3((P.Lq + kOwn * NW - 1) / (kOwn * NW), P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
+                                     (const T*)V, bias, expiry, bitmap, (T*)O, lse, P, use_bitmap);
     timing_mark(0, true, st);
-    count_launch();
-    return check_launch();
+    return rc;
 }
 
 template <typename T, int D, int kOwn, int NW>
@@ -426,14 +425,14 @@ int bwd_t(const Prob& P, const void* Q, const void* K, const void* V, const void
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     const size_t rows = (size_t)P.B * P.Hq * P.L;
     float* Dv = reinterpret_cast<float*>((char*)ws + kWsHeaderBytes);
-    launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P);
+    int rc = launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P);
+    if (rc) return rc;
     int use_bitmap = !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0;
     timing_mark(1, false, st);
-    launch_overlapped(kern, dim3((P.L + kOwn * NW - 1) / (kOwn * NW), P.Hkv + P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
-                      (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap);
+    rc = launch_overlapped(kern, dim3((P.L + kOwn * NW - 1) / (kOwn * NW), P.Hkv + P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
+                           (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap);
     timing_mark(1, true, st);
-    count_launch(2);
-    return check_launch();
+    return rc;
 }
 
 // CTA size: 32 rows (four per warp, eight warps) when that gives every SM a CTA; else 8 rows (two per warp, four warps), where a

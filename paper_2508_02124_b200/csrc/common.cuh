@@ -78,8 +78,9 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
 // made of: step of 2 x 1000 rows, d = 64: 112 -> 103 us, prefill of 4096 keys 123 -> 107 us. (Letting the next kernel in early,
 // with griddepcontrol.launch_dependents at the top, was slower everywhere: its waiting CTAs take the places that the running
 // kernel's CTAs leave unevenly, 218 -> 239 us for 2048 rows of a 16384-key prefill, 2998 -> 3071 us for its training step.)
+// Returns a dma_status; a caller that gets an error launches nothing more, since the later kernels read what this one writes.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
+inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -97,7 +98,12 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 b
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...) != cudaSuccess) {
+        cudaGetLastError();              // (consumed here: it is not the next call's error)
+        return DMA_ERR_CUDA;
+    }
+    count_launch();
+    return DMA_OK;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -669,12 +669,9 @@ template <typename T, int D>
 int launch_typed(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, void* o, float* lse,
                  const int* kept, int64_t kept_stride, int* tickets, float* partial, cudaStream_t st) {
     const int per = split_keys(P), nsplit = (P.w + per - 1) / per;
-    if (launch_overlapped(decode_attn_kernel<T, D>, dim3(nsplit, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
-                          delta, ld, kept, kept_stride, partial, P.w, per, P.Hq, P.G, P.scale * 1.4426950408889634f, nsplit, P.ks[0], P.ks[1],
-                          P.ks[2], P.vs[0], P.vs[1], P.vs[2], tickets, (T*)o, lse) != cudaSuccess)
-        return DMA_ERR_CUDA;
-    count_launch();
-    return check_launch();
+    return launch_overlapped(decode_attn_kernel<T, D>, dim3(nsplit, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
+                             delta, ld, kept, kept_stride, partial, P.w, per, P.Hq, P.G, P.scale * 1.4426950408889634f, nsplit, P.ks[0], P.ks[1],
+                             P.ks[2], P.vs[0], P.vs[1], P.vs[2], tickets, (T*)o, lse);
 }
 
 }  // namespace
@@ -726,11 +723,8 @@ static int launch_select(const Prob& P, const float* delta, int64_t ld, int* lis
     };
     auto kern = state ? pick(std::true_type{}) : pick(std::false_type{});
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelectShared)) != cudaSuccess) return DMA_ERR_CUDA;
-    if (launch_overlapped(kern, dim3((unsigned)(P.B * P.Hq) * nrank), dim3(kSelectThreads), sizeof(SelectShared), st, nrank, delta, ld, P.L, P.w,
-                          slice, list, list_stride, tickets) != cudaSuccess)
-        return DMA_ERR_CUDA;
-    count_launch();
-    return check_launch();
+    return launch_overlapped(kern, dim3((unsigned)(P.B * P.Hq) * nrank), dim3(kSelectThreads), sizeof(SelectShared), st, nrank, delta, ld, P.L, P.w,
+                             slice, list, list_stride, tickets);
 }
 
 int launch_decode(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, void* o, float* lse,
@@ -757,14 +751,12 @@ template <typename T, int D>
 static int launch_step_typed(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, int* state,
                              void* o, float* lse, float* partial, cudaStream_t st) {
     const int ns = list_splits(P);
-    if (launch_overlapped(decode_list_attn_kernel<T, D>, dim3(ns, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
+    const int rc = launch_overlapped(decode_list_attn_kernel<T, D>, dim3(ns, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
                           delta, ld, (const int*)state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns, P.ks[0], P.ks[1],
-                          P.ks[2], P.vs[0], P.vs[1], P.vs[2]) != cudaSuccess ||
-        launch_overlapped(decode_step_combine_kernel<T, D>, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
-                          ld, P.L, P.w_cap, state) != cudaSuccess)
-        return DMA_ERR_CUDA;
-    count_launch(2);
-    return check_launch();
+                          P.ks[2], P.vs[0], P.vs[1], P.vs[2]);
+    if (rc) return rc;
+    return launch_overlapped(decode_step_combine_kernel<T, D>, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
+                             ld, P.L, P.w_cap, state);
 }
 
 // One decoding step with the carried state: P.L counts the cached keys INCLUDING the one appended for this step.

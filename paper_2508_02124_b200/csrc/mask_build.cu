@@ -660,10 +660,8 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
         const size_t bytes = (HqP * P.Hkv * D + HqP * rows) * sizeof(float);
         auto kern = rows == 64 ? delta_full_kernel<T, D, 64> : delta_full_kernel<T, D, kFewRows>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return DMA_ERR_CUDA;
-        launch_overlapped(kern, dim3((j_end - j_begin + rows - 1) / rows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.Hkv,
-                          P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
-        count_launch();
-        return check_launch();
+        return launch_overlapped(kern, dim3((j_end - j_begin + rows - 1) / rows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.Hkv,
+                                 P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
     }
     // two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles grid-stride; short ranges (one appended key
     // of a decoding step) get one CTA per tile
@@ -673,9 +671,7 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     dim3 grid(per_pair, P.Hkv, P.B);
     size_t smem = (size_t)P.G * (D + 2 * 128) * sizeof(float);
     if (smem > 48 * 1024) return DMA_ERR_UNSUPPORTED;
-    launch_overlapped(delta_kernel<T, D>, grid, dim3(256), smem, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
-    count_launch();
-    return check_launch();
+    return launch_overlapped(delta_kernel<T, D>, grid, dim3(256), smem, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
 }
 
 // delta for the keys [j_begin, j_end) only, into rows of ld entries (a decoding cache that grows)
@@ -718,8 +714,8 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
     const int64_t bitmap_words = (int64_t)BH * P.Tr * P.Wd;        // zeroed by the kernel after the deltas
     if (P.w >= P.L && !cu) {   // every visible key is kept
         size_t n = (size_t)BH * P.L;
-        launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, bitmap_words);
-        count_launch();
+        rc = launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, bitmap_words);
+        if (rc) return rc;
     } else {
         // rank tree: sorted chunks and the low levels, one merge pass per further level, then one walk per key
         const int Lc = nchunk * kChunk, m = tree_levels(Lc);
@@ -727,30 +723,28 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
         auto* buf0 = reinterpret_cast<unsigned long long*>((char*)ws + kWsHeaderBytes);
         auto* buf1 = buf0 + keys;
         uint2* lev = reinterpret_cast<uint2*>(buf1 + keys);
-        launch_overlapped(chunk_sort_kernel, dim3(nchunk, BH), dim3(kChunk), 0, st, 1, bias, buf0, P.L, nchunk, lev, m, bitmap, bitmap_words);
-        int launches = 2;
+        rc = launch_overlapped(chunk_sort_kernel, dim3(nchunk, BH), dim3(kChunk), 0, st, 1, bias, buf0, P.L, nchunk, lev, m, bitmap, bitmap_words);
+        if (rc) return rc;
         if (Lc > kChunk) {
-            launch_overlapped(tree_block_kernel, dim3((Lc + kBlockKeys - 1) / kBlockKeys, BH), dim3(kBlockThreads), kBlockSmem, st, 1, buf0, buf1, lev, Lc, m);
+            rc = launch_overlapped(tree_block_kernel, dim3((Lc + kBlockKeys - 1) / kBlockKeys, BH), dim3(kBlockThreads), kBlockSmem, st, 1, buf0, buf1, lev, Lc, m);
+            if (rc) return rc;
             std::swap(buf0, buf1);
-            ++launches;
         }
         int l = m - 13;                                          // level of the nodes of 2 * kBlockKeys keys
-        for (int R = kBlockKeys; R < Lc; R *= 2, --l, ++launches) {
-            launch_overlapped(tree_merge_kernel, dim3((Lc + kMergeOut - 1) / kMergeOut, BH), dim3(kMergeThreads), 0, st, 1, buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
+        for (int R = kBlockKeys; R < Lc; R *= 2, --l) {
+            rc = launch_overlapped(tree_merge_kernel, dim3((Lc + kMergeOut - 1) / kMergeOut, BH), dim3(kMergeThreads), 0, st, 1, buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
+            if (rc) return rc;
             std::swap(buf0, buf1);
         }
         const dim3 grid((P.L + 255) / 256, BH);
-        launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev, expiry,
-                          P.L, Lc, P.w, m, cu, nseq);
-        count_launch(launches);
+        rc = launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev,
+                               expiry, P.L, Lc, P.w, m, cu, nseq);
+        if (rc) return rc;
     }
-    if ((rc = check_launch())) return rc;
 
     size_t smem = (size_t)(P.Tr + 1) * sizeof(int);
     if (smem > 48 * 1024) return DMA_ERR_UNSUPPORTED;
-    launch_overlapped(bitmap_kernel, dim3(P.Tc, BH), dim3(128), smem, st, 1, expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
-    count_launch();
-    return check_launch();
+    return launch_overlapped(bitmap_kernel, dim3(P.Tc, BH), dim3(128), smem, st, 1, expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
 }
 
 }  // namespace dma

@@ -516,11 +516,11 @@ static int launch_typed(const Prob& P, const void* V, const float* W, const floa
     const size_t smem = (size_t)P.G * (D + 8 * (D + 1) + 8 * 2 * kRows) * sizeof(float);
     auto kern = P.G == 1 ? mask_bwd_kernel<T, D, 1> : P.G == 2 ? mask_bwd_kernel<T, D, 2> : P.G == 4 ? mask_bwd_kernel<T, D, 4> : mask_bwd_kernel<T, D, 0>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
-    launch_overlapped(kern, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
-                      P.G, P.vs[0], P.vs[1], P.vs[2]);
-    launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(P.Hq), dim3((D == 128 ? 4 : 8) * (D + 1)), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G, nblk);
-    count_launch(2);
-    return check_launch();
+    const int rc = launch_overlapped(kern, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
+                                     P.G, P.vs[0], P.vs[1], P.vs[2]);
+    if (rc) return rc;
+    return launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(P.Hq), dim3((D == 128 ? 4 : 8) * (D + 1)), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G,
+                             nblk);
 }
 
 template <typename T, int RW>
@@ -531,11 +531,10 @@ static int launch_full(const Prob& P, const void* V, const float* W, const float
     const size_t smem = ((size_t)R * C + (size_t)R * HqP + (size_t)P.Hq * R) * sizeof(float);
     if (cudaFuncSetAttribute(mask_bwd_full_kernel<T, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return DMA_ERR_CUDA;
-    launch_overlapped(mask_bwd_full_kernel<T, RW>, dim3(nblk, P.B), dim3(kFullThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
-                                                                          P.Hkv, P.d, P.vs[0], P.vs[1], P.vs[2]);
-    launch_overlapped(mask_bwd_full_reduce_kernel, dim3((C + 1 + 127) / 128, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
-    count_launch(2);
-    return check_launch();
+    const int rc = launch_overlapped(mask_bwd_full_kernel<T, RW>, dim3(nblk, P.B), dim3(kFullThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV,
+                                     (float*)ws, P.L, P.Hq, P.Hkv, P.d, P.vs[0], P.vs[1], P.vs[2]);
+    if (rc) return rc;
+    return launch_overlapped(mask_bwd_full_reduce_kernel, dim3((C + 1 + 127) / 128, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
 }
 
 template <typename T>

@@ -9,6 +9,7 @@ from paper_2508_02124_b200 import workloads as wl
 from helpers import assert_close, problem_of
 
 pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
 
 
 def run_case(case, seed):
@@ -76,3 +77,23 @@ def test_group_sizes_and_ragged_units(G, L, d, dtype):
     not full, and warps that take several units."""
     run_case(wl.small(wl.CONFIGS["2"], name="mask-bwd-units", backward=True, B=1, Hq=2 * G, Hkv=2, L=L, d=d, w=max(1, L // 4), dtype=dtype, seed=L + G),
              seed=13)
+
+
+def test_refused_launch_ends_the_call():
+    """More KV heads than a grid has rows: the first kernel cannot be launched, which the call reports. Then nothing else runs (the
+    second kernel would sum a workspace that nobody wrote), and the next call does not find the error."""
+    H = 65600
+    p = dma.problem(1, H, H, 1, 64, 1)
+    f32 = dict(dtype=torch.float32, device=DEV)
+    V, dV = torch.zeros(1, 1, H, 64, dtype=torch.bfloat16, device=DEV), torch.zeros(1, 1, H, 64, dtype=torch.bfloat16, device=DEV)
+    W, A, bias, dM = torch.zeros(H, 64, **f32), torch.ones(H, **f32), torch.ones(1, H, 1, **f32), torch.zeros(1, H, 1, **f32)
+    dW, dA = torch.full((H, 64), 7.0, **f32), torch.full((H,), 7.0, **f32)
+    before = dma.dma_launch_count()
+    with pytest.raises(dma.DmaError) as err:
+        dma.dma_mask_bwd(p, V, W, A, bias, dM, dV, dW, dA)
+    assert err.value.status == -6
+    torch.cuda.synchronize()
+    assert dma.dma_launch_count() == before
+    assert bool((dW == 7.0).all()) and bool((dA == 7.0).all())
+    q = dma.problem(1, 4, 4, 1, 64, 1)
+    dma.dma_mask_bwd(q, V[:, :, :4].contiguous(), W[:4], A[:4], bias[:, :4].contiguous(), dM[:, :4].contiguous(), dV[:, :, :4].contiguous())
