@@ -26,6 +26,7 @@
 //     shared-memory copy of dS^T), so the compute warps store step n+1 while the MMAs of step n still read step n's;
 //   - dQ^T = K^T dS^T keeps M = 128 with the K tile loaded a second time into the unused half of its buffer: lanes
 //     64-127 repeat lanes 0-63, so all four drain warps work, two per 32 channels, each on half of the step's rows.
+#include <algorithm>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -797,19 +798,28 @@ static size_t bwd_rows64(const Prob& P) { return ((((size_t)P.B * P.Hq * P.L) + 
 static size_t bwd_acc_floats(const Prob& P) { return (size_t)P.B * P.Hq * P.Tr * 128 * P.d; }     // rows padded to whole query tiles
 static size_t bwd_perm_ints(const Prob& P) { return (((size_t)P.B * P.Hq * P.Tc * 128) + 63) / 64 * 64; }
 
-// Tile mode: a CTA owns a key tile of one KV head and walks all its query heads. Where that leaves fewer than two CTAs per SM,
-// the group's heads are dealt out to several CTAs, whose parts of dK and dV go to slots of their own: the serial walk of the
-// heaviest CTA (2 G L / 128 steps) is what a short sequence waits for. Two batch entries of 1000 rows, 16 / 4 heads, d = 64:
-// main kernel 68.7 -> 37.5 us with four CTAs per KV head. A divisor of G, so that every (key, query head) keeps one writer of dM.
+// Tile mode: a CTA owns a key tile of one KV head and walks all its query heads. Where few CTAs wait for the heaviest one, the
+// group's heads are dealt out to several CTAs, whose parts of dK and dV go to slots of their own. The number is the divisor of G
+// (every (key, query head) keeps one writer of dM) with the shortest estimate, in 64-row steps: the heaviest CTA's walk of
+// 2 G Tr / n and kCtaSteps of fixed cost (prologue, write-out of dK and dV, its slot's pass through memory); with more CTAs than
+// SMs also the work per SM and one more fixed cost for the uneven end. Fitted to 62 shapes of 1 to 64 tiles, 16 to 256 CTAs and
+// groups of 2 to 16 heads, each timed with every divisor: within 7 % of the best one everywhere. us with one / the rule's / every
+// divisor that leaves under 296 CTAs room: 2 x 1000 rows, 16 / 4 heads, d = 64 73 / 39 / 39, 8 x 512 rows, 16 / 4 heads, d = 128
+// 73 / 78 / 101, 32 x 128 rows 45 / 45 / 92, 2048 rows, 32 / 8 heads 192 / 131 / 156.
+constexpr int kMostSplitCtas = 384;        // (no shape gained from more; the slots' space is bounded by it)
 int tc_bwd_splits(const Prob& P) {
     if (P.flags & DMA_FLAG_COMPACT_KV) return 1;
     if (P.bwd_split) return P.bwd_split;
-    const int64_t ctas = (int64_t)P.B * P.Hkv * P.Tc;
-    int n = 1;
-    while (n < P.G && ctas * n < 2 * 148) {
-        do ++n; while (P.G % n);
-    }
-    return n;
+    constexpr double kCtaSteps = 7.0, kSms = 148.0;
+    const double ctas = (double)P.B * P.Hkv * P.Tc;
+    auto steps = [&](int n) {
+        const double heaviest = kCtaSteps + 2.0 * P.Tr * P.G / n;
+        return ctas * n <= kSms ? heaviest : std::max(heaviest, ctas * (kCtaSteps * n + (P.Tr + 1.0) * P.G) / kSms + kCtaSteps);
+    };
+    int best = 1;
+    for (int n = 2; n <= P.G && ctas * n <= kMostSplitCtas; ++n)
+        if (P.G % n == 0 && steps(n) < steps(best)) best = n;
+    return best;
 }
 // copies of the dK, dV accumulators (0: the main kernel writes dK, dV itself)
 static size_t bwd_slots(const Prob& P) {

@@ -1,0 +1,43 @@
+"""Workspace sizes, host side: what the entry points ask for and accept. No GPU: a call whose arguments pass is told apart by its
+next check, which finds no device."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2508_02124_b200 import binding as dma
+from paper_2508_02124_b200 import build as dma_build
+
+no_device = pytest.mark.skipif(torch.cuda.is_available(), reason="tells accepted calls by the missing device")
+ERR_WORKSPACE, ERR_CUDA = -5, -6
+
+
+@pytest.fixture(scope="module")
+def lib():
+    dma_build.build()
+    return dma.lib()
+
+
+def backward(lib, p, ws_bytes):
+    a = ctypes.c_void_p(4096)
+    return lib.dma_attn_bwd(ctypes.byref(p), *([a] * 13), a, ctypes.c_size_t(ws_bytes), ctypes.c_void_p(0))
+
+
+def backward_bytes(B, Hq, Hkv, L, d, slots):
+    """Header, D (whole 64 rows), the dQ accumulator of whole query tiles, `slots` copies of the dK and dV accumulators."""
+    return 256 + 4 * (-(-B * Hq * L // 64) * 64 + B * Hq * -(-L // 128) * 128 * d + 2 * slots * B * L * Hkv * d)
+
+
+@no_device
+@pytest.mark.parametrize("B,Hq,Hkv,L,n", [
+    (2, 16, 4, 1000, 4),                       # 64 key tiles for 148 SMs
+    (1, 32, 8, 2048, 2), (1, 16, 4, 4096, 2),  # 128 tiles, long walks
+    (8, 16, 4, 512, 2), (32, 16, 4, 128, 1),   # 128 tiles, short walks: another CTA costs what it takes over
+    (16, 16, 4, 512, 1), (1, 32, 16, 2048, 1),  # 256 tiles
+    (1, 16, 1, 2048, 16), (1, 16, 1, 8192, 4), (1, 6, 2, 1500, 3), (1, 8, 8, 512, 1)])
+def test_tile_backward_split(lib, B, Hq, Hkv, L, n):
+    """The number of CTAs that share a KV head's query heads, seen through the slots that the call needs."""
+    p = dma.problem(B, Hq, Hkv, L, 128, L, flags=dma.DMA_FLAG_TILE_PATH)
+    need = backward_bytes(B, Hq, Hkv, L, 128, n if n > 1 else 0)
+    assert backward(lib, p, need) == ERR_CUDA
+    assert backward(lib, p, need - 1) == ERR_WORKSPACE
