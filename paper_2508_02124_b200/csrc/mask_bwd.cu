@@ -479,16 +479,17 @@ __global__ void __launch_bounds__(512) mask_bwd_full_reduce_kernel(const float* 
     }
 }
 
-// rows per CTA: the largest of 64, 32, 16, 8 whose tile fits 200 KiB of shared memory (0: none does) and, down to 32, gives
-// every SM a CTA (training step of 4096 keys, 512 channels, 16 heads: 273 us with 64 CTAs of 64 rows, 265 with 32 rows, 272 with
-// 16, whose partial sums weigh more)
+// rows per CTA: the largest of 64, 32, 16, 8 whose tile fits 200 KiB of shared memory (0: none does); 32 instead of 64 where
+// twice the CTAs still run at once, one per SM (both kernels, us, 64 / 32 rows, 16 heads, 512 channels: 4096 keys 38 / 27, but
+// 4800 keys, 75 CTAs, 39 / 48 and 8192 keys 40 / 52: two waves of half the length cost more than one). Not 16: the partial sums
+// weigh more (training step of 4096 keys 265 us with 32 rows, 272 with 16).
 static int full_rows(const Prob& P) {
     const size_t C = (size_t)P.Hkv * P.d, HqP = (P.Hq + 7) & ~7;
     auto fits = [&](int R) { return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= 200 * 1024; };
     int R = 64;
     while (R >= 8 && !fits(R)) R >>= 1;
     if (R < 8) return 0;
-    while (R > 32 && (int64_t)P.B * ((P.L + R - 1) / R) < 148) R >>= 1;
+    if (R == 64 && 2 * (int64_t)P.B * ((P.L + R - 1) / R) <= 148) R = 32;
     return R;
 }
 

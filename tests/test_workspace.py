@@ -41,3 +41,21 @@ def test_tile_backward_split(lib, B, Hq, Hkv, L, n):
     need = backward_bytes(B, Hq, Hkv, L, 128, n if n > 1 else 0)
     assert backward(lib, p, need) == ERR_CUDA
     assert backward(lib, p, need - 1) == ERR_WORKSPACE
+
+
+def mask_backward(lib, p, ws_bytes):
+    a = ctypes.c_void_p(4096)
+    return lib.dma_mask_bwd(ctypes.byref(p), *([a] * 8), a, ctypes.c_size_t(ws_bytes), ctypes.c_void_p(0))
+
+
+@no_device
+@pytest.mark.parametrize("B,Hq,Hkv,L,d,rows", [
+    (1, 16, 4, 4096, 128, 32), (1, 16, 4, 4736, 128, 32),     # at most 74 CTAs of 64 rows: twice as many still run at once
+    (1, 16, 4, 4737, 128, 64), (1, 16, 4, 8192, 128, 64), (1, 8, 8, 8192, 64, 64), (2, 8, 4, 3000, 128, 64),
+    (1, 16, 4, 16384, 128, 64), (1, 32, 8, 8192, 128, 32)])   # 1024 channels: 64 rows do not fit
+def test_full_weight_backward_rows(lib, B, Hq, Hkv, L, d, rows):
+    """Rows per CTA of the mask backward with full sampling weights, seen through the partial sums that the call needs."""
+    p = dma.problem(B, Hq, Hkv, L, d, 64, flags=dma.DMA_FLAG_FULL_DELTA)
+    need = B * -(-L // rows) * Hq * (Hkv * d + 1) * 4
+    assert mask_backward(lib, p, need) == ERR_CUDA
+    assert mask_backward(lib, p, need - 1) == ERR_WORKSPACE
