@@ -72,12 +72,13 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
 // launches that overlap the tail of the kernel before them (programmatic dependent launch)
 // ---------------------------------------------------------------------------------------------
 // A kernel launched this way may become resident once every CTA of the previous kernel of the stream has left the chip or is
-// about to, instead of after that kernel's completion has been reported. Every such kernel calls pdl_enter() with ALL its
-// global pointers before its first access to global memory: it returns once the previous kernel has completed and its writes
-// are visible. What is saved is the launch latency between dependent kernels, about 1 to 2 us each, which short kernels are
-// made of: step of 2 x 1000 rows, d = 64: 112 -> 103 us, prefill of 4096 keys 123 -> 107 us. (Letting the next kernel in early,
-// with griddepcontrol.launch_dependents at the top, was slower everywhere: its waiting CTAs take the places that the running
-// kernel's CTAs leave unevenly, 218 -> 239 us for 2048 rows of a 16384-key prefill, 2998 -> 3071 us for its training step.)
+// about to, instead of after that kernel's completion has been reported. Every such kernel calls pdl_enter() (or
+// pdl_enter_restrict()) with ALL its global pointers before its first access to global memory: it returns once the previous
+// kernel has completed and its writes are visible. What is saved is the launch latency between dependent kernels, about 1 to 2 us
+// each, which short kernels are made of: step of 2 x 1000 rows, d = 64: 112 -> 103 us, prefill of 4096 keys 123 -> 107 us.
+// (Letting the next kernel in early, with griddepcontrol.launch_dependents at the top, was slower everywhere: its waiting CTAs
+// take the places that the running kernel's CTAs leave unevenly, 218 -> 239 us for 2048 rows of a 16384-key prefill, 2998 ->
+// 3071 us for its training step.)
 // Returns a dma_status; a caller that gets an error launches nothing more, since the later kernels read what this one writes.
 template <typename... KArgs, typename... Args>
 inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
@@ -116,6 +117,20 @@ __device__ __forceinline__ void pdl_enter(Ts&... ptrs) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     auto pin = [](auto& p) { asm volatile("" : "+l"(p) :: "memory"); };
     (pin(ptrs), ...);
+}
+
+// The same wait for kernels that its pins slow down. A pointer that has passed through asm is no longer __restrict__: the loads
+// through it wait for every store before them, those to shared memory included. Here the pointers move by a zero that only the
+// asm statement knows, so that the addresses depend on the wait and the pointers stay __restrict__. For the kernels of
+// mask_build.cu; us with pdl_enter / this (without overlap or pins before): full sampling weights of 32 heads, 1024 channels, mask
+// build of 16384 keys 204 / 163 (165), of 8192 keys 131 / 91 (91), delta of 8 x 65536 keys, 32 heads 574 / 566 (558), mask build
+// of 32 heads, 16384 keys 76 / 73 (76). The kernels of the other files gain and lose by it (fp32 forward of two heads, 256 rows
+// 12.3 / 14.2, mask backward of 4096 keys 13.8 / 14.2) and keep the pins.
+template <typename... Ts>
+__device__ __forceinline__ void pdl_enter_restrict(Ts&... ptrs) {
+    int64_t zero;
+    asm volatile("griddepcontrol.wait;\n\tmov.s64 %0, 0;" : "=l"(zero) :: "memory");
+    ((ptrs += zero), ...);
 }
 
 __device__ __forceinline__ float to_f32(float x) { return x; }

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? 2 : 1) delta_kernel(cons
     const int hk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = lane % LPR, grp = lane / LPR;
-    pdl_enter(V, W, A, delta);
+    pdl_enter_restrict(V, W, A, delta);
     const int ntiles = (L - j_off + kRows - 1) / kRows;        // keys [j_off, L) of a row of ld entries
     const T* Vb = V + b * vs_b + hk * vs_h + sub * 8;
     auto request = [&](int tile, Raw (&raw)[kPass]) {
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V
     int mine = 0;                         // the head (within a batch) this lane ends up with: sub, bit-reversed
 #pragma unroll
     for (int m = 1, t = LPR >> 1; m < LPR; m <<= 1, t >>= 1) mine |= (sub & m) ? t : 0;
-    pdl_enter(V, W, A, delta);
+    pdl_enter_restrict(V, W, A, delta);
     for (int i = tid; i < HqP * C; i += 256) sW[i] = i < Hq * C ? W[i] : 0.0f;
     __syncthreads();
     for (int r0 = 0; r0 < kFullRows; r0 += kPass) {
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kChunk) chunk_sort_kernel(const float* __restr
                                                             uint2* __restrict__ lev, int m, uint32_t* __restrict__ bitmap, int64_t bitmap_words) {
     __shared__ unsigned long long s[2][kChunk];
     const int bh = blockIdx.y, c = blockIdx.x, t = threadIdx.x, j = c * kChunk + t;
-    pdl_enter(delta, sorted, lev, bitmap);
+    pdl_enter_restrict(delta, sorted, lev, bitmap);
     zero_share(bitmap, bitmap_words);
     // padding sorts below every real key (delta > 0) and keeps its index in the low word
     unsigned long long v = j < L ? sort_key(delta[(size_t)bh * L + j], j) : (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const unsigne
                                                                    unsigned long long* __restrict__ dst,
                                                                    uint2* __restrict__ lev, int Lc, int m) {
     extern __shared__ __align__(16) unsigned long long sk[];         // two buffers of kBlockKeys keys
-    pdl_enter(src, dst, lev);
+    pdl_enter_restrict(src, dst, lev);
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
     const int base = blockIdx.x * kBlockKeys, nreal = min(kBlockKeys, Lc - base);
     const size_t Wl = (size_t)Lc / 32;
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kMergeThreads) tree_merge_kernel(const unsigne
                                                                    uint2* __restrict__ lev_l, int Lc, int R, int m) {
     __shared__ __align__(16) unsigned long long sA[kMergeOut], sB[kMergeOut];
     __shared__ int s_a0;
-    pdl_enter(src, dst, lev_l);
+    pdl_enter_restrict(src, dst, lev_l);
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int o0 = blockIdx.x * kMergeOut;                       // first output position of this CTA within the head
     const int base = o0 & ~(2 * R - 1), t0 = o0 - base;
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
                                                           int32_t* __restrict__ expiry, int L, int Lc, int w, int m,
                                                           const int32_t* __restrict__ cu, int nseq) {
     const int r = blockIdx.x * 256 + threadIdx.x, bh = blockIdx.y;
-    pdl_enter(sorted, lev, expiry, cu);
+    pdl_enter_restrict(sorted, lev, expiry, cu);
     if (r >= L) return;                                          // ranks from L on are padding
     const int j = (int)(0xFFFFFFFFu - (uint32_t)sorted[(size_t)bh * Lc + r]);
     const size_t W = (size_t)Lc / 32;
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
 
 __global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v, uint32_t* bitmap, int64_t bitmap_words) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_enter(p, bitmap);
+    pdl_enter_restrict(p, bitmap);
     zero_share(bitmap, bitmap_words);
     if (i < n) p[i] = v;
 }
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(128) bitmap_kernel(const int32_t* __restrict__
                                                      int L, int bm, int bn, int Tr, int Wd, int causal) {
     extern __shared__ int diff[];                 // [Tr + 1]
     const int kt = blockIdx.x, bh = blockIdx.y, t = threadIdx.x;
-    pdl_enter(expiry, bitmap);
+    pdl_enter_restrict(expiry, bitmap);
     for (int i = t; i <= Tr; i += blockDim.x) diff[i] = 0;
     __syncthreads();
     const int jend = min(L, (kt + 1) * bn);
