@@ -117,7 +117,9 @@ typedef struct {
 } dma_problem_t;
 
 /* Bytes of device workspace each stage needs for this problem (any pointer may be NULL to skip it).
- * Each workspace begins with a 256-byte header whose first int32 is the device status word. */
+ * Each workspace begins with a 256-byte header whose first int32 is the device status word.
+ * No size falls as L or B grows (all else equal): a workspace taken for the longest sequence and the largest batch serves
+ * the shorter and smaller ones. */
 int dma_query_workspace(const dma_problem_t* p, size_t* mask_ws, size_t* fwd_ws, size_t* bwd_ws);
 
 /* Number of uint32 words of the bitmap, [B, Hq, Tr, ceil(Tc/32)] with Tr = ceil(L/tile_m), Tc = ceil(L/tile_n). */

@@ -65,7 +65,7 @@ int resolve(const dma_problem_t* p, Prob* o) {
     o->B = p->B; o->Hq = p->Hq; o->Hkv = p->Hkv; o->L = p->L; o->d = p->d; o->G = p->Hq / p->Hkv;
     o->w = p->w < p->L ? p->w : p->L;
     o->w_cap = p->w;
-    o->Lq = p->L; o->q_off = 0; o->bwd_split = 0;
+    o->Lq = p->L; o->q_off = 0; o->bwd_split = 0; o->chose_compact = false;
     o->dtype = p->dtype; o->flags = p->flags; o->causal = p->causal;
     o->bm = p->tile_m ? p->tile_m : 128;
     o->bn = p->tile_n ? p->tile_n : 128;
@@ -87,6 +87,7 @@ int resolve(const dma_problem_t* p, Prob* o) {
         // the library's choice (a function of the descriptor alone): with a window of at most a quarter of the
         // sequence the token-compacted kernels do O(L w d) work where walking tiles does O(L^2 d) on scattered masks
         o->flags |= DMA_FLAG_COMPACT_KV;
+        o->chose_compact = true;
     }
     return DMA_OK;
 }
@@ -100,6 +101,7 @@ static bool use_tensor_cores(const Prob& P) {
 static size_t fwd_ws_any(const Prob& P) { return use_tensor_cores(P) ? tc_fwd_ws_bytes(P) : (size_t)kWsHeaderBytes; }
 
 static size_t bwd_ws_any(const Prob& P) { return use_tensor_cores(P) ? tc_bwd_ws_bytes(P) : simt_bwd_ws_bytes(P); }
+static size_t bwd_need_any(const Prob& P) { return use_tensor_cores(P) ? tc_bwd_need(P) : simt_bwd_ws_bytes(P); }
 
 static int fwd_any(const Prob& P, const void* Q, const void* K, const void* V, const float* bias, const int32_t* expiry,
                    const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st) {
@@ -134,7 +136,7 @@ int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* 
         return DMA_ERR_ALIGN;
     const bool tc = use_tensor_cores(P);
     if ((P.flags & DMA_FLAG_COMPACT_KV) && !tc) return DMA_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < bwd_ws_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
+    if (!ws || ws_bytes < bwd_need_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
     if ((rc = device_ok())) return rc;
     // (the tensor-core path's first kernel clears the workspace header)
     if (!tc && cudaMemsetAsync(ws, 0, kWsHeaderBytes, st) != cudaSuccess) return DMA_ERR_CUDA;

@@ -827,10 +827,25 @@ static size_t bwd_slots(const Prob& P) {
     return tc_bwd_splits(P) > 1 ? (size_t)tc_bwd_splits(P) : 0;
 }
 
+static size_t bwd_base_bytes(const Prob& P) { return kWsHeaderBytes + (bwd_rows64(P) + bwd_acc_floats(P)) * sizeof(float); }
+// what the call uses beyond that
+static size_t bwd_extra_bytes(const Prob& P) {
+    const size_t perm = P.flags & DMA_FLAG_COMPACT_KV ? bwd_perm_ints(P) * sizeof(int) : 0;
+    return perm + 2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
+}
+
+size_t tc_bwd_need(const Prob& P) { return bwd_base_bytes(P) + bwd_extra_bytes(P); }
+
+// The slots of the split go away where a longer sequence or a larger batch has CTAs enough, but a workspace of that size serves
+// the shorter ones too: the bound for all of them, n CTAs for each of B Hkv Tc key tiles with n <= G and n B Hkv Tc <=
+// kMostSplitCtas.
 size_t tc_bwd_ws_bytes(const Prob& P) {
-    size_t n = kWsHeaderBytes + (bwd_rows64(P) + bwd_acc_floats(P)) * sizeof(float);
-    if (P.flags & DMA_FLAG_COMPACT_KV) n += bwd_perm_ints(P) * sizeof(int);
-    return n + 2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
+    size_t extra = bwd_extra_bytes(P);
+    if (P.G > 1 && (!(P.flags & DMA_FLAG_COMPACT_KV) || P.chose_compact)) {
+        const size_t ctas = std::min((size_t)P.B * P.Hq * P.Tc, (size_t)kMostSplitCtas);
+        extra = std::max(extra, 2 * ctas * 128 * P.d * sizeof(float));
+    }
+    return bwd_base_bytes(P) + extra;
 }
 
 int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,

@@ -16,7 +16,8 @@ struct Prob {
     int B, Hq, Hkv, L, d, G;
     int w;                 // min(w, L)
     int w_cap;             // w as given (the capacity of an incremental decoding state)
-    int dtype, flags;
+    int dtype, flags;      // flags: the caller's and what they imply (DMA_FLAG_COMPACT_KV also where the library chose it)
+    bool chose_compact;    // token-compacted execution is the library's choice: a shorter sequence may walk tiles
     int causal;            // 1: key j visible to rows i >= j; 0: to every row (the key's first row is 0 instead of j)
     int bm, bn, Tr, Tc, Wd;   // bitmap tile sizes, tile counts, uint32 words per bitmap row
     int bwd_split;            // CTAs that share a KV head in the tile-mode backward (0: tc_bwd_splits chooses)
@@ -58,7 +59,8 @@ int launch_simt_bwd(const Prob& P, const void* Q, const void* K, const void* V, 
 size_t tc_fwd_ws_bytes(const Prob& P);
 int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
                   const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st);
-size_t tc_bwd_ws_bytes(const Prob& P);
+size_t tc_bwd_need(const Prob& P);         // what the call uses
+size_t tc_bwd_ws_bytes(const Prob& P);     // what is asked for: at least the need of every shorter sequence and smaller batch
 int tc_bwd_splits(const Prob& P);
 // dma_attn_bwd on a part of a problem: with the split of the whole one, so that the parts' results are the whole's
 int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* K, const void* V, const void* O, const void* dO,

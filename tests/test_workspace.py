@@ -59,3 +59,40 @@ def test_full_weight_backward_rows(lib, B, Hq, Hkv, L, d, rows):
     need = B * -(-L // rows) * Hq * (Hkv * d + 1) * 4
     assert mask_backward(lib, p, need) == ERR_CUDA
     assert mask_backward(lib, p, need - 1) == ERR_WORKSPACE
+
+
+# ---- a workspace taken for the longest sequence and the largest batch serves the others --------------------------------------
+LENGTHS = sorted({1, 7, 100, 127, 128, 129, 255, 300, 513, 900, 1000, 1151, 1152, 1153, 1279, 1280, 1281, 1500, 2047, 2048, 2049, 2500,
+                  3000, 4095, 4096, 4097, 4607, 4608, 4609, 4736, 4737, 6000, 8063, 8064, 8191, 8192, 8193, 9408, 9409, 9472, 16383, 16384,
+                  16385, 20000, 32768})
+BATCHES = [1, 2, 3, 4, 5, 8, 16, 37, 64]
+HEADS = [(32, 8), (16, 2), (16, 4), (16, 1), (12, 4), (6, 2), (32, 32), (8, 8), (14, 2), (1, 1)]
+
+
+def never_falls(size, make):
+    """size(make(B, L)) over all pairs: not below that of any shorter sequence or smaller batch."""
+    table = [[size(make(B, L)) for L in LENGTHS] for B in BATCHES]
+    for row in table:
+        assert row == sorted(row), [(L, n) for L, n, m in zip(LENGTHS, row, row[1:] + [row[-1]]) if n > m]
+    for i, L in enumerate(LENGTHS):
+        col = [row[i] for row in table]
+        assert col == sorted(col), (L, list(zip(BATCHES, col)))
+
+
+@pytest.mark.parametrize("flags", [0, dma.DMA_FLAG_TILE_PATH, dma.DMA_FLAG_COMPACT_KV, dma.DMA_FLAG_COMPACT_KV | dma.DMA_FLAG_DETERMINISTIC])
+@pytest.mark.parametrize("Hq,Hkv", HEADS)
+def test_attention_and_mask_workspaces_never_fall(lib, Hq, Hkv, flags):
+    for d in (64, 128):
+        for w in (1, 256, 1280, 4096):
+            for causal in ((1, 0) if flags == 0 else (1,)):
+                for i in range(3):
+                    never_falls(lambda p: dma.dma_query_workspace(p)[i], lambda B, L: dma.problem(B, Hq, Hkv, L, d, w, causal=causal, flags=flags))
+
+
+@no_device
+@pytest.mark.parametrize("B,Hq,Hkv,L,d,w", [(1, 32, 8, 8192, 128, 4096), (1, 16, 2, 8192, 64, 2048), (4, 16, 4, 1000, 64, 256), (2, 32, 8, 16384, 128, 2048)])
+def test_backward_accepts_a_workspace_of_a_longer_sequence(lib, B, Hq, Hkv, L, d, w):
+    ws = dma.dma_query_workspace(dma.problem(B, Hq, Hkv, L, d, w))[2]
+    for n in (n for n in LENGTHS if n <= L):
+        for b in range(1, B + 1):
+            assert backward(lib, dma.problem(b, Hq, Hkv, n, d, w), ws) == ERR_CUDA, (b, n)
