@@ -11,6 +11,7 @@
 //   decode_list_attn_kernel, decode_step_combine_kernel   the same for a kept set that is carried from step to step
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -658,11 +659,18 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
 
 // Splits of a row's kept list: few enough that all CTAs are resident at once (two per SM), which matters when a step is
 // short, but no longer than kMaxSplit keys, so that a large batch still comes in waves that balance.
+constexpr int kResident = 2 * 148;
 int split_keys(const Prob& P) {
     const int64_t bh = (int64_t)P.B * P.Hq;
     int per = kMinSplit;
-    while (per < kMaxSplit && bh * ((P.w + per - 1) / per) > 2 * 148) per += kMinSplit;
+    while (per < kMaxSplit && bh * ((P.w + per - 1) / per) > kResident) per += kMinSplit;
     return per;
+}
+// The most splits of all rows that a call with at most P.w kept keys and at most P.B * P.Hq rows has. (The splits of one call
+// fall where a longer list takes longer splits.)
+size_t most_splits(const Prob& P) {
+    const size_t bh = (size_t)P.B * P.Hq, few = bh * ((P.w + kMinSplit - 1) / kMinSplit), many = bh * ((P.w + kMaxSplit - 1) / kMaxSplit);
+    return std::max(std::min(few, (size_t)kResident), many);
 }
 
 template <typename T, int D>
@@ -683,19 +691,18 @@ struct DecodeWs {
     int* tickets;
     int* kept;
     float* partial;
-    size_t bytes;
+    size_t bytes;              // no fewer than for any shorter cache and smaller batch
 };
 static DecodeWs decode_ws(const Prob& P, void* ws) {
     const size_t bh = (size_t)P.B * P.Hq;
-    const int per = split_keys(P), ns = (P.w + per - 1) / per;
-    const size_t splits = (size_t)(ns > list_splits(P) ? ns : list_splits(P));
+    const size_t splits = std::max(most_splits(P), bh * list_splits(P));
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     DecodeWs w;
     size_t off = kWsHeaderBytes;
     char* base = (char*)ws;
     w.tickets = reinterpret_cast<int*>(base + off); off += up(bh * sizeof(int));
     w.kept = reinterpret_cast<int*>(base + off); off += up(bh * P.w * sizeof(int));
-    w.partial = reinterpret_cast<float*>(base + off); off += bh * splits * (P.d + 2) * sizeof(float);
+    w.partial = reinterpret_cast<float*>(base + off); off += splits * (P.d + 2) * sizeof(float);
     w.bytes = off;
     return w;
 }

@@ -96,3 +96,21 @@ def test_backward_accepts_a_workspace_of_a_longer_sequence(lib, B, Hq, Hkv, L, d
     for n in (n for n in LENGTHS if n <= L):
         for b in range(1, B + 1):
             assert backward(lib, dma.problem(b, Hq, Hkv, n, d, w), ws) == ERR_CUDA, (b, n)
+
+
+@pytest.mark.parametrize("Hq,Hkv", HEADS)
+@pytest.mark.parametrize("w", [1, 100, 600, 1152, 1200, 1280, 2048, 5000, 16384])
+def test_decode_workspace_never_falls(lib, Hq, Hkv, w):
+    never_falls(dma.dma_decode_workspace, lambda B, N: dma.problem(B, Hq, Hkv, N, 128, w))
+
+
+@no_device
+@pytest.mark.parametrize("B,Hq,w", [(1, 32, 1280), (1, 32, 1200), (2, 32, 600), (1, 1, 2048)])
+def test_decoding_calls_accept_the_last_step_s_workspace(lib, B, Hq, w):
+    a, z = ctypes.c_void_p(4096), ctypes.c_void_p(0)
+    ws = ctypes.c_size_t(dma.dma_decode_workspace(dma.problem(B, Hq, Hq, 16384, 128, w)))
+    for N in (n for n in LENGTHS if n <= 16384):
+        p, ld = ctypes.byref(dma.problem(B, Hq, Hq, N, 128, w)), ctypes.c_int64(16384)
+        assert lib.dma_decode(p, a, a, a, a, ld, a, a, z, a, ws, z) == ERR_CUDA, N
+        assert lib.dma_decode_step(p, a, a, a, a, ld, a, a, a, a, ws, z) == ERR_CUDA, N
+        assert lib.dma_decode_state_init(p, a, ld, a, a, ws, z) == ERR_CUDA, N
