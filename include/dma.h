@@ -214,7 +214,8 @@ int dma_attn_bwd(const dma_problem_t* p, const void* Q, const void* K, const voi
  * V, bias (the delta written by dma_mask_build), dM: inputs. dV [B,L,Hkv,d] (layout and strides of V, element type of
  * the problem) is IN/OUT: the contribution is added to what it holds (the attention backward's dV), in fp32, and
  * rounded once. dW_delta [Hq,d] and dA [Hq] fp32 are overwritten; their sums are formed in a fixed order (no
- * floating-point atomics). ws: dma_mask_bwd_workspace() bytes. All pointers device memory, 16-byte aligned. */
+ * floating-point atomics). ws: dma_mask_bwd_workspace() bytes, a size that does not fall as L or B grows. All pointers device
+ * memory, 16-byte aligned. */
 int dma_mask_bwd_workspace(const dma_problem_t* p, size_t* bytes);
 int dma_mask_bwd(const dma_problem_t* p, const void* V, const float* W_delta, const float* A, const float* bias,
                  const float* dM, void* dV, float* dW_delta, float* dA, void* ws, size_t ws_bytes, void* cuda_stream);

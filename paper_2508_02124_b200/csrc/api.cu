@@ -230,7 +230,7 @@ int dma_mask_bwd(const dma_problem_t* p, const void* V, const float* W_delta, co
     if (!V || !W_delta || !A || !bias || !dM || !dV || !dW_delta || !dA) return DMA_ERR_NULL;
     if (!aligned16(V) || !aligned16(W_delta) || !aligned16(bias) || !aligned16(dM) || !aligned16(dV) || !aligned16(dW_delta))
         return DMA_ERR_ALIGN;
-    if (!ws || ws_bytes < mask_bwd_ws_bytes(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
+    if (!ws || ws_bytes < mask_bwd_need(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
     if ((rc = device_ok())) return rc;
     return launch_mask_bwd(P, V, W_delta, A, bias, dM, dV, dW_delta, dA, ws, (cudaStream_t)cuda_stream);
 }

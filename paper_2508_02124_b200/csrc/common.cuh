@@ -34,6 +34,7 @@ int check_launch();                                       // cudaGetLastError ->
 
 // stage launchers (each returns a dma_status); defined in the stage's .cu file
 size_t mask_ws_bytes(const Prob& P);
+size_t mask_bwd_need(const Prob& P);       // as tc_bwd_need, tc_bwd_ws_bytes
 size_t mask_bwd_ws_bytes(const Prob& P);
 int launch_delta_range(const Prob& P, const void* V, const float* W, const float* A, float* delta, int64_t ld, int j_begin,
                        int j_end, cudaStream_t st);

@@ -5,6 +5,7 @@
 // HBM-bound: V and dV rows are read once, dV written once. A CTA walks keys of one (batch, KV head) with all G query heads of
 // the group; its dW / dA sums go to the workspace and a second kernel adds them in a fixed order (no floating-point atomics:
 // the result does not depend on the launch schedule).
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -479,15 +480,17 @@ __global__ void __launch_bounds__(512) mask_bwd_full_reduce_kernel(const float* 
     }
 }
 
+static bool full_fits(const Prob& P, int R) {
+    const size_t C = (size_t)P.Hkv * P.d, HqP = (P.Hq + 7) & ~7;
+    return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= 200 * 1024;
+}
 // rows per CTA: the largest of 64, 32, 16, 8 whose tile fits 200 KiB of shared memory (0: none does); 32 instead of 64 where
 // twice the CTAs still run at once, one per SM (both kernels, us, 64 / 32 rows, 16 heads, 512 channels: 4096 keys 38 / 27, but
 // 4800 keys, 75 CTAs, 39 / 48 and 8192 keys 40 / 52: two waves of half the length cost more than one). Not 16: the partial sums
 // weigh more (training step of 4096 keys 265 us with 32 rows, 272 with 16).
 static int full_rows(const Prob& P) {
-    const size_t C = (size_t)P.Hkv * P.d, HqP = (P.Hq + 7) & ~7;
-    auto fits = [&](int R) { return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= 200 * 1024; };
     int R = 64;
-    while (R >= 8 && !fits(R)) R >>= 1;
+    while (R >= 8 && !full_fits(P, R)) R >>= 1;
     if (R < 8) return 0;
     if (R == 64 && 2 * (int64_t)P.B * ((P.L + R - 1) / R) <= 148) R = 32;
     return R;
@@ -501,13 +504,26 @@ int ctas_per_pair(const Prob& P) {
 
 }  // namespace
 
-size_t mask_bwd_ws_bytes(const Prob& P) {
+static size_t full_partial_bytes(const Prob& P, size_t ctas) { return ctas * P.Hq * ((size_t)P.Hkv * P.d + 1) * sizeof(float); }
+static size_t partial_bytes(const Prob& P, size_t ctas) { return ctas * P.G * (P.d + 1) * sizeof(float); }
+
+size_t mask_bwd_need(const Prob& P) {
     if (P.flags & DMA_FLAG_FULL_DELTA) {
         const int R = full_rows(P);
-        if (R == 0) return 0;
-        return (size_t)P.B * ((P.L + R - 1) / R) * P.Hq * ((size_t)P.Hkv * P.d + 1) * sizeof(float);
+        return R == 0 ? 0 : full_partial_bytes(P, (size_t)P.B * ((P.L + R - 1) / R));
     }
-    return (size_t)P.B * P.Hkv * ctas_per_pair(P) * P.G * (P.d + 1) * sizeof(float);
+    return partial_bytes(P, (size_t)P.B * P.Hkv * ctas_per_pair(P));
+}
+
+// CTAs go down where a longer sequence takes 64 rows per CTA instead of 32, or where more pairs leave no room for a second CTA per
+// pair, but a workspace of that size serves the smaller problems too: the bound for all of them.
+size_t mask_bwd_ws_bytes(const Prob& P) {
+    if (P.flags & DMA_FLAG_FULL_DELTA) {
+        const size_t half = std::min((size_t)P.B * ((P.L + 31) / 32), (size_t)148);        // (of 32 rows, while they run at once)
+        return full_fits(P, 64) ? std::max(mask_bwd_need(P), full_partial_bytes(P, half)) : mask_bwd_need(P);
+    }
+    const size_t pairs = (size_t)P.B * P.Hkv;                              // (pairs * ceil(296 / pairs) < pairs + 296)
+    return partial_bytes(P, std::min(pairs * ((P.L + 8 * kRows - 1) / (8 * kRows)), pairs + 2 * 148 - 1));
 }
 
 template <typename T, int D>

@@ -114,3 +114,20 @@ def test_decoding_calls_accept_the_last_step_s_workspace(lib, B, Hq, w):
         assert lib.dma_decode(p, a, a, a, a, ld, a, a, z, a, ws, z) == ERR_CUDA, N
         assert lib.dma_decode_step(p, a, a, a, a, ld, a, a, a, a, ws, z) == ERR_CUDA, N
         assert lib.dma_decode_state_init(p, a, ld, a, a, ws, z) == ERR_CUDA, N
+
+
+@pytest.mark.parametrize("flags", [0, dma.DMA_FLAG_FULL_DELTA])
+@pytest.mark.parametrize("Hq,Hkv", HEADS)
+def test_mask_backward_workspace_never_falls(lib, Hq, Hkv, flags):
+    for d in (64, 128):
+        never_falls(dma.dma_mask_bwd_workspace, lambda B, L: dma.problem(B, Hq, Hkv, L, d, 64, flags=flags))
+
+
+@no_device
+@pytest.mark.parametrize("flags", [0, dma.DMA_FLAG_FULL_DELTA])
+@pytest.mark.parametrize("B,Hq,Hkv,L", [(1, 16, 4, 16384), (3, 16, 4, 4737), (64, 8, 8, 1000)])
+def test_mask_backward_accepts_a_workspace_of_a_longer_sequence(lib, B, Hq, Hkv, L, flags):
+    ws = dma.dma_mask_bwd_workspace(dma.problem(B, Hq, Hkv, L, 64, 64, flags=flags))
+    for n in (n for n in LENGTHS if n <= L):
+        for b in range(1, B + 1):
+            assert mask_backward(lib, dma.problem(b, Hq, Hkv, n, 64, 64, flags=flags), ws) == ERR_CUDA, (b, n)
