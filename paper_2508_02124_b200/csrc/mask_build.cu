@@ -215,6 +215,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? 2 : 1) delta_kernel(cons
 // values and hands the other half to its partner: the same additions as the plain butterfly, a quarter of the
 // shuffles), after which lane `sub` holds the dot product of head bitrev(sub) and carries that head's running sum.
 // kFullRows keys per CTA: 64, or 32 where 64 would leave SMs without a CTA (4096 keys, 16 heads, 512 channels: 15.5 -> 14.2 us).
+constexpr size_t kFullSmem = 200 * 1024;     // the most dynamic shared memory of a CTA
+
 template <typename T, int D, int kFullRows>
 __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V, const float* __restrict__ W,
                                                          const float* __restrict__ A, float* __restrict__ delta,
@@ -654,12 +656,13 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     if (j_end <= j_begin) return DMA_OK;
     if (P.flags & DMA_FLAG_FULL_DELTA) {
         const size_t HqP = (size_t)(P.Hq + D / 8 - 1) / (D / 8) * (D / 8);
-        if ((HqP * P.Hkv * D + HqP * 64) * sizeof(float) > 200 * 1024) return DMA_ERR_UNSUPPORTED;
+        if ((HqP * P.Hkv * D + HqP * 64) * sizeof(float) > kFullSmem) return DMA_ERR_UNSUPPORTED;
         constexpr int kFewRows = D == 128 ? 32 : 64;          // (one pass of the CTA covers 32 rows at d = 128, 64 at d = 64)
         const int rows = (int64_t)P.B * ((j_end - j_begin + 63) / 64) < 148 ? kFewRows : 64;
         const size_t bytes = (HqP * P.Hkv * D + HqP * rows) * sizeof(float);
         auto kern = rows == 64 ? delta_full_kernel<T, D, 64> : delta_full_kernel<T, D, kFewRows>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return DMA_ERR_CUDA;
+        // (state of the function, which other threads' calls share: always the limit)
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFullSmem) != cudaSuccess) return DMA_ERR_CUDA;
         return launch_overlapped(kern, dim3((j_end - j_begin + rows - 1) / rows, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.Hkv,
                                  P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
     }
@@ -688,7 +691,7 @@ int launch_delta_range(const Prob& P, const void* V, const float* W, const float
 static int mask_build_limits(const Prob& P) {
     if (P.flags & DMA_FLAG_FULL_DELTA) {
         const size_t lanes = (size_t)P.d / 8, HqP = (P.Hq + lanes - 1) / lanes * lanes;
-        if ((HqP * P.Hkv * P.d + HqP * 64) * sizeof(float) > 200 * 1024) return DMA_ERR_UNSUPPORTED;
+        if ((HqP * P.Hkv * P.d + HqP * 64) * sizeof(float) > kFullSmem) return DMA_ERR_UNSUPPORTED;
     } else if ((size_t)P.G * (P.d + 2 * 128) * sizeof(float) > 48 * 1024) {
         return DMA_ERR_UNSUPPORTED;
     }

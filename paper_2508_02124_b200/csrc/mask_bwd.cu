@@ -15,6 +15,7 @@ namespace {
 
 constexpr int kRows = 8;       // keys per warp and unit
 constexpr int kThreads = 256;
+constexpr int kMaxGroup = 16;  // query heads per KV head
 
 __device__ __forceinline__ void load8f(const float* p, float (&v)[8]) {
     const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
@@ -313,6 +314,7 @@ __global__ void __launch_bounds__((D == 128 ? 4 : 8) * (D + 1)) mask_bwd_reduce_
 //   3  dW partial [h][col] = sum_rows dz v: a thread owns a column and walks the rows (no cross-thread sums)
 //   4  the value tile is overwritten by sum_h dz W[h][col], then added to dV
 // partial [B * blocks][Hq][C + 1]; mask_bwd_full_reduce_kernel adds them in a fixed order.
+constexpr size_t kFullSmem = 200 * 1024;    // the most dynamic shared memory of a CTA
 constexpr int kFullThreads = 512;     // 16 warps: the kernel is bound by instruction issue and latency, not by registers
 
 template <typename T, int RW>
@@ -482,7 +484,7 @@ __global__ void __launch_bounds__(512) mask_bwd_full_reduce_kernel(const float* 
 
 static bool full_fits(const Prob& P, int R) {
     const size_t C = (size_t)P.Hkv * P.d, HqP = (P.Hq + 7) & ~7;
-    return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= 200 * 1024;
+    return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= kFullSmem;
 }
 // rows per CTA: the largest of 64, 32, 16, 8 whose tile fits 200 KiB of shared memory (0: none does); 32 instead of 64 where
 // twice the CTAs still run at once, one per SM (both kernels, us, 64 / 32 rows, 16 heads, 512 channels: 4096 keys 38 / 27, but
@@ -530,9 +532,11 @@ template <typename T, int D>
 static int launch_typed(const Prob& P, const void* V, const float* W, const float* A, const float* delta, const float* dM,
                         void* dV, float* dW, float* dA, void* ws, cudaStream_t st) {
     const int nblk = ctas_per_pair(P);
-    const size_t smem = (size_t)P.G * (D + 8 * (D + 1) + 8 * 2 * kRows) * sizeof(float);
+    constexpr size_t smem_head = (D + 8 * (D + 1) + 8 * 2 * kRows) * sizeof(float);
+    const size_t smem = P.G * smem_head;
     auto kern = P.G == 1 ? mask_bwd_kernel<T, D, 1> : P.G == 2 ? mask_bwd_kernel<T, D, 2> : P.G == 4 ? mask_bwd_kernel<T, D, 4> : mask_bwd_kernel<T, D, 0>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
+    // (state of the function, which other threads' calls share: always the limit)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxGroup * smem_head)) != cudaSuccess) return DMA_ERR_CUDA;
     const int rc = launch_overlapped(kern, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
                                      P.G, P.vs[0], P.vs[1], P.vs[2]);
     if (rc) return rc;
@@ -546,7 +550,7 @@ static int launch_full(const Prob& P, const void* V, const float* W, const float
     constexpr int R = RW * 8;
     const int nblk = (P.L + R - 1) / R, C = P.Hkv * P.d, HqP = (P.Hq + 7) & ~7;
     const size_t smem = ((size_t)R * C + (size_t)R * HqP + (size_t)P.Hq * R) * sizeof(float);
-    if (cudaFuncSetAttribute(mask_bwd_full_kernel<T, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(mask_bwd_full_kernel<T, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFullSmem) != cudaSuccess)
         return DMA_ERR_CUDA;
     const int rc = launch_overlapped(mask_bwd_full_kernel<T, RW>, dim3(nblk, P.B), dim3(kFullThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV,
                                      (float*)ws, P.L, P.Hq, P.Hkv, P.d, P.vs[0], P.vs[1], P.vs[2]);
@@ -571,7 +575,7 @@ int launch_mask_bwd(const Prob& P, const void* V, const float* W, const float* A
     if (P.flags & DMA_FLAG_FULL_DELTA)
         return P.dtype == DMA_BF16 ? launch_full_rows<__nv_bfloat16>(P, V, W, A, delta, dM, dV, dW, dA, ws, st)
                                    : launch_full_rows<float>(P, V, W, A, delta, dM, dV, dW, dA, ws, st);
-    if (P.G > 16) return DMA_ERR_UNSUPPORTED;
+    if (P.G > kMaxGroup) return DMA_ERR_UNSUPPORTED;
     if (P.dtype == DMA_BF16) {
         return P.d == 128 ? launch_typed<__nv_bfloat16, 128>(P, V, W, A, delta, dM, dV, dW, dA, ws, st)
                           : launch_typed<__nv_bfloat16, 64>(P, V, W, A, delta, dM, dV, dW, dA, ws, st);

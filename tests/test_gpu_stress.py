@@ -209,3 +209,43 @@ def test_list_kernel_shared_memory_size_in_a_fresh_process(w):
     code = f"import sys; sys.path[:0] = [{here!r}, {os.path.dirname(here)!r}]; import test_gpu_stress as t; assert t.lists_of_eight_pairs({w})()"
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("flags,heads", [(0, [(5, 1), (16, 1)]), (dma.DMA_FLAG_FULL_DELTA, [(4, 1), (32, 8)])])
+def test_mask_kernels_shared_memory_sizes_from_two_threads(flags, heads):
+    """Two threads whose mask kernels take different amounts of shared memory (26 / 82 KB, and 4 / 139 KB with full sampling
+    weights): the limit is state of the kernel that both share."""
+    import threading
+
+    def work(Hq, Hkv):
+        g = torch.Generator(DEV).manual_seed(Hq)
+        L, d = 1000, 128
+        V = torch.randn(1, L, Hkv, d, generator=g, device=DEV).to(torch.bfloat16)
+        W = torch.randn(Hq, Hkv * d if flags else d, generator=g, device=DEV) / 16
+        A, dM = torch.rand(Hq, generator=g, device=DEV), torch.randn(1, Hq, L, generator=g, device=DEV)
+        p = dma.problem(1, Hq, Hkv, L, d, 100, flags=flags)
+
+        def run():
+            dV = torch.zeros_like(V)
+            bias, e, _ = dma.dma_mask_build(p, V, W, A)
+            _, dW, dA = dma.dma_mask_bwd(p, V, W, A, bias, dM, dV)
+            torch.cuda.current_stream().synchronize()
+            return bias, e, dV, dW, dA
+
+        return run, run()
+
+    jobs, bad = [work(*h) for h in heads], []
+
+    def worker(run, ref):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                bad.extend(i for i in range(200) if not all(torch.equal(a, b) for a, b in zip(run(), ref)))
+        except Exception as ex:
+            bad.append(repr(ex))
+
+    threads = [threading.Thread(target=worker, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad[:5]
