@@ -66,6 +66,8 @@ struct SharedStorage {
     int n_iters;
     int abort_flag;
 };
+static_assert(kStages == 2 && offsetof(SharedStorage, bext) == offsetof(SharedStorage, aext) + 2 * 4096,
+              "token-compacted mode takes aext and bext as six blocks of 2 KB in a row: ones, two stages of two tiles, zeros");
 
 struct FwdParams {
     const float* bias;

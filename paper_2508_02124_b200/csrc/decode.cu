@@ -585,7 +585,7 @@ __device__ __forceinline__ void decode_state_update(const float* __restrict__ de
 }
 
 // attention over the row's kept list as it is AFTER the appended key N - 1 is taken into account (the stored state still
-// describes the first N - 1 keys; decode_state_update_kernel brings it up to date afterwards)
+// describes the first N - 1 keys; decode_step_combine_kernel brings it up to date afterwards)
 template <typename T, int D>
 __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const T* __restrict__ q, const T* __restrict__ K,
                                                                         const T* __restrict__ V, const float* __restrict__ delta,
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
         if (c == 0) lse[bh] = lt > 0.0f ? 0.6931471805599453f * (m_all + log2f(lt)) : -INFINITY;
     }
     // incremental decoding: the attention kernel has read the row's state, which can now take in the appended key
-    if (state) decode_state_update(delta, ld, N, w_cap, state, bh);
+    decode_state_update(delta, ld, N, w_cap, state, bh);
 }
 
 

@@ -534,3 +534,25 @@ def test_compact_forward_bits_do_not_depend_on_how_the_lists_were_made(Hq):
     bmp1 = torch.full((dma.dma_bitmap_words(p1),), -1, dtype=torch.int32, device="cuda")
     O1, lse1 = dma.dma_attn_fwd(p1, inp["Q"], inp["K"], inp["V"], bias1, e1, bmp1)
     assert torch.equal(O1[:, :L], O) and torch.equal(lse1[..., :L], lse)
+
+
+def test_overflow_of_gathered_lists_made_for_several_pairs():
+    """148 heads of 4096 rows: eight pairs of query tiles per CTA. A mask that keeps every key where w promises 64 is reported, both
+    where a pair's own list overflows (rows 256 on) and where the keys of the whole group do not fit (rows 2048 on); the next call
+    with the same workspace, on a mask within w, is clean."""
+    Hq, L, d, w = 148, 4096, 64, 64
+    case = wl.small(C2, B=1, Hq=Hq, Hkv=Hq // 2, L=L, d=d, w=w, seed=3, name="list-overflow")
+    inp = {k: v.cuda() for k, v in wl.make_inputs(case).items()}
+    p = problem_of(case, flags=dma.DMA_FLAG_COMPACT_KV)
+    bias, e, _ = dma.dma_mask_build(p, inp["V"], inp["W_delta"], inp["A"])
+    ws = torch.empty(dma.dma_query_workspace(p)[1], dtype=torch.uint8, device="cuda")
+    forward = lambda q0, rows, ex: dma.dma_attn_fwd_chunk(p, q0, inp["Q"][:, q0:q0 + rows].contiguous(), inp["K"], inp["V"], bias, ex, ws=ws)   # noqa: E731
+    want = forward(0, L, e)
+    assert dma.dma_read_status(ws) == 0
+    dense = torch.full_like(e, L)
+    for q0, rows in ((0, L), (0, 2048), (2048, 2048)):
+        forward(q0, rows, dense)
+        assert dma.dma_read_status(ws) == -8, (q0, rows)
+        got = forward(0, L, e)
+        assert dma.dma_read_status(ws) == 0
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])

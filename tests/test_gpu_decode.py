@@ -88,3 +88,23 @@ def test_selection_at_the_edges_of_the_register_and_cluster_sizes(N, w, kind):
     assert torch.equal(idx.cpu().long(), want)
     state = dma.dma_decode_state_init(p, delta.cuda(), dma.dma_decode_state(p, "cuda"))
     assert dma.decode_state_sets(state, w) == [r.tolist() for r in want[0]]
+
+
+@pytest.mark.parametrize("N,w", [(33, 7), (16384, 2048), (40000, 100), (262177, 20000)])
+@pytest.mark.parametrize("share", [0.0001, 0.5])
+def test_selection_with_infinite_weights(N, w, share):
+    """exp overflows to infinity in earnest (a large gate): such keys come first, the lower index among them, whether fewer or more
+    than w. (A row with fewer still ranks the finite ones, over a range of bit patterns that ends at infinity.)"""
+    g = torch.Generator().manual_seed(N)
+    BH = 2
+    delta = torch.exp(torch.randn(1, BH, N, generator=g))
+    delta[torch.rand(1, BH, N, generator=g) < share] = float("inf")
+    delta[..., N // 2] = float("inf")
+    p = dma.problem(1, BH, 1, N, 64, w)
+    K = torch.zeros(1, N, 1, 64, dtype=torch.bfloat16, device="cuda")
+    q = torch.zeros(1, BH, 64, dtype=torch.bfloat16, device="cuda")
+    _, _, idx = dma.dma_decode(p, q, K, K, delta.cuda(), want_idx=True)
+    want = torch.sort(torch.sort(delta, dim=-1, descending=True, stable=True)[1][..., :w], dim=-1)[0]
+    assert torch.equal(idx.cpu().long(), want)
+    state = dma.dma_decode_state_init(p, delta.cuda(), dma.dma_decode_state(p, "cuda"))
+    assert dma.decode_state_sets(state, w) == [r.tolist() for r in want[0]]
