@@ -241,27 +241,28 @@ __global__ void rowdot_kernel(const T* __restrict__ O, const T* __restrict__ dO,
     if (lane == 0) Dv[row] = s;
 }
 
-// Grid: (blocks of BM keys or rows, Hkv + Hq, B). blockIdx.y < Hkv: dK, dV, dM of BM keys of that KV head; else dQ of BM rows
-// of query head blockIdx.y - Hkv.
+// Grid: (Hkv + Hq heads of nblk blocks each, B). Head y < Hkv: dK, dV, dM of BM keys of that KV head; else dQ of BM rows of query
+// head y - Hkv. (The heads are not blockIdx.y, which ends at 65535: calls with that many query heads are accepted.)
 template <typename T, int D, int kOwn, int NW>
 __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
                                                            const T* __restrict__ dO, const float* __restrict__ lse, const float* __restrict__ Dv,
                                                            const float* __restrict__ bias, const int32_t* __restrict__ expiry,
                                                            const uint32_t* __restrict__ bitmap, T* __restrict__ dQ, T* __restrict__ dK,
-                                                           T* __restrict__ dV, float* __restrict__ dM, Prob P, int use_bitmap) {
+                                                           T* __restrict__ dV, float* __restrict__ dM, Prob P, int use_bitmap, int nblk) {
     constexpr int LD = D + 4, BM = kOwn * NW;
     extern __shared__ __align__(16) float sm[];
     float* sA = sm;                              // stationary rows: K, V (or Q, dO), [BM][D] each
     float* sY = sA + 2 * BM * D;                 // two buffers of Q, dO (or K, V) tiles, [kTile][LD] each
     float* sP = sY + 4 * kTile * LD;             // [NW][2][kOwn][kTile]
-    const int b = blockIdx.z, L = P.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.y, head = blockIdx.x / nblk, blk = blockIdx.x % nblk;
+    const int L = P.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_enter(Q, K, V, dO, lse, Dv, bias, expiry, bitmap, dQ, dK, dV, dM);
     float* wts = sP + warp * 2 * kOwn * kTile;
     const float* own1 = sA + warp * kOwn * D;
     const float* own2 = own1 + BM * D;
 
-    if ((int)blockIdx.y < P.Hkv) {
-        const int hk = blockIdx.y, j0 = blockIdx.x * BM;       // (causal: the first keys have the longest walks)
+    if (head < P.Hkv) {
+        const int hk = head, j0 = blk * BM;       // (causal: the first keys have the longest walks)
         stage_rows<T, D, D>(sA, K + b * P.ks[0] + hk * P.ks[2], P.ks[1], j0, BM, L);
         stage_rows<T, D, D>(sA + BM * D, V + b * P.vs[0] + hk * P.vs[2], P.vs[1], j0, BM, L);
         float adk[kOwn][D / 32], adv[kOwn][D / 32];
@@ -339,8 +340,8 @@ __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__
             store_row<T, D>(dV + b * P.vs[0] + (int64_t)j * P.vs[1] + hk * P.vs[2], adv[a], 1.0f, lane);
         }
     } else {
-        const int h = (int)blockIdx.y - P.Hkv, hk = h / P.G, bh = b * P.Hq + h;
-        const int i0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * BM;
+        const int h = head - P.Hkv, hk = h / P.G, bh = b * P.Hq + h;
+        const int i0 = (nblk - 1 - blk) * BM;
         stage_rows<T, D, D>(sA, Q + b * P.qs[0] + h * P.qs[2], P.qs[1], i0, BM, L);
         stage_rows<T, D, D>(sA + BM * D, dO + b * P.os[0] + h * P.os[2], P.os[1], i0, BM, L);
         float adq[kOwn][D / 32], li[kOwn], di[kOwn];
@@ -428,9 +429,10 @@ int bwd_t(const Prob& P, const void* Q, const void* K, const void* V, const void
     int rc = launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P);
     if (rc) return rc;
     int use_bitmap = !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0;
+    const int nblk = (P.L + kOwn * NW - 1) / (kOwn * NW);
     timing_mark(1, false, st);
-    rc = launch_overlapped(kern, dim3((P.L + kOwn * NW - 1) / (kOwn * NW), P.Hkv + P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
-                           (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap);
+    rc = launch_overlapped(kern, dim3((unsigned)nblk * (unsigned)(P.Hkv + P.Hq), P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
+                           (const T*)V, (const T*)dO, lse, Dv, bias, expiry, bitmap, (T*)dQ, (T*)dK, (T*)dV, dM, P, use_bitmap, nblk);
     timing_mark(1, true, st);
     return rc;
 }

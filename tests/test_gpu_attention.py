@@ -556,3 +556,23 @@ def test_overflow_of_gathered_lists_made_for_several_pairs():
         got = forward(0, L, e)
         assert dma.dma_read_status(ws) == 0
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def test_fp32_backward_of_more_heads_than_a_grid_has_rows():
+    """32 768 query heads that share no KV head: with as many KV heads the dK / dV and dQ parts together are 65 536 heads, one more
+    than a grid has rows. Against plain torch in 64 bits; every gradient of every head (8 keys, all kept)."""
+    H, L, d = 32768, 8, 64
+    g = torch.Generator("cuda").manual_seed(5)
+    Q, K, V, dO = (torch.randn(1, L, H, d, generator=g, device="cuda") for _ in range(4))
+    p = dma.problem(1, H, H, L, d, L, dtype=torch.float32)
+    bias, e, bmp = dma.dma_mask_build(p, V, torch.zeros(H, d, device="cuda"), torch.ones(H, device="cuda"))
+    O, lse = dma.dma_attn_fwd(p, Q, K, V, bias, e, bmp)
+    got = dma.dma_attn_bwd(p, Q, K, V, O, dO, lse, bias, e, bmp)
+    q, k, v, go = (t[0].transpose(0, 1).double() for t in (Q, K, V, dO))                 # [H, L, d]
+    hide = torch.ones(L, L, dtype=torch.bool, device="cuda").triu(1)
+    pr = torch.softmax((q @ k.mT / d ** 0.5 + bias[0, :, None].double()).masked_fill(hide, float("-inf")), -1)
+    ds = pr * (go @ v.mT - (go * (pr @ v)).sum(-1, keepdim=True))
+    ref = [ds @ k / d ** 0.5, ds.mT @ q / d ** 0.5, pr.mT @ go]
+    for name, a, r in zip(("dQ", "dK", "dV"), got, ref):
+        assert_close(a, r.transpose(0, 1)[None].cpu().numpy(), "fp32", name)
+    assert_close(got[3], ds.sum(1)[None].cpu().numpy(), "fp32", "dM")
