@@ -666,10 +666,14 @@ int split_keys(const Prob& P) {
     while (per < kMaxSplit && bh * ((P.w + per - 1) / per) > kResident) per += kMinSplit;
     return per;
 }
-// The most splits of all rows that a call with at most P.w kept keys and at most P.B * P.Hq rows has. (The splits of one call
+// The kept keys per row that a workspace is sized for: the window, whatever the cached length up to 65536, so that a loop may take
+// its workspace at any step. (A window of 2^31 - 1, "keep all", is the longer cache's length.)
+int held_keys(const Prob& P) { return std::min(P.w_cap, std::max(P.L, 1 << 16)); }
+
+// The most splits of all rows that a call with at most `keep` kept keys and at most P.B * P.Hq rows has. (The splits of one call
 // fall where a longer list takes longer splits.)
-size_t most_splits(const Prob& P) {
-    const size_t bh = (size_t)P.B * P.Hq, few = bh * ((P.w + kMinSplit - 1) / kMinSplit), many = bh * ((P.w + kMaxSplit - 1) / kMaxSplit);
+size_t most_splits(const Prob& P, int keep) {
+    const size_t bh = (size_t)P.B * P.Hq, few = bh * ((keep + kMinSplit - 1) / kMinSplit), many = bh * ((keep + kMaxSplit - 1) / kMaxSplit);
     return std::max(std::min(few, (size_t)kResident), many);
 }
 
@@ -684,7 +688,7 @@ int launch_typed(const Prob& P, const void* q, const void* K, const void* V, con
 
 }  // namespace
 
-static int list_splits(const Prob& P) { return (P.w_cap + kListSplit - 1) / kListSplit; }
+static int list_splits(const Prob& P) { return (held_keys(P) + kListSplit - 1) / kListSplit; }
 
 // header | tickets | kept lists | partials of the larger of the two attention kernels' split counts
 struct DecodeWs {
@@ -695,13 +699,14 @@ struct DecodeWs {
 };
 static DecodeWs decode_ws(const Prob& P, void* ws) {
     const size_t bh = (size_t)P.B * P.Hq;
-    const size_t splits = std::max(most_splits(P), bh * list_splits(P));
+    const int keep = held_keys(P);
+    const size_t splits = std::max(most_splits(P, keep), bh * list_splits(P));
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     DecodeWs w;
     size_t off = kWsHeaderBytes;
     char* base = (char*)ws;
     w.tickets = reinterpret_cast<int*>(base + off); off += up(bh * sizeof(int));
-    w.kept = reinterpret_cast<int*>(base + off); off += up(bh * P.w * sizeof(int));
+    w.kept = reinterpret_cast<int*>(base + off); off += up(bh * keep * sizeof(int));
     w.partial = reinterpret_cast<float*>(base + off); off += splits * (P.d + 2) * sizeof(float);
     w.bytes = off;
     return w;
