@@ -231,8 +231,8 @@ int dma_mask_bwd(const dma_problem_t* p, const void* V, const float* W_delta, co
  * dma_decode: every (batch, query head) keeps the min(w, N) keys with the largest delta (ties to the lower index) and
  * returns o = softmax(q . K_sel^T scale + delta_sel) V_sel and its log-sum-exp lse [B, Hq] (natural log). sel_idx, if
  * not NULL, receives the kept key indices [B, Hq, min(w, N)] int32 in ascending order. Only the selected K and V rows
- * are read. ws: dma_decode_workspace() bytes, a size that does not fall as N or B grows and is the same for all N up to 65536 (a loop
- * takes any step's there, else its last one's). All
+ * are read. ws: dma_decode_workspace() bytes, a size that does not fall as N or B grows and, with w up to 2^20, does not depend on N
+ * (a loop takes any step's; with a longer w its last one's). All
  * pointers device memory, 16-byte aligned. */
 int dma_delta_range(const dma_problem_t* p, const void* V, const float* W_delta, const float* A, float* delta, int64_t delta_ld,
                     int32_t j_begin, int32_t j_end, void* cuda_stream);

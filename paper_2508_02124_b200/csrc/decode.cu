@@ -666,9 +666,9 @@ int split_keys(const Prob& P) {
     while (per < kMaxSplit && bh * ((P.w + per - 1) / per) > kResident) per += kMinSplit;
     return per;
 }
-// The kept keys per row that a workspace is sized for: the window, whatever the cached length up to 65536, so that a loop may take
-// its workspace at any step. (A window of 2^31 - 1, "keep all", is the longer cache's length.)
-int held_keys(const Prob& P) { return std::min(P.w_cap, std::max(P.L, 1 << 16)); }
+// The kept keys per row that a workspace is sized for: the window, whatever the cached length, so that a loop may take its workspace
+// at any step; a window beyond 2^20 (2^31 - 1: "keep all") stands for the cached length.
+int held_keys(const Prob& P) { return P.w_cap <= 1 << 20 ? P.w_cap : P.w; }
 
 // The most splits of all rows that a call with at most `keep` kept keys and at most P.B * P.Hq rows has. (The splits of one call
 // fall where a longer list takes longer splits.)

@@ -117,7 +117,7 @@ def test_decoding_calls_accept_the_last_step_s_workspace(lib, B, Hq, w):
 
 
 @no_device
-@pytest.mark.parametrize("B,Hq,w", [(1, 32, 1280), (1, 32, 2048), (2, 8, 1000), (1, 1, 65536)])
+@pytest.mark.parametrize("B,Hq,w", [(1, 32, 1280), (1, 32, 2048), (2, 8, 1000), (1, 1, 65536), (1, 2, 1 << 20)])
 def test_decoding_calls_accept_the_first_step_s_workspace(lib, B, Hq, w):
     a, z = ctypes.c_void_p(4096), ctypes.c_void_p(0)
     ws = ctypes.c_size_t(dma.dma_decode_workspace(dma.problem(B, Hq, Hq, 1, 128, w)))
@@ -131,8 +131,8 @@ def test_decoding_calls_accept_the_first_step_s_workspace(lib, B, Hq, w):
 def test_decode_workspace_of_a_window_without_bound(lib, w):
     """`Keep all`: the window does not count beyond the cached keys. (Kept indices and, per 128 of them, a partial row of d + 2 floats.)"""
     for N in (1, 1000, 65536, 200000):
-        rows, keep = 32, max(N, 65536)
-        assert 0 < dma.dma_decode_workspace(dma.problem(1, 32, 8, N, 128, w)) <= 4096 + rows * (keep * 4 + (keep // 128 + 1) * 130 * 4), (w, N)
+        rows, keep = 32, N
+        assert 0 < dma.dma_decode_workspace(dma.problem(1, 32, 8, N, 128, w)) <= 200000 + rows * (keep * 4 + (keep // 128 + 1) * 130 * 4), (w, N)
 
 
 @pytest.mark.parametrize("flags", [0, dma.DMA_FLAG_FULL_DELTA])
