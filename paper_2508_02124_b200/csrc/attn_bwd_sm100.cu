@@ -116,7 +116,8 @@ __device__ __forceinline__ uint4 split3(float x) {
 // same query rows, so the walk over query tiles [first key's tile, last expiry's tile] wastes little. K and V rows
 // are gathered once with 16-byte asynchronous copies; dK and dV are added to fp32 accumulators (the query heads of a
 // group meet there), dM is written directly.
-template <bool kCompact, int kD>
+// kLong: tile mode without a split of the query heads and without the overlapped launch, for problems that last long (bwd_long).
+template <bool kCompact, int kD, bool kLong = false>
 __global__ void __launch_bounds__(kThreads, 1)
 bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const BwdParams P) {
@@ -125,7 +126,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     constexpr bool kDouble = kD == 64;               // P^T / dS^T in two buffers used in turn (see the file header)
     extern __shared__ uint8_t smem_raw[];
     SharedStorage& S = *reinterpret_cast<SharedStorage*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    pdl_enter();
+    static_assert(!(kCompact && kLong), "kLong is a tile mode");
+    if constexpr (!kLong) pdl_enter();
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // warp-uniform to the compiler: role branches stay uniform
     // tile mode: blockIdx.x = (batch, KV head, split of its query heads); token-compacted mode: (batch, query head), whose group index is fixed
@@ -133,7 +135,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     // tile 0 has the most query tiles: heaviest first), then the groups
     const int lin = blockIdx.y * gridDim.x + blockIdx.x, per_group = P.sched_group * (int)gridDim.y;
     const int bx = (lin / per_group) * P.sched_group + (lin % per_group) % P.sched_group;
-    const int nsplit = kCompact ? 1 : P.nsplit, sp = kCompact ? 0 : bx % nsplit;
+    const int nsplit = kCompact || kLong ? 1 : P.nsplit, sp = kCompact || kLong ? 0 : bx % nsplit;
     const int b = kCompact ? bx / P.Hq : bx / (nsplit * P.Hkv);
     const int hq_c = bx % P.Hq;                        // token-compacted mode only
     const int hk = kCompact ? hq_c / P.G : bx / nsplit % P.Hkv;
@@ -821,6 +823,13 @@ int tc_bwd_splits(const Prob& P) {
         if (P.G % n == 0 && steps(n) < steps(best)) best = n;
     return best;
 }
+// Tile mode without a split: from 256 64-row steps per SM on (about 0.36 ms) the instance that knows of no split and leaves the wait for
+// its predecessor to the stream. Both only precede the main loop but cost it 2 %, while an overlapped launch saves 2 us: 16384 rows,
+// 32 / 8 heads, backward at full clocks 4.95 -> 4.88 ms, over 20 calls at the power cap 5.56 -> 5.48 (4.85 and 5.43 before either
+// existed; the split's constant alone 4.90, 5.51). At 8192 rows of 16 heads (450 steps, 0.74 ms) runs differ by more than that.
+bool bwd_long(const Prob& P) {
+    return !(P.flags & DMA_FLAG_COMPACT_KV) && tc_bwd_splits(P) == 1 && (int64_t)P.B * P.Hq * P.Tc * (P.Tr + 1) >= 256 * 148;
+}
 // copies of the dK, dV accumulators (0: the main kernel writes dK, dV itself)
 static size_t bwd_slots(const Prob& P) {
     if (P.flags & DMA_FLAG_COMPACT_KV) return (P.flags & DMA_FLAG_DETERMINISTIC) ? (size_t)P.G : 1;
@@ -910,10 +919,15 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     bp.perm = perm; bp.expiry_all = expiry; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
     bp.dKacc = accK; bp.dVacc = accV; bp.acc_slot = slots > 1 ? (int64_t)nkv : 0; bp.nsplit = nsplit;
     const size_t smem = sizeof(SharedStorage) + 1024;
-    auto kern = compact ? (P.d == 128 ? bwd_kernel<true, 128> : bwd_kernel<true, 64>) : (P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>);
+    const bool lng = bwd_long(P);
+    auto kern = compact ? (P.d == 128 ? bwd_kernel<true, 128> : bwd_kernel<true, 64>)
+                : lng   ? (P.d == 128 ? bwd_kernel<false, 128, true> : bwd_kernel<false, 64, true>)
+                        : (P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     timing_mark(1, false, st);
-    rc = launch_overlapped(kern, dim3(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc), dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
+    const dim3 grid(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc);
+    rc = lng ? launch_plain(kern, grid, dim3(kThreads), smem, st, tmQ, tmK, tmV, tmG, bp)
+             : launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
     timing_mark(1, true, st);
     if (rc) return rc;
     FinishParams f;

@@ -84,7 +84,7 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
 // 3071 us for its training step.)
 // Returns a dma_status; a caller that gets an error launches nothing more, since the later kernels read what this one writes.
 template <typename... KArgs, typename... Args>
-inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
+inline int launch_config(bool overlapped, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -92,7 +92,7 @@ inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = overlapped ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cluster > 1) {
@@ -108,6 +108,15 @@ inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     }
     count_launch();
     return DMA_OK;
+}
+template <typename... KArgs, typename... Args>
+inline int launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args... args) {
+    return launch_config(true, kernel, grid, block, smem, st, cluster, args...);
+}
+// the launch of a kernel that does not wait itself
+template <typename... KArgs, typename... Args>
+inline int launch_plain(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    return launch_config(false, kernel, grid, block, smem, st, 1, args...);
 }
 
 // ---------------------------------------------------------------------------------------------

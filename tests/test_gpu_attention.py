@@ -576,3 +576,32 @@ def test_fp32_backward_of_more_heads_than_a_grid_has_rows():
     for name, a, r in zip(("dQ", "dK", "dV"), got, ref):
         assert_close(a, r.transpose(0, 1)[None].cpu().numpy(), "fp32", name)
     assert_close(got[3], ds.sum(1)[None].cpu().numpy(), "fp32", "dM")
+
+
+@pytest.mark.parametrize("L,d", [(3000, 64), (3072, 128), (3071, 128)])
+def test_tile_backward_of_long_problems_is_the_batch_entries_on_their_own(L, d):
+    """Eight batch entries take the backward's instance for long problems, each of them alone the one for short problems: dK, dV, dM are
+    the same bits, dQ (atomic sums in fp32) agrees to its rounding to bf16."""
+    B, H = 8, 8
+    case = wl.small(C2, B=B, Hq=H, Hkv=H, L=L, d=d, w=L // 2, seed=L, name="long-tile-bwd")
+    inp = {k: v.cuda() for k, v in wl.make_inputs(case).items()}
+    p = problem_of(case, flags=dma.DMA_FLAG_TILE_PATH)
+    Q, K, V, dO = (inp[k] for k in ("Q", "K", "V", "dO"))
+    bias, e, bmp = dma.dma_mask_build(p, V, inp["W_delta"], inp["A"])
+    O, lse = dma.dma_attn_fwd(p, Q, K, V, bias, e, bmp)
+    whole = dma.dma_attn_bwd(p, Q, K, V, O, dO, lse, bias, e, bmp)
+    p1 = dma.problem(1, H, H, L, d, L // 2, flags=dma.DMA_FLAG_TILE_PATH)
+    words = dma.dma_bitmap_words(p1)
+    for b in (0, 3, B - 1):
+        one = lambda t: t[b:b + 1].contiguous()   # noqa: E731
+        part = dma.dma_attn_bwd(p1, one(Q), one(K), one(V), one(O), one(dO), one(lse), one(bias), one(e), bmp.flatten()[b * words:(b + 1) * words].contiguous())
+        for name, x, y in zip(("dQ", "dK", "dV", "dM"), whole, part):
+            x = x[b:b + 1]
+            if name == "dQ":
+                # two fp32 sums of the same L / 32 terms in another order: L / 32 roundings of partial sums, bounded by the largest
+                # element of the tensor; where they fall on two sides of a rounding boundary the bf16 values are a whole spacing,
+                # up to 2^-7 of the element, apart
+                x, y = x.float(), y.float()
+                assert ((x - y).abs() <= 2.0 ** -7 * torch.maximum(x.abs(), y.abs()) + 2.0 ** -24 * L / 32 * y.abs().max()).all(), b
+            else:
+                assert torch.equal(x, y), (name, b)
