@@ -518,9 +518,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_attn_kernel(const T* _
 //         [4..7] unused
 //   int32 [8 .. 8 + w)       the kept key indices, in no particular order
 // A step costs O(w), whatever the number of cached keys: no scan of the delta row.
-// kept keys per CTA of the list attention kernel: at w = 2048 and 32 rows 256 CTAs, all resident at once, with two batches per
-// warp (32 tokens 402 us; 457 with 128 keys, whose 512 CTAs come in two waves)
-constexpr int kListSplit = 256;
+constexpr int kListSplit = 256;                     // most kept keys per CTA of the list attention kernel (list_split)
 
 __device__ __forceinline__ int state_stride(int w_cap) { return kStateHeader + ((w_cap + 3) & ~3); }
 
@@ -586,14 +584,14 @@ __device__ __forceinline__ void decode_state_update(const float* __restrict__ de
 
 // attention over the row's kept list as it is AFTER the appended key N - 1 is taken into account (the stored state still
 // describes the first N - 1 keys; decode_step_combine_kernel brings it up to date afterwards)
-template <typename T, int D>
+template <typename T, int D, int kSplit>
 __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const T* __restrict__ q, const T* __restrict__ K,
                                                                         const T* __restrict__ V, const float* __restrict__ delta,
                                                                         int64_t ld, const int* __restrict__ state, int w_cap,
                                                                         float* __restrict__ partial, int N, int Hq, int G,
                                                                         float scale_log2, int nsplit, int64_t ks_b, int64_t ks_l,
                                                                         int64_t ks_h, int64_t vs_b, int64_t vs_l, int64_t vs_h) {
-    __shared__ int list[kListSplit];
+    __shared__ int list[kSplit];
     const int split = blockIdx.x, bh = blockIdx.y, b = bh / Hq, h = bh % Hq, hk = h / G;
     const int tid = threadIdx.x;
     pdl_enter(q, K, V, delta, state, partial);
@@ -601,13 +599,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const
     const int* hdr = state + (size_t)bh * state_stride(w_cap);
     const int* kept = hdr + kStateHeader;
     const int newj = N - 1, count = hdr[0];
-    const int e = split * kListSplit + tid;
-    const int held = tid < kListSplit && e < w_cap ? kept[e] : 0;          // (in flight together with the header)
+    const int e = split * kSplit + tid;
+    const int held = tid < kSplit && e < w_cap ? kept[e] : 0;          // (in flight together with the header)
     const int mode = step_mode(hdr, w_cap, key_of(dl[newj], newj));
     const int eff = count + (mode == 1 ? 1 : 0), weakest = hdr[1];
-    if (tid < kListSplit && e < eff) list[tid] = (e >= count || (mode == 2 && e == weakest)) ? newj : held;
+    if (tid < kSplit && e < eff) list[tid] = (e >= count || (mode == 2 && e == weakest)) ? newj : held;
     __syncthreads();
-    decode_attend<T, D>(list, max(0, min(kListSplit, eff - split * kListSplit)), q, K, V, dl,
+    decode_attend<T, D>(list, max(0, min(kSplit, eff - split * kSplit)), q, K, V, dl,
                         partial + ((size_t)bh * nsplit + split) * (D + 2), bh, b, hk, scale_log2, ks_b, ks_l, ks_h, vs_b, vs_l, vs_h);
 }
 
@@ -688,7 +686,18 @@ int launch_typed(const Prob& P, const void* q, const void* K, const void* V, con
 
 }  // namespace
 
-static int list_splits(const Prob& P) { return (held_keys(P) + kListSplit - 1) / kListSplit; }
+// Kept keys per CTA of a step with the carried state: 128 where all CTAs have an SM to themselves, else 256, two batches per warp.
+// Eight captured steps, us, 128 / 256 keys: one row of w = 2048 70 / 74, 8 rows of 256 66 / 72, 16 rows of 1024 (128 CTAs) 72 /
+// 76, but 16 rows of 2048 (256 CTAs) 96 / 96, one row of 32768 182 / 162, 32 rows of 2048 121 / 111, 256 rows of 4096 1127 / 926.
+static int list_split(const Prob& P) {
+    const int64_t ctas = (int64_t)P.B * P.Hq * ((held_keys(P) + kMinSplit - 1) / kMinSplit);
+    return ctas <= 148 ? kMinSplit : kListSplit;
+}
+// the most splits of all rows that a step with at most `keep` kept keys and at most P.B * P.Hq rows has
+static size_t most_list_splits(const Prob& P, int keep) {
+    const size_t bh = (size_t)P.B * P.Hq;
+    return std::max(std::min(bh * ((keep + kMinSplit - 1) / kMinSplit), (size_t)148), bh * ((keep + kListSplit - 1) / kListSplit));
+}
 
 // header | tickets | kept lists | partials of the larger of the two attention kernels' split counts
 struct DecodeWs {
@@ -700,7 +709,7 @@ struct DecodeWs {
 static DecodeWs decode_ws(const Prob& P, void* ws) {
     const size_t bh = (size_t)P.B * P.Hq;
     const int keep = held_keys(P);
-    const size_t splits = std::max(most_splits(P, keep), bh * list_splits(P));
+    const size_t splits = std::max(most_splits(P, keep), most_list_splits(P, keep));
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     DecodeWs w;
     size_t off = kWsHeaderBytes;
@@ -762,8 +771,9 @@ int launch_decode_state_init(const Prob& P, const float* delta, int64_t ld, int*
 template <typename T, int D>
 static int launch_step_typed(const Prob& P, const void* q, const void* K, const void* V, const float* delta, int64_t ld, int* state,
                              void* o, float* lse, float* partial, cudaStream_t st) {
-    const int ns = list_splits(P);
-    const int rc = launch_overlapped(decode_list_attn_kernel<T, D>, dim3(ns, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
+    const int per = list_split(P), ns = (held_keys(P) + per - 1) / per;
+    auto kern = per == kMinSplit ? decode_list_attn_kernel<T, D, kMinSplit> : decode_list_attn_kernel<T, D, kListSplit>;
+    const int rc = launch_overlapped(kern, dim3(ns, P.B * P.Hq), dim3(kAttnThreads), 0, st, 1, (const T*)q, (const T*)K, (const T*)V,
                           delta, ld, (const int*)state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns, P.ks[0], P.ks[1],
                           P.ks[2], P.vs[0], P.vs[1], P.vs[2]);
     if (rc) return rc;

@@ -57,7 +57,9 @@ def run(case, n0, steps, seed=5, tie_head=False):
 @pytest.mark.parametrize("kw,n0,steps", [
     (dict(B=1, Hq=2, Hkv=2, L=64, d=64, w=8, dtype="fp32"), 0, 40),          # from an empty cache through the fill-up
     (dict(B=2, Hq=4, Hkv=2, L=400, d=64, w=100, dtype="bf16"), 90, 60),      # prefill below w: appends, then replacements
-    (dict(B=1, Hq=8, Hkv=2, L=1200, d=128, w=300, dtype="bf16"), 1100, 50),  # two list splits, the second ragged
+    (dict(B=1, Hq=8, Hkv=2, L=1200, d=128, w=300, dtype="bf16"), 1100, 50),  # splits of 128 keys (24 CTAs), the last ragged
+    (dict(B=2, Hq=8, Hkv=2, L=1200, d=64, w=1152, dtype="bf16"), 1130, 40),  # 144 CTAs of 128 keys, the last of each row filling up
+    (dict(B=2, Hq=8, Hkv=2, L=1200, d=64, w=1170, dtype="bf16"), 1140, 40),  # 160 would be more than SMs: 256 keys, ragged
     (dict(B=1, Hq=4, Hkv=4, L=300, d=128, w=1, dtype="fp32"), 200, 40),      # a single kept key
     (dict(B=1, Hq=4, Hkv=1, L=200, d=128, w=4096, dtype="bf16"), 150, 30),   # w above the cache: everything is kept
 ])

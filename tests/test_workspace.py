@@ -105,7 +105,7 @@ def test_decode_workspace_never_falls(lib, Hq, Hkv, w):
 
 
 @no_device
-@pytest.mark.parametrize("B,Hq,w", [(1, 32, 1280), (1, 32, 1200), (2, 32, 600), (1, 1, 2048)])
+@pytest.mark.parametrize("B,Hq,w", [(1, 32, 1280), (1, 32, 1200), (2, 32, 600), (1, 1, 2048), (3, 8, 1024), (1, 40, 512)])
 def test_decoding_calls_accept_the_last_step_s_workspace(lib, B, Hq, w):
     a, z = ctypes.c_void_p(4096), ctypes.c_void_p(0)
     ws = ctypes.c_size_t(dma.dma_decode_workspace(dma.problem(B, Hq, Hq, 16384, 128, w)))
@@ -114,6 +114,9 @@ def test_decoding_calls_accept_the_last_step_s_workspace(lib, B, Hq, w):
         assert lib.dma_decode(p, a, a, a, a, ld, a, a, z, a, ws, z) == ERR_CUDA, N
         assert lib.dma_decode_step(p, a, a, a, a, ld, a, a, a, a, ws, z) == ERR_CUDA, N
         assert lib.dma_decode_state_init(p, a, ld, a, a, ws, z) == ERR_CUDA, N
+    for b in range(1, B):                                    # (fewer rows may take shorter splits, hence more of them)
+        p = ctypes.byref(dma.problem(b, Hq, Hq, 4096, 128, w))
+        assert lib.dma_decode_step(p, a, a, a, a, ld, a, a, a, a, ws, z) == ERR_CUDA, b
 
 
 @no_device
