@@ -80,3 +80,11 @@ def test_binding_refuses_tensors_of_another_element_type():
         dma.dma_attn_fwd(p, V, V, V, None, None, None)
     with pytest.raises(TypeError):
         dma.problem(1, 2, 2, 8, 64, 4, dtype=torch.float16)
+
+
+def test_typed_calls_match_the_header():
+    text = re.sub(r"/\*.*?\*/", "", open(os.path.join(ROOT, "include", "dma.h")).read(), flags=re.S)
+    for name, kinds in dma._SIGNATURES.items():
+        args = re.search(r"\b" + name + r"\s*\(([^;]*)\)\s*;", text).group(1).split(",")
+        assert kinds == "".join("P" if "dma_problem_t" in a else "v" if "*" in a else "z" if "size_t" in a else "l" if "int64_t" in a else "i"
+                                for a in args), name
