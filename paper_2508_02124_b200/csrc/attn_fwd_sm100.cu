@@ -19,7 +19,10 @@
 // kD = 64 (its own instantiations): Q, K and V tiles are one 16 KB half tile each (the second half of every buffer stays
 // unused), S = Q K^T has four k-steps and the ninth, O_w takes 64 columns.
 // The log-sum-exp replaces Alg. 1's (l, m) pair.
+#include <algorithm>
+#include <cmath>
 #include <cstdlib>
+#include <type_traits>
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
@@ -61,10 +64,17 @@ struct SharedStorage {
                                               // bits 8-15: 16-key blocks that hold a key some row of the query tile may keep
     uint32_t sched[kMaxSched];                // key tile | use by tile 0 << 30 | use by tile 1 << 31
     uint64_t q_full, k_full[kStages], v_full[kStages], k_empty[kStages], v_empty[kStages];
-    uint64_t s_full[2], p_half[2], p_ready[2], o_done[2];
+    uint64_t s_full[2], p_half[2], p_ready[2], o_done[2], merge;
     uint32_t tmem_base;
     int n_iters;
     int abort_flag;
+    // One query tile per CTA (kSplit): a group's flags, `fast`, and what its per-element test reads are in two slots that its entries take
+    // in turn. Token-compacted: group 1's len and jidx. Tile mode: a byte per column, expiry[j] relative to the query tile's first row, cut
+    // to [0, 128]: row r of the tile keeps the key iff r is below it (and, in the diagonal tile, not below the column).
+    union {
+        struct { alignas(16) int len1[2][128], jidx1[2][128]; };
+        alignas(16) uint8_t last[2][2][128];
+    };
 };
 static_assert(kStages == 2 && offsetof(SharedStorage, bext) == offsetof(SharedStorage, aext) + 2 * 4096,
               "token-compacted mode takes aext and bext as six blocks of 2 KB in a row: ones, two stages of two tiles, zeros");
@@ -108,11 +118,15 @@ constexpr int kWarpProducer = 0, kWarpIssuer = 1, kWarpStager0 = 2, kWarpStager1
 // rows are constant) and flags the 32-column chunks that still need the per-element test.
 // kBlockSkip: MMA-block skipping inside executed tiles (DMA_FLAG_BLOCK_SKIP), a separate instantiation so that the
 // default kernel carries none of its code (the kernel is sensitive to the size of its service warps' loops).
-template <bool kCompact, bool kBlockSkip, int kD>
+// kSplit: the CTA owns ONE query tile and its two softmax groups take the key tiles (slices) in turn, entry t of the schedule by
+// group t & 1; group 1 hands its O, row max and row sum over in shared memory at the end. A CTA's walk is then half as long, for grids
+// that leave SMs idle (tc_fwd_tiles).
+template <bool kCompact, bool kBlockSkip, int kD, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const FwdParams P) {
     static_assert(kD == 128 || kD == 64, "head dimensions of the tensor-core kernels");
+    static_assert(!(kSplit && kBlockSkip), "no blocks are skipped where the groups share a query tile");
     constexpr int kHalves = kD / 64;                         // 64-channel (128-byte) swizzled half tiles per operand tile
     constexpr uint32_t kLoadBytes = kHalves * (kTileBytes / 2);
     extern __shared__ uint8_t smem_raw[];
@@ -122,9 +136,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // warp-uniform to the compiler: role branches stay uniform
     const int bh = blockIdx.x, b = bh / P.Hq, h = bh % P.Hq, hk = h / P.G;
     const int npairs = (P.Trq + 1) / 2;
-    const int pair = npairs - 1 - (int)blockIdx.y;          // heaviest query tiles first
-    const int qt0 = 2 * pair, qt1 = 2 * pair + 1;           // query tiles inside the chunk (the whole sequence unless P.q_off / P.Lq say otherwise)
-    const bool has1 = qt1 < P.Trq;
+    const int unit = (kSplit ? P.Trq : npairs) - 1 - (int)blockIdx.y;  // pair of query tiles (kSplit: query tile), heaviest first
+    const int pair = kSplit ? unit >> 1 : unit;
+    const int qt0 = kSplit ? unit : 2 * pair, qt1 = kSplit ? unit : 2 * pair + 1;   // query tiles inside the chunk (the whole sequence unless P.q_off / P.Lq say otherwise)
+    const bool has1 = !kSplit && qt1 < P.Trq;
     const int lpair = (kCompact && !P.causal) ? 0 : pair;   // non-causal: all rows of a head keep the same keys, one list serves every pair
     volatile int* abort_flag = &S.abort_flag;
 
@@ -142,6 +157,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             mbar_init(&S.p_ready[w], 4);
             mbar_init(&S.o_done[w], 1);
         }
+        mbar_init(&S.merge, 4);
         S.abort_flag = 0;
         S.n_iters = 0;
         fence_barrier_init();
@@ -150,6 +166,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         tmem_alloc(&S.tmem_base, 512);
         tmem_relinquish();
     }
+    // tile mode: the workspace header is cleared here (a wait that times out writes the status a second later at the earliest)
+    if (!kCompact && blockIdx.x == 0 && blockIdx.y == 0 && tid < kWsHeaderBytes / 4) P.status[tid] = 0;
     if (warp == kWarpProducer) {
         // schedule: ascending key tiles that at least one of the two query tiles uses
         if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
@@ -159,7 +177,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const int listed = P.ccnt[(size_t)bh * npairs + lpair];
             if (listed > P.ccap && lane == 0) atomicExch(P.status, (int32_t)DMA_ERR_MASK_OVERFLOW);
             n = min((min(listed, P.ccap) + 127) / 128, kMaxSched);
-            for (int t = lane; t < n; t += 32) S.sched[t] = (uint32_t)t | (1u << 30) | (has1 ? (1u << 31) : 0u);
+            for (int t = lane; t < n; t += 32) S.sched[t] = (uint32_t)t | (kSplit ? 1u << (30 + (t & 1)) : (1u << 30) | (has1 ? (1u << 31) : 0u));
         } else {
             const int kt_last = min(has1 ? qt1 : qt0, P.Tc - 1);
             for (int base = 0; base <= kt_last; base += 32) {
@@ -170,7 +188,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     u1 = has1 && kt <= qt1 && (P.ignore_bitmap || bitmap_test(P.bitmap, P.Tr, P.Wd, bh, qt1, kt));
                 }
                 const uint32_t act = __ballot_sync(0xffffffffu, u0 | u1);
-                if (u0 | u1) S.sched[n + __popc(act & ((1u << lane) - 1))] = (uint32_t)kt | (u0 << 30) | (u1 << 31);
+                const int at = n + __popc(act & ((1u << lane) - 1));
+                if (u0 | u1) S.sched[at] = (uint32_t)kt | (kSplit ? 1u << (30 + (at & 1)) : (u0 << 30) | (u1 << 31));
                 n += __popc(act);
             }
         }
@@ -193,13 +212,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + lane_base + w * 128;
         const uint32_t tO = tmem + lane_base + 256 + w * 128;
+        const uint32_t rows4 = (uint32_t)r * 0x01010101u;
         float m_ref = -INFINITY, r_ref = 0.0f, l = 0.0f;
         int n_used = 0;
         bool ok = true;
         for (int it = 0; it < n_iters && ok; ++it) {
             const uint32_t entry = S.sched[it];
             if (!use_bit(entry, w)) continue;
-            const int st = it % kStages, j0 = (int)(entry & 0xFFFFF) * 128;
+            const int st = kSplit ? n_used & 1 : it % kStages, j0 = (int)(entry & 0xFFFFF) * 128;
             ok = mbar_wait_warp(&S.s_full[w], n_used & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
@@ -229,10 +249,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if ((tile_flags >> q) & 1u) {
+                        const int* le = kSplit && w ? S.len1[st] : S.len[st];
+                        const int* ji = kSplit && w ? S.jidx1[st] : S.jidx[st];
 #pragma unroll
                         for (int c = 32 * q; c < 32 * q + 32; c += 4) {
-                            const int4 ee = *reinterpret_cast<const int4*>(&S.len[st][c]);
-                            const int4 jj = *reinterpret_cast<const int4*>(&S.jidx[st][c]);
+                            const int4 ee = *reinterpret_cast<const int4*>(&le[c]);
+                            const int4 jj = *reinterpret_cast<const int4*>(&ji[c]);
                             const int ev[4] = {ee.x, ee.y, ee.z, ee.w}, jv[4] = {jj.x, jj.y, jj.z, jj.w};
 #pragma unroll
                             for (int u = 0; u < 4; ++u) x[c + u] = (jv[u] <= i && i < ev[u]) ? x[c + u] : -INFINITY;
@@ -248,6 +270,24 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) mxa[u] = mxa[u] < -1e20f ? -INFINITY : mxa[u];
+            } else if constexpr (kSplit) {
+                // four columns per word, bit 7 of a byte: r < last, and in the diagonal tile column <= r
+                const bool diag = (int)(entry & 0xFFFFF) == qt;
+                const uint32_t step = diag ? 0x04040404u : 0u, seen0 = diag ? 0x80808080u + rows4 - 0x03020100u : 0x80808080u;
+#pragma unroll
+                for (int h4 = 0; h4 < 8; ++h4) {
+                    const uint4 t4 = *reinterpret_cast<const uint4*>(&S.last[st][w][16 * h4]);
+                    const uint32_t tw[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        const int c = 16 * h4 + 4 * g;
+                        const uint32_t keep = (tw[g] + (0x7F7F7F7Fu - rows4)) & (seen0 - (uint32_t)(4 * h4 + g) * step);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) x[c + u] = (keep & (0x80u << (8 * u))) ? x[c + u] : -INFINITY;
+                        mxa[g & 1] = max3(mxa[g & 1], x[c], x[c + 1]);
+                        mxa[2 + (g & 1)] = max3(mxa[2 + (g & 1)], x[c + 2], x[c + 3]);
+                    }
+                }
             } else {
 #pragma unroll
                 for (int c = 0; c < 128; c += 4) {
@@ -350,10 +390,50 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         // epilogue: O_w / l -> bf16 rows, log-sum-exp in natural log
         const bool exists = w == 0 || has1;
-        if (ok && exists && n_used > 0) ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
+        if (ok && (exists || kSplit) && n_used > 0) ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
+        // kSplit: group 1 leaves its row max, row sum and O (chunks of four channels, rows innermost) in what only it has used: the second
+        // query tile's buffer and stage 1 of K and V, which no load or product touches once its last P V is done
+        float* other = reinterpret_cast<float*>(S.q[1]);
+        auto other_o = [&](int c) { return reinterpret_cast<float4*>(c < 64 ? S.k[1] : S.v[1]) + ((c & 63) >> 2) * 128 + r; };
+        float f0 = 1.0f, f1 = 0.0f;
+        if constexpr (kSplit) {
+            if (ok && w == 1) {
+                tc_fence_after();
+                other[r] = m_ref;
+                other[128 + r] = r_ref;
+                other[256 + r] = l;
+                if (n_used > 0) {
+#pragma unroll
+                    for (int c = 0; c < kD / 32; ++c) {
+                        uint32_t o[32];
+                        tmem_ld32(tO + c * 32, o);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int u = 0; u < 32; u += 4)
+                            *other_o(c * 32 + u) = make_float4(__uint_as_float(o[u]), __uint_as_float(o[u + 1]), __uint_as_float(o[u + 2]), __uint_as_float(o[u + 3]));
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.merge);
+            }
+            if (ok && w == 0) {
+                ok = mbar_wait_warp(&S.merge, 0, abort_flag);
+                if (ok) {
+                    const float m1 = other[r], r1 = other[128 + r], l1 = other[256 + r];
+                    const bool mine = m_ref >= m1;
+                    const float m = mine ? m_ref : m1, rr = mine ? r_ref : r1;
+                    f0 = m_ref == -INFINITY ? 0.0f : ex2(fmaf(m_ref - m, P.scale_log2, rr - r_ref));
+                    f1 = m1 == -INFINITY ? 0.0f : ex2(fmaf(m1 - m, P.scale_log2, rr - r1));
+                    l = l * f0 + l1 * f1;
+                    m_ref = m;
+                    r_ref = rr;
+                }
+            }
+        }
         if (ok && exists) {
             tc_fence_after();
             const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+            const bool second = kSplit && n_iters > 1;       // (group 1 had an entry)
             __nv_bfloat16* orow = P.O + b * P.os_b + (int64_t)il * P.os_l + h * P.os_h;
 #pragma unroll
             for (int c = 0; c < kD / 32; ++c) {
@@ -364,6 +444,16 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 } else {
 #pragma unroll
                     for (int u = 0; u < 32; ++u) o[u] = 0;
+                }
+                if (second) {
+#pragma unroll
+                    for (int u = 0; u < 32; u += 4) {
+                        const float4 y = *other_o(c * 32 + u);
+                        o[u] = __float_as_uint(__uint_as_float(o[u]) * f0 + y.x * f1);
+                        o[u + 1] = __float_as_uint(__uint_as_float(o[u + 1]) * f0 + y.y * f1);
+                        o[u + 2] = __float_as_uint(__uint_as_float(o[u + 2]) * f0 + y.z * f1);
+                        o[u + 3] = __float_as_uint(__uint_as_float(o[u + 3]) * f0 + y.w * f1);
+                    }
                 }
                 if (il < P.Lq) {
 #pragma unroll
@@ -493,22 +583,27 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         }
                     }
                 }
-                // what this stage holds was last read by the softmax groups before they released P of slice it - kStages,
-                // hence before its P V, and by that slice's S products, which were issued before that P V
-                if (it >= kStages) ok = mbar_wait_warp(&S.v_empty[st], ((it / kStages) - 1) & 1, abort_flag);
+                // What this slot holds was last read by the softmax groups before they released P of slice it - kStages,
+                // hence before its P V, and by that slice's S products, which were issued before that P V. kSplit: the group's
+                // slot was last read for its entry before the last one, and the last one's S product was issued after that P V
+                const int slot = kSplit ? (it >> 1) & 1 : st;
+                if (it >= kStages) ok = kSplit ? mbar_wait_warp(&S.s_full[it & 1], ((it >> 1) - 1) & 1, abort_flag)
+                                               : mbar_wait_warp(&S.v_empty[st], ((it / kStages) - 1) & 1, abort_flag);
                 if (!ok) break;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const int c = lane + 32 * t;
-                    S.jidx[st][c] = jv[t] >= 0 ? (P.causal ? jv[t] : 0) : 0x7fffffff;  // first row of the key; padding: never <= a row index
-                    S.len[st][c] = ev[t];
+                    (kSplit && (it & 1) ? S.jidx1 : S.jidx)[slot][c] = jv[t] >= 0 ? (P.causal ? jv[t] : 0) : 0x7fffffff;  // first row of the key; padding: never <= a row index
+                    (kSplit && (it & 1) ? S.len1 : S.len)[slot][c] = ev[t];
 #pragma unroll
-                    for (int w = 0; w < 2; ++w)
-                        *reinterpret_cast<uint4*>(ext + (1 + st * 2 + w) * 2048 + c * 16) =
+                    for (int w = 0; w < 2; ++w) {
+                        if (kSplit && w != (it & 1)) continue;
+                        *reinterpret_cast<uint4*>(ext + (1 + slot * 2 + w) * 2048 + c * 16) =
                             make_uint4(b0[w][t], b0[w][t] == kNegBig ? 0u : b1[t], 0u, 0u);
+                    }
                     jv[t] = jn[t]; bv[t] = bn[t]; ev[t] = en[t]; jn[t] = jnn[t];
                 }
-                if (lane < 2) S.fast[st][lane] = (lane ? flags[1] : flags[0]) | ((kBlockSkip ? (lane ? live[1] : live[0]) : 0xFFu) << 8);
+                if (lane < 2 && (!kSplit || lane == (it & 1))) S.fast[slot][lane] = (lane ? flags[1] : flags[0]) | ((kBlockSkip ? (lane ? live[1] : live[0]) : 0xFFu) << 8);
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.k_full[st]);
@@ -644,12 +739,19 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                             aw[t][m - 1] = (r >= th[2 * m - 3] ? kOne : 0u) | (r >= th[2 * m - 2] ? (kOne << 16) : 0u);
                     }
                 }
-                // fast[st] / len[st] were last read by the softmax groups before they released P of tile it - kStages
-                // (hence before its P V); the operand blocks were last read by the S products of tile it - 1
-                if (it >= kStages) ok = mbar_wait_warp(&S.v_empty[st], ((it / kStages) - 1) & 1, abort_flag);
-                if (ok && it >= 1) ok = mbar_wait_warp(&S.k_empty[(it - 1) % kStages], ((it - 1) / kStages) & 1, abort_flag);
+                const int slot = kSplit ? (it >> 1) & 1 : st;
+                if constexpr (kSplit) {
+                    // The group's operand blocks were last read by its last S product, and the slot by the group before it released P of the
+                    // entry before that one, hence before that S product was issued. k_full takes one arrival per entry: not before its last phase is over.
+                    if (it >= kStages) ok = mbar_wait_warp(&S.k_empty[st], ((it / kStages) - 1) & 1, abort_flag);
+                } else {
+                    // fast[st] / len[st] were last read by the softmax groups before they released P of tile it - kStages
+                    // (hence before its P V); the operand blocks were last read by the S products of tile it - 1
+                    if (it >= kStages) ok = mbar_wait_warp(&S.v_empty[st], ((it / kStages) - 1) & 1, abort_flag);
+                    if (ok && it >= 1) ok = mbar_wait_warp(&S.k_empty[(it - 1) % kStages], ((it - 1) / kStages) & 1, abort_flag);
+                }
                 if (!ok) break;
-                if (w == 0) {
+                if (!kSplit && w == 0) {
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
                         S.len[st][lane + 32 * t] = ev[t];
@@ -659,6 +761,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
                         const int c = lane + 32 * t;
+                        if constexpr (kSplit) S.last[slot][w][c] = (uint8_t)min(max(ev[t] - i0, 0), 128);     // (columns beyond L: expiry 0)
                         uint32_t wd[8];
                         wd[0] = b0[t];
                         wd[1] = b1[t];
@@ -671,7 +774,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         *reinterpret_cast<uint4*>(arow) = make_uint4(kOne | (kOne << 16), aw[t][0], aw[t][1], aw[t][2]);
                         *reinterpret_cast<uint4*>(arow + 128) = make_uint4(aw[t][3], aw[t][4], aw[t][5], aw[t][6]);
                     }
-                    if (lane == 0) S.fast[st][w] = (fast ? 1u : 0u) | (live8 << 8);
+                    if (lane == 0) S.fast[slot][w] = (fast ? 1u : 0u) | (live8 << 8);
                 }
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -707,8 +810,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // load on the critical path: 1.98 -> 2.55 ms at L = 16384), so it stayed out.
             uint32_t live[2] = {0xFFu, 0xFFu};          // marks of the key tile whose S product was issued last, per query tile
             bool o_started[2] = {false, false};         // the O accumulator has been written (first product: no accumulate)
-            auto issue_s = [&](int w, int st) {
-                const uint64_t dq = dQ0 + (uint64_t)(w * (kTileBytes >> 4)), dk = dK0 + (uint64_t)(st * (kTileBytes >> 4));
+            auto issue_s = [&](int w, int st, int slot) {
+                const uint64_t dq = dQ0 + (uint64_t)(kSplit ? 0 : w * (kTileBytes >> 4)), dk = dK0 + (uint64_t)(st * (kTileBytes >> 4));
                 const uint32_t d_tmem = tmem_u + w * 128;
                 if (elect_one()) {
 #pragma unroll
@@ -716,19 +819,61 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         const uint32_t off = ((kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32) >> 4;
                         mma_ss(d_tmem, dq + off, dk + off, idesc_s, kk > 0);
                     }
-                    if constexpr (kCompact) mma_ss(d_tmem, dOnes, dRows + kNextBlock * (uint64_t)(st * 2 + w), idesc_s, 1u);
+                    if constexpr (kCompact) mma_ss(d_tmem, dOnes, dRows + kNextBlock * (uint64_t)(slot * 2 + w), idesc_s, 1u);
                     else mma_ss(d_tmem, dA0 + (uint64_t)(w * (4096 >> 4)), dB0 + (uint64_t)(w * (4096 >> 4)), idesc_s, 1u);
                     tc_commit(&S.s_full[w]);
                 }
                 __syncwarp();
                 // the block marks of this key tile, for its P V product later on: read AFTER the issue (a shared-memory load
                 // costs hundreds of cycles while the MMAs stream their operands, and the S products are on the critical path)
-                if constexpr (kBlockSkip) live[w] = *reinterpret_cast<volatile uint32_t*>(&S.fast[st][w]) >> 8;     // (every lane reads the same word; first used at the P V issue)
+                if constexpr (kBlockSkip) live[w] = *reinterpret_cast<volatile uint32_t*>(&S.fast[slot][w]) >> 8;     // (every lane reads the same word; first used at the P V issue)
             };
             const uint32_t both = (1u << 30) | (has1 ? (1u << 31) : 0u);     // token-compacted mode: every slice serves both tiles
             int n_p[2] = {0, 0};
             bool ok = mbar_wait_warp(&S.q_full, 0, abort_flag);
-            if (ok && n_iters_u > 0) {
+            if constexpr (kSplit) {
+                // entry it: group and stage it & 1, the group's entry number it >> 1. Both groups start at once; the next S product of a group
+                // is issued right behind its P V, so that the other group's softmax runs beside both
+                auto start = [&](int it) {
+                    const int w = it & 1;
+                    ok = mbar_wait_warp(&S.k_full[w], (it >> 1) & 1, abort_flag);
+                    if constexpr (kCompact) fence_proxy_async();
+                    if (!ok) return;
+                    tc_fence_after();
+                    issue_s(w, w, (it >> 1) & 1);
+                    if (elect_one()) tc_commit(&S.k_empty[w]);
+                    __syncwarp();
+                };
+                if (ok && n_iters_u > 0) start(0);
+                if (ok && n_iters_u > 1) start(1);
+                for (int it = 0; it < n_iters_u && ok; ++it) {
+                    const int w = it & 1, ph = (it >> 1) & 1;
+                    const uint64_t dv = dV0 + (uint64_t)(w * (kTileBytes >> 4));
+                    const uint32_t d_tmem = tmem_u + 256 + w * 128, a_tmem = tmem_u + w * 128;
+                    ok = mbar_wait_warp(&S.v_full[w], ph, abort_flag);
+                    if constexpr (kCompact) fence_proxy_async();
+                    if (ok) ok = mbar_wait_warp(&S.p_half[w], ph, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_ts(d_tmem, a_tmem + kk * 8, dv + (uint64_t)((kk * 2048) >> 4), idesc_pv, kk > 0 || it > 1 ? 1u : 0u);
+                    }
+                    __syncwarp();
+                    ok = mbar_wait_warp(&S.p_ready[w], ph, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int kk = 4; kk < 8; ++kk) mma_ts(d_tmem, a_tmem + kk * 8, dv + (uint64_t)((kk * 2048) >> 4), idesc_pv, 1u);
+                        tc_commit(&S.o_done[w]);
+                        tc_commit(&S.v_empty[w]);
+                    }
+                    __syncwarp();
+                    if (it + 2 < n_iters_u) start(it + 2);
+                }
+            } else if (ok && n_iters_u > 0) {
                 ok = mbar_wait_warp(&S.k_full[0], 0, abort_flag);
                 if (ok) {
                     if constexpr (kCompact) fence_proxy_async();
@@ -741,13 +886,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                             // two softmax groups stay in step: they contend for the issue slots and then wait for the MMAs
                             // together (L = 16384, w = 2048: 694 -> 680 us; 700 before the stager ran ahead)
                             if (kCompact && w == 1) ok = mbar_wait_warp(&S.p_half[0], 0, abort_flag);
-                            if (ok) issue_s(w, 0);
+                            if (ok) issue_s(w, 0, 0);
                         }
                     if (elect_one()) tc_commit(&S.k_empty[0]);
                     __syncwarp();
                 }
             }
-            for (int it = 0; it < n_iters_u && ok; ++it) {
+            for (int it = 0; !kSplit && it < n_iters_u && ok; ++it) {
                 const int st = it % kStages, nst = (it + 1) % kStages;
                 const uint32_t entry = kCompact ? both : __shfl_sync(0xffffffffu, S.sched[it], 0);
                 const uint32_t next = it + 1 >= n_iters_u ? 0u : kCompact ? both : __shfl_sync(0xffffffffu, S.sched[it + 1], 0);
@@ -816,7 +961,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                             if (ok) tc_fence_after();
                             k_ready = true;
                         }
-                        if (ok) issue_s(w, nst);
+                        if (ok) issue_s(w, nst, nst);
                     }
                 }
                 if (ok) {
@@ -1024,15 +1169,43 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
     return kWsHeaderBytes + cnt_bytes + compact_lists(P) * compact_cap(P) * sizeof(int);
 }
 
+// Query tiles per CTA: two, or one whose key tiles are dealt out to the two softmax groups where that shortens the call. Both grids
+// are estimated in steps of a CTA (two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs; the pair's
+// steps in tile mode are longer where many keys expire per tile, i.e. in short sequences. Fitted to 64 shapes of 1 to 128 heads and
+// 183 to 15889 keys, each timed with both: the faster one, or within 4 %, everywhere. Forward, us, two tiles / one: 16 heads of 1000
+// keys 37 / 18, 8 heads of 500 23 / 12, 8 heads of 4096 (w = 2048) 76 / 45, a chunk of 1185 rows of 18445 keys, one head 82 / 53, but 64
+// heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568.
+// The two add in different orders. A chunk of 16 query tiles and more always takes two, so that a head's rows come out the same however
+// many heads share the call.
+int tc_fwd_tiles(const Prob& P) {
+    if (P.fwd_split) return P.fwd_split;
+    constexpr double kOneSteps = 2.25, kTwoSteps = 3.0, kSms = 148.0;
+    const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2;
+    const double heads = (double)P.B * P.Hq;
+    if (P.flags & DMA_FLAG_COMPACT_KV) {                     // lists of about the same length
+        if (P.Lq < P.L && Trq >= 16) return 2;
+        const double n = std::min((int64_t)P.w + (P.causal ? 256 : 0), (int64_t)P.L) / 128.0;
+        return std::ceil(heads * Trq / kSms) * (n / 2 + kTwoSteps) < std::ceil(heads * npairs / kSms) * (n + kTwoSteps) ? 1 : 2;
+    }
+    const double total = Trq * (Trq + 1) / 2.0;              // walks grow with the row: the last tile's is the longest
+    const double one = std::max(Trq / 2.0 + kOneSteps, heads * (total / 2 + Trq * kOneSteps) / kSms);
+    const double two = (1.0 + 2.0 / Trq) * std::max(Trq + kTwoSteps, heads * (total / 2 + npairs * kTwoSteps) / kSms);
+    return one < two ? 1 : 2;
+}
+
 int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
                   const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st) {
     const bool compact = (P.flags & DMA_FLAG_COMPACT_KV) != 0;
     if (P.Tc > kMaxSched) return DMA_ERR_UNSUPPORTED;
     const bool block_skip = (P.flags & DMA_FLAG_BLOCK_SKIP) != 0;
-    auto kern = P.d == 128 ? (compact ? (block_skip ? fwd_kernel<true, true, 128> : fwd_kernel<true, false, 128>)
-                                      : (block_skip ? fwd_kernel<false, true, 128> : fwd_kernel<false, false, 128>))
-                           : (compact ? (block_skip ? fwd_kernel<true, true, 64> : fwd_kernel<true, false, 64>)
-                                      : (block_skip ? fwd_kernel<false, true, 64> : fwd_kernel<false, false, 64>));
+    const bool split = tc_fwd_tiles(P) == 1;
+    auto pick = [&](auto d_tag) {
+        constexpr int kD = decltype(d_tag)::value;
+        if (split) return compact ? fwd_kernel<true, false, kD, true> : fwd_kernel<false, false, kD, true>;
+        return compact ? (block_skip ? fwd_kernel<true, true, kD, false> : fwd_kernel<true, false, kD, false>)
+                       : (block_skip ? fwd_kernel<false, true, kD, false> : fwd_kernel<false, false, kD, false>);
+    };
+    auto kern = P.d == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
     {
         cudaFuncAttributes fa;       // (before anything is enqueued)
         if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs != kLaunchRegs) return DMA_ERR_CUDA;
@@ -1078,7 +1251,7 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
     fp.os_b = P.os[0]; fp.os_l = P.os[1]; fp.os_h = P.os[2];
     fp.ks_b = P.ks[0]; fp.ks_l = P.ks[1]; fp.ks_h = P.ks[2]; fp.vs_b = P.vs[0]; fp.vs_l = P.vs[1]; fp.vs_h = P.vs[2];
     const size_t smem = sizeof(SharedStorage) + 1024;
-    dim3 grid(P.B * P.Hq, npairs);
+    dim3 grid(P.B * P.Hq, split ? Trq : npairs);
     timing_mark(0, false, st);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     rc = launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, fp);
