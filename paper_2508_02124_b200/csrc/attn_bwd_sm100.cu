@@ -88,7 +88,7 @@ struct BwdParams {
     // token-compacted mode: per (batch, query head) a permutation of the keys (padded with L to a multiple of 128) that
     // groups keys of similar lifetime; a CTA owns 128 consecutive entries of one query head's permutation
     const int* perm;
-    const int32_t* expiry_all;
+    const int2* items;         // what each CTA does: [B, Hq, gridDim.y] (WorkItem)
     int causal;                // 0: key j is visible to every row (token-compacted mode only): its first row is 0 instead of j
     const __nv_bfloat16* Kg;    // K, V base pointers for the row gathers (ks_*, vs_* strides)
     const __nv_bfloat16* Vg;
@@ -101,6 +101,12 @@ struct BwdParams {
     int64_t ks_b, ks_l, ks_h, vs_b, vs_l, vs_h;
 };
 
+
+// Token-compacted mode: one CTA's work, a key tile of the head's permutation and a part of its walk over the query tiles q0 .. q1:
+//   x = key tile | part << 16 | parts << 24 (-1: nothing)     y = q0 | q1 << 16
+constexpr int kMostParts = 8;
+// 64-row steps of a walk (the sequence's last tile may have one only)
+__device__ __forceinline__ int walk_steps(int q0, int q1, int L) { return min(2 * (q1 - q0 + 1) - (q1 * 128 + 64 >= L ? 1 : 0), kMaxSteps); }
 
 // x as three bf16 terms (hi, mid, lo: 24 significant bits) in elements 0-2 of a 16-byte core-matrix row
 __device__ __forceinline__ uint4 split3(float x) {
@@ -139,15 +145,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     const int b = kCompact ? bx / P.Hq : bx / (nsplit * P.Hkv);
     const int hq_c = bx % P.Hq;                        // token-compacted mode only
     const int hk = kCompact ? hq_c / P.G : bx / nsplit % P.Hkv;
-    const int kt = (lin % per_group) / P.sched_group;
+    const int at = (lin % per_group) / P.sched_group;
+    const int2 item = kCompact ? P.items[(size_t)bx * gridDim.y + at] : make_int2(at, 0);
+    if (kCompact && item.x < 0) return;                // no more items for this head
+    const int kt = kCompact ? item.x & 0xFFFF : at;
     const int j0 = kt * 128;
     const int* my_perm = kCompact ? P.perm + ((size_t)bx * P.Tc + kt) * 128 : nullptr;
     volatile int* abort_flag = &S.abort_flag;
-    if constexpr (kCompact) {
-        // keys that no row keeps are sorted to the end of the permutation: a tile that starts with one holds nothing else
-        const int jf = my_perm[0];
-        if (jf >= P.L || P.expiry_all[(size_t)bx * P.L + jf] <= (P.causal ? jf : 0)) return;
-    }
 
     if (tid == 0) {
         mbar_init(&S.kv_full, 1);
@@ -166,6 +170,33 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         S.abort_flag = 0;
         S.n_steps = 0;
         fence_barrier_init();
+        if constexpr (!kCompact) {                     // K and V need no schedule: they are under way while it is built
+            mbar_arrive_expect_tx(&S.kv_full, (kD == 128 ? 4 : 3) * (kKVBytes / 2));
+            for (int hf = 0; hf < 2; ++hf) {           // d = 64: both halves of the K buffer hold the same 64 channels
+                tma_load_4d(&S.k[hf * (kKVBytes / 2)], &tmK, &S.kv_full, kD == 128 ? hf * 64 : 0, j0, hk, b);
+                if (hf < kHalves) tma_load_4d(&S.v[hf * (kKVBytes / 2)], &tmV, &S.kv_full, hf * 64, j0, hk, b);
+            }
+        }
+    }
+    if (kCompact && warp < 8) {
+        // The compute warps gather the CTA's 128 K and V rows into the swizzled tile layout, 16 rows each (8 lanes per 128-byte half row, 4
+        // rows per instruction; padding entries are zero-filled), while the schedule is built. (One warp after the schedule: the first
+        // product was issued 10500 clk after the start instead of 6000, as long as two steps.)
+        const int rsub = lane >> 3, c = lane & 7;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = warp * 16 + 4 * q + rsub, j = my_perm[r];
+            const int64_t jr = min(j, P.L - 1);
+            const int64_t krow = b * P.ks_b + jr * P.ks_l + hk * P.ks_h + c * 8, vrow = b * P.vs_b + jr * P.vs_l + hk * P.vs_h + c * 8;
+            const uint32_t off = r * 128 + ((c ^ (r & 7)) << 4);
+            const int nb = j < P.L ? 16 : 0;
+            cp_async16(S.k + off, P.Kg + krow, nb);
+            cp_async16(S.k + off + kKVBytes / 2, P.Kg + krow + (kD == 128 ? 64 : 0), nb);     // d = 64: the same 64 channels once more
+            cp_async16(S.v + off, P.Vg + vrow, nb);
+            if constexpr (kD == 128) cp_async16(S.v + off + kKVBytes / 2, P.Vg + vrow + 64, nb);
+        }
+        cp_async_wait_all();
+        fence_proxy_async();                           // (the barrier below hands the rows to the MMA issuers)
     }
     if (warp == 13) {
         tmem_alloc(&S.tmem_base, 512);
@@ -176,34 +207,20 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmG); }
         int n = 0;
         if constexpr (kCompact) {
-            // query tiles from the first key's tile to the tile of the last row that keeps one of the keys
-            int jmin = 0x7fffffff, emax = 0;
-            for (int t = 0; t < 4; ++t) {
-                const int j = my_perm[lane + 32 * t];
-                const int e = j < P.L ? P.expiry_all[(size_t)bx * P.L + j] : 0;
-                const int first = P.causal ? j : 0;
-                if (e > first) { jmin = min(jmin, first); emax = max(emax, e); }
-            }
-            for (int o = 16; o; o >>= 1) {
-                jmin = min(jmin, __shfl_xor_sync(0xffffffffu, jmin, o));
-                emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-            }
-            if (emax > 0) {
-                // The walk goes BACKWARDS, from the last row that keeps one of the keys to the first key's row: the CTAs
-                // of neighbouring entries of the permutation share their expiry band, i.e. the END of their walks, and start
-                // about together, so walking down from there they pass the same query rows (the Q / dO tiles they load, the
-                // dQ accumulator rows they add to) at about the same time, while those are in L2; walking up, each from its
-                // own first key, they passed a row at times spread over the life of the whole group.
-                const int g = hq_c % P.G, q0 = jmin / 128, q1 = (emax - 1) / 128;
-                n = 2 * (q1 - q0 + 1);
-                if (q1 * 128 + 64 >= P.L) n -= 1;       // the last tile has one 64-row step only
-                n = min(n, kMaxSteps);
-                for (int qt = q0 + lane; qt <= q1; qt += 32) {
+            // Query tiles from the first key's tile to the tile of the last row that keeps one of the keys, or a part of that walk. The walk
+            // goes BACKWARDS, from the last row that keeps one of the keys to the first key's row: the CTAs
+            // of neighbouring entries of the permutation share their expiry band, i.e. the END of their walks, and start
+            // about together, so walking down from there they pass the same query rows (the Q / dO tiles they load, the
+            // dQ accumulator rows they add to) at about the same time, while those are in L2; walking up, each from its
+            // own first key, they passed a row at times spread over the life of the whole group.
+            const int g = hq_c % P.G, q0 = item.y & 0xFFFF, q1 = item.y >> 16, part = (item.x >> 16) & 0xFF, parts = item.x >> 24;
+            const int all = walk_steps(q0, q1, P.L), p0 = all * part / parts, p1 = all * (part + 1) / parts;
+            n = p1 - p0;
+            for (int qt = q0 + lane; qt <= q1; qt += 32) {
 #pragma unroll
-                    for (int hf = 0; hf < 2; ++hf) {
-                        const int pos = n - 1 - (2 * (qt - q0) + hf);
-                        if (pos >= 0) S.sched[pos] = (uint16_t)((g << 11) | (qt << 1) | hf);
-                    }
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int pos = all - 1 - (2 * (qt - q0) + hf);
+                    if (pos >= p0 && pos < p1) S.sched[pos - p0] = (uint16_t)((g << 11) | (qt << 1) | hf);
                 }
             }
         } else {
@@ -354,61 +371,61 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                          : mbar_wait_warp(&S.pds_free[0], (n_steps - 1) & 1, abort_flag);
         if (ok) {
             tc_fence_after();
-            __nv_bfloat16* dk = P.dK + b * P.ks_b + (int64_t)j * P.ks_l + hk * P.ks_h;
-            __nv_bfloat16* dv = P.dV + b * P.vs_b + (int64_t)j * P.vs_l + hk * P.vs_h;
-            const size_t arow = ((size_t)(b * P.L + min(j, P.L - 1)) * P.Hkv + hk) * kD +      // accumulator row
-                                (size_t)(kCompact ? hq_c % P.G : sp) * (size_t)P.acc_slot;
+            // A thread holds 32 channels of its key's row. The warp turns each such block of 32 rows around in shared memory (the Q stages, which
+            // the last MMAs have left; 16-byte chunks swizzled by the row), so that eight lanes write 128 consecutive bytes of a row, and the
+            // block after it is on its way from tensor memory meanwhile. What is left is the stores and reductions themselves, 14 to 32 bytes per clock:
+            // 10000 -> 6800 clk for fp32 parts, 9300 -> 7700 for reductions, 6000 either way for bf16 rows.
+            uint8_t* turn = S.q[0] + warp * 4096;
+            static_assert(sizeof(S.q) >= 8 * 4096, "a block of 32 x 32 floats per compute warp");
+            const int rsub = lane >> 3, ch = lane & 7;
+            int jr[8];                                             // keys of the rows this lane writes a part of
 #pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                const float mul = which == 0 ? P.scale : 1.0f;
-                __nv_bfloat16* out = which == 0 ? dk : dv;
-                float* acc = (which == 0 ? P.dKacc : P.dVacc) + arow;
+            for (int t = 0; t < 8; ++t) jr[t] = __shfl_sync(0xffffffffu, j, 4 * t + rsub);
+            uint32_t o[32];
+            auto fetch = [&](int blk) { tmem_ld32(tmem + lane_base + (blk < kHalves ? cDK : cDV) + (hsel * kHalves + blk % kHalves) * 32, o); };
 #pragma unroll
-                for (int cc = 0; cc < kHalves; ++cc) {
-                    const int c = hsel * kHalves + cc;
-                    uint32_t o[32];
-                    if (n_steps > 0) {
-                        tmem_ld32(tmem + lane_base + (which == 0 ? cDK : cDV) + c * 32, o);
-                        tc_wait_ld();
-                    } else {
+            for (int u = 0; u < 32; ++u) o[u] = 0u;
+            if (n_steps > 0) fetch(0);
+#pragma unroll 1
+            for (int blk = 0; blk < 2 * kHalves; ++blk) {
+                const bool isK = blk < kHalves;
+                const int col = (hsel * kHalves + blk % kHalves) * 32 + ch * 4;
+                if (n_steps > 0) tc_wait_ld_dep(o);
 #pragma unroll
-                        for (int u = 0; u < 32; ++u) o[u] = 0;
-                    }
-                    if constexpr (kCompact) {
-                        // unscaled sums into the fp32 accumulators: the group's query heads add into the same rows
-                        if (j < P.L && n_steps > 0) {
-                            if (P.acc_slot) {          // this (key, query head) pair is written by this thread alone
+                for (int q = 0; q < 8; ++q)
+                    *reinterpret_cast<uint4*>(turn + lane * 128 + ((q ^ (lane & 7)) << 4)) = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+                if (n_steps > 0 && blk + 1 < 2 * kHalves) fetch(blk + 1);
+                __syncwarp();
+                float4 x[8];
 #pragma unroll
-                                for (int u = 0; u < 32; u += 4)
-                                    *reinterpret_cast<float4*>(acc + c * 32 + u) = make_float4(__uint_as_float(o[u]), __uint_as_float(o[u + 1]),
-                                                                                              __uint_as_float(o[u + 2]), __uint_as_float(o[u + 3]));
-                            } else {
-#pragma unroll
-                                for (int u = 0; u < 32; u += 4)
-                                    red_add_v4(acc + c * 32 + u, __uint_as_float(o[u]), __uint_as_float(o[u + 1]), __uint_as_float(o[u + 2]),
-                                               __uint_as_float(o[u + 3]));
-                            }
-                        }
-                    } else if (nsplit > 1) {
-                        // this split's part of the group sum (unscaled; zeros where it had nothing to add), to its own slot
-                        if (j < P.L) {
-#pragma unroll
-                            for (int u = 0; u < 32; u += 4)
-                                *reinterpret_cast<float4*>(acc + c * 32 + u) = make_float4(__uint_as_float(o[u]), __uint_as_float(o[u + 1]),
-                                                                                          __uint_as_float(o[u + 2]), __uint_as_float(o[u + 3]));
-                        }
-                    } else if (j < P.L) {
-#pragma unroll
-                        for (int u = 0; u < 32; u += 8) {
-                            uint4 pkt;
-                            pkt.x = pack_bf16(__uint_as_float(o[u]) * mul, __uint_as_float(o[u + 1]) * mul);
-                            pkt.y = pack_bf16(__uint_as_float(o[u + 2]) * mul, __uint_as_float(o[u + 3]) * mul);
-                            pkt.z = pack_bf16(__uint_as_float(o[u + 4]) * mul, __uint_as_float(o[u + 5]) * mul);
-                            pkt.w = pack_bf16(__uint_as_float(o[u + 6]) * mul, __uint_as_float(o[u + 7]) * mul);
-                            *reinterpret_cast<uint4*>(out + c * 32 + u) = pkt;
-                        }
-                    }
+                for (int t = 0; t < 8; ++t) {
+                    const int row = 4 * t + rsub;
+                    x[t] = *reinterpret_cast<const float4*>(turn + row * 128 + ((ch ^ (row & 7)) << 4));
                 }
+                if (kCompact || nsplit > 1) {
+                    // Unscaled sums in fp32. Token-compacted: the group's query heads add into the same rows, or (slots) this (key, query head) pair is
+                    // written by this CTA alone. Tile mode: this split's part, zeros where it had nothing to add.
+                    float* acc = (isK ? P.dKacc : P.dVacc) + (size_t)(kCompact ? hq_c % P.G : sp) * (size_t)P.acc_slot +
+                                 ((size_t)b * P.L * P.Hkv + hk) * kD + col;
+                    const bool red = kCompact && P.acc_slot == 0;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) {
+                        float* row = acc + (int64_t)jr[t] * (P.Hkv * kD);
+                        if (jr[t] < P.L && (!kCompact || n_steps > 0)) {
+                            if (red) red_add_v4(row, x[t].x, x[t].y, x[t].z, x[t].w);
+                            else *reinterpret_cast<float4*>(row) = x[t];
+                        }
+                    }
+                } else {
+                    const float mul = isK ? P.scale : 1.0f;
+                    __nv_bfloat16* out = (isK ? P.dK + b * P.ks_b + hk * P.ks_h : P.dV + b * P.vs_b + hk * P.vs_h) + col;
+                    const int64_t out_l = isK ? P.ks_l : P.vs_l;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+                        if (jr[t] < P.L)
+                            *reinterpret_cast<uint2*>(out + jr[t] * out_l) = make_uint2(pack_bf16(x[t].x * mul, x[t].y * mul), pack_bf16(x[t].z * mul, x[t].w * mul));
+                }
+                __syncwarp();                                      // (the block has been read)
             }
         }
     } else if (warp < 12) {
@@ -461,35 +478,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     } else {
         if (warp == 12) {
             // ============================ producer ============================
-            if constexpr (kCompact) {
-                if (n_steps > 0) {
-                // gather the CTA's 128 K and V rows into the swizzled tile layout (8 lanes per 128-byte half row,
-                // 4 rows per instruction; padding entries are zero-filled)
-                const int rsub = lane >> 3, c = lane & 7;
-#pragma unroll 4
-                for (int q = 0; q < 32; ++q) {
-                    const int r = 4 * q + rsub, j = my_perm[r];
-                    const int64_t jr = min(j, P.L - 1);
-                    const int64_t krow = b * P.ks_b + jr * P.ks_l + hk * P.ks_h + c * 8, vrow = b * P.vs_b + jr * P.vs_l + hk * P.vs_h + c * 8;
-                    const uint32_t off = r * 128 + ((c ^ (r & 7)) << 4);
-                    const int nb = j < P.L ? 16 : 0;
-                    cp_async16(S.k + off, P.Kg + krow, nb);
-                    cp_async16(S.k + off + kKVBytes / 2, P.Kg + krow + (kD == 128 ? 64 : 0), nb);     // d = 64: the same 64 channels once more
-                    cp_async16(S.v + off, P.Vg + vrow, nb);
-                    if constexpr (kD == 128) cp_async16(S.v + off + kKVBytes / 2, P.Vg + vrow + 64, nb);
-                }
-                cp_async_wait_all();
-                fence_proxy_async();
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&S.kv_full);
-            } else if (lane == 0) {
-                mbar_arrive_expect_tx(&S.kv_full, (kD == 128 ? 4 : 3) * (kKVBytes / 2));
-                for (int hf = 0; hf < 2; ++hf) {           // d = 64: both halves of the K buffer hold the same 64 channels
-                    tma_load_4d(&S.k[hf * (kKVBytes / 2)], &tmK, &S.kv_full, kD == 128 ? hf * 64 : 0, j0, hk, b);
-                    if (hf < kHalves) tma_load_4d(&S.v[hf * (kKVBytes / 2)], &tmV, &S.kv_full, hf * 64, j0, hk, b);
-                }
-            }
             bool ok = true;
             for (int n = 0; n < n_steps && ok; ++n) {
                 const uint32_t e = S.sched[n];
@@ -555,7 +543,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const uint64_t dX0 = smem_desc_plain(smem_u32(S.qext[0]), 128, 256);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             const int n_steps_u = __shfl_sync(0xffffffffu, n_steps, 0);
-            bool ok = mbar_wait_warp(&S.kv_full, 0, abort_flag);
+            bool ok = kCompact || mbar_wait_warp(&S.kv_full, 0, abort_flag);
             for (int n = 0; n < n_steps_u && ok; ++n) {
                 const int st = n % kStages;
                 ok = mbar_wait_warp(&S.qd_full[st], (n / kStages) & 1, abort_flag);
@@ -641,15 +629,121 @@ struct PrepareParams {
     int64_t zero_n[3];          // floats
     int64_t zero_part[3];       // 16-byte chunks per CTA
     int32_t* status;            // the workspace header
+    // token-compacted mode: the first perm_ctas CTAs (one per (batch, query head), 1024 threads) make the head's permutation and work items
+    int perm_ctas;
+    const int32_t* expiry;
+    int* perm;
+    int2* items;
+    int Tc, causal, max_items;
+    int walk;                   // steps of a walk that one CTA takes at most
+    int longest_first;          // order of a head's items: by length, or as the permutation has them
 };
 constexpr int kPrepareRows = 4;     // rows per lane group
+constexpr int kPermThreads = 1024;
 
-template <int kLanes>
-__global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepareParams P) {
+// Token-compacted mode: per (batch, query head) a stable counting sort of the keys by the band their expiry falls in (latest expiry
+// first; keys that no row keeps go last). Within a band the keys stay in index order, so 128 consecutive entries start at nearby rows
+// and expire within one band of each other: on i.i.d. importance at L = 16384, w = 2048 the walk covers 1.4 x the (row, key) pairs
+// actually kept, against 4.3 x for tiles of consecutive keys. Bands of L / 8 rows, 128 to 2048, at most 62 (counted offline over windows of
+// L / 16 to L / 4: within 3 % of the best width at 4096, 8192 and 16384 keys; 2048-row bands cover 15 % more at 4096). Padded with L up to Tc * 128.
+// One CTA of 1024 threads per (batch, head). Per 1024-key chunk every warp ranks its 32 keys within their class
+// (match_any), the per-warp class counts are turned into start positions by 64 threads (one per class, a running sum over
+// the 32 warps and over the chunks), and every key is written to its place: stable in key order, three barriers per chunk.
+// Then the work items: a warp per key tile finds its walk, walks longer than P.walk steps are cut into equal parts, and with
+// P.longest_first the items are ranked by length, so that no long one starts late.
+struct PermShared {
+    int hist[64];
+    int offs[64];                 // next free position of each class
+    int cnt[32][64];              // per warp and class: keys in this chunk, then their start position
+    int bounds[1024];             // walk of each key tile, q0 | q1 << 16, or -1
+    int parts[1024], len[1024];
+};
+__device__ __forceinline__ void lifetime_perm(const PrepareParams& P, PermShared& S) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bh = blockIdx.x, L = P.L, Tc = P.Tc;
+    const int32_t* e = P.expiry + (size_t)bh * L;
+    int* out = P.perm + (size_t)bh * Tc * 128;
+    const int band = max((L + 61) / 62, min(2048, max(128, L / 8)));
+    auto cls = [&](int j) { return e[j] > (P.causal ? j : 0) ? 1 + (e[j] - 1) / band : 0; };
+    if (tid < 64) S.hist[tid] = 0;
+    __syncthreads();
+    for (int j = tid; j < L; j += kPermThreads) atomicAdd(&S.hist[cls(j)], 1);
+    __syncthreads();
+    if (tid == 0) {
+        int run = 0;
+        for (int c = 63; c >= 0; --c) { S.offs[c] = run; run += S.hist[c]; }
+    }
+    __syncthreads();
+    for (int base = 0; base < L; base += kPermThreads) {
+        const int j = base + tid;
+        const int c = j < L ? cls(j) : -1;
+        const uint32_t same = __match_any_sync(0xffffffffu, c);
+        const int leader = __ffs(same) - 1, rank = __popc(same & ((1u << lane) - 1));
+        S.cnt[warp][lane] = 0;
+        S.cnt[warp][lane + 32] = 0;
+        __syncwarp();
+        if (lane == leader && c >= 0) S.cnt[warp][c] = __popc(same);
+        __syncthreads();
+        if (tid < 64) {
+            int run = S.offs[tid];
+            for (int w = 0; w < 32; ++w) {
+                const int n = S.cnt[w][tid];
+                S.cnt[w][tid] = run;
+                run += n;
+            }
+            S.offs[tid] = run;
+        }
+        __syncthreads();
+        if (c >= 0) out[S.cnt[warp][c] + rank] = j;
+        __syncthreads();
+    }
+    for (int t = L + tid; t < Tc * 128; t += kPermThreads) out[t] = L;
+    __syncthreads();                                        // (the CTA reads its own entries back)
+    for (int t = warp; t < Tc; t += 32) {
+        int first = 0x7fffffff, last = 0;
+        for (int u = 0; u < 4; ++u) {
+            const int j = out[t * 128 + lane + 32 * u];
+            const int ej = j < L ? e[j] : 0, f = P.causal ? j : 0;
+            if (ej > f) { first = min(first, f); last = max(last, ej); }
+        }
+        first = __reduce_min_sync(0xffffffffu, first);
+        last = __reduce_max_sync(0xffffffffu, last);
+        if (lane == 0) {
+            const int q0 = first >> 7, q1 = (last - 1) >> 7, n = last > 0 ? walk_steps(q0, q1, L) : 0;
+            const int parts = min(min(kMostParts, P.max_items / Tc), (n + P.walk - 1) / P.walk);        // (0: no row keeps a key of the tile)
+            S.bounds[t] = q0 | (q1 << 16);
+            S.parts[t] = parts;
+            S.len[t] = parts ? n / parts : 0;
+        }
+    }
+    __syncthreads();
+    int2* items = P.items + (size_t)bh * P.max_items;
+    if (tid < Tc) {
+        const int parts = S.parts[tid], len = S.len[tid];
+        int at = 0;
+        for (int u = 0; u < Tc; ++u) at += (P.longest_first ? S.len[u] > len || (S.len[u] == len && u < tid) : u < tid) ? S.parts[u] : 0;
+        for (int q = 0; q < parts; ++q) items[at + q] = make_int2(tid | (q << 16) | (parts << 24), S.bounds[tid]);
+    }
+    int total = 0;
+    for (int u = lane; u < Tc; u += 32) total += S.parts[u];
+    total = __reduce_add_sync(0xffffffffu, total);
+    for (int t = total + tid; t < P.max_items; t += kPermThreads) items[t] = make_int2(-1, 0);
+}
+
+template <int kLanes, bool kPerm>
+__global__ void __launch_bounds__(kPerm ? kPermThreads : 256) bwd_prepare_kernel(const PrepareParams P) {
+    constexpr int nthr = kPerm ? kPermThreads : 256;
     pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x < kWsHeaderBytes / 4) P.status[threadIdx.x] = 0;
-    const int sub = threadIdx.x % kLanes, per_cta = 256 / kLanes;
-    const uint32_t rows = (uint32_t)P.B * P.Hq * P.L, r0 = blockIdx.x * per_cta * kPrepareRows + threadIdx.x / kLanes;
+    if constexpr (kPerm) {
+        __shared__ PermShared S;
+        if ((int)blockIdx.x < P.perm_ctas) {
+            lifetime_perm(P, S);
+            return;
+        }
+    }
+    const int cta = (int)blockIdx.x - (kPerm ? P.perm_ctas : 0);
+    const int sub = threadIdx.x % kLanes, per_cta = nthr / kLanes;
+    const uint32_t rows = (uint32_t)P.B * P.Hq * P.L, r0 = cta * per_cta * kPrepareRows + threadIdx.x / kLanes;
     uint4 a[kPrepareRows], g[kPrepareRows];
 #pragma unroll
     for (int n = 0; n < kPrepareRows; ++n) {
@@ -661,10 +755,10 @@ __global__ void __launch_bounds__(256) bwd_prepare_kernel(const PrepareParams P)
     }
 #pragma unroll
     for (int z = 0; z < 3; ++z) {
-        const int64_t n4 = P.zero_n[z] >> 2, e0 = P.zero_part[z] * blockIdx.x, e1 = min(n4, e0 + P.zero_part[z]);
+        const int64_t n4 = P.zero_n[z] >> 2, e0 = P.zero_part[z] * cta, e1 = min(n4, e0 + P.zero_part[z]);
         float4* dst = reinterpret_cast<float4*>(P.zero[z]);
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) dst[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (blockIdx.x == 0 && threadIdx.x < (P.zero_n[z] & 3)) P.zero[z][4 * n4 + threadIdx.x] = 0.0f;
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += nthr) dst[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (cta == 0 && threadIdx.x < (P.zero_n[z] & 3)) P.zero[z][4 * n4 + threadIdx.x] = 0.0f;
     }
 #pragma unroll
     for (int n = 0; n < kPrepareRows; ++n) {
@@ -742,63 +836,12 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
 
 }  // namespace
 
-// Token-compacted mode: per (batch, query head) a stable counting sort of the keys by the band their expiry falls in
-// (band size >= 2048 rows, at most 62 bands; latest expiry first; keys that no row keeps go last). Within a band the
-// keys stay in index order, so 128 consecutive entries start at nearby rows and expire within one band of each other:
-// on i.i.d. importance at L = 16384, w = 2048 the walk covers 1.4 x the (row, key) pairs actually kept, against 4.3 x
-// for tiles of consecutive keys. Padded with L up to Tc * 128.
-// One CTA of 1024 threads per (batch, head). Per 1024-key chunk every warp ranks its 32 keys within their class
-// (match_any), the per-warp class counts are turned into start positions by 64 threads (one per class, a running sum over
-// the 32 warps and over the chunks), and every key is written to its place: stable in key order, three barriers per chunk.
-__global__ void __launch_bounds__(1024) lifetime_perm_kernel(const int32_t* __restrict__ expiry, int* __restrict__ perm, int L, int Tc, int causal) {
-    __shared__ int hist[64];
-    __shared__ int offs[64];                 // next free position of each class
-    __shared__ int cnt[32][64];              // per warp and class: keys in this chunk, then their start position
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    pdl_enter(expiry, perm);
-    const int32_t* e = expiry + (size_t)blockIdx.x * L;
-    int* out = perm + (size_t)blockIdx.x * Tc * 128;
-    const int band = max(2048, (L + 61) / 62);
-    auto cls = [&](int j) { return e[j] > (causal ? j : 0) ? 1 + (e[j] - 1) / band : 0; };
-    if (tid < 64) hist[tid] = 0;
-    __syncthreads();
-    for (int j = tid; j < L; j += 1024) atomicAdd(&hist[cls(j)], 1);
-    __syncthreads();
-    if (tid == 0) {
-        int run = 0;
-        for (int c = 63; c >= 0; --c) { offs[c] = run; run += hist[c]; }
-    }
-    __syncthreads();
-    for (int base = 0; base < L; base += 1024) {
-        const int j = base + tid;
-        const int c = j < L ? cls(j) : -1;
-        const uint32_t same = __match_any_sync(0xffffffffu, c);
-        const int leader = __ffs(same) - 1, rank = __popc(same & ((1u << lane) - 1));
-        cnt[warp][lane] = 0;
-        cnt[warp][lane + 32] = 0;
-        __syncwarp();
-        if (lane == leader && c >= 0) cnt[warp][c] = __popc(same);
-        __syncthreads();
-        if (tid < 64) {
-            int run = offs[tid];
-            for (int w = 0; w < 32; ++w) {
-                const int n = cnt[w][tid];
-                cnt[w][tid] = run;
-                run += n;
-            }
-            offs[tid] = run;
-        }
-        __syncthreads();
-        if (c >= 0) out[cnt[warp][c] + rank] = j;
-        __syncthreads();
-    }
-    for (int t = L + tid; t < Tc * 128; t += 1024) out[t] = L;
-}
-
-// workspace layout: header | D [rows] | dQ accumulator [B x Hq x (Tr x 128) x d] | (token-compacted mode) permutation | dK, dV accumulators
+// workspace layout: header | D [rows] | dQ accumulator [B x Hq x (Tr x 128) x d] | (token-compacted mode) permutation, work items | dK, dV accumulators
 static size_t bwd_rows64(const Prob& P) { return ((((size_t)P.B * P.Hq * P.L) + 63) / 64) * 64; }
 static size_t bwd_acc_floats(const Prob& P) { return (size_t)P.B * P.Hq * P.Tr * 128 * P.d; }     // rows padded to whole query tiles
-static size_t bwd_perm_ints(const Prob& P) { return (((size_t)P.B * P.Hq * P.Tc * 128) + 63) / 64 * 64; }
+// permutation and work items
+static size_t bwd_perm_ints(const Prob& P) { return (size_t)P.B * P.Hq * P.Tc * 128; }
+static size_t bwd_item_ints(const Prob& P) { return ((size_t)P.B * P.Hq * P.Tc * 2 * kMostParts + 63) / 64 * 64; }
 
 // Tile mode: a CTA owns a key tile of one KV head and walks all its query heads. Where few CTAs wait for the heaviest one, the
 // group's heads are dealt out to several CTAs, whose parts of dK and dV go to slots of their own. The number is the divisor of G
@@ -830,6 +873,23 @@ int tc_bwd_splits(const Prob& P) {
 bool bwd_long(const Prob& P) {
     return !(P.flags & DMA_FLAG_COMPACT_KV) && tc_bwd_splits(P) == 1 && (int64_t)P.B * P.Hq * P.Tc * (P.Tr + 1) >= 256 * 148;
 }
+// Token-compacted mode: the longest walk of one CTA, in 64-row steps. A long-lived key's tile is walked over all later rows, 2 L / 128 steps,
+// which few heads cannot hide behind other tiles: then walks are cut into parts of about what an SM gets of the whole work (its share of
+// the kept pairs, and half as much again that the tiles' walks cover beyond them), on the z axis of the grid. dK, dV (and dM) take the
+// parts' sums through the atomics that the heads of a group need anyway; with DMA_FLAG_DETERMINISTIC nothing is cut.
+// Backward, us, whole walks / this rule and items by length: one head of 9663 keys (w = 1442) 233 / 66, 2 heads of 4728 (w = 1044) 117 /
+// 46, 8 heads of 8192 (w = 1024) 240 / 188, 16 heads of 4096 (w = 1024) 202 / 164 (nothing cut, long walks first), 32 heads of 16384
+// 2282 / 2221 (K and V gathered by eight warps). Cutting every walk above 0.8 of the share was slower where the longest exceeds it by little
+// (16 heads, w = 2375 of 14353 keys).
+static int bwd_walk(const Prob& P) {
+    const int longest = 2 * P.Tr;
+    if (P.flags & DMA_FLAG_DETERMINISTIC) return longest;
+    const double w = P.w, pairs = P.causal ? w * (w + 1) / 2 + (P.L - w) * w : w * P.L;
+    const double share = (P.causal ? 1.55 : 1.0) * P.B * P.Hq * pairs / (128.0 * 64.0) / 148.0;
+    if (longest <= 1.3 * share) return longest;
+    return std::max(std::max(16, (int)(0.8 * share)), (longest + kMostParts - 1) / kMostParts);
+}
+
 // copies of the dK, dV accumulators (0: the main kernel writes dK, dV itself)
 static size_t bwd_slots(const Prob& P) {
     if (P.flags & DMA_FLAG_COMPACT_KV) return (P.flags & DMA_FLAG_DETERMINISTIC) ? (size_t)P.G : 1;
@@ -839,7 +899,7 @@ static size_t bwd_slots(const Prob& P) {
 static size_t bwd_base_bytes(const Prob& P) { return kWsHeaderBytes + (bwd_rows64(P) + bwd_acc_floats(P)) * sizeof(float); }
 // what the call uses beyond that
 static size_t bwd_extra_bytes(const Prob& P) {
-    const size_t perm = P.flags & DMA_FLAG_COMPACT_KV ? bwd_perm_ints(P) * sizeof(int) : 0;
+    const size_t perm = P.flags & DMA_FLAG_COMPACT_KV ? (bwd_perm_ints(P) + bwd_item_ints(P)) * sizeof(int) : 0;
     return perm + 2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
 }
 
@@ -869,7 +929,8 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     int* perm = reinterpret_cast<int*>(acc + bwd_acc_floats(P));
     const size_t slots = bwd_slots(P);
     const int nsplit = tc_bwd_splits(P);
-    float* accK = reinterpret_cast<float*>(perm + (compact ? bwd_perm_ints(P) : 0));
+    int2* items = reinterpret_cast<int2*>(perm + bwd_perm_ints(P));
+    float* accK = reinterpret_cast<float*>(perm + (compact ? bwd_perm_ints(P) + bwd_item_ints(P) : 0));
     float* accV = accK + slots * nkv;
     CUtensorMap tmQ, tmK, tmV, tmG;
     int rc;
@@ -884,13 +945,17 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     pp.zero[0] = acc; pp.zero_n[0] = (int64_t)bwd_acc_floats(P);
     pp.zero[1] = dM; pp.zero_n[1] = (int64_t)rows;                                       // two partial sums are added per key
     pp.zero[2] = accK; pp.zero_n[2] = compact ? (int64_t)(2 * slots * nkv) : 0;
-    const int per_cta = 256 / (P.d / 8) * kPrepareRows;
+    const int threads = compact ? kPermThreads : 256, per_cta = threads / (P.d / 8) * kPrepareRows;
     const unsigned prep_ctas = (unsigned)((rows + per_cta - 1) / per_cta);
     for (int z = 0; z < 3; ++z) pp.zero_part[z] = ((pp.zero_n[z] >> 2) + prep_ctas - 1) / prep_ctas;
-    if ((rc = launch_overlapped(P.d == 128 ? bwd_prepare_kernel<16> : bwd_prepare_kernel<8>, dim3(prep_ctas), dim3(256), 0, st, 1, pp))) return rc;
-    if (compact) {
-        if ((rc = launch_overlapped(lifetime_perm_kernel, dim3(P.B * P.Hq), dim3(1024), 0, st, 1, expiry, perm, P.L, P.Tc, P.causal))) return rc;
-    }
+    const int walk = compact ? bwd_walk(P) : 1, max_items = compact ? P.Tc * ((2 * P.Tr + walk - 1) / walk) : P.Tc;
+    pp.perm_ctas = compact ? P.B * P.Hq : 0;
+    pp.expiry = expiry; pp.perm = perm; pp.items = items; pp.Tc = P.Tc; pp.causal = P.causal; pp.max_items = max_items; pp.walk = walk;
+    // (of more rows than one scheduling group, below, the order of the permutation keeps the rows in use in L2)
+    pp.longest_first = (double)P.B * P.Hq * P.L * P.d * 8 <= 160.0 * 1024 * 1024 ? 1 : 0;
+    auto prepare = compact ? (P.d == 128 ? bwd_prepare_kernel<16, true> : bwd_prepare_kernel<8, true>)
+                           : (P.d == 128 ? bwd_prepare_kernel<16, false> : bwd_prepare_kernel<8, false>);
+    if ((rc = launch_overlapped(prepare, dim3(pp.perm_ctas + prep_ctas), dim3(threads), 0, st, 1, pp))) return rc;
     BwdParams bp;
     bp.lse = lse; bp.Dv = Dv; bp.bias = bias; bp.expiry = expiry; bp.bitmap = bitmap; bp.dQacc = acc; bp.Lblk = P.Tr * 8;
     bp.dK = (__nv_bfloat16*)dK; bp.dV = (__nv_bfloat16*)dV; bp.dM = dM; bp.status = (int32_t*)ws;
@@ -916,7 +981,7 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     }
     bp.scale = P.scale; bp.scale_log2 = P.scale * 1.4426950408889634f; bp.inv_scale = 1.0f / P.scale;
     bp.ks_b = P.ks[0]; bp.ks_l = P.ks[1]; bp.ks_h = P.ks[2]; bp.vs_b = P.vs[0]; bp.vs_l = P.vs[1]; bp.vs_h = P.vs[2];
-    bp.perm = perm; bp.expiry_all = expiry; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
+    bp.perm = perm; bp.items = items; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
     bp.dKacc = accK; bp.dVacc = accV; bp.acc_slot = slots > 1 ? (int64_t)nkv : 0; bp.nsplit = nsplit;
     const size_t smem = sizeof(SharedStorage) + 1024;
     const bool lng = bwd_long(P);
@@ -925,7 +990,7 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
                         : (P.d == 128 ? bwd_kernel<false, 128> : bwd_kernel<false, 64>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     timing_mark(1, false, st);
-    const dim3 grid(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, P.Tc);
+    const dim3 grid(compact ? P.B * P.Hq : P.B * P.Hkv * nsplit, max_items);
     rc = lng ? launch_plain(kern, grid, dim3(kThreads), smem, st, tmQ, tmK, tmV, tmG, bp)
              : launch_overlapped(kern, grid, dim3(kThreads), smem, st, 1, tmQ, tmK, tmV, tmG, bp);
     timing_mark(1, true, st);
