@@ -4,11 +4,11 @@
 //
 // Kernels
 //   delta_kernel        V read once (HBM-bound); z, softplus, exp in a fixed fp32 operation order
-//   chunk_sort_kernel   256-key chunks of (delta bits, ~index) keys sorted in shared memory
 //   tree_block_kernel, tree_merge_kernel, expiry_tree_kernel
-//                       selection as a rank tree: the merge passes that finish the sort leave one bit per key and level,
-//                       and a key's expiry (the w-th smallest index among the keys that beat it) is a walk of log2(L) steps
-//   bitmap_kernel       per key tile: union of the query-tile intervals its keys are kept in
+//                       selection as a rank tree: the passes of a merge sort of (delta bits, ~index) keys leave one bit per key and
+//                       level, and a key's expiry (the w-th smallest index among the keys that beat it) is a walk of log2(L) steps.
+//                       Heads of up to 4096 keys: sort, walk and bitmap in the one block kernel
+//   bitmap_square_kernel, bitmap_kernel   per key tile: union of the query-tile intervals its keys are kept in
 #include <mutex>
 #include <utility>
 #include <type_traits>
@@ -18,7 +18,7 @@
 namespace dma {
 namespace {
 
-constexpr int kChunk = 256;   // keys per sorted chunk (= threads of the sort kernel)
+constexpr int kChunk = 256;   // the sort pads a head to a multiple of this many keys
 
 // ---- fixed-order fp32 routines: every step is one correctly rounded IEEE operation -----------------------
 
@@ -310,70 +310,6 @@ __device__ __forceinline__ void zero_share(uint32_t* p, int64_t n) {
     for (int64_t i = n * cta / ctas + threadIdx.x; i < n * (cta + 1) / ctas; i += blockDim.x) p[i] = 0u;
 }
 
-// Chunks are written in DESCENDING order, padding keys (beyond L) carry their index and sort below every real key, and
-// the kernel also emits the eight lowest levels of the rank tree (node sizes 256 ... 2, see below) by splitting the sorted
-// chunk on one index bit per level.
-__global__ void __launch_bounds__(kChunk) chunk_sort_kernel(const float* __restrict__ delta,
-                                                            unsigned long long* __restrict__ sorted, int L, int nchunk,
-                                                            uint2* __restrict__ lev, int m, uint32_t* __restrict__ bitmap, int64_t bitmap_words) {
-    __shared__ unsigned long long s[2][kChunk];
-    const int bh = blockIdx.y, c = blockIdx.x, t = threadIdx.x, j = c * kChunk + t;
-    pdl_enter_restrict(delta, sorted, lev, bitmap);
-    zero_share(bitmap, bitmap_words);
-    // padding sorts below every real key (delta > 0) and keeps its index in the low word
-    unsigned long long v = j < L ? sort_key(delta[(size_t)bh * L + j], j) : (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
-    // bitonic network, ascending; thread t holds position t. Partners less than 32 apart exchange by shuffle, the six
-    // wider exchanges go through shared memory (two buffers in turn: one barrier each).
-    int nb = 0;
-#pragma unroll
-    for (int k = 2; k <= kChunk; k <<= 1) {
-        const bool up = (t & k) == 0;
-#pragma unroll
-        for (int mm = k >> 1; mm > 0; mm >>= 1) {
-            unsigned long long o;
-            if (mm >= 32) {
-                s[nb][t] = v;
-                __syncthreads();
-                o = s[nb][t ^ mm];
-                nb ^= 1;
-            } else {
-                o = __shfl_xor_sync(0xffffffffu, v, mm);
-            }
-            const bool want_min = ((t & mm) == 0) == up;
-            v = want_min ? (v < o ? v : o) : (v > o ? v : o);
-        }
-    }
-    s[0][t] = v;
-    __syncthreads();
-    const unsigned long long mine = s[0][kChunk - 1 - t];        // position t of the descending order
-    sorted[((size_t)bh * nchunk + c) * kChunk + t] = mine;
-    // Levels with node size Bs = 256, 128, ..., 2: a node is an aligned block of Bs key indices, its sequence the block's
-    // keys in descending order, its bit the half of the block a key lies in. Splitting a node's sequence stably on that
-    // bit gives the sequences of its two children.
-    __shared__ uint8_t cur[2][kChunk];
-    __shared__ uint32_t wbits[kChunk / 32];
-    const int lane = t & 31, warp = t >> 5;
-    const size_t W = (size_t)nchunk * (kChunk / 32);
-    cur[0][t] = (uint8_t)((0xFFFFFFFFu - (uint32_t)mine) & (kChunk - 1));
-    __syncthreads();
-#pragma unroll
-    for (int lv = 0; lv < 8; ++lv) {
-        const int Bs = kChunk >> lv, v = cur[lv & 1][t], bit = (v >> (7 - lv)) & 1;
-        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-        if (lane == 0) wbits[warp] = bal;
-        __syncthreads();
-        const int node_start = t & ~(Bs - 1);
-        uint32_t cumw = 0;                                      // ones of the node before this word
-        for (int k = node_start >> 5; k < warp; ++k) cumw += __popc(wbits[k]);
-        const uint32_t below = (1u << lane) - 1u, in_node = Bs >= 32 ? 0xffffffffu : (((1u << Bs) - 1u) << (node_start & 31));
-        const int ones_before = (int)cumw + __popc(bal & below & in_node);
-        if (lane == 0) lev[((size_t)bh * m + (m - 8 + lv)) * W + (size_t)c * (kChunk / 32) + warp] = make_uint2(cumw, bal);
-        const int npos = node_start + (bit ? Bs / 2 + ones_before : (t - node_start) - ones_before);
-        cur[(lv + 1) & 1][npos] = (uint8_t)v;
-        __syncthreads();
-    }
-}
-
 // ---- selection as a rank tree -------------------------------------------------------------------------------
 // expiry[j] is the w-th smallest INDEX among the keys that beat j, i.e. among the first r entries of the head's keys in
 // descending order, r = rank of j. That is a quantile query on a prefix, answered by a tree over key indices: the node of an
@@ -382,99 +318,278 @@ __global__ void __launch_bounds__(kChunk) chunk_sort_kernel(const float* __restr
 // node and z of them in its lower half, the k-th smallest index is in the lower half iff k <= z. log2(L) steps of one
 // 8-byte load each, for every key in parallel, whatever w.
 // The tree is what a bottom-up merge sort leaves behind: merging the sorted lower and upper half of a block yields the
-// block's sorted sequence, and "this output came from the upper half" is the node's bit. chunk_sort_kernel builds the
-// levels up to 256 keys; one tree_merge_kernel launch per level does the rest (runs of R keys -> runs of 2R).
+// block's sorted sequence, and "this output came from the upper half" is the node's bit. tree_block_kernel builds the
+// levels up to 1024 or 4096 keys; one tree_merge_kernel launch per level does the rest (runs of R keys -> runs of 2R).
 // Level l (0 = root) of head bh lives at lev[(bh * m + l) * W + position / 32]: x = ones of the node before this word,
 // y = the bits. A trailing run shorter than R (L is not a power of two) merges with what exists; the nodes stay
 // left-aligned, which is all a query needs (it never looks past the real keys).
 constexpr int kMergeThreads = 256;
 constexpr int kMergeOut = 1024;       // outputs per CTA of tree_merge_kernel (four per thread)
-constexpr int kBlockKeys = 4096;      // keys one CTA of tree_block_kernel merges in shared memory
-constexpr int kBlockThreads = 1024;
+constexpr int kBlockKeys = 4096, kSmallBlock = 1024;      // keys one CTA of tree_block_kernel sorts in shared memory
+constexpr int kBlockThreads = 512;
 
-// Four consecutive outputs of the merge of two descending runs A (na keys) and B (nb keys), starting at output x:
-// i = how many of the first x outputs come from A (the first i for which "A[i] goes before the last B taken" fails), then
-// four merge steps. Keys are distinct and non-zero; 0 stands for "run exhausted". Returns i; prov bit u = output u came from B.
-__device__ __forceinline__ int merge4(const unsigned long long* A, int na, const unsigned long long* B, int nb, int x,
-                                      unsigned long long (&out)[4], uint32_t& prov) {
-    int lo = max(0, x - nb), hi = min(x, na);
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (A[mid] > B[x - mid - 1]) lo = mid + 1; else hi = mid;
-    }
-    int i = lo, k = x - lo;
-    unsigned long long a = i < na ? A[i] : 0ull, b = k < nb ? B[k] : 0ull;
-    prov = 0u;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const bool takeA = a > b;
-        out[u] = takeA ? a : b;
-        prov |= takeA ? 0u : 1u << u;
-        if (takeA) { ++i; a = i < na ? A[i] : 0ull; } else { ++k; b = k < nb ? B[k] : 0ull; }
-    }
-    return lo;
+// Comparator of two keys: the larger one to x.
+__device__ __forceinline__ void order_desc(unsigned long long& x, unsigned long long& y) {
+    const bool swap = y > x;
+    const unsigned long long t = swap ? y : x;
+    y = swap ? x : y;
+    x = t;
 }
 
-// the 32-bit word of eight neighbouring threads' four provenance bits each (valid in the lanes with lane % 8 == 0)
-__device__ __forceinline__ uint32_t gather_nibbles(uint32_t prov, int lane) {
-    uint32_t wv = prov << (4 * (lane & 7));
-    wv |= __shfl_xor_sync(0xffffffffu, wv, 1);
-    wv |= __shfl_xor_sync(0xffffffffu, wv, 2);
-    wv |= __shfl_xor_sync(0xffffffffu, wv, 4);
+// kN consecutive outputs of the merge of two descending runs A (na keys) and B (nb keys), starting at output x.
+// i = how many of the first x outputs come from A: the first i for which "A[i] goes before the last B taken" fails, found by quartering the
+// range `steps` times (at least (log2 of the shorter run's length + 1) / 2, rounded up) without a branch. Then the kN largest of A[i ..]
+// and B[x - i ..] are the pairwise larger ones of one list and the other reversed, and a bitonic network orders them: all loads are in
+// flight together, where kN steps of a merge would wait for one another. Keys are distinct and non-zero; 0 stands for "run exhausted".
+// Returns i. at(p): the key at position p of the array that holds both, A from pa on and B from pb on.
+template <int kN, typename At>
+__device__ __forceinline__ int merge_outputs(At&& at, int pa, int na, int pb, int nb, int x, int steps, unsigned long long (&out)[kN]) {
+    int lo = max(0, x - nb), hi = min(x, na);
+    for (int t = 0; t < steps; ++t) {
+        const int len = hi - lo, m2 = lo + (len >> 1), m1 = lo + (len >> 2), m3 = m2 + ((hi - m2) >> 1);
+        auto before = [&](int mid) {                                 // (an empty range probes A[0] against itself: false)
+            const bool in = mid < hi;
+            return at(in ? pa + mid : pa) > at(in ? pb + x - mid - 1 : pa);
+        };
+        const bool p1 = before(m1), p2 = before(m2), p3 = before(m3);
+        lo = p3 ? m3 + 1 : p2 ? m2 + 1 : p1 ? m1 + 1 : lo;
+        hi = !p1 ? min(m1, hi) : !p2 ? m2 : !p3 ? min(m3, hi) : hi;
+    }
+    unsigned long long b[kN];
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+        out[u] = lo + u < na ? at(pa + lo + u) : 0ull;
+        b[u] = x - lo + u < nb ? at(pb + x - lo + u) : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < kN; ++u) out[u] = out[u] > b[kN - 1 - u] ? out[u] : b[kN - 1 - u];
+#pragma unroll
+    for (int h = kN / 2; h; h >>= 1)
+#pragma unroll
+        for (int u = 0; u < kN; ++u)
+            if (!(u & h)) order_desc(out[u], out[u + h]);
+    return lo;
+}
+// Which of the keys lie in the upper half of their block of 2 R = 2 << bit keys (a key's low word is ~index; R a power of two, blocks aligned)
+template <int kN>
+__device__ __forceinline__ uint32_t upper_half(const unsigned long long (&key)[kN], int bit) {
+    uint32_t prov = 0u;
+#pragma unroll
+    for (int u = 0; u < kN; ++u) prov |= ((~(uint32_t)key[u] >> bit) & 1u) << u;
+    return prov;
+}
+
+// the 32-bit word of 32 / kN neighbouring threads' kN provenance bits each (valid in the lanes with lane % (32 / kN) == 0)
+template <int kN>
+__device__ __forceinline__ uint32_t gather_bits(uint32_t prov, int lane) {
+    uint32_t wv = prov << (kN * (lane & (32 / kN - 1)));
+#pragma unroll
+    for (int m = 1; m < 32 / kN; m <<= 1) wv |= __shfl_xor_sync(0xffffffffu, wv, m);
     return wv;
 }
 
-// Levels with nodes of 512 ... 4096 keys in one launch: a CTA holds 4096 keys (16 sorted chunks) in shared memory and
-// merges runs of R = 256, 512, 1024, 2048, four consecutive outputs per thread. A node's bit says whether the output came
-// from the upper run, and the count of such outputs before a word is the word's position minus the A keys taken so far.
-__global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const unsigned long long* __restrict__ src,
-                                                                   unsigned long long* __restrict__ dst,
-                                                                   uint2* __restrict__ lev, int Lc, int m) {
-    extern __shared__ __align__(16) unsigned long long sk[];         // two buffers of kBlockKeys keys
-    pdl_enter_restrict(src, dst, lev);
-    const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-    const int base = blockIdx.x * kBlockKeys, nreal = min(kBlockKeys, Lc - base);
+// Place of key p in the block kernel's buffers: one 8-byte word is skipped after every 16, so that neighbouring threads, whose searches and
+// outputs lie 4 or 8 keys apart, use different banks (16 heads of 4096 keys in blocks of 4096, all levels merged in shared memory: mask build 34 -> 30 us).
+__host__ __device__ constexpr int padded(int p) { return p + (p >> 4); }
+
+// ones among the first c entries (c >= 1) of the node that starts at position s of a level; word(q) is the level's word of position q
+template <typename Word>
+__device__ __forceinline__ int ones_of(Word&& word, int s, int c) {
+    const int q = s + c - 1;                                     // last entry of the prefix
+    const uint2 wd = word(q);
+    const uint32_t upto = (2u << (q & 31)) - 1u, from = ~((1u << (s & 31)) - 1u);             // a node smaller than a word starts inside it
+    return (int)wd.x + __popc(wd.y & upto & from);
+}
+
+// Expiry of the key j at rank r of its head; word(l, q) is the word of position q in level l (0: the root).
+// kMode 2 (non-causal): every row sees every key, so the key is kept by all rows iff fewer than w keys beat it.
+// kMode 1: sequences packed along the key axis (sequence s owns the keys cu[s] <= j < cu[s+1]). A key competes only with
+// the keys of its own sequence [s0, s1): of the first r keys of the head, n0 have an index below s0 (a first walk, along
+// the path of s0, adds up the lower halves it leaves to its left), so the w-th beater inside the sequence is the
+// (n0 + w)-th smallest index overall, if that exists and lies below s1; otherwise the key lives to the end of its sequence.
+template <int kMode, typename Word>
+__device__ __forceinline__ int expiry_of(Word&& word, int r, int j, int L, int w, int m, const int32_t* cu, int nseq) {
+    int s0 = 0, s1 = L, k = w;
+    if (kMode == 1) {
+        int lo = 0, hi = nseq;                                   // largest s with cu[s] <= j
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (cu[mid] <= j) lo = mid; else hi = mid;
+        }
+        s0 = max(cu[lo], 0);
+        s1 = min(cu[lo + 1], L);
+        if (r >= w && s0 > 0) {
+            int c = r, s = 0, n0 = 0;
+            for (int l = 0; l < m && c > 0; ++l) {
+                const int half = 1 << (m - 1 - l);
+                const int ones = ones_of([&](int q) { return word(l, q); }, s, c);
+                if (s0 & half) { n0 += c - ones; c = ones; s += half; } else { c -= ones; }
+            }
+            k = w + n0;
+        }
+    }
+    if (r < k) return s1;                                        // fewer than w keys beat it (inside its sequence): never dropped
+    if (kMode == 2) return 0;
+    int c = r, s = 0;                                            // k-th smallest among the first c entries of the node starting at s
+    for (int l = 0; l < m; ++l) {
+        const int half = 1 << (m - 1 - l);
+        const int ones = ones_of([&](int q) { return word(l, q); }, s, c), zeros = c - ones;
+        if (k <= zeros) c = zeros; else { k -= zeros; c = ones; s += half; }
+    }
+    return (kMode == 1 && s >= s1) ? s1 : max(j, s);
+}
+
+// Bitmap words of square tiles (bm = bn): all keys of key tile kt that any row keeps enter in query tile kt (non-causal: 0), so the union of
+// their intervals ends with the latest expiry of the tile, `last` (0: no key kept).
+__device__ __forceinline__ uint32_t bitmap_word(const int* last, int kt0, int n, int qt, int bm, int causal) {
+    uint32_t word = 0u;
+    for (int k = 0; k < n; ++k) word |= (qt >= (causal ? kt0 + k : 0) && qt * bm < last[k]) ? 1u << k : 0u;
+    return word;
+}
+
+// All levels with nodes of up to kBlock keys in one launch, a CTA per block of kBlock keys. A thread takes kPer consecutive keys; the
+// levels inside a thread and inside a warp (up to 32 kPer keys) are bitonic merges in registers and by shuffles, the wider runs are merged
+// in shared memory, kPer consecutive outputs per thread. A node's bit is a bit of the key's index, and the count of ones before a word is,
+// in shared memory, the word's position minus the A keys taken so far. Padding keys (beyond L) sort below every real key (delta > 0)
+// and keep their index in the low word.
+// kMode >= 0: the head is one block (Lc = its padded length <= kBlock) and the CTA goes on from the tree in shared memory: expiry (the modes of
+// expiry_of) and, with Tr > 0 (square tiles, at most 32), the bitmap. Otherwise sorted keys and levels go to global memory.
+// 1024 keys are bound by latency, each level a chain of probes or shuffles (8.5 us); 4096 on one SM by its integer pipe (issue slots 57 %
+// busy, 24 us), which is why few heads take blocks of 1024 and two merge launches more (launch_mask_build).
+template <int kBlock, int kMode>
+__global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const float* __restrict__ delta, unsigned long long* __restrict__ sorted,
+                                                                   uint2* __restrict__ lev, int L, int Lc, int m, int32_t* __restrict__ expiry,
+                                                                   uint32_t* __restrict__ bitmap, int w, const int32_t* __restrict__ cu, int nseq,
+                                                                   int bm, int Tr, int causal, int64_t zero_words) {
+    constexpr int kPer = kBlock > 2048 ? 8 : 4, kWarpKeys = 32 * kPer, kWarpBit = kPer == 8 ? 8 : 7;
+    static_assert(kWarpKeys == 1 << kWarpBit && kPer * kBlockThreads >= kBlock, "a thread's keys, a warp's keys");
+    constexpr int kWords = kBlock / 32;
+    extern __shared__ __align__(16) unsigned long long sk[];         // two buffers of keys; kMode >= 0: the levels
+    __shared__ int last[32];
+    const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = blockIdx.x * kBlock, nreal = min(kBlock, Lc - base);
     const size_t Wl = (size_t)Lc / 32;
     unsigned long long* cur = sk;
-    unsigned long long* nxt = sk + kBlockKeys;
+    unsigned long long* nxt = sk + padded(kBlock);
+    uint2* slev = reinterpret_cast<uint2*>(sk + 2 * padded(kBlock)); // [level][kWords]
+    pdl_enter_restrict(delta, sorted, lev, expiry, bitmap, cu);
+    if (zero_words) zero_share(bitmap, zero_words);
+    // the word of position p of the block in the level of nodes of 2 << bit keys
+    auto put_word = [&](int bit, int p, uint32_t before, uint32_t bits) {
+        if (kMode >= 0) slev[(m - 1 - bit) * kWords + (p >> 5)] = make_uint2(before, bits);
+        else lev[((size_t)bh * m + (m - 1 - bit)) * Wl + ((base + p) >> 5)] = make_uint2(before, bits);
+    };
+    constexpr int kPerWord = 32 / kPer;                              // threads per word of a level
+    const int o = kPer * tid;                                        // this thread's keys, and its outputs of every level: o .. o + kPer - 1 of the block
+    const bool exists = o < nreal;                                   // (all of a warp's or none: nreal is a multiple of 256)
+    unsigned long long key[kPer];
+    if (exists) {
 #pragma unroll
-    for (int k = 0; k < kBlockKeys / kBlockThreads; ++k) {
-        const int i = tid + k * kBlockThreads;
-        cur[i] = i < nreal ? src[(size_t)bh * Lc + base + i] : 0ull;
+        for (int u = 0; u < kPer; ++u) {
+            const int j = base + o + u;
+            key[u] = j < L ? sort_key(delta[(size_t)bh * L + j], j) : (unsigned long long)(0xFFFFFFFFu - (unsigned)j);
+        }
+        // a level in order in the warp's registers: the bits, and per word the ones of its node before it
+        auto emit = [&](int bit) {
+            const uint32_t wv = gather_bits<kPer>(upper_half(key, bit), lane);
+            const int words = max(1, (2 << bit) / 32), word = (lane / kPerWord) & (words - 1), ones = __popc(wv);
+            int upto = ones;
+            for (int d = 1; d < words; d <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, upto, d * kPerWord);
+                if (word >= d) upto += y;
+            }
+            if (lane % kPerWord == 0) put_word(bit, o, (uint32_t)(upto - ones), wv);
+        };
+#pragma unroll
+        for (int h = 1; h < kPer; h *= 2) {                          // in the thread: runs of h keys, the second one reversed against the first
+#pragma unroll
+            for (int g = 0; g < kPer; g += 2 * h) {
+#pragma unroll
+                for (int u = 0; u < h; ++u) order_desc(key[g + u], key[g + 2 * h - 1 - u]);
+#pragma unroll
+                for (int d = h / 2; d; d >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 2 * h; ++u)
+                        if (!(u & d)) order_desc(key[g + u], key[g + u + d]);
+            }
+            emit(h == 1 ? 0 : h == 2 ? 1 : 2);
+        }
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {                                // in the warp: runs of kPer << t keys
+#pragma unroll
+            for (int d = t; d >= 0; --d) {
+                // first the second run reversed against the first, then the distances of 2^(t-1) .. 1 threads
+                const int mask = d == t ? (2 << t) - 1 : 1 << d;
+                const bool upper = (lane >> d) & 1;
+                unsigned long long y[kPer];
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) y[u] = __shfl_xor_sync(0xffffffffu, key[d == t ? kPer - 1 - u : u], mask);
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) key[u] = (key[u] > y[u]) != upper ? key[u] : y[u];
+            }
+#pragma unroll
+            for (int d = kPer / 2; d; d >>= 1)
+#pragma unroll
+                for (int u = 0; u < kPer; ++u)
+                    if (!(u & d)) order_desc(key[u], key[u + d]);
+            emit(kWarpBit - 5 + t);
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) cur[padded(o) + u] = key[u];
     }
     __syncthreads();
-    const int o = 4 * tid;                                       // this thread's outputs: o .. o + 3 of the block
-    int l = m - 9;
-    for (int R = kChunk; R < kBlockKeys && R < Lc; R *= 2, --l) {
-        const int pair = o & ~(2 * R - 1), x = o - pair;
+    for (int bit = kWarpBit; (1 << bit) < kBlock && (1 << bit) < Lc; ++bit) {        // wider runs, of R = 1 << bit keys
+        const int R = 1 << bit, pair = o & ~(2 * R - 1), x = o - pair;
         const int na = max(0, min(R, nreal - pair)), nb = max(0, min(R, nreal - pair - R));
-        unsigned long long out[4];
-        uint32_t prov;
-        const int i0 = merge4(cur + pair, na, cur + pair + R, nb, x, out, prov);
-        const bool exists = o < nreal;                           // (runs are whole chunks: all four outputs exist or none)
+        int i0 = 0;
         if (exists) {
-            *reinterpret_cast<ulonglong2*>(nxt + o) = make_ulonglong2(out[0], out[1]);
-            *reinterpret_cast<ulonglong2*>(nxt + o + 2) = make_ulonglong2(out[2], out[3]);
+            i0 = merge_outputs<kPer>([&](int p) { return cur[padded(p)]; }, pair, na, pair + R, nb, x, bit / 2 + 1, key);
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) nxt[padded(o) + u] = key[u];
         }
-        const uint32_t wv = gather_nibbles(exists ? prov : 0u, lane);
-        if ((lane & 7) == 0 && exists) lev[((size_t)bh * m + l) * Wl + (size_t)((base + o) >> 5)] = make_uint2((uint32_t)(x - i0), wv);
+        const uint32_t wv = gather_bits<kPer>(exists ? upper_half(key, bit) : 0u, lane);
+        if (lane % kPerWord == 0 && exists) put_word(bit, o, (uint32_t)(x - i0), wv);
         unsigned long long* tmp = cur; cur = nxt; nxt = tmp;
         __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < kBlockKeys / kBlockThreads; ++k) {
-        const int i = tid + k * kBlockThreads;
-        if (i < nreal) dst[(size_t)bh * Lc + base + i] = cur[i];
+    if constexpr (kMode < 0) {
+        for (int i = tid; i < nreal; i += kBlockThreads) sorted[(size_t)bh * Lc + base + i] = cur[padded(i)];
+    } else {
+        int* sexp = reinterpret_cast<int*>(nxt);
+        for (int r = tid; r < L; r += kBlockThreads) {
+            const int j = (int)(0xFFFFFFFFu - (uint32_t)cur[padded(r)]);
+            sexp[j] = expiry_of<kMode>([&](int l, int q) { return slev[l * kWords + (q >> 5)]; }, r, j, L, w, m, cu, nseq);
+        }
+        __syncthreads();
+        if (Tr > 0) {                                                // a warp per key tile
+            for (int kt = warp; kt < Tr; kt += kBlockThreads / 32) {
+                int top = 0;
+                for (int j = kt * bm + lane; j < min(L, kt * bm + bm); j += 32) {
+                    const int e = sexp[j];
+                    expiry[(size_t)bh * L + j] = e;
+                    top = max(top, e > (causal ? j : 0) ? e : 0);
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+                if (lane == 0) last[kt] = top;
+            }
+            __syncthreads();
+            if (tid < Tr) bitmap[(size_t)bh * Tr + tid] = bitmap_word(last, 0, Tr, tid, bm, causal);
+        } else {
+            for (int j = tid; j < L; j += kBlockThreads) expiry[(size_t)bh * L + j] = sexp[j];
+        }
     }
 }
 
-// One level per launch for runs of R >= 4096 keys: a CTA produces 1024 consecutive outputs of one pair of runs. Warp 0
+// Shared memory of tree_block_kernel
+constexpr size_t block_smem(int keys, bool whole) { return 2 * (size_t)padded(keys) * sizeof(unsigned long long) + (whole ? 12 * (keys / 32) * sizeof(uint2) : 0); }
+
+// One level per launch for runs of R >= 1024 keys: a CTA produces 1024 consecutive outputs of one pair of runs. Warp 0
 // finds where they start in the two runs (32 probes per round), the CTA stages up to 1024 keys of each run in shared
 // memory, and every thread merges four outputs from there.
 __global__ void __launch_bounds__(kMergeThreads) tree_merge_kernel(const unsigned long long* __restrict__ src,
                                                                    unsigned long long* __restrict__ dst,
                                                                    uint2* __restrict__ lev_l, int Lc, int R, int m) {
-    __shared__ __align__(16) unsigned long long sA[kMergeOut], sB[kMergeOut];
+    __shared__ __align__(16) unsigned long long sAB[2 * kMergeOut];       // A | B
     __shared__ int s_a0;
     pdl_enter_restrict(src, dst, lev_l);
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -503,30 +618,25 @@ __global__ void __launch_bounds__(kMergeThreads) tree_merge_kernel(const unsigne
 #pragma unroll
     for (int k = 0; k < kMergeOut / kMergeThreads; ++k) {
         const int i = tid + k * kMergeThreads;
-        sA[i] = i < la ? A[a0 + i] : 0ull;
-        sB[i] = i < lb ? Bv[b0 + i] : 0ull;
+        sAB[i] = i < la ? A[a0 + i] : 0ull;
+        sAB[kMergeOut + i] = i < lb ? Bv[b0 + i] : 0ull;
     }
     __syncthreads();
     const int x = 4 * tid;
     const bool exists = t0 + x < na + nb;
     unsigned long long out[4];
-    uint32_t prov;
-    const int i0 = merge4(sA, la, sB, lb, x, out, prov);
+    const int i0 = merge_outputs<4>([&](int p) { return sAB[p]; }, 0, la, kMergeOut, lb, x, 6, out);      // (staged runs of up to 1024 keys)
+    const uint32_t prov = upper_half(out, 31 - __clz(R));
     if (exists) {
         unsigned long long* d = dst + (size_t)bh * Lc + o0 + x;
         *reinterpret_cast<ulonglong2*>(d) = make_ulonglong2(out[0], out[1]);
         *reinterpret_cast<ulonglong2*>(d + 2) = make_ulonglong2(out[2], out[3]);
     }
-    const uint32_t wv = gather_nibbles(exists ? prov : 0u, lane);
+    const uint32_t wv = gather_bits<4>(exists ? prov : 0u, lane);
     if ((lane & 7) == 0 && exists) lev_l[(size_t)bh * m * (Lc / 32) + ((o0 + x) >> 5)] = make_uint2((uint32_t)(b0 + x - i0), wv);
 }
 
 // One thread per rank r of a head: the key at rank r, the walk down the tree, expiry[j] = max(j, index found).
-// kMode 2 (non-causal): every row sees every key, so the key is kept by all rows iff fewer than w keys beat it.
-// kMode 1: sequences packed along the key axis (sequence s owns the keys cu[s] <= j < cu[s+1]). A key competes only with
-// the keys of its own sequence [s0, s1): of the first r keys of the head, n0 have an index below s0 (a first walk, along
-// the path of s0, adds up the lower halves it leaves to its left), so the w-th beater inside the sequence is the
-// (n0 + w)-th smallest index overall, if that exists and lies below s1; otherwise the key lives to the end of its sequence.
 template <int kMode>
 __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long long* __restrict__ sorted, const uint2* __restrict__ lev,
                                                           int32_t* __restrict__ expiry, int L, int Lc, int w, int m,
@@ -536,60 +646,38 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
     if (r >= L) return;                                          // ranks from L on are padding
     const int j = (int)(0xFFFFFFFFu - (uint32_t)sorted[(size_t)bh * Lc + r]);
     const size_t W = (size_t)Lc / 32;
-    const uint2* lv0 = lev + (size_t)bh * m * W;
-    // ones among the first c entries of the node that starts at position s of a level
-    auto ones_of = [](const uint2* lv, int s, int c) {
-        const int q = s + c - 1;                                 // last entry of the prefix (c >= 1)
-        const uint2 wd = lv[q >> 5];
-        const uint32_t upto = (2u << (q & 31)) - 1u, from = ~((1u << (s & 31)) - 1u);         // a node smaller than a word starts inside it
-        return (int)wd.x + __popc(wd.y & upto & from);
-    };
-    int s0 = 0, s1 = L, k = w;
-    if (kMode == 1) {
-        int lo = 0, hi = nseq;                                   // largest s with cu[s] <= j
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (cu[mid] <= j) lo = mid; else hi = mid;
-        }
-        s0 = max(cu[lo], 0);
-        s1 = min(cu[lo + 1], L);
-        if (r >= w && s0 > 0) {
-            const uint2* lv = lv0;
-            int c = r, s = 0, n0 = 0;
-            for (int l = 0; l < m && c > 0; ++l, lv += W) {
-                const int half = 1 << (m - 1 - l);
-                const int ones = ones_of(lv, s, c);
-                if (s0 & half) { n0 += c - ones; c = ones; s += half; } else { c -= ones; }
-            }
-            k = w + n0;
-        }
-    }
-    int e;
-    if (r < k) {
-        e = s1;                                                  // fewer than w keys beat it (inside its sequence): never dropped
-    } else if (kMode == 2) {
-        e = 0;
-    } else {
-        const uint2* lv = lv0;
-        int c = r, s = 0;                                        // k-th smallest among the first c entries of the node starting at s
-        for (int l = 0; l < m; ++l, lv += W) {
-            const int half = 1 << (m - 1 - l);
-            const int ones = ones_of(lv, s, c), zeros = c - ones;
-            if (k <= zeros) c = zeros; else { k -= zeros; c = ones; s += half; }
-        }
-        e = (kMode == 1 && s >= s1) ? s1 : max(j, s);
-    }
-    expiry[(size_t)bh * L + j] = e;
+    const uint2* lv = lev + (size_t)bh * m * W;
+    expiry[(size_t)bh * L + j] = expiry_of<kMode>([&](int l, int q) { return lv[l * W + (q >> 5)]; }, r, j, L, w, m, cu, nseq);
 }
 
 __global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v, uint32_t* bitmap, int64_t bitmap_words) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_enter_restrict(p, bitmap);
-    zero_share(bitmap, bitmap_words);
+    if (bitmap_words) zero_share(bitmap, bitmap_words);
     if (i < n) p[i] = v;
 }
 
-// One CTA per (key tile, head): key j is kept by rows [j, expiry[j]), i.e. by query tiles j/bm .. (expiry[j]-1)/bm.
+// Square tiles of a multiple of 32 rows: one CTA per (word of 32 key tiles, head), a warp per key tile finds the latest expiry, then a thread per
+// query tile forms its word: no atomics, and the bitmap needs no zeros. A difference array per key tile and
+// atomics into the bitmap took 7.8 us for 32 heads of 16384 keys.
+__global__ void __launch_bounds__(1024) bitmap_square_kernel(const int32_t* __restrict__ expiry, uint32_t* __restrict__ bitmap,
+                                                             int L, int bm, int T, int Wd, int causal) {
+    __shared__ int last[32];
+    const int kt0 = blockIdx.x * 32, bh = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j0 = (kt0 + warp) * bm;
+    pdl_enter_restrict(expiry, bitmap);
+    int top = 0;
+    for (int j = j0 + lane; j < min(L, j0 + bm); j += 32) {
+        const int e = expiry[(size_t)bh * L + j];
+        top = max(top, e > (causal ? j : 0) ? e : 0);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) last[warp] = top;
+    __syncthreads();
+    for (int qt = threadIdx.x; qt < T; qt += 1024)
+        bitmap[((size_t)bh * T + qt) * Wd + blockIdx.x] = bitmap_word(last, kt0, min(32, T - kt0), qt, bm, causal);
+}
+
+// Any other tiles. One CTA per (key tile, head): key j is kept by rows [j, expiry[j]), i.e. by query tiles j/bm .. (expiry[j]-1)/bm.
 // A difference array over query tiles forms the union; bits are OR-ed into the (pre-zeroed) bitmap.
 // (non-causal mode: key j is kept by rows [0, expiry[j]), so its interval of query tiles starts at tile 0)
 __global__ void __launch_bounds__(128) bitmap_kernel(const int32_t* __restrict__ expiry, uint32_t* __restrict__ bitmap,
@@ -633,6 +721,7 @@ __global__ void __launch_bounds__(128) bitmap_kernel(const int32_t* __restrict__
 }  // namespace
 
 constexpr int kStaticChunk = kChunk;
+constexpr int kFewWhole = 3072;              // padded keys of a head that one CTA takes whole although few heads leave SMs idle
 
 // levels of the rank tree over a head of Lc (a multiple of 256) keys: the smallest m with 2^m >= Lc
 static int tree_levels(int Lc) {
@@ -703,8 +792,6 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
                       uint32_t* bitmap, void* ws, cudaStream_t st, const int32_t* cu, int nseq) {
     int rc;
     if ((rc = mask_build_limits(P))) return rc;          // an error return means that no kernel has been launched
-    constexpr size_t kBlockSmem = 2 * (size_t)kBlockKeys * sizeof(unsigned long long);
-    if (cudaFuncSetAttribute(tree_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlockSmem) != cudaSuccess) return DMA_ERR_CUDA;
     if (P.dtype == DMA_BF16)
         rc = P.d == 128 ? launch_delta<__nv_bfloat16, 128>(P, V, W, A, bias, st)
                         : launch_delta<__nv_bfloat16, 64>(P, V, W, A, bias, st);
@@ -714,40 +801,54 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
 
     const int BH = P.B * P.Hq;
     const int nchunk = (P.L + kChunk - 1) / kChunk;
-    const int64_t bitmap_words = (int64_t)BH * P.Tr * P.Wd;        // zeroed by the kernel after the deltas
+    // (the general bitmap kernel ORs bits into zeros that an earlier kernel of the stage leaves)
+    const bool square = P.bm == P.bn && P.bm % 32 == 0;
+    const int64_t zero_words = square ? 0 : (int64_t)BH * P.Tr * P.Wd;
     if (P.w >= P.L && !cu) {   // every visible key is kept
         size_t n = (size_t)BH * P.L;
-        rc = launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, bitmap_words);
+        rc = launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, zero_words);
         if (rc) return rc;
     } else {
-        // rank tree: sorted chunks and the low levels, one merge pass per further level, then one walk per key
+        // rank tree: sorted blocks, one merge pass per further level, then one walk per key; or everything in the block kernel.
+        // Blocks of 4096 keys keep few SMs busy for long where there are few; mask build, us, before (256-key chunks, blocks of 4096) / now:
+        // 8 heads of 500 keys 14.4 / 8.4, 16 of 1000 18.6 / 12.1, 8 of 2048 20.2 / 16.7, 16 of 2500 24.1 / 22.5, 16 of 4096 26.5 / 23.9 (28.8 whole),
+        // 8 of 13000 36 / 33 (38 in blocks of 4096), 128 of 4096 68 / 48, 32 of 16384 73 / 60, of 65536 292 / 229. A cluster of four CTAs per
+        // 4096 keys, which merged and walked through distributed shared memory: 26.2 at 16 heads of 4096, 37 at 8 of 13000.
         const int Lc = nchunk * kChunk, m = tree_levels(Lc);
+        const bool few = (int64_t)BH * ((Lc + kSmallBlock - 1) / kSmallBlock) <= 2 * 148, whole = Lc <= (few ? kFewWhole : kBlockKeys);
+        const int per_block = whole ? (Lc <= kSmallBlock ? kSmallBlock : kBlockKeys) : few ? kSmallBlock : kBlockKeys;
+        const bool fused_bitmap = whole && square && P.Tr <= 32;
         const size_t keys = (size_t)BH * Lc, Wl = (size_t)Lc / 32;
         auto* buf0 = reinterpret_cast<unsigned long long*>((char*)ws + kWsHeaderBytes);
         auto* buf1 = buf0 + keys;
         uint2* lev = reinterpret_cast<uint2*>(buf1 + keys);
-        rc = launch_overlapped(chunk_sort_kernel, dim3(nchunk, BH), dim3(kChunk), 0, st, 1, bias, buf0, P.L, nchunk, lev, m, bitmap, bitmap_words);
+        const int mode = !whole ? -1 : cu ? 1 : P.causal ? 0 : 2;
+        auto pick = [&](auto n) {
+            constexpr int kN = decltype(n)::value;
+            return mode < 0 ? tree_block_kernel<kN, -1> : mode == 0 ? tree_block_kernel<kN, 0> : mode == 1 ? tree_block_kernel<kN, 1> : tree_block_kernel<kN, 2>;
+        };
+        auto block = per_block == kSmallBlock ? pick(std::integral_constant<int, kSmallBlock>{}) : pick(std::integral_constant<int, kBlockKeys>{});
+        // (state of the function, which other threads' calls share: always the limit)
+        if (cudaFuncSetAttribute(block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)block_smem(kBlockKeys, true)) != cudaSuccess) return DMA_ERR_CUDA;
+        rc = launch_overlapped(block, dim3((Lc + per_block - 1) / per_block, BH), dim3(kBlockThreads), block_smem(per_block, whole), st, 1, bias, buf0, lev, P.L, Lc, m,
+                               expiry, fused_bitmap || zero_words ? bitmap : nullptr, P.w, cu, nseq, P.bm, fused_bitmap ? P.Tr : 0, P.causal, zero_words);
         if (rc) return rc;
-        if (Lc > kChunk) {
-            rc = launch_overlapped(tree_block_kernel, dim3((Lc + kBlockKeys - 1) / kBlockKeys, BH), dim3(kBlockThreads), kBlockSmem, st, 1, buf0, buf1, lev, Lc, m);
-            if (rc) return rc;
-            std::swap(buf0, buf1);
-        }
-        int l = m - 13;                                          // level of the nodes of 2 * kBlockKeys keys
-        for (int R = kBlockKeys; R < Lc; R *= 2, --l) {
+        if (fused_bitmap) return DMA_OK;
+        int l = m - (per_block == kSmallBlock ? 11 : 13);         // level of the nodes of two blocks
+        for (int R = per_block; !whole && R < Lc; R *= 2, --l) {
             rc = launch_overlapped(tree_merge_kernel, dim3((Lc + kMergeOut - 1) / kMergeOut, BH), dim3(kMergeThreads), 0, st, 1, buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
             if (rc) return rc;
             std::swap(buf0, buf1);
         }
-        const dim3 grid((P.L + 255) / 256, BH);
-        rc = launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev,
-                               expiry, P.L, Lc, P.w, m, cu, nseq);
-        if (rc) return rc;
+        if (!whole) {
+            const dim3 grid((P.L + 255) / 256, BH);
+            rc = launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev,
+                                   expiry, P.L, Lc, P.w, m, cu, nseq);
+            if (rc) return rc;
+        }
     }
-
-    size_t smem = (size_t)(P.Tr + 1) * sizeof(int);
-    if (smem > 48 * 1024) return DMA_ERR_UNSUPPORTED;
-    return launch_overlapped(bitmap_kernel, dim3(P.Tc, BH), dim3(128), smem, st, 1, expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
+    if (square) return launch_overlapped(bitmap_square_kernel, dim3(P.Wd, BH), dim3(1024), 0, st, 1, expiry, bitmap, P.L, P.bm, P.Tr, P.Wd, P.causal);
+    return launch_overlapped(bitmap_kernel, dim3(P.Tc, BH), dim3(128), (size_t)(P.Tr + 1) * sizeof(int), st, 1, expiry, bitmap, P.L, P.bm, P.bn, P.Tr, P.Wd, P.causal);
 }
 
 }  // namespace dma
