@@ -778,9 +778,10 @@ __global__ void __launch_bounds__(kPerm ? kPermThreads : 256) bwd_prepare_kernel
 // After the main kernel, in one launch (HBM-bound): the first q_blocks CTAs turn the blocked fp32 dQ accumulator (see
 // BwdParams::dQacc) into bf16 dQ in the caller's layout, softmax scale applied; the others the fp32 dK, dV accumulators
 // [B, L, Hkv, d] where the main kernel did not write dK, dV itself.
-//   dQ: one CTA per (batch, head, 16-row block, or two of them at d = 64); a thread takes two neighbouring channels (they share
-//   their chunk position) and four rows: two 16-byte loads, four 4-byte stores that the lanes of a warp, consecutive channel
-//   pairs, make whole 128-byte lines of.
+//   dQ: kFinishBlocks 2 KB blocks (16 rows x 32 channels) per warp, read as they lie (512 consecutive bytes per instruction, all of a
+//   warp's loads in flight), turned around as bf16 in shared memory and written 256 (d = 64: 128) consecutive bytes per row. Reading
+//   a channel pair's rows per thread instead, 16 bytes out of every 128, took 32 passes per load: at L = 16384 with 32 heads of 128 channels
+//   121 us (backward 2221 -> 2097), 16 heads of 4096 (backward 163 -> 159).
 //   dK, dV: 8 elements per thread. nslots > 1: the accumulator is nslots copies, slot_stride elements apart, added in slot
 //   order (a fixed order: the result is then the same bits from run to run).
 struct FinishParams {
@@ -789,30 +790,54 @@ struct FinishParams {
     __nv_bfloat16* dQ;
     __nv_bfloat16* out[2];
     int q_blocks, kv_blocks;    // CTAs of dQ, of each of dK and dV
-    int L, Hq, Hkv, Lblk, d, nslots;
+    int L, Hq, Hkv, Lblk, nslots;
     int64_t nkv;                // elements of dK
     uint32_t q_rows16;          // 16-row blocks of dQ in all
     int64_t qs[3], st[2][3];
     float scale;
 };
 
+constexpr int kFinishBlocks = 2;
+
+template <int kD>
 __global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
+    constexpr int kCh = kD / 32, kRowBlocks = 8 / kCh * kFinishBlocks;     // channel blocks of a row, 16-row blocks of a CTA
+    constexpr int kPitch = kD / 2 + 4;                                     // 4-byte words per row: 16-byte aligned, rows 4 apart 16 banks apart
+    __shared__ __align__(16) uint32_t turn[kRowBlocks * 16 * kPitch];
     pdl_enter();
     if ((int)blockIdx.x < P.q_blocks) {
-        const int per = P.d * 2, t = threadIdx.x % per;                    // threads per 16-row block
-        const uint32_t blk = blockIdx.x * (256 / per) + threadIdx.x / per;
-        if (blk >= P.q_rows16) return;
-        const int bh = (int)(blk / (uint32_t)P.Lblk), rb = (int)(blk - (uint32_t)bh * P.Lblk), h = bh % P.Hq, b = bh / P.Hq;
-        const int pairs = P.d >> 1, c = 2 * (t % pairs), q = t / pairs;    // channel pair, quad of rows
-        const int cc = c & 31;
-        const float* src = P.dQacc + (size_t)blk * P.d * 16 + (c >> 5) * 512 + cc * 16 + ((q ^ ((cc >> 1) & 3)) << 2);
-        const float4 x = *reinterpret_cast<const float4*>(src), y = *reinterpret_cast<const float4*>(src + 16);
-        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
-        __nv_bfloat16* out = P.dQ + b * P.qs[0] + h * P.qs[2] + c;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ch = warp % kCh;
+        const uint32_t blk0 = blockIdx.x * kRowBlocks;
+        float4 x[kFinishBlocks][4];
 #pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
-            const int i = rb * 16 + 4 * q + rr;
-            if (i < P.L) *reinterpret_cast<uint32_t*>(out + (int64_t)i * P.qs[1]) = ptx::pack_bf16(xs[rr] * P.scale, ys[rr] * P.scale);
+        for (int n = 0; n < kFinishBlocks; ++n) {
+            const uint32_t blk = min(blk0 + warp / kCh + n * (8 / kCh), P.q_rows16 - 1);
+            const float4* src = reinterpret_cast<const float4*>(P.dQacc + ((size_t)blk * kCh + ch) * 512) + lane;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[n][u] = src[32 * u];
+        }
+#pragma unroll
+        for (int n = 0; n < kFinishBlocks; ++n) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int c = 8 * u + (lane >> 2), q = (lane & 3) ^ ((c >> 1) & 3);       // channel of the block, quad of rows (BwdParams::dQacc)
+                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(turn + ((warp / kCh + n * (8 / kCh)) * 16 + 4 * q) * kPitch) + ch * 32 + c;
+                dst[0] = __float2bfloat16_rn(x[n][u].x * P.scale);
+                dst[2 * kPitch] = __float2bfloat16_rn(x[n][u].y * P.scale);
+                dst[4 * kPitch] = __float2bfloat16_rn(x[n][u].z * P.scale);
+                dst[6 * kPitch] = __float2bfloat16_rn(x[n][u].w * P.scale);
+            }
+        }
+        __syncthreads();
+        constexpr int kParts = kD / 8;                                     // 16-byte parts of a row
+#pragma unroll
+        for (int t = threadIdx.x; t < kRowBlocks * 16 * kParts; t += 256) {
+            const int r = t / kParts, part = t % kParts;
+            const uint32_t blk = blk0 + r / 16;
+            if (blk >= P.q_rows16) continue;
+            const int bh = (int)(blk / (uint32_t)P.Lblk), i = (int)(blk - (uint32_t)bh * P.Lblk) * 16 + r % 16, h = bh % P.Hq, b = bh / P.Hq;
+            if (i < P.L)
+                *reinterpret_cast<uint4*>(P.dQ + b * P.qs[0] + (int64_t)i * P.qs[1] + h * P.qs[2] + part * 8) = *reinterpret_cast<const uint4*>(turn + r * kPitch + part * 4);
         }
         return;
     }
@@ -820,8 +845,8 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
     const int64_t e = ((int64_t)(blk % P.kv_blocks) * 256 + threadIdx.x) * 8;
     if (e >= P.nkv) return;
     const float* acc = P.acc[which];
-    const uint32_t row = (uint32_t)(e >> (P.d == 128 ? 7 : 6)), bl = row / (uint32_t)P.Hkv;
-    const int c = (int)(e & (P.d - 1)), h = (int)(row - bl * P.Hkv), b = (int)(bl / (uint32_t)P.L), i = (int)(bl - (uint32_t)b * P.L);
+    const uint32_t row = (uint32_t)(e / kD), bl = row / (uint32_t)P.Hkv;
+    const int c = (int)(e % kD), h = (int)(row - bl * P.Hkv), b = (int)(bl / (uint32_t)P.L), i = (int)(bl - (uint32_t)b * P.L);
     float4 a = *reinterpret_cast<const float4*>(acc + e), bb = *reinterpret_cast<const float4*>(acc + e + 4);
     for (int sl = 1; sl < P.nslots; ++sl) {
         const float4 a2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e), b2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e + 4);
@@ -997,13 +1022,14 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     if (rc) return rc;
     FinishParams f;
     f.dQacc = acc; f.acc[0] = accK; f.acc[1] = accV; f.dQ = (__nv_bfloat16*)dQ; f.out[0] = (__nv_bfloat16*)dK; f.out[1] = (__nv_bfloat16*)dV;
-    f.L = P.L; f.Hq = P.Hq; f.Hkv = P.Hkv; f.Lblk = P.Tr * 8; f.d = P.d; f.nslots = (int)slots; f.nkv = (int64_t)nkv;
+    f.L = P.L; f.Hq = P.Hq; f.Hkv = P.Hkv; f.Lblk = P.Tr * 8; f.nslots = (int)slots; f.nkv = (int64_t)nkv;
     f.q_rows16 = (uint32_t)((size_t)P.B * P.Hq * P.Tr * 8);
-    f.q_blocks = (int)(((size_t)f.q_rows16 * P.d * 2 + 255) / 256);
+    const int per = 8 / (P.d / 32) * kFinishBlocks;                        // 16-row blocks per CTA
+    f.q_blocks = (int)((f.q_rows16 + per - 1) / per);
     f.kv_blocks = (int)((nkv / 8 + 255) / 256);
     for (int t = 0; t < 3; ++t) { f.qs[t] = P.qs[t]; f.st[0][t] = P.ks[t]; f.st[1][t] = P.vs[t]; }
     f.scale = P.scale;
-    return launch_overlapped(bwd_finish_kernel, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
+    return launch_overlapped(P.d == 128 ? bwd_finish_kernel<128> : bwd_finish_kernel<64>, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
 }
 
 }  // namespace dma
