@@ -154,7 +154,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     volatile int* abort_flag = &S.abort_flag;
 
     if (tid == 0) {
-        mbar_init(&S.kv_full, 1);
+        mbar_init(&S.kv_full, kCompact ? 8 : 1);        // one arrival per gathering warp | TMA bytes
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&S.qd_full[s], 2);      // TMA bytes + the staged vectors
             mbar_init(&S.qd_empty[s], 1);
@@ -195,8 +195,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             cp_async16(S.v + off, P.Vg + vrow, nb);
             if constexpr (kD == 128) cp_async16(S.v + off + kKVBytes / 2, P.Vg + vrow + 64, nb);
         }
-        cp_async_wait_all();
-        fence_proxy_async();                           // (the barrier below hands the rows to the MMA issuers)
     }
     if (warp == 13) {
         tmem_alloc(&S.tmem_base, 512);
@@ -272,6 +270,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         float2 dm2 = make_float2(0.0f, 0.0f);
         int len = 0, cur_g = -1;
         bool ok = true;
+        if constexpr (kCompact) {
+            cp_async_wait_all();       // (behind the barrier, so that the first Q and dO are requested meanwhile: 16 heads of 4096 keys, backward, 161.0 -> 157.6 us)
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.kv_full);
+        }
         for (int n = 0; n < n_steps && ok; ++n) {
             const uint32_t e = S.sched[n];
             const int g = (int)(e >> 11), i0 = (int)((e >> 1) & 0x3FF) * 128 + (int)(e & 1) * 64;
@@ -543,7 +547,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const uint64_t dX0 = smem_desc_plain(smem_u32(S.qext[0]), 128, 256);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             const int n_steps_u = __shfl_sync(0xffffffffu, n_steps, 0);
-            bool ok = kCompact || mbar_wait_warp(&S.kv_full, 0, abort_flag);
+            bool ok = mbar_wait_warp(&S.kv_full, 0, abort_flag);
+            if constexpr (kCompact) fence_proxy_async();     // the gathered rows were written through the generic proxy
             for (int n = 0; n < n_steps_u && ok; ++n) {
                 const int st = n % kStages;
                 ok = mbar_wait_warp(&S.qd_full[st], (n / kStages) & 1, abort_flag);
