@@ -64,10 +64,11 @@ struct SharedStorage {
                                               // bits 8-15: 16-key blocks that hold a key some row of the query tile may keep
     uint32_t sched[kMaxSched];                // key tile | use by tile 0 << 30 | use by tile 1 << 31
     uint64_t q_full, k_full[kStages], v_full[kStages], k_empty[kStages], v_empty[kStages];
-    uint64_t s_full[2], p_half[2], p_ready[2], o_done[2], merge;
+    uint64_t s_full[2], p_half[2], p_ready[2], o_done[2], merge, ref_set[2][4];
     uint32_t tmem_base;
     int n_iters;
     int abort_flag;
+    float ref[2][128];                         // kSplit: each row's reference maximum after the group's last entry
     // One query tile per CTA (kSplit): a group's flags, `fast`, and what its per-element test reads are in two slots that its entries take
     // in turn. Token-compacted: group 1's len and jidx. Tile mode: a byte per column, expiry[j] relative to the query tile's first row, cut
     // to [0, 128]: row r of the tile keeps the key iff r is below it (and, in the diagonal tile, not below the column).
@@ -76,6 +77,7 @@ struct SharedStorage {
         alignas(16) uint8_t last[2][2][128];
     };
 };
+static_assert(sizeof(SharedStorage) + 1024 <= 232448, "shared memory of a CTA");
 static_assert(kStages == 2 && offsetof(SharedStorage, bext) == offsetof(SharedStorage, aext) + 2 * 4096,
               "token-compacted mode takes aext and bext as six blocks of 2 KB in a row: ones, two stages of two tiles, zeros");
 
@@ -158,6 +160,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             mbar_init(&S.o_done[w], 1);
         }
         mbar_init(&S.merge, 4);
+        for (int q = 0; q < 8; ++q) mbar_init(&S.ref_set[q >> 2][q & 3], 1);
         S.abort_flag = 0;
         S.n_iters = 0;
         fence_barrier_init();
@@ -304,7 +307,26 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // The running max m_ref stays in score units and the exponent is formed as (x - m_ref) * c: the difference
             // is exact for the entries that matter, whatever the magnitude of the bias.
             const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
-            const float m_new = fmaxf(m_ref, mx);
+            float m_new = fmaxf(m_ref, mx);
+            bool grown = false;
+            if constexpr (kSplit) {
+                // Both groups follow the one sequence of references that a walk over all entries takes: entry it - 1's comes from the other group
+                // (the warp with the same rows), and this entry's is published before the exponentials. P then has the same bits as
+                // with two query tiles per CTA, and O differs by the order of fp32 sums only. (With a reference of its own per group P
+                // was rounded at other places: O as accurate, but 1.7e-3 away, and dA, a sum that cancels, by up to 1e-2.)
+                float before = -INFINITY;
+                if (it > 0) {
+                    ok = mbar_wait_warp(&S.ref_set[w ^ 1][warp & 3], ((it - 1) >> 1) & 1, abort_flag);
+                    if (!ok) break;
+                    before = S.ref[w ^ 1][r];
+                }
+                m_new = fmaxf(before, mx);
+                if (it > 0 && !__any_sync(0xffffffffu, m_new > before + P.rescale_gap)) m_new = before;
+                S.ref[w][r] = m_new;               // (the other group has read the value before it published its own last one)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.ref_set[w][warp & 3]);
+                grown = __any_sync(0xffffffffu, m_new != m_ref);
+            }
             auto stab_resid = [&](float m) {           // m c - stab(m); 0 for m = -inf
                 const float mm = (m == -INFINITY) ? 0.0f : m;
                 const float Mm = mm * P.scale_log2;
@@ -313,7 +335,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             if (n_used == 0) {
                 m_ref = m_new;
                 r_ref = stab_resid(m_ref);
-            } else if (__any_sync(0xffffffffu, m_new > m_ref + P.rescale_gap)) {
+            } else if (kSplit ? grown : __any_sync(0xffffffffu, m_new > m_ref + P.rescale_gap)) {
                 // O_w *= 2^(stab(m_ref) - stab(m_new)): the previous P V product must have landed first
                 ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
                 if (!ok) break;
