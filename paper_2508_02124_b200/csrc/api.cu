@@ -106,7 +106,7 @@ static size_t bwd_need_any(const Prob& P) { return use_tensor_cores(P) ? tc_bwd_
 static int fwd_any(const Prob& P, const void* Q, const void* K, const void* V, const float* bias, const int32_t* expiry,
                    const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st) {
     if (use_tensor_cores(P)) return launch_tc_fwd(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, st);
-    return launch_simt_fwd(P, Q, K, V, bias, expiry, bitmap, O, lse, st);
+    return launch_simt_fwd(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, st);
 }
 
 static int bwd_any(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO, const float* lse,
@@ -133,12 +133,10 @@ int attn_fwd_part(const dma_problem_t* p, int tiles, const void* Q, const void* 
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(bias) || !aligned16(expiry) ||
         !aligned16(lse))
         return DMA_ERR_ALIGN;
-    const bool tc = use_tensor_cores(P);
-    if ((P.flags & DMA_FLAG_COMPACT_KV) && !tc) return DMA_ERR_UNSUPPORTED;
+    if ((P.flags & DMA_FLAG_COMPACT_KV) && !use_tensor_cores(P)) return DMA_ERR_UNSUPPORTED;
     if (!ws || ws_bytes < fwd_ws_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
     if ((rc = device_ok())) return rc;
-    // (the tensor-core path's first kernel clears the workspace header)
-    if (!tc && cudaMemsetAsync(ws, 0, kWsHeaderBytes, st) != cudaSuccess) return DMA_ERR_CUDA;
+    // (the stage's first kernel clears the workspace header)
     return fwd_any(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, st);
 }
 
@@ -153,12 +151,10 @@ int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* 
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(dO) || !aligned16(dQ) ||
         !aligned16(dK) || !aligned16(dV) || !aligned16(dM) || !aligned16(lse))
         return DMA_ERR_ALIGN;
-    const bool tc = use_tensor_cores(P);
-    if ((P.flags & DMA_FLAG_COMPACT_KV) && !tc) return DMA_ERR_UNSUPPORTED;
+    if ((P.flags & DMA_FLAG_COMPACT_KV) && !use_tensor_cores(P)) return DMA_ERR_UNSUPPORTED;
     if (!ws || ws_bytes < bwd_need_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
     if ((rc = device_ok())) return rc;
-    // (the tensor-core path's first kernel clears the workspace header)
-    if (!tc && cudaMemsetAsync(ws, 0, kWsHeaderBytes, st) != cudaSuccess) return DMA_ERR_CUDA;
+    // (the stage's first kernel clears the workspace header)
     return bwd_any(P, Q, K, V, O, dO, lse, bias, expiry, bitmap, dQ, dK, dV, dM, ws, st);
 }
 
@@ -351,9 +347,7 @@ int dma_attn_fwd_chunk(const dma_problem_t* p, int32_t q_begin, int32_t q_len, c
     if (use_tensor_cores(P)) P.flags |= DMA_FLAG_COMPACT_KV;   // the gathered-key kernel has no tile alignment between rows and keys
     if (!ws || ws_bytes < fwd_ws_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
     if ((rc = device_ok())) return rc;
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (!use_tensor_cores(P) && cudaMemsetAsync(ws, 0, kWsHeaderBytes, st) != cudaSuccess) return DMA_ERR_CUDA;
-    return fwd_any(P, Q, K, V, bias, expiry, nullptr, O, lse, ws, st);
+    return fwd_any(P, Q, K, V, bias, expiry, nullptr, O, lse, ws, (cudaStream_t)cuda_stream);
 }
 
 int dma_attn_bwd(const dma_problem_t* p, const void* Q, const void* K, const void* V, const void* O, const void* dO,

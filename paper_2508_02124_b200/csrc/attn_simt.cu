@@ -140,7 +140,7 @@ template <typename T, int D, int kOwn, int NW>
 __global__ void __launch_bounds__(32 * NW) simt_fwd_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
                                                            const float* __restrict__ bias, const int32_t* __restrict__ expiry,
                                                            const uint32_t* __restrict__ bitmap, T* __restrict__ O, float* __restrict__ lse,
-                                                           Prob P, int use_bitmap) {
+                                                           Prob P, int use_bitmap, int32_t* __restrict__ status) {
     constexpr int LD = D + 4, BM = kOwn * NW;
     extern __shared__ __align__(16) float sm[];
     float* sQ = sm;                              // [BM][D]
@@ -150,7 +150,9 @@ __global__ void __launch_bounds__(32 * NW) simt_fwd_kernel(const T* __restrict__
     const int i0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * BM, L = P.L;       // first row inside the chunk (longest walks first)
     const int ia0 = P.q_off + i0;                // its position in the sequence
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    pdl_enter(Q, K, V, bias, expiry, bitmap, O, lse);
+    pdl_enter(Q, K, V, bias, expiry, bitmap, O, lse, status);
+    static_assert(32 * NW >= kWsHeaderBytes / 4, "one CTA clears the workspace header");       // (a memset in front of the kernel is 2 us and keeps it from overlapping)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < kWsHeaderBytes / 4) status[threadIdx.x] = 0;
     const T* q = Q + b * P.qs[0] + h * P.qs[2];
     const T* k = K + b * P.ks[0] + hk * P.ks[2];
     const T* v = V + b * P.vs[0] + hk * P.vs[2];
@@ -227,10 +229,11 @@ __global__ void __launch_bounds__(32 * NW) simt_fwd_kernel(const T* __restrict__
 
 // D_i = dO_i . O_i  (Alg. 2): one warp per (b, h, i)
 template <typename T>
-__global__ void rowdot_kernel(const T* __restrict__ O, const T* __restrict__ dO, float* __restrict__ Dv, Prob P) {
+__global__ void rowdot_kernel(const T* __restrict__ O, const T* __restrict__ dO, float* __restrict__ Dv, Prob P, int32_t* __restrict__ status) {
     const long row = (long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x % 32;
-    pdl_enter(O, dO, Dv);
+    pdl_enter(O, dO, Dv, status);
+    if (blockIdx.x == 0 && threadIdx.x < kWsHeaderBytes / 4) status[threadIdx.x] = 0;         // (the stage's first kernel clears the workspace header)
     if (row >= (long)P.B * P.Hq * P.L) return;
     const int i = row % P.L, h = (row / P.L) % P.Hq, b = row / ((long)P.L * P.Hq);
     const T* o = O + b * P.os[0] + (int64_t)i * P.os[1] + h * P.os[2];
@@ -404,7 +407,7 @@ __global__ void __launch_bounds__(32 * NW) simt_bwd_kernel(const T* __restrict__
 
 template <typename T, int D, int kOwn, int NW>
 int fwd_t(const Prob& P, const void* Q, const void* K, const void* V, const float* bias, const int32_t* expiry,
-          const uint32_t* bitmap, void* O, float* lse, cudaStream_t st) {
+          const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st) {
     constexpr size_t smem = (size_t)(kOwn * NW * D + 4 * kTile * (D + 4) + NW * kOwn * kTile) * sizeof(float);
     auto kern = simt_fwd_kernel<T, D, kOwn, NW>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
@@ -412,7 +415,7 @@ int fwd_t(const Prob& P, const void* Q, const void* K, const void* V, const floa
     int use_bitmap = bitmap && !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0 && P.q_off % kTile == 0;
     timing_mark(0, false, st);
     const int rc = launch_overlapped(kern, dim3((P.Lq + kOwn * NW - 1) / (kOwn * NW), P.Hq, P.B), dim3(32 * NW), smem, st, 1, (const T*)Q, (const T*)K,
-                                     (const T*)V, bias, expiry, bitmap, (T*)O, lse, P, use_bitmap);
+                                     (const T*)V, bias, expiry, bitmap, (T*)O, lse, P, use_bitmap, (int32_t*)ws);
     timing_mark(0, true, st);
     return rc;
 }
@@ -426,7 +429,7 @@ int bwd_t(const Prob& P, const void* Q, const void* K, const void* V, const void
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DMA_ERR_CUDA;
     const size_t rows = (size_t)P.B * P.Hq * P.L;
     float* Dv = reinterpret_cast<float*>((char*)ws + kWsHeaderBytes);
-    int rc = launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P);
+    int rc = launch_overlapped(rowdot_kernel<T>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, 1, (const T*)O, (const T*)dO, Dv, P, (int32_t*)ws);
     if (rc) return rc;
     int use_bitmap = !(P.flags & DMA_FLAG_IGNORE_BITMAP) && P.bm % kTile == 0 && P.bn % kTile == 0;
     const int nblk = (P.L + kOwn * NW - 1) / (kOwn * NW);
@@ -451,14 +454,14 @@ size_t simt_bwd_ws_bytes(const Prob& P) {
 }
 
 int launch_simt_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
-                    const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, cudaStream_t st) {
+                    const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st) {
     const bool small = small_grid(P, P.Lq, P.Hq);
     auto pick = [&](auto t_tag) {
         using T = decltype(t_tag);
         return P.d == 128 ? (small ? fwd_t<T, 128, 2, 4> : fwd_t<T, 128, 4, 8>) : (small ? fwd_t<T, 64, 2, 4> : fwd_t<T, 64, 4, 8>);
     };
     auto f = P.dtype == DMA_FP32 ? pick(float()) : pick(__nv_bfloat16());
-    return f(P, Q, K, V, bias, expiry, bitmap, O, lse, st);
+    return f(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, st);
 }
 
 int launch_simt_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,

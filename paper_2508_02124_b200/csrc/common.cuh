@@ -53,7 +53,7 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
 
 size_t simt_bwd_ws_bytes(const Prob& P);
 int launch_simt_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
-                    const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, cudaStream_t st);
+                    const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st);
 int launch_simt_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,
                     const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ,
                     void* dK, void* dV, float* dM, void* ws, cudaStream_t st);
