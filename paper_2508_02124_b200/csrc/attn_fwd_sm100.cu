@@ -1045,10 +1045,12 @@ int make_tmap_bf16(CUtensorMap* m, const void* base, int B, int L, int H, int d,
 // made from those: the head is read once per 256 group rows. group = 1: the lists are made straight from the head.
 // Every warp owns a contiguous part of what it reads, 128 keys at a time (four coalesced loads per lane in flight), and writes
 // from the sum of the earlier parts' counts. Padded with -1 to the next multiple of 128.
-constexpr int kListThreads = 256, kListWarps = 8;
+constexpr int kListGroup = 8;               // most pairs per CTA
+constexpr int kWideListKeys = 8192;
 constexpr int kListSmem = 100 * 1024;       // the most dynamic shared memory a CTA takes: two fit on an SM
 
-__global__ void __launch_bounds__(kListThreads) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
+template <int kListWarps>
+__global__ void __launch_bounds__(32 * kListWarps) compact_lists_kernel(const int32_t* __restrict__ expiry, int* __restrict__ cidx,
                                                                      int* __restrict__ ccnt, int L, int npairs, int cap, int causal,
                                                                      int q_off, int32_t* __restrict__ status, int group, int ccap) {
     extern __shared__ int2 cand[];                       // group > 1: (key, expiry) of the keys some row of the group keeps
@@ -1195,23 +1197,23 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
 // Query tiles per CTA: two, or one whose key tiles are dealt out to the two softmax groups where that shortens the call. Both grids
 // are estimated in steps of a CTA (two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs; the pair's
 // steps in tile mode are longer where many keys expire per tile, i.e. in short sequences. Fitted to 64 shapes of 1 to 128 heads and
-// 183 to 15889 keys, each timed with both: the faster one, or within 4 %, everywhere. Forward, us, two tiles / one: 16 heads of 1000
-// keys 37 / 18, 8 heads of 500 23 / 12, 8 heads of 4096 (w = 2048) 76 / 45, a chunk of 1185 rows of 18445 keys, one head 82 / 53, but 64
+// 183 to 15889 keys, each timed with both, and then moved by 5 to 10 % towards two for the hand-over of references: forward, us, two
+// tiles / one: 16 heads of 1000 keys 37 / 19, 8 heads of 500 25 / 13, 8 heads of 4096 (w = 2048) 78 / 50, 172 rows of 26817 keys, 4 heads 109 / 71, but 64
 // heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568.
 // The two add in different orders. A chunk of 16 query tiles and more always takes two, so that a head's rows come out the same however
 // many heads share the call.
 int tc_fwd_tiles(const Prob& P) {
     if (P.fwd_split) return P.fwd_split;
-    constexpr double kOneSteps = 2.25, kTwoSteps = 3.0, kSms = 148.0;
+    constexpr double kOneSteps = 2.5, kTwoSteps = 3.0, kSms = 148.0;
     const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2;
     const double heads = (double)P.B * P.Hq;
     if (P.flags & DMA_FLAG_COMPACT_KV) {                     // lists of about the same length
         if (P.Lq < P.L && Trq >= 16) return 2;
         const double n = std::min((int64_t)P.w + (P.causal ? 256 : 0), (int64_t)P.L) / 128.0;
-        return std::ceil(heads * Trq / kSms) * (n / 2 + kTwoSteps) < std::ceil(heads * npairs / kSms) * (n + kTwoSteps) ? 1 : 2;
+        return 1.1 * std::ceil(heads * Trq / kSms) * (n / 2 + kTwoSteps) < std::ceil(heads * npairs / kSms) * (n + kTwoSteps) ? 1 : 2;
     }
     const double total = Trq * (Trq + 1) / 2.0;              // walks grow with the row: the last tile's is the longest
-    const double one = std::max(Trq / 2.0 + kOneSteps, heads * (total / 2 + Trq * kOneSteps) / kSms);
+    const double one = 1.05 * std::max(Trq / 2.0 + kOneSteps, heads * (total / 2 + Trq * kOneSteps) / kSms);
     const double two = (1.0 + 2.0 / Trq) * std::max(Trq + kTwoSteps, heads * (total / 2 + npairs * kTwoSteps) / kSms);
     return one < two ? 1 : 2;
 }
@@ -1251,12 +1253,17 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
         // one pair / this rule: 32 heads of 65536 keys 539 / 141, of 16384 keys 49 / 25 (a scalar two-pass scan per pair: 781, 69)
         const int cap = compact_cap(P);
         int group = 1;
-        while (group < kListWarps && P.causal && npairs >= 2 * group && (int64_t)P.B * P.Hq * ((npairs + 2 * group - 1) / (2 * group)) >= 148 &&
+        while (group < kListGroup && P.causal && npairs >= 2 * group && (int64_t)P.B * P.Hq * ((npairs + 2 * group - 1) / (2 * group)) >= 148 &&
                (size_t)(cap + 2 * group * 256) * sizeof(int2) <= (size_t)kListSmem) group *= 2;
         const size_t smem = group > 1 ? (size_t)(cap + group * 256) * sizeof(int2) : 0;
+        // one pair per CTA: a long head takes twice the warps (us, forward, 8 / 16 / 32 warps: 500 rows of 20000 keys, 8 heads 57.0 / 53.5 / 56.2,
+        // 2048 of 16384, 32 heads 119.9 / 118.1 / 127.1, but 16 heads of 4096 73.8 / 74.3 / 79.0)
+        const bool wide = group == 1 && P.L >= kWideListKeys;
+        auto lists = wide ? compact_lists_kernel<2 * kListGroup> : compact_lists_kernel<kListGroup>;
+        const int threads = wide ? 64 * kListGroup : 32 * kListGroup;
         // (the limit is state of the function, which other threads' calls share: always the same value)
-        if (smem && cudaFuncSetAttribute(compact_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kListSmem) != cudaSuccess) return DMA_ERR_CUDA;
-        if ((rc = launch_overlapped(compact_lists_kernel, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(kListThreads), smem, st, 1,
+        if (smem && cudaFuncSetAttribute(lists, cudaFuncAttributeMaxDynamicSharedMemorySize, kListSmem) != cudaSuccess) return DMA_ERR_CUDA;
+        if ((rc = launch_overlapped(lists, dim3((unsigned)(P.B * P.Hq * ((npairs + group - 1) / group))), dim3(threads), smem, st, 1,
                                     expiry, cidx, ccnt, P.L, npairs, cap, P.causal, P.q_off, (int32_t*)ws, group, cap + group * 256)))
             return rc;                 // the forward kernel must not run on lists that nobody wrote
         fp.cidx = cidx; fp.ccnt = ccnt; fp.ccap = compact_cap(P);
