@@ -100,14 +100,18 @@ _SIGNATURES = {
     "dma_decode_state_init": "Pvlvvzv", "dma_decode_step": "Pvvvvlvvvvzv", "dma_step_host": "Pivvvvvvvvvvvvvzv",
     "dma_read_status": "vv", "dma_selftest_wait_timeout": "vzv"}
 _KINDS = {"P": ctypes.POINTER(dma_problem_t), "v": ctypes.c_void_p, "i": ctypes.c_int32, "l": ctypes.c_int64, "z": ctypes.c_size_t}
-_typed = {}
+_typed = {}                  # name -> function object with typed parameters
+_typed_lib = None            # a handle of its own: the function objects of lib() stay untyped
 
 
 def _typed_fn(name):
+    global _typed_lib
     f = _typed.get(name)
     if f is None:
-        lib()                                  # (raises where the library is missing)
-        f = ctypes.CDLL(LIB_PATH)[name]        # a function object of its own: those of lib() stay untyped
+        if _typed_lib is None:
+            lib()                              # (raises where the library is missing)
+            _typed_lib = ctypes.CDLL(LIB_PATH)
+        f = _typed_lib[name]
         f.argtypes = [_KINDS[k] for k in _SIGNATURES[name]]
         _typed[name] = f
     return f
