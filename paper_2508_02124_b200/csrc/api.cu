@@ -65,7 +65,7 @@ int resolve(const dma_problem_t* p, Prob* o) {
     o->B = p->B; o->Hq = p->Hq; o->Hkv = p->Hkv; o->L = p->L; o->d = p->d; o->G = p->Hq / p->Hkv;
     o->w = p->w < p->L ? p->w : p->L;
     o->w_cap = p->w;
-    o->Lq = p->L; o->q_off = 0; o->fwd_split = 0; o->bwd_split = 0; o->chose_compact = false;
+    o->Lq = p->L; o->q_off = 0; o->bwd_split = 0; o->chose_compact = false;
     o->dtype = p->dtype; o->flags = p->flags; o->causal = p->causal;
     o->bm = p->tile_m ? p->tile_m : 128;
     o->bn = p->tile_n ? p->tile_n : 128;
@@ -121,23 +121,6 @@ static int device_ok() {
     if (cudaGetDevice(&dev) != cudaSuccess) return DMA_ERR_CUDA;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return DMA_ERR_CUDA;
     return major == 10 ? DMA_OK : DMA_ERR_CUDA;
-}
-
-int attn_fwd_part(const dma_problem_t* p, int tiles, const void* Q, const void* K, const void* V, const float* bias, const int32_t* expiry,
-                  const uint32_t* bitmap, void* O, float* lse, void* ws, size_t ws_bytes, cudaStream_t st) {
-    Prob P;
-    int rc = resolve(p, &P);
-    if (rc) return rc;
-    P.fwd_split = tiles;
-    if (!Q || !K || !V || !bias || !expiry || !bitmap || !O || !lse) return DMA_ERR_NULL;
-    if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(bias) || !aligned16(expiry) ||
-        !aligned16(lse))
-        return DMA_ERR_ALIGN;
-    if ((P.flags & DMA_FLAG_COMPACT_KV) && !use_tensor_cores(P)) return DMA_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < fwd_ws_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
-    if ((rc = device_ok())) return rc;
-    // (the stage's first kernel clears the workspace header)
-    return fwd_any(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, st);
 }
 
 int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* K, const void* V, const void* O, const void* dO,
@@ -322,7 +305,18 @@ int dma_decode_step(const dma_problem_t* p, const void* q, const void* K, const 
 int dma_attn_fwd(const dma_problem_t* p, const void* Q, const void* K, const void* V, const float* bias,
                  const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, size_t ws_bytes,
                  void* cuda_stream) {
-    return dma::attn_fwd_part(p, 0, Q, K, V, bias, expiry, bitmap, O, lse, ws, ws_bytes, (cudaStream_t)cuda_stream);
+    Prob P;
+    int rc = resolve(p, &P);
+    if (rc) return rc;
+    if (!Q || !K || !V || !bias || !expiry || !bitmap || !O || !lse) return DMA_ERR_NULL;
+    if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(bias) || !aligned16(expiry) ||
+        !aligned16(lse))
+        return DMA_ERR_ALIGN;
+    if ((P.flags & DMA_FLAG_COMPACT_KV) && !use_tensor_cores(P)) return DMA_ERR_UNSUPPORTED;
+    if (!ws || ws_bytes < fwd_ws_any(P) || !aligned16(ws)) return DMA_ERR_WORKSPACE;
+    if ((rc = device_ok())) return rc;
+    // (the stage's first kernel clears the workspace header)
+    return fwd_any(P, Q, K, V, bias, expiry, bitmap, O, lse, ws, (cudaStream_t)cuda_stream);
 }
 
 int dma_attn_fwd_chunk(const dma_problem_t* p, int32_t q_begin, int32_t q_len, const void* Q, const void* K, const void* V,

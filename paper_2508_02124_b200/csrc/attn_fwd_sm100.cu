@@ -68,7 +68,6 @@ struct SharedStorage {
     uint32_t tmem_base;
     int n_iters;
     int abort_flag;
-    float ref[2][128];                         // kSplit: each row's reference maximum after the group's last entry
     // One query tile per CTA (kSplit): a group's flags, `fast`, and what its per-element test reads are in two slots that its entries take
     // in turn. Token-compacted: group 1's len and jidx. Tile mode: a byte per column, expiry[j] relative to the query tile's first row, cut
     // to [0, 128]: row r of the tile keeps the key iff r is below it (and, in the diagonal tile, not below the column).
@@ -121,8 +120,9 @@ constexpr int kWarpProducer = 0, kWarpIssuer = 1, kWarpStager0 = 2, kWarpStager1
 // kBlockSkip: MMA-block skipping inside executed tiles (DMA_FLAG_BLOCK_SKIP), a separate instantiation so that the
 // default kernel carries none of its code (the kernel is sensitive to the size of its service warps' loops).
 // kSplit: the CTA owns ONE query tile and its two softmax groups take the key tiles (slices) in turn, entry t of the schedule by
-// group t & 1; group 1 hands its O, row max and row sum over in shared memory at the end. A CTA's walk is then half as long, for grids
-// that leave SMs idle (tc_fwd_tiles).
+// group t & 1. A CTA's walk is then half as long, for grids that leave SMs idle (fwd_tiles). Both groups' products go to one
+// accumulator in the order of the schedule, and the row references and row sums are handed from entry to entry: O and lse have the bits
+// of the kernel with two query tiles, so that they do not depend on how many heads share the call.
 template <bool kCompact, bool kBlockSkip, int kD, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -159,7 +159,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             mbar_init(&S.p_ready[w], 4);
             mbar_init(&S.o_done[w], 1);
         }
-        mbar_init(&S.merge, 4);
+        mbar_init(&S.merge, kSplit ? 8 : 4);      // (unused with two query tiles; with another count than its neighbours' that instance was 1.5 % slower)
         for (int q = 0; q < 8; ++q) mbar_init(&S.ref_set[q >> 2][q & 3], 1);
         S.abort_flag = 0;
         S.n_iters = 0;
@@ -214,9 +214,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const int i = P.q_off + il;                         // its position in the sequence
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + lane_base + w * 128;
-        const uint32_t tO = tmem + lane_base + 256 + w * 128;
+        const uint32_t tO = tmem + lane_base + 256 + (kSplit ? 0 : w * 128);
         const uint32_t rows4 = (uint32_t)r * 0x01010101u;
         float m_ref = -INFINITY, r_ref = 0.0f, l = 0.0f;
+        float f_last = 1.0f, s_last = 0.0f;                 // kSplit: the group's last entry, its factor and its row sum, not yet handed over
+        // kSplit, in the second query tile's buffer: per group and row the reference maximum after the group's last entry and the row sum up
+        // to its entry before that one; in the end f_last and s_last
+        float2 (*handed)[128] = reinterpret_cast<float2 (*)[128]>(S.q[1]);
         int n_used = 0;
         bool ok = true;
         for (int it = 0; it < n_iters && ok; ++it) {
@@ -309,37 +313,45 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
             float m_new = fmaxf(m_ref, mx);
             bool grown = false;
+            float before = -INFINITY;
             if constexpr (kSplit) {
-                // Both groups follow the one sequence of references that a walk over all entries takes: entry it - 1's comes from the other group
-                // (the warp with the same rows), and this entry's is published before the exponentials. P then has the same bits as
-                // with two query tiles per CTA, and O differs by the order of fp32 sums only. (With a reference of its own per group P
-                // was rounded at other places: O as accurate, but 1.7e-3 away, and dA, a sum that cancels, by up to 1e-2.)
-                float before = -INFINITY;
+                // Entry it - 1's reference comes from the other group (the warp with the same rows), this entry's is published before the
+                // exponentials. (With a reference of its own per group P was rounded at other places: O 1.7e-3 away, dA, a sum that
+                // cancels, by up to 1e-2.) The row sum travels with it two entries late, when its terms are known.
+                float2 from = make_float2(-INFINITY, 0.0f);                 // (row sum up to entry it - 3)
                 if (it > 0) {
                     ok = mbar_wait_warp(&S.ref_set[w ^ 1][warp & 3], ((it - 1) >> 1) & 1, abort_flag);
                     if (!ok) break;
-                    before = S.ref[w ^ 1][r];
+                    from = handed[w ^ 1][r];
                 }
+                before = from.x;
                 m_new = fmaxf(before, mx);
-                if (it > 0 && !__any_sync(0xffffffffu, m_new > before + P.rescale_gap)) m_new = before;
-                S.ref[w][r] = m_new;               // (the other group has read the value before it published its own last one)
+                grown = it > 0 && __any_sync(0xffffffffu, m_new > before + P.rescale_gap);
+                if (it > 0 && !grown) m_new = before;
+                // (the other group has read the values before it published its own last ones)
+                handed[w][r] = make_float2(m_new, __fadd_rn(__fmul_rn(from.y, f_last), s_last));
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.ref_set[w][warp & 3]);
-                grown = __any_sync(0xffffffffu, m_new != m_ref);
+                f_last = 1.0f;
             }
             auto stab_resid = [&](float m) {           // m c - stab(m); 0 for m = -inf
                 const float mm = (m == -INFINITY) ? 0.0f : m;
                 const float Mm = mm * P.scale_log2;
                 return fabsf(Mm) < kSmallStab ? fmaf(mm, P.scale_log2, -Mm) : 0.0f;
             };
-            if (n_used == 0) {
+            if (kSplit ? !grown : n_used == 0) {
                 m_ref = m_new;
-                r_ref = stab_resid(m_ref);
-            } else if (kSplit ? grown : __any_sync(0xffffffffu, m_new > m_ref + P.rescale_gap)) {
-                // O_w *= 2^(stab(m_ref) - stab(m_new)): the previous P V product must have landed first
-                ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
+                if constexpr (!kSplit) r_ref = stab_resid(m_ref);
+            } else if (kSplit || __any_sync(0xffffffffu, m_new > m_ref + P.rescale_gap)) {
+                // O_w *= 2^(stab(m_ref) - stab(m_new)): the previous P V product must have landed first (kSplit: that of entry it - 1, after which
+                // nothing is added until this entry's P is released)
+                ok = kSplit ? mbar_wait_warp(&S.o_done[w ^ 1], ((it - 1) >> 1) & 1, abort_flag) : mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
+                if constexpr (kSplit) {
+                    m_ref = before;
+                    r_ref = stab_resid(before);
+                }
                 const float r_new = stab_resid(m_new);
                 const float f = (m_new == -INFINITY) ? 1.0f : (m_ref == -INFINITY) ? 0.0f : ex2(fmaf(m_ref - m_new, P.scale_log2, r_new - r_ref));
 #pragma unroll
@@ -352,7 +364,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     tmem_st32(tO + c * 32, o);
                 }
                 tc_wait_st();
-                l *= f;
+                if constexpr (kSplit) f_last = f;
+                else l *= f;
                 m_ref = m_new;
                 r_ref = r_new;
             }
@@ -362,7 +375,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // fp32 range stay safe). r_ref = m_ref c - stab(m_ref) travels with m_ref.
             const float m_use = (m_ref == -INFINITY) ? 0.0f : m_ref;
             const float M = m_use * P.scale_log2, nM = -M;
-            const float resid = r_ref;
+            const float resid = kSplit ? stab_resid(m_ref) : r_ref;
             const bool small = __all_sync(0xffffffffu, fabsf(M) < kSmallStab);
             float sa[4] = {0.f, 0.f, 0.f, 0.f};
             if (small) {
@@ -403,63 +416,45 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     }
                 }
             }
-            l += (sa[0] + sa[1]) + (sa[2] + sa[3]);
+            if constexpr (kSplit) s_last = (sa[0] + sa[1]) + (sa[2] + sa[3]);
+            else l += (sa[0] + sa[1]) + (sa[2] + sa[3]);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.p_ready[w]);      // one arrival per warp: 128 serialised arrivals cost ~400 cycles
             ++n_used;
         }
-        // epilogue: O_w / l -> bf16 rows, log-sum-exp in natural log
-        const bool exists = w == 0 || has1;
-        if (ok && (exists || kSplit) && n_used > 0) ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
-        // kSplit: group 1 leaves its row max, row sum and O (chunks of four channels, rows innermost) in what only it has used: the second
-        // query tile's buffer and stage 1 of K and V, which no load or product touches once its last P V is done
-        float* other = reinterpret_cast<float*>(S.q[1]);
-        auto other_o = [&](int c) { return reinterpret_cast<float4*>(c < 64 ? S.k[1] : S.v[1]) + ((c & 63) >> 2) * 128 + r; };
-        float f0 = 1.0f, f1 = 0.0f;
+        // epilogue: O_w / l -> bf16 rows, log-sum-exp in natural log. kSplit: each group writes half of the channels
+        const bool exists = w == 0 || has1 || kSplit;
         if constexpr (kSplit) {
-            if (ok && w == 1) {
-                tc_fence_after();
-                other[r] = m_ref;
-                other[128 + r] = r_ref;
-                other[256 + r] = l;
-                if (n_used > 0) {
-#pragma unroll
-                    for (int c = 0; c < kD / 32; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(tO + c * 32, o);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int u = 0; u < 32; u += 4)
-                            *other_o(c * 32 + u) = make_float4(__uint_as_float(o[u]), __uint_as_float(o[u + 1]), __uint_as_float(o[u + 2]), __uint_as_float(o[u + 3]));
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&S.merge);
+            handed[2 + w][r] = make_float2(f_last, s_last);
+            __syncwarp();
+            if (ok && lane == 0) mbar_arrive(&S.merge);
+            if (ok) ok = mbar_wait_warp(&S.merge, 0, abort_flag);
+            const int a = (n_iters - 1) & 1;                     // the group of the last entry
+            if (ok && n_iters > 0) {
+                m_ref = handed[a][r].x;
+                l = handed[a][r].y;
+                const float m_use = m_ref == -INFINITY ? 0.0f : m_ref, M = m_use * P.scale_log2;
+                r_ref = fabsf(M) < kSmallStab ? fmaf(m_use, P.scale_log2, -M) : 0.0f;
+                if (n_iters > 1) l = __fadd_rn(__fmul_rn(l, handed[2 + (a ^ 1)][r].x), handed[2 + (a ^ 1)][r].y);
+                l = __fadd_rn(__fmul_rn(l, handed[2 + a][r].x), handed[2 + a][r].y);
             }
-            if (ok && w == 0) {
-                ok = mbar_wait_warp(&S.merge, 0, abort_flag);
-                if (ok) {
-                    const float m1 = other[r], r1 = other[128 + r], l1 = other[256 + r];
-                    const bool mine = m_ref >= m1;
-                    const float m = mine ? m_ref : m1, rr = mine ? r_ref : r1;
-                    f0 = m_ref == -INFINITY ? 0.0f : ex2(fmaf(m_ref - m, P.scale_log2, rr - r_ref));
-                    f1 = m1 == -INFINITY ? 0.0f : ex2(fmaf(m1 - m, P.scale_log2, rr - r1));
-                    l = l * f0 + l1 * f1;
-                    m_ref = m;
-                    r_ref = rr;
-                }
-            }
+            // (the entry before the last one first: a wait for a phase that is two ahead would not wait)
+            if (ok && n_iters > 1) ok = mbar_wait_warp(&S.o_done[a ^ 1], ((n_iters - 2) >> 1) & 1, abort_flag);
+            if (ok && n_iters > 0) ok = mbar_wait_warp(&S.o_done[a], ((n_iters - 1) >> 1) & 1, abort_flag);
+        } else if (ok && exists && n_used > 0) {
+            ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
         }
         if (ok && exists) {
             tc_fence_after();
             const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-            const bool second = kSplit && n_iters > 1;       // (group 1 had an entry)
+            if constexpr (kSplit) n_used = n_iters;
             __nv_bfloat16* orow = P.O + b * P.os_b + (int64_t)il * P.os_l + h * P.os_h;
             constexpr int kUnroll = kCompact && !kSplit ? 1 : kD / 32;     // (rolled: 8 bytes of spills less, 32 heads of 16384 keys 690 -> 666 us; unrolled where calls are short, 9.4 / 10.0 us)
 #pragma unroll kUnroll
             for (int c = 0; c < kD / 32; ++c) {
+                if (kSplit && c / (kD / 64) != w) continue;          // (each group writes half of the channels)
                 uint32_t o[32];
                 if (n_used > 0) {
                     tmem_ld32(tO + c * 32, o);
@@ -467,16 +462,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 } else {
 #pragma unroll
                     for (int u = 0; u < 32; ++u) o[u] = 0;
-                }
-                if (second) {
-#pragma unroll
-                    for (int u = 0; u < 32; u += 4) {
-                        const float4 y = *other_o(c * 32 + u);
-                        o[u] = __float_as_uint(__uint_as_float(o[u]) * f0 + y.x * f1);
-                        o[u + 1] = __float_as_uint(__uint_as_float(o[u + 1]) * f0 + y.y * f1);
-                        o[u + 2] = __float_as_uint(__uint_as_float(o[u + 2]) * f0 + y.z * f1);
-                        o[u + 3] = __float_as_uint(__uint_as_float(o[u + 3]) * f0 + y.w * f1);
-                    }
                 }
                 if (il < P.Lq) {
 #pragma unroll
@@ -490,7 +475,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     }
                 }
             }
-            if (il < P.Lq) P.lse[(size_t)bh * P.Lq + il] = l > 0.0f ? 0.6931471805599453f * ((m_ref * P.scale_log2 - r_ref) + log2f(l)) : -INFINITY;
+            if (il < P.Lq && (!kSplit || w == 0)) P.lse[(size_t)bh * P.Lq + il] = l > 0.0f ? 0.6931471805599453f * ((m_ref * P.scale_log2 - r_ref) + log2f(l)) : -INFINITY;
         }
     } else {
         setmaxnreg_dec<88>();   // 4 warps x 80 registers released = 8 warps x 40 acquired above
@@ -872,7 +857,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 for (int it = 0; it < n_iters_u && ok; ++it) {
                     const int w = it & 1, ph = (it >> 1) & 1;
                     const uint64_t dv = dV0 + (uint64_t)(w * (kTileBytes >> 4));
-                    const uint32_t d_tmem = tmem_u + 256 + w * 128, a_tmem = tmem_u + w * 128;
+                    const uint32_t d_tmem = tmem_u + 256, a_tmem = tmem_u + w * 128;
                     ok = mbar_wait_warp(&S.v_full[w], ph, abort_flag);
                     if constexpr (kCompact) fence_proxy_async();
                     if (ok) ok = mbar_wait_warp(&S.p_half[w], ph, abort_flag);
@@ -881,7 +866,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
-                            mma_ts(d_tmem, a_tmem + kk * 8, dv + (uint64_t)((kk * 2048) >> 4), idesc_pv, kk > 0 || it > 1 ? 1u : 0u);
+                            mma_ts(d_tmem, a_tmem + kk * 8, dv + (uint64_t)((kk * 2048) >> 4), idesc_pv, kk > 0 || it > 0 ? 1u : 0u);
                     }
                     __syncwarp();
                     ok = mbar_wait_warp(&S.p_ready[w], ph, abort_flag);
@@ -1197,18 +1182,14 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
 // Query tiles per CTA: two, or one whose key tiles are dealt out to the two softmax groups where that shortens the call. Both grids
 // are estimated in steps of a CTA (two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs; the pair's
 // steps in tile mode are longer where many keys expire per tile, i.e. in short sequences. Fitted to 64 shapes of 1 to 128 heads and
-// 183 to 15889 keys, each timed with both, and then moved by 5 to 10 % towards two for the hand-over of references: forward, us, two
+// 183 to 15889 keys, each timed with both before rows had their references from both groups, and then moved by 5 to 10 % towards two: forward, us, two
 // tiles / one: 16 heads of 1000 keys 37 / 19, 8 heads of 500 25 / 13, 8 heads of 4096 (w = 2048) 78 / 50, 172 rows of 26817 keys, 4 heads 109 / 71, but 64
-// heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568.
-// The two add in different orders. A chunk of 16 query tiles and more always takes two, so that a head's rows come out the same however
-// many heads share the call.
-int tc_fwd_tiles(const Prob& P) {
-    if (P.fwd_split) return P.fwd_split;
+// heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568. The results are the same bits.
+static int fwd_tiles(const Prob& P) {
     constexpr double kOneSteps = 2.5, kTwoSteps = 3.0, kSms = 148.0;
     const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2;
     const double heads = (double)P.B * P.Hq;
     if (P.flags & DMA_FLAG_COMPACT_KV) {                     // lists of about the same length
-        if (P.Lq < P.L && Trq >= 16) return 2;
         const double n = std::min((int64_t)P.w + (P.causal ? 256 : 0), (int64_t)P.L) / 128.0;
         return 1.1 * std::ceil(heads * Trq / kSms) * (n / 2 + kTwoSteps) < std::ceil(heads * npairs / kSms) * (n + kTwoSteps) ? 1 : 2;
     }
@@ -1223,7 +1204,7 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
     const bool compact = (P.flags & DMA_FLAG_COMPACT_KV) != 0;
     if (P.Tc > kMaxSched) return DMA_ERR_UNSUPPORTED;
     const bool block_skip = (P.flags & DMA_FLAG_BLOCK_SKIP) != 0;
-    const bool split = tc_fwd_tiles(P) == 1;
+    const bool split = fwd_tiles(P) == 1;
     auto pick = [&](auto d_tag) {
         constexpr int kD = decltype(d_tag)::value;
         if (split) return compact ? fwd_kernel<true, false, kD, true> : fwd_kernel<false, false, kD, true>;

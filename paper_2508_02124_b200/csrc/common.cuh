@@ -20,7 +20,6 @@ struct Prob {
     bool chose_compact;    // token-compacted execution is the library's choice: a shorter sequence may walk tiles
     int causal;            // 1: key j visible to rows i >= j; 0: to every row (the key's first row is 0 instead of j)
     int bm, bn, Tr, Tc, Wd;   // bitmap tile sizes, tile counts, uint32 words per bitmap row
-    int fwd_split;            // query tiles per CTA of the tensor-core forward: 1 or 2 (0: tc_fwd_tiles chooses)
     int bwd_split;            // CTAs that share a KV head in the tile-mode backward (0: tc_bwd_splits chooses)
     int Lq, q_off;            // forward over a chunk of query rows: Q, O, lse hold the rows q_off .. q_off + Lq - 1 (Lq = L, q_off = 0: all)
     float scale;
@@ -61,10 +60,6 @@ int launch_simt_bwd(const Prob& P, const void* Q, const void* K, const void* V, 
 size_t tc_fwd_ws_bytes(const Prob& P);
 int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,
                   const int32_t* expiry, const uint32_t* bitmap, void* O, float* lse, void* ws, cudaStream_t st);
-int tc_fwd_tiles(const Prob& P);
-// dma_attn_fwd on a part of a problem: with the query tiles per CTA of the whole one, so that the parts' results are the whole's
-int attn_fwd_part(const dma_problem_t* p, int tiles, const void* Q, const void* K, const void* V, const float* bias, const int32_t* expiry,
-                  const uint32_t* bitmap, void* O, float* lse, void* ws, size_t ws_bytes, cudaStream_t st);
 size_t tc_bwd_need(const Prob& P);         // what the call uses
 size_t tc_bwd_ws_bytes(const Prob& P);     // what is asked for: at least the need of every shorter sequence and smaller batch
 int tc_bwd_splits(const Prob& P);

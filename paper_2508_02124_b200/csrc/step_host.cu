@@ -186,7 +186,7 @@ int dma_step_host(const dma_problem_t* p, int backward, const void* hQ, const vo
     sub.B = GB; sub.Hq = nqh; sub.Hkv = nkh;
     Prob whole;
     if ((rc = resolve(p, &whole))) return cleanup(rc);
-    const int tiles = tc_fwd_tiles(whole), split = tc_bwd_splits(whole);   // (of the whole problem: the groups' results are then those of one call on it)
+    const int split = tc_bwd_splits(whole);          // (of the whole problem: the groups' gradients are then those of one call on it)
     const int64_t qs[3] = {(int64_t)L * p->Hq * d, (int64_t)p->Hq * d, d}, ks[3] = {(int64_t)L * p->Hkv * d, (int64_t)p->Hkv * d, d};
     for (int i = 0; i < 3; ++i) { sub.q_stride[i] = sub.o_stride[i] = qs[i]; sub.k_stride[i] = sub.v_stride[i] = ks[i]; }
     const size_t f_ws = Lo.f_ws - (size_t)NG * kWsHeaderBytes, b_ws = Lo.b_ws - (size_t)NG * kWsHeaderBytes;
@@ -203,7 +203,7 @@ int dma_step_host(const dma_problem_t* p, int backward, const void* hQ, const vo
         if ((rc = dma_mask_build(&sub, a + Lo.V + G.k * esz, (float*)(a + Lo.W) + G.hq0 * w_per_head, (float*)(a + Lo.A) + G.hq0, bias,
                                  expiry, bitmap, a + Lo.ws_mask, Lo.m_ws, st))) return cleanup(rc);
         if (!wait(st, e[kKQ])) return cleanup(DMA_ERR_CUDA);
-        if ((rc = attn_fwd_part(&sub, tiles, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, bias, expiry, bitmap,
+        if ((rc = dma_attn_fwd(&sub, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, bias, expiry, bitmap,
                                a + Lo.O + G.q * esz, lse, wsf, f_ws, st))) return cleanup(rc);
         const cudaMemcpyKind out = cudaMemcpyDeviceToHost;
         ok = rec(e[kO], st) && wait(s_out, e[kO]) &&
