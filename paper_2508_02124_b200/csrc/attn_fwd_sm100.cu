@@ -1185,7 +1185,9 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
 // 183 to 15889 keys, each timed with both before rows had their references from both groups, and then moved by 5 to 10 % towards two: forward, us, two
 // tiles / one: 16 heads of 1000 keys 37 / 19, 8 heads of 500 25 / 13, 8 heads of 4096 (w = 2048) 78 / 50, 172 rows of 26817 keys, 4 heads 109 / 71, but 64
 // heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568. The results are the same bits.
+// DMA_FLAG_BLOCK_SKIP is for two tiles: its marks are read where one group walks every entry.
 static int fwd_tiles(const Prob& P) {
+    if (P.flags & DMA_FLAG_BLOCK_SKIP) return 2;
     constexpr double kOneSteps = 2.5, kTwoSteps = 3.0, kSms = 148.0;
     const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2;
     const double heads = (double)P.B * P.Hq;

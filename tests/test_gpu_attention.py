@@ -244,6 +244,30 @@ def test_mma_block_skipping_does_not_change_the_result():
             assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1]), (case.name, path)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("path", [dma.DMA_FLAG_TILE_PATH, dma.DMA_FLAG_COMPACT_KV])
+def test_mma_block_skipping_leaves_dead_blocks_out(path, d):
+    """Infinite value rows of 16 keys that the last query tile's rows no longer keep, one MMA block of an active tile and of the gathered list:
+    a product over that block would be 0 x inf."""
+    dev = torch.device("cuda:0")
+    case = wl.small(C2, B=1, Hq=1, Hkv=1, L=512, w=512, d=d, backward=False, name="block-skip infinite")
+    inp = wl.make_inputs(case)
+    e = torch.full((1, 1, 512), 512, dtype=torch.int32)
+    e[0, 0, :16], e[0, 0, 16] = 384, 17                       # (240 keys are kept by all rows of the second pair of tiles: the 16 are a block of its list)
+    bmp = torch.from_numpy(oracle.bitmap_from_expiry(e.numpy()).view(np.int32)).to(dev)
+    bias = torch.zeros(1, 1, 512)
+    V = inp["V"].clone()
+    V[:, :16] = float("inf")
+    p = problem_of(case, flags=path | dma.DMA_FLAG_BLOCK_SKIP)
+    ws = torch.empty(dma.dma_query_workspace(p)[1], dtype=torch.uint8, device=dev)
+    O, lse = dma.dma_attn_fwd(p, inp["Q"].to(dev), inp["K"].to(dev), V.to(dev), bias.to(dev), e.to(dev), bmp, ws=ws)
+    assert dma.dma_read_status(ws) == 0
+    rows = np.arange(384, 512, dtype=np.int32)
+    Or, lr = oracle.forward(*(f64(inp[k]) for k in ("Q", "K", "V")), f64(bias), expiry=e.numpy(), rows=rows)
+    assert_close(O[:, 384:], Or, case.dtype, "O")
+    assert_close(lse[:, :, 384:], lr, case.dtype, "lse", lse=True)
+
+
 def test_largest_supported_lengths():
     """The longest sequences the tensor-core kernels take: L = 131072 (1024 key tiles, the forward schedule's capacity; with
     a group of 4 query heads per KV head also the capacity of the backward's step list), forward and backward, tile path and
