@@ -198,8 +198,9 @@ int dma_attn_fwd_chunk(const dma_problem_t* p, int32_t q_begin, int32_t q_len, c
  * dK and dV are summed over the Hq/Hkv query heads that share a KV head; dM is per query head.
  * dQ is accumulated with floating-point atomics on the tensor-core paths: its rounding depends on execution order. dK, dV
  * (and O, lse of the forward) are reproducible bit for bit from run to run on the tile path, every gradient on the CUDA-core
- * path; with token-compacted execution dK and dV are accumulated with atomics too, and so is dM where few heads let several CTAs
- * share a key tile's rows: they vary in the last bits unless DMA_FLAG_DETERMINISTIC is set. */
+ * path; with token-compacted execution dM is, and dK and dV are with one or two query heads per KV head. With more, the heads' sums meet
+ * in atomics too: dK and dV vary in the last bits unless DMA_FLAG_DETERMINISTIC is set. How sums are split is a function of the
+ * descriptor, B and Hq included: in another batch a head's dK, dV and dM may differ in the last bits (its O and lse do not). */
 int dma_attn_bwd(const dma_problem_t* p, const void* Q, const void* K, const void* V,
                  const void* O, const void* dO, const float* lse,
                  const float* bias, const int32_t* expiry, const uint32_t* bitmap,

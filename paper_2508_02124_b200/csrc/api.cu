@@ -65,7 +65,7 @@ int resolve(const dma_problem_t* p, Prob* o) {
     o->B = p->B; o->Hq = p->Hq; o->Hkv = p->Hkv; o->L = p->L; o->d = p->d; o->G = p->Hq / p->Hkv;
     o->w = p->w < p->L ? p->w : p->L;
     o->w_cap = p->w;
-    o->Lq = p->L; o->q_off = 0; o->bwd_split = 0; o->chose_compact = false;
+    o->Lq = p->L; o->q_off = 0; o->bwd_split = 0; o->bwd_heads = 0; o->chose_compact = false;
     o->dtype = p->dtype; o->flags = p->flags; o->causal = p->causal;
     o->bm = p->tile_m ? p->tile_m : 128;
     o->bn = p->tile_n ? p->tile_n : 128;
@@ -123,13 +123,14 @@ static int device_ok() {
     return major == 10 ? DMA_OK : DMA_ERR_CUDA;
 }
 
-int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* K, const void* V, const void* O, const void* dO,
+int attn_bwd_part(const dma_problem_t* p, int split, int heads, const void* Q, const void* K, const void* V, const void* O, const void* dO,
                   const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ, void* dK, void* dV,
                   float* dM, void* ws, size_t ws_bytes, cudaStream_t st) {
     Prob P;
     int rc = resolve(p, &P);
     if (rc) return rc;
     P.bwd_split = split;
+    P.bwd_heads = heads;
     if (!Q || !K || !V || !O || !dO || !lse || !bias || !expiry || !bitmap || !dQ || !dK || !dV || !dM) return DMA_ERR_NULL;
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(dO) || !aligned16(dQ) ||
         !aligned16(dK) || !aligned16(dV) || !aligned16(dM) || !aligned16(lse))
@@ -347,7 +348,7 @@ int dma_attn_fwd_chunk(const dma_problem_t* p, int32_t q_begin, int32_t q_len, c
 int dma_attn_bwd(const dma_problem_t* p, const void* Q, const void* K, const void* V, const void* O, const void* dO,
                  const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ, void* dK,
                  void* dV, float* dM, void* ws, size_t ws_bytes, void* cuda_stream) {
-    return dma::attn_bwd_part(p, 0, Q, K, V, O, dO, lse, bias, expiry, bitmap, dQ, dK, dV, dM, ws, ws_bytes, (cudaStream_t)cuda_stream);
+    return dma::attn_bwd_part(p, 0, 0, Q, K, V, O, dO, lse, bias, expiry, bitmap, dQ, dK, dV, dM, ws, ws_bytes, (cudaStream_t)cuda_stream);
 }
 
 int dma_read_status(const void* ws, void* cuda_stream) {

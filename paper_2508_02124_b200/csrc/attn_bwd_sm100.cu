@@ -65,6 +65,20 @@ struct SharedStorage {
     uint32_t tmem_base;
     int n_steps;
     int abort_flag;
+    int part, block;                                 // token-compacted mode: the walk's part, and where its dK and dV go (WalkBlocks; -1: to the accumulators)
+    int cut;                                         // what the first part notes for the last kernel: WalkBlocks::where but for the row (0: nothing)
+};
+
+// Token-compacted mode: the sums of walks that are cut into parts. What a key gets must not depend on which part ends first where it did
+// not depend on order without cuts: dM, and dK and dV with one or two query heads per KV head (a sum of two addends onto a zero has one
+// value). The first `direct` parts of a walk add their dK and dV to the accumulators, two with one query head, one with two, all of them with
+// more, whose sums vary in any case. The others have a block each, `cap` of them per (batch, query head), and every part but the
+// first has a place for its dM; the last kernel adds these in the order of the parts.
+struct WalkBlocks {
+    float* kv;                  // [B, Hq, cap] x dK [128 keys][d] | dV [128][d], unscaled
+    float* m;                   // [B, Hq, key tile, part - 1] x two halves of the query columns [2][128]
+    int* where;                 // [B, Hq, L], zeros before: row of the key in its tile | parts - 1 << 7 | first block << 10 | key tile << 19. NULL: no walk is cut
+    int cap, direct;
 };
 
 struct BwdParams {
@@ -88,7 +102,8 @@ struct BwdParams {
     // token-compacted mode: per (batch, query head) a permutation of the keys (padded with L to a multiple of 128) that
     // groups keys of similar lifetime; a CTA owns 128 consecutive entries of one query head's permutation
     const int* perm;
-    const int2* items;         // what each CTA does: [B, Hq, gridDim.y] (WorkItem)
+    const int2* items;         // what each CTA does: [B, Hq, gridDim.y]
+    WalkBlocks blocks;
     int causal;                // 0: key j is visible to every row (token-compacted mode only): its first row is 0 instead of j
     const __nv_bfloat16* Kg;    // K, V base pointers for the row gathers (ks_*, vs_* strides)
     const __nv_bfloat16* Vg;
@@ -103,8 +118,10 @@ struct BwdParams {
 
 
 // Token-compacted mode: one CTA's work, a key tile of the head's permutation and a part of its walk over the query tiles q0 .. q1:
-//   x = key tile | part << 16 | parts << 24 (-1: nothing)     y = q0 | q1 << 16
+//   x = key tile | part << 10 | parts << 13 | block << 17 (-1: nothing)     y = q0 | q1 << 16
+// block: of the parts that have none the first that has
 constexpr int kMostParts = 8;
+constexpr int kWalkBlocks = 296;               // blocks of a call in all (39 MB at d = 128): parts are about an SM's share of the work, 148 / 0.8 of them in all
 // 64-row steps of a walk (the sequence's last tile may have one only)
 __device__ __forceinline__ int walk_steps(int q0, int q1, int L) { return min(2 * (q1 - q0 + 1) - (q1 * 128 + 64 >= L ? 1 : 0), kMaxSteps); }
 
@@ -121,7 +138,7 @@ __device__ __forceinline__ uint4 split3(float x) {
 // key permutation instead of 128 consecutive keys of a KV head: keys that live equally long are kept by about the
 // same query rows, so the walk over query tiles [first key's tile, last expiry's tile] wastes little. K and V rows
 // are gathered once with 16-byte asynchronous copies; dK and dV are added to fp32 accumulators (the query heads of a
-// group meet there), dM is written directly.
+// group meet there), dM, the sum of two halves of the query columns, to zeros.
 // kLong: tile mode without a split of the query heads and without the overlapped launch, for problems that last long (bwd_long).
 template <bool kCompact, int kD, bool kLong = false>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -148,7 +165,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     const int at = (lin % per_group) / P.sched_group;
     const int2 item = kCompact ? P.items[(size_t)bx * gridDim.y + at] : make_int2(at, 0);
     if (kCompact && item.x < 0) return;                // no more items for this head
-    const int kt = kCompact ? item.x & 0xFFFF : at;
+    const int kt = kCompact ? item.x & 0x3FF : at;
     const int j0 = kt * 128;
     const int* my_perm = kCompact ? P.perm + ((size_t)bx * P.Tc + kt) * 128 : nullptr;
     volatile int* abort_flag = &S.abort_flag;
@@ -169,6 +186,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         mbar_init(&S.dq_free, 4);         // one arrival per drain warp
         S.abort_flag = 0;
         S.n_steps = 0;
+        if constexpr (kCompact) {
+            const int part = (item.x >> 10) & 7, later = ((item.x >> 13) & 0xF) - 1, block = item.x >> 17;
+            S.part = part;
+            S.block = part >= P.blocks.direct ? block : -1;
+            S.cut = part == 0 && later > 0 ? later << 7 | block << 10 | kt << 19 : 0;
+        }
         fence_barrier_init();
         if constexpr (!kCompact) {                     // K and V need no schedule: they are under way while it is built
             mbar_arrive_expect_tx(&S.kv_full, (kD == 128 ? 4 : 3) * (kKVBytes / 2));
@@ -211,7 +234,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // about together, so walking down from there they pass the same query rows (the Q / dO tiles they load, the
             // dQ accumulator rows they add to) at about the same time, while those are in L2; walking up, each from its
             // own first key, they passed a row at times spread over the life of the whole group.
-            const int g = hq_c % P.G, q0 = item.y & 0xFFFF, q1 = item.y >> 16, part = (item.x >> 16) & 0xFF, parts = item.x >> 24;
+            const int g = hq_c % P.G, q0 = item.y & 0xFFFF, q1 = item.y >> 16, part = (item.x >> 10) & 7, parts = (item.x >> 13) & 0xF;
             const int all = walk_steps(q0, q1, P.L), p0 = all * part / parts, p1 = all * (part + 1) / parts;
             n = p1 - p0;
             for (int qt = q0 + lane; qt <= q1; qt += 32) {
@@ -368,7 +391,10 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.pds_ready[pb]);
         }
-        if (cur_g >= 0 && j < P.L) atomicAdd(&P.dM[(size_t)(b * P.Hq + hk * P.G + cur_g) * P.L + j], dm2.x + dm2.y);
+        const int block = kCompact ? S.block : -1, part = kCompact ? S.part : 0, cut = kCompact ? S.cut : 0;
+        if (cut && hsel == 0 && j < P.L) P.blocks.where[(size_t)bx * P.L + j] = r | cut;
+        if (part) P.blocks.m[(((size_t)bx * P.Tc + kt) * (kMostParts - 1) + part - 1) * 256 + hsel * 128 + r] = dm2.x + dm2.y;
+        else if (cur_g >= 0 && j < P.L) atomicAdd(&P.dM[(size_t)(b * P.Hq + hk * P.G + cur_g) * P.L + j], dm2.x + dm2.y);
         // epilogue: dK (scaled) and dV rows to global memory; warps w and w+4 each write one half of the channels
         if (ok && n_steps > 0)
             ok = kDouble ? mbar_wait_warp(&S.pds_free[(n_steps - 1) & 1], ((n_steps - 1) >> 1) & 1, abort_flag)
@@ -406,7 +432,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     const int row = 4 * t + rsub;
                     x[t] = *reinterpret_cast<const float4*>(turn + row * 128 + ((ch ^ (row & 7)) << 4));
                 }
-                if (kCompact || nsplit > 1) {
+                if (kCompact && block >= 0) {
+                    float* dst = P.blocks.kv + (((size_t)bx * P.blocks.cap + block) * 2 + (isK ? 0 : 1)) * (128 * kD) + quad * (32 * kD) + col;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) *reinterpret_cast<float4*>(dst + (4 * t + rsub) * kD) = x[t];
+                } else if (kCompact || nsplit > 1) {
                     // Unscaled sums in fp32. Token-compacted: the group's query heads add into the same rows, or (slots) this (key, query head) pair is
                     // written by this CTA alone. Tile mode: this split's part, zeros where it had nothing to add.
                     float* acc = (isK ? P.dKacc : P.dVacc) + (size_t)(kCompact ? hq_c % P.G : sp) * (size_t)P.acc_slot +
@@ -639,6 +669,7 @@ struct PrepareParams {
     const int32_t* expiry;
     int* perm;
     int2* items;
+    int cap, direct;            // as WalkBlocks
     int Tc, causal, max_items;
     int walk;                   // steps of a walk that one CTA takes at most
     int longest_first;          // order of a head's items: by length, or as the permutation has them
@@ -654,14 +685,14 @@ constexpr int kPermThreads = 1024;
 // One CTA of 1024 threads per (batch, head). Per 1024-key chunk every warp ranks its 32 keys within their class
 // (match_any), the per-warp class counts are turned into start positions by 64 threads (one per class, a running sum over
 // the 32 warps and over the chunks), and every key is written to its place: stable in key order, three barriers per chunk.
-// Then the work items: a warp per key tile finds its walk, walks longer than P.walk steps are cut into equal parts, and with
-// P.longest_first the items are ranked by length, so that no long one starts late.
+// Then the work items: a warp per key tile finds its walk, walks longer than P.walk steps are cut into equal parts (as long as the head has
+// blocks left for them, in the permutation's order), and with P.longest_first the items are ranked by length, so that no long one starts late.
 struct PermShared {
     int hist[64];
     int offs[64];                 // next free position of each class
     int cnt[32][64];              // per warp and class: keys in this chunk, then their start position
-    int bounds[1024];             // walk of each key tile, q0 | q1 << 16, or -1
-    int parts[1024], len[1024];
+    int bounds[1024];             // walk of each key tile, q0 | q1 << 16 (meaningless where parts = 0)
+    int parts[1024], len[1024], first[1024];
 };
 __device__ __forceinline__ void lifetime_perm(const PrepareParams& P, PermShared& S) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bh = blockIdx.x, L = P.L, Tc = P.Tc;
@@ -721,12 +752,33 @@ __device__ __forceinline__ void lifetime_perm(const PrepareParams& P, PermShared
         }
     }
     __syncthreads();
+    if (P.max_items > Tc) {                                 // walks are cut
+        const int later = tid < Tc ? max(S.parts[tid] - P.direct, 0) : 0;
+        int to = later;                                     // blocks up to this tile's, in the permutation's order
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, to, o);
+            if (lane >= o) to += t;
+        }
+        if (lane == 31) S.hist[warp] = to;
+        __syncthreads();
+        to += __reduce_add_sync(0xffffffffu, lane < warp ? S.hist[lane] : 0);
+        const int from = min(to - later, P.cap);
+        to = min(to, P.cap);
+        if (tid < Tc) {
+            S.first[tid] = from;
+            if (S.parts[tid] > 0) {
+                S.parts[tid] = min(S.parts[tid], P.direct + to - from);
+                S.len[tid] = walk_steps(S.bounds[tid] & 0xFFFF, S.bounds[tid] >> 16, L) / S.parts[tid];
+            }
+        }
+        __syncthreads();
+    }
     int2* items = P.items + (size_t)bh * P.max_items;
     if (tid < Tc) {
         const int parts = S.parts[tid], len = S.len[tid];
         int at = 0;
         for (int u = 0; u < Tc; ++u) at += (P.longest_first ? S.len[u] > len || (S.len[u] == len && u < tid) : u < tid) ? S.parts[u] : 0;
-        for (int q = 0; q < parts; ++q) items[at + q] = make_int2(tid | (q << 16) | (parts << 24), S.bounds[tid]);
+        for (int q = 0; q < parts; ++q) items[at + q] = make_int2(tid | q << 10 | parts << 13 | (parts > 1 ? S.first[tid] + max(q - P.direct, 0) : 0) << 17, S.bounds[tid]);
     }
     int total = 0;
     for (int u = lane; u < Tc; u += 32) total += S.parts[u];
@@ -788,7 +840,8 @@ __global__ void __launch_bounds__(kPerm ? kPermThreads : 256) bwd_prepare_kernel
 //   a channel pair's rows per thread instead, 16 bytes out of every 128, took 32 passes per load: at L = 16384 with 32 heads of 128 channels
 //   121 us (backward 2221 -> 2097), 16 heads of 4096 (backward 163 -> 159).
 //   dK, dV: 8 elements per thread. nslots > 1: the accumulator is nslots copies, slot_stride elements apart, added in slot
-//   order (a fixed order: the result is then the same bits from run to run).
+//   order (a fixed order: the result is then the same bits from run to run). Where walks were cut, the blocks of the group's heads after that.
+//   dM: only where walks were cut, a thread per key.
 struct FinishParams {
     const float* dQacc;
     const float* acc[2];        // of dK, dV
@@ -796,16 +849,19 @@ struct FinishParams {
     __nv_bfloat16* out[2];
     int q_blocks, kv_blocks;    // CTAs of dQ, of each of dK and dV
     int L, Hq, Hkv, Lblk, nslots;
-    int64_t nkv;                // elements of dK
+    int64_t nkv, rows;          // elements of dK, of dM
     uint32_t q_rows16;          // 16-row blocks of dQ in all
     int64_t qs[3], st[2][3];
     float scale;
+    WalkBlocks blocks;
+    float* dM;
 };
 
 constexpr int kFinishBlocks = 1;       // (two: more loads in flight, but 8 heads of 500 keys, backward, 21.3 -> 22.1 us, 32 heads of 16384 2139 -> 2154)
 
-template <int kD>
-__global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
+// kBlocks: walks have left blocks
+template <int kD, bool kBlocks>
+__device__ __forceinline__ void finish(const FinishParams& P) {
     constexpr int kCh = kD / 32, kRowBlocks = 8 / kCh * kFinishBlocks;     // channel blocks of a row, 16-row blocks of a CTA
     constexpr int kPitch = kD / 2 + 4;                                     // 4-byte words per row: 16-byte aligned, rows 4 apart 16 banks apart
     __shared__ __align__(16) uint32_t turn[kRowBlocks * 16 * kPitch];
@@ -847,15 +903,42 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
         return;
     }
     const int blk = (int)blockIdx.x - P.q_blocks, which = blk / P.kv_blocks;
+    if (blk >= 2 * P.kv_blocks) {
+        const int64_t row = (int64_t)(blk - 2 * P.kv_blocks) * 256 + threadIdx.x;
+        const int at = row < P.rows ? P.blocks.where[row] : 0, n = (at >> 7) & 7;
+        if (n == 0) return;
+        const float* m = P.blocks.m + ((size_t)(row / P.L) * (P.Lblk / 8) + (at >> 19)) * ((kMostParts - 1) * 256) + (at & 127);
+        float sum = P.dM[row];
+#pragma unroll 4
+        for (int p = 0; p < n; ++p) sum += m[p * 256] + m[p * 256 + 128];
+        P.dM[row] = sum;
+        return;
+    }
     const int64_t e = ((int64_t)(blk % P.kv_blocks) * 256 + threadIdx.x) * 8;
     if (e >= P.nkv) return;
     const float* acc = P.acc[which];
+    auto add = [](float4& x, float4& y, const float* p) {
+        const float4 x2 = *reinterpret_cast<const float4*>(p), y2 = *reinterpret_cast<const float4*>(p + 4);
+        x.x += x2.x; x.y += x2.y; x.z += x2.z; x.w += x2.w; y.x += y2.x; y.y += y2.y; y.z += y2.z; y.w += y2.w;
+    };
     const uint32_t row = (uint32_t)(e / kD), bl = row / (uint32_t)P.Hkv;
     const int c = (int)(e % kD), h = (int)(row - bl * P.Hkv), b = (int)(bl / (uint32_t)P.L), i = (int)(bl - (uint32_t)b * P.L);
+    int at[2] = {0, 0};                                                    // (blocks: one or two query heads per KV head)
+    if constexpr (kBlocks) {
+        at[0] = P.blocks.where[(size_t)(b * P.Hq + h * (P.Hq / P.Hkv)) * P.L + i];
+        if (P.Hq != P.Hkv) at[1] = P.blocks.where[(size_t)(b * P.Hq + h * 2 + 1) * P.L + i];
+    }
     float4 a = *reinterpret_cast<const float4*>(acc + e), bb = *reinterpret_cast<const float4*>(acc + e + 4);
-    for (int sl = 1; sl < P.nslots; ++sl) {
-        const float4 a2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e), b2 = *reinterpret_cast<const float4*>(acc + sl * P.nkv + e + 4);
-        a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w; bb.x += b2.x; bb.y += b2.y; bb.z += b2.z; bb.w += b2.w;
+    for (int sl = 1; sl < P.nslots; ++sl) add(a, bb, acc + sl * P.nkv + e);
+    if constexpr (kBlocks) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const int n = ((at[g] >> 7) & 7) + 1 - P.blocks.direct;
+            const float* src = P.blocks.kv + (((size_t)(b * P.Hq + h * (P.Hq / P.Hkv) + g) * P.blocks.cap + ((at[g] >> 10) & 0x1FF)) * 2 + which) * (128 * kD) +
+                               (at[g] & 127) * kD + c;
+#pragma unroll 2
+            for (int p = 0; p < n; ++p) add(a, bb, src + p * (2 * 128 * kD));
+        }
     }
     const float scale = which == 0 ? P.scale : 1.0f;
     uint4 o;
@@ -864,14 +947,28 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) {
     *reinterpret_cast<uint4*>(P.out[which] + b * P.st[which][0] + (int64_t)i * P.st[which][1] + h * P.st[which][2] + c) = o;
 }
 
+template <int kD>
+__global__ void __launch_bounds__(256) bwd_finish_kernel(const FinishParams P) { finish<kD, false>(P); }
+// (registers for six CTAs per SM instead of four: 8 heads of 8192 keys, backward 189 -> 185 us)
+template <int kD>
+__global__ void __launch_bounds__(256, 6) bwd_finish_blocks_kernel(const FinishParams P) { finish<kD, true>(P); }
+
 }  // namespace
 
-// workspace layout: header | D [rows] | dQ accumulator [B x Hq x (Tr x 128) x d] | (token-compacted mode) permutation, work items | dK, dV accumulators
+// workspace layout: header | D [rows] | dQ accumulator [B x Hq x (Tr x 128) x d] | (token-compacted mode) permutation, work items, where each
+// key's walk left its later parts' sums | dK, dV accumulators | those sums
 static size_t bwd_rows64(const Prob& P) { return ((((size_t)P.B * P.Hq * P.L) + 63) / 64) * 64; }
 static size_t bwd_acc_floats(const Prob& P) { return (size_t)P.B * P.Hq * P.Tr * 128 * P.d; }     // rows padded to whole query tiles
 // permutation and work items
 static size_t bwd_perm_ints(const Prob& P) { return (size_t)P.B * P.Hq * P.Tc * 128; }
 static size_t bwd_item_ints(const Prob& P) { return ((size_t)P.B * P.Hq * P.Tc * 2 * kMostParts + 63) / 64 * 64; }
+// What cut walks take (WalkBlocks). Walks are never cut with DMA_FLAG_DETERMINISTIC.
+static bool bwd_may_cut(const Prob& P) { return (P.flags & DMA_FLAG_COMPACT_KV) && !(P.flags & DMA_FLAG_DETERMINISTIC); }
+static int bwd_heads(const Prob& P) { return P.bwd_heads ? P.bwd_heads : P.B * P.Hq; }
+static size_t bwd_where_ints(const Prob& P) { return bwd_may_cut(P) ? bwd_rows64(P) : 0; }
+static size_t bwd_part_floats(const Prob& P) { return bwd_may_cut(P) ? (size_t)P.B * P.Hq * P.Tc * (kMostParts - 1) * 256 : 0; }
+static size_t bwd_blocks(const Prob& P) { return bwd_may_cut(P) && P.G <= 2 ? std::min((size_t)P.B * P.Hq * P.Tc * (kMostParts - 1), (size_t)kWalkBlocks) : 0; }
+static int bwd_blocks_per_head(const Prob& P) { return P.G <= 2 ? std::min(P.Tc * (kMostParts - 1), kWalkBlocks / bwd_heads(P)) : 0; }
 
 // Tile mode: a CTA owns a key tile of one KV head and walks all its query heads. Where few CTAs wait for the heaviest one, the
 // group's heads are dealt out to several CTAs, whose parts of dK and dV go to slots of their own. The number is the divisor of G
@@ -905,17 +1002,17 @@ bool bwd_long(const Prob& P) {
 }
 // Token-compacted mode: the longest walk of one CTA, in 64-row steps. A long-lived key's tile is walked over all later rows, 2 L / 128 steps,
 // which few heads cannot hide behind other tiles: then walks are cut into parts of about what an SM gets of the whole work (its share of
-// the kept pairs, and half as much again that the tiles' walks cover beyond them), on the z axis of the grid. dK, dV (and dM) take the
-// parts' sums through the atomics that the heads of a group need anyway; with DMA_FLAG_DETERMINISTIC nothing is cut.
-// Backward, us, whole walks / this rule and items by length: one head of 9663 keys (w = 1442) 233 / 66, 2 heads of 4728 (w = 1044) 117 /
-// 46, 8 heads of 8192 (w = 1024) 240 / 188, 16 heads of 4096 (w = 1024) 202 / 164 (nothing cut, long walks first), 32 heads of 16384
-// 2282 / 2221 (K and V gathered by eight warps). Cutting every walk above 0.8 of the share was slower where the longest exceeds it by little
-// (16 heads, w = 2375 of 14353 keys).
+// the kept pairs, and half as much again that the tiles' walks cover beyond them), which are work items of their own. The later parts' sums
+// go through blocks (WalkBlocks); with DMA_FLAG_DETERMINISTIC nothing is cut.
+// Backward, us, whole walks / this rule and items by length: one head of 9663 keys (w = 1442) 233 / 60, 2 heads of 4728 (w = 1044) 117 /
+// 47, 8 heads of 8192 (w = 1024) 240 / 183, 16 heads of 4096 (w = 1024) 202 / 157 (nothing cut, long walks first), 32 heads of 16384
+// 2282 / 2060 (K and V gathered by eight warps). The blocks cost 1 to 3 us of that: with all parts on the accumulators 57, 45, 180. Cutting every
+// walk above 0.8 of the share was slower where the longest exceeds it by little (16 heads, w = 2375 of 14353 keys).
 static int bwd_walk(const Prob& P) {
     const int longest = 2 * P.Tr;
     if (P.flags & DMA_FLAG_DETERMINISTIC) return longest;
     const double w = P.w, pairs = P.causal ? w * (w + 1) / 2 + (P.L - w) * w : w * P.L;
-    const double share = (P.causal ? 1.55 : 1.0) * P.B * P.Hq * pairs / (128.0 * 64.0) / 148.0;
+    const double share = (P.causal ? 1.55 : 1.0) * bwd_heads(P) * pairs / (128.0 * 64.0) / 148.0;
     if (longest <= 1.3 * share) return longest;
     return std::max(std::max(16, (int)(0.8 * share)), (longest + kMostParts - 1) / kMostParts);
 }
@@ -929,8 +1026,8 @@ static size_t bwd_slots(const Prob& P) {
 static size_t bwd_base_bytes(const Prob& P) { return kWsHeaderBytes + (bwd_rows64(P) + bwd_acc_floats(P)) * sizeof(float); }
 // what the call uses beyond that
 static size_t bwd_extra_bytes(const Prob& P) {
-    const size_t perm = P.flags & DMA_FLAG_COMPACT_KV ? (bwd_perm_ints(P) + bwd_item_ints(P)) * sizeof(int) : 0;
-    return perm + 2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d * sizeof(float);
+    const size_t perm = P.flags & DMA_FLAG_COMPACT_KV ? (bwd_perm_ints(P) + bwd_item_ints(P) + bwd_where_ints(P)) * sizeof(int) : 0;
+    return perm + (2 * bwd_slots(P) * (size_t)P.B * P.L * P.Hkv * P.d + bwd_part_floats(P) + bwd_blocks(P) * 2 * 128 * P.d) * sizeof(float);
 }
 
 size_t tc_bwd_need(const Prob& P) { return bwd_base_bytes(P) + bwd_extra_bytes(P); }
@@ -960,8 +1057,15 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     const size_t slots = bwd_slots(P);
     const int nsplit = tc_bwd_splits(P);
     int2* items = reinterpret_cast<int2*>(perm + bwd_perm_ints(P));
-    float* accK = reinterpret_cast<float*>(perm + (compact ? bwd_perm_ints(P) + bwd_item_ints(P) : 0));
+    const size_t where_ints = compact ? bwd_where_ints(P) : 0;
+    int* where = reinterpret_cast<int*>(items) + bwd_item_ints(P);
+    float* accK = reinterpret_cast<float*>(compact ? where + where_ints : perm);
     float* accV = accK + slots * nkv;
+    WalkBlocks blocks;
+    blocks.cap = bwd_blocks_per_head(P);
+    blocks.direct = P.G > 2 ? kMostParts : 3 - P.G;
+    blocks.m = accV + slots * nkv;
+    blocks.kv = blocks.m + bwd_part_floats(P);
     CUtensorMap tmQ, tmK, tmV, tmG;
     int rc;
     if ((rc = make_tmap_bf16(&tmQ, Q, P.B, P.L, P.Hq, P.d, P.qs, 64))) return rc;
@@ -973,13 +1077,16 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     pp.os_b = P.os[0]; pp.os_l = P.os[1]; pp.os_h = P.os[2];
     pp.status = (int32_t*)ws;
     pp.zero[0] = acc; pp.zero_n[0] = (int64_t)bwd_acc_floats(P);
-    pp.zero[1] = dM; pp.zero_n[1] = (int64_t)rows;                                       // two partial sums are added per key
+    pp.zero[1] = dM; pp.zero_n[1] = (int64_t)rows;                                       // two sums, over the halves of the query columns, are added per key
     pp.zero[2] = accK; pp.zero_n[2] = compact ? (int64_t)(2 * slots * nkv) : 0;
+    const int walk = compact ? bwd_walk(P) : 1, max_items = compact ? P.Tc * ((2 * P.Tr + walk - 1) / walk) : P.Tc;
+    blocks.where = compact && max_items > P.Tc ? where : nullptr;
+    if (blocks.where) { pp.zero[2] = reinterpret_cast<float*>(where); pp.zero_n[2] += (int64_t)where_ints; }   // (the accumulators are behind it)
     const int threads = compact ? kPermThreads : 256, per_cta = threads / (P.d / 8) * kPrepareRows;
     const unsigned prep_ctas = (unsigned)((rows + per_cta - 1) / per_cta);
     for (int z = 0; z < 3; ++z) pp.zero_part[z] = ((pp.zero_n[z] >> 2) + prep_ctas - 1) / prep_ctas;
-    const int walk = compact ? bwd_walk(P) : 1, max_items = compact ? P.Tc * ((2 * P.Tr + walk - 1) / walk) : P.Tc;
     pp.perm_ctas = compact ? P.B * P.Hq : 0;
+    pp.cap = blocks.cap; pp.direct = blocks.direct;
     pp.expiry = expiry; pp.perm = perm; pp.items = items; pp.Tc = P.Tc; pp.causal = P.causal; pp.max_items = max_items; pp.walk = walk;
     // (of more rows than one scheduling group, below, the order of the permutation keeps the rows in use in L2)
     pp.longest_first = (double)P.B * P.Hq * P.L * P.d * 8 <= 160.0 * 1024 * 1024 ? 1 : 0;
@@ -1011,7 +1118,7 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     }
     bp.scale = P.scale; bp.scale_log2 = P.scale * 1.4426950408889634f; bp.inv_scale = 1.0f / P.scale;
     bp.ks_b = P.ks[0]; bp.ks_l = P.ks[1]; bp.ks_h = P.ks[2]; bp.vs_b = P.vs[0]; bp.vs_l = P.vs[1]; bp.vs_h = P.vs[2];
-    bp.perm = perm; bp.items = items; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
+    bp.perm = perm; bp.items = items; bp.blocks = blocks; bp.causal = P.causal; bp.Kg = (const __nv_bfloat16*)K; bp.Vg = (const __nv_bfloat16*)V;
     bp.dKacc = accK; bp.dVacc = accV; bp.acc_slot = slots > 1 ? (int64_t)nkv : 0; bp.nsplit = nsplit;
     const size_t smem = sizeof(SharedStorage) + 1024;
     const bool lng = bwd_long(P);
@@ -1034,7 +1141,12 @@ int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, co
     f.kv_blocks = (int)((nkv / 8 + 255) / 256);
     for (int t = 0; t < 3; ++t) { f.qs[t] = P.qs[t]; f.st[0][t] = P.ks[t]; f.st[1][t] = P.vs[t]; }
     f.scale = P.scale;
-    return launch_overlapped(P.d == 128 ? bwd_finish_kernel<128> : bwd_finish_kernel<64>, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0)), dim3(256), 0, st, 1, f);
+    f.blocks = blocks; f.dM = dM; f.rows = (int64_t)rows;
+    const int m_blocks = blocks.where ? (int)((rows + 255) / 256) : 0;
+    auto finish = blocks.where && P.G <= 2 ? (P.d == 128 ? bwd_finish_blocks_kernel<128> : bwd_finish_blocks_kernel<64>)
+                                           : (P.d == 128 ? bwd_finish_kernel<128> : bwd_finish_kernel<64>);
+    return launch_overlapped(finish, dim3(f.q_blocks + (slots ? 2 * f.kv_blocks : 0) + m_blocks), dim3(256), 0, st,
+                             1, f);
 }
 
 }  // namespace dma

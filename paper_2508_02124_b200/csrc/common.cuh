@@ -21,6 +21,7 @@ struct Prob {
     int causal;            // 1: key j visible to rows i >= j; 0: to every row (the key's first row is 0 instead of j)
     int bm, bn, Tr, Tc, Wd;   // bitmap tile sizes, tile counts, uint32 words per bitmap row
     int bwd_split;            // CTAs that share a KV head in the tile-mode backward (0: tc_bwd_splits chooses)
+    int bwd_heads;            // (batch, query head) pairs by which the token-compacted backward cuts its walks (0: B Hq)
     int Lq, q_off;            // forward over a chunk of query rows: Q, O, lse hold the rows q_off .. q_off + Lq - 1 (Lq = L, q_off = 0: all)
     float scale;
     int64_t qs[3], ks[3], vs[3], os[3];   // batch, seq, head strides in elements
@@ -63,8 +64,8 @@ int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, co
 size_t tc_bwd_need(const Prob& P);         // what the call uses
 size_t tc_bwd_ws_bytes(const Prob& P);     // what is asked for: at least the need of every shorter sequence and smaller batch
 int tc_bwd_splits(const Prob& P);
-// dma_attn_bwd on a part of a problem: with the split of the whole one, so that the parts' results are the whole's
-int attn_bwd_part(const dma_problem_t* p, int split, const void* Q, const void* K, const void* V, const void* O, const void* dO,
+// dma_attn_bwd on a part of a problem: with the split and the walks of the whole one, so that the parts' results are the whole's
+int attn_bwd_part(const dma_problem_t* p, int split, int heads, const void* Q, const void* K, const void* V, const void* O, const void* dO,
                   const float* lse, const float* bias, const int32_t* expiry, const uint32_t* bitmap, void* dQ, void* dK, void* dV,
                   float* dM, void* ws, size_t ws_bytes, cudaStream_t st);
 int launch_tc_bwd(const Prob& P, const void* Q, const void* K, const void* V, const void* O, const void* dO,

@@ -213,7 +213,7 @@ int dma_step_host(const dma_problem_t* p, int backward, const void* hQ, const vo
             char* wsb = a + Lo.ws_bwd + (size_t)g * kWsHeaderBytes;
             float* dM = (float*)(a + Lo.dM) + (size_t)g * Lo.gh;
             if (!ok || !wait(st, e[kdO])) return cleanup(DMA_ERR_CUDA);
-            if ((rc = attn_bwd_part(&sub, split, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, a + Lo.O + G.q * esz,
+            if ((rc = attn_bwd_part(&sub, split, whole.B * whole.Hq, a + Lo.Q + G.q * esz, a + Lo.K + G.k * esz, a + Lo.V + G.k * esz, a + Lo.O + G.q * esz,
                                    a + Lo.dO + G.q * esz, lse, bias, expiry, bitmap, a + Lo.dQ + G.q * esz, a + Lo.dK + G.k * esz,
                                    a + Lo.dV + G.k * esz, dM, wsb, b_ws, st))) return cleanup(rc);
             ok = rec(e[kG], st) && wait(s_out, e[kG]) &&

@@ -53,6 +53,17 @@ def test_equals_the_device_entry_points(case):
         assert_close(got["dQ"], dev["dQ"].double().cpu().numpy(), case.dtype, "dQ")
 
 
+@pytest.mark.parametrize("B,H,L,d,w", [(1, 16, 4096, 64, 1000), (2, 8, 2500, 128, 600)])
+def test_parts_cut_their_walks_as_the_whole_does(B, H, L, d, w):
+    """Token-compacted, one query head per KV head: the backward of a part alone would cut its walks, that of the whole problem does not."""
+    case = wl.small(C2, B=B, Hq=H, Hkv=H, L=L, w=w, d=d, backward=True, name="host token-compacted")
+    inp = wl.make_inputs(case)
+    got, dev = host_step(case, inp), gpu_run(case, inp)
+    for k in ("O", "lse", "dK", "dV", "dM"):
+        assert torch.equal(got[k], dev[k].cpu()), k
+    assert_close(got["dQ"], dev["dQ"].double().cpu().numpy(), case.dtype, "dQ")
+
+
 def test_against_the_oracle():
     case = wl.small(C2, B=2, Hq=8, Hkv=4, L=512, w=96, backward=True, name="host oracle")
     inp = wl.make_inputs(case)
