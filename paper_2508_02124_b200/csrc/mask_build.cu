@@ -663,10 +663,12 @@ __global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v, uint32_t* bitma
 __global__ void __launch_bounds__(1024) bitmap_square_kernel(const int32_t* __restrict__ expiry, uint32_t* __restrict__ bitmap,
                                                              int L, int bm, int T, int Wd, int causal) {
     __shared__ int last[32];
-    const int kt0 = blockIdx.x * 32, bh = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j0 = (kt0 + warp) * bm;
+    const int kt0 = blockIdx.x * 32, bh = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_enter_restrict(expiry, bitmap);
     int top = 0;
-    for (int j = j0 + lane; j < min(L, j0 + bm); j += 32) {
+    // (a tile side may be anything: neither a tile beyond the last nor the end of one is formed, they need not fit 32 bits)
+    const int j0 = kt0 + warp < T ? (kt0 + warp) * bm : L, jend = bm < L - j0 ? j0 + bm : L;
+    for (int j = j0 + lane; j < jend; j += 32) {
         const int e = expiry[(size_t)bh * L + j];
         top = max(top, e > (causal ? j : 0) ? e : 0);
     }

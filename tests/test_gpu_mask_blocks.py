@@ -52,6 +52,16 @@ def test_ties_documents_and_other_rows(H, L):
     assert np.array_equal(e, oracle.select_noncausal(dl, L // 4))
 
 
+@pytest.mark.parametrize("side", [4096, 8192, 1 << 26, 1 << 27, 1 << 30])
+@pytest.mark.parametrize("L,w", [(300, 400), (700, 90), (5000, 800), (9000, 9000)])
+def test_tiles_longer_than_the_sequence(L, w, side):
+    """Also where 32 sides, a word's worth of tiles, are more than 32 bits hold."""
+    dl, e, bitmap = build(2, L, w, seed=L, tile=(side, side))
+    ref = oracle.select_expiry(dl, min(w, L))
+    assert np.array_equal(e, ref)
+    assert np.array_equal(bitmap, oracle.bitmap_from_expiry(ref, side, side))
+
+
 @pytest.mark.parametrize("tile", [(64, 64), (96, 96), (160, 160), (32, 32), (48, 48), (128, 64), (64, 128)])
 @pytest.mark.parametrize("L", [900, 4000, 5000])
 def test_tiles(L, tile):
