@@ -84,10 +84,16 @@ def _elem(p, *tensors):
             raise TypeError(f"tensor of {t.dtype} passed for a problem whose element type is {want}")
 
 
+# torch's own calls for the handle alone, where this release of it has them
+_raw_stream, _raw_device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+
 def _stream():
     """The current stream of the current device, as torch.cuda.current_stream().cuda_stream says it. That call builds a Stream
     object, 5.7 us a time, which was 40 % of the host's share of a decoding token; asking for the handle alone is 0.3 us."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 # Parameter types of the calls that take device pointers: P problem, v pointer, i int32, l int64, z size_t. ctypes then converts

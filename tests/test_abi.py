@@ -82,6 +82,19 @@ def test_binding_refuses_tensors_of_another_element_type():
         dma.problem(1, 2, 2, 8, 64, 4, dtype=torch.float16)
 
 
+@pytest.mark.parametrize("gone", ["_raw_stream", "_raw_device", None])
+def test_stream_handle(gone, monkeypatch):
+    """With torch's calls for the handle, and by its public interface where a release has moved them."""
+    class Stream:
+        cuda_stream = 77
+    monkeypatch.setattr(dma, "_raw_stream", lambda device: 1000 + device)
+    monkeypatch.setattr(dma, "_raw_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    if gone:
+        monkeypatch.setattr(dma, gone, None)
+    assert dma._stream() == (77 if gone else 1003)
+
+
 def test_typed_calls_match_the_header():
     text = re.sub(r"/\*.*?\*/", "", open(os.path.join(ROOT, "include", "dma.h")).read(), flags=re.S)
     for name, kinds in dma._SIGNATURES.items():
