@@ -15,9 +15,12 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
+SHAPES = [(1, 1, 0), (5, 2, 0), (128, 128, 0), (129, 40, 0), (256, 256, 0), (300, 30, 0), (640, 500, 0), (897, 64, 0),
+          (2050, 100, 0), (2305, 512, 0), (700, 90, 1), (1000, 128, 129), (2500, 300, 250)]
+
+
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("L,w,rows", [(1, 1, 0), (5, 2, 0), (128, 128, 0), (129, 40, 0), (256, 256, 0), (300, 30, 0), (640, 500, 0), (897, 64, 0),
-                                      (2050, 100, 0), (2305, 512, 0), (700, 90, 1), (1000, 128, 129), (2500, 300, 250)])
+@pytest.mark.parametrize("L,w,rows", SHAPES)
 def test_one_query_tile_per_cta(L, w, rows, d):
     case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=1, L=L, w=w, d=d, name=f"one tile L{L} w{w} d{d}")
     inp = wl.make_inputs(case)
@@ -64,3 +67,47 @@ def test_bits_do_not_depend_on_the_batch(L, w, rows, B, flags, d):
     Or, lr = oracle.forward(*(f64(inp[k]) for k in ("Q", "K", "V")), dl.astype(np.float64), expiry=e, rows=kept)
     assert_close(out[1][0][:1], Or, case.dtype, f"{case.name}: O")
     assert_close(out[1][1][:1], lr, case.dtype, f"{case.name}: lse", lse=True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("L,w,rows", SHAPES)
+def test_two_query_tiles_on_the_small_shapes(L, w, rows, d):
+    """DMA_FLAG_BLOCK_SKIP always takes two query tiles per CTA: odd tile counts, ragged ends, w = 1, w >= L, both walks."""
+    case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=1, L=L, w=w, d=d, name=f"two tiles L{L} w{w} d{d}")
+    inp = wl.make_inputs(case)
+    p, bias, expiry, bitmap = gpu_mask(case, inp)
+    Q, K, V = (inp[k].to(DEV) for k in ("Q", "K", "V"))
+    for path in (0,) if rows else (dma.DMA_FLAG_TILE_PATH, dma.DMA_FLAG_COMPACT_KV):
+        out = []
+        for flags in (path, path | dma.DMA_FLAG_BLOCK_SKIP):
+            p = dma.problem(1, 2, 1, L, d, w, flags=flags)
+            if rows:
+                out.append(dma.dma_attn_fwd_chunk(p, L - rows, Q[:, L - rows:].contiguous(), K, V, bias, expiry))
+            else:
+                out.append(dma.dma_attn_fwd(p, Q, K, V, bias, expiry, bitmap))
+        torch.cuda.synchronize()
+        assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1]), path
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_pairs_whose_tiles_use_different_key_tiles(d):
+    """Documents that begin inside a pair of query tiles: one tile skips the key tiles its partner needs and enters the walk late. 64 heads take
+    two query tiles per CTA, two heads one."""
+    L, cu = 1100, torch.tensor([0, 77, 384, 520, 700, 1100], dtype=torch.int32, device=DEV)
+    case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=2, L=L, w=64, d=d, name="late entry")
+    inp = wl.make_inputs(case)
+    W, A = inp["W_delta"].to(DEV), inp["A"].to(DEV)
+    out = {}
+    for B, flags in ((1, dma.DMA_FLAG_SIMT), (1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (32, 0), (32, 0), (32, 0)):
+        p = dma.problem(B, 2, 2, L, d, 64, flags=flags)
+        Q, K, V = (inp[k].to(DEV).repeat(B, 1, 1, 1) for k in ("Q", "K", "V"))
+        mask = dma.dma_mask_build_varlen(p, V, W, A, cu)
+        O, lse = dma.dma_attn_fwd(p, Q, K, V, *mask)
+        torch.cuda.synchronize()
+        if flags == dma.DMA_FLAG_SIMT:
+            assert_close(O, np.asarray(oracle.forward(*(f64(inp[k]) for k in ("Q", "K", "V")), f64(mask[0]), expiry=mask[1].cpu().numpy())[0]), case.dtype, "O")
+            out["O"], out["lse"] = O.float(), lse
+            continue
+        assert float((O.float() - out["O"]).abs().max()) <= 3e-2 and float((lse - out["lse"]).abs().max()) <= 1e-3 * max(1.0, float(out["lse"].abs().max()))
+        bits = out.setdefault("bits", (O[0], lse[0]))
+        assert all(torch.equal(x, bits[0]) for x in O) and all(torch.equal(x, bits[1]) for x in lse), (B, flags)
