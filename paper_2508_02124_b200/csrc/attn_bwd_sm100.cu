@@ -204,7 +204,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     if (kCompact && warp < 8) {
         // The compute warps gather the CTA's 128 K and V rows into the swizzled tile layout, 16 rows each (8 lanes per 128-byte half row, 4
         // rows per instruction; padding entries are zero-filled), while the schedule is built. (One warp after the schedule: the first
-        // product was issued 10500 clk after the start instead of 6000, as long as two steps.)
+        // product was issued 10500 clk after the CTA's start, now 4200 to 4900 in the median.)
         const int rsub = lane >> 3, c = lane & 7;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -404,7 +404,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // A thread holds 32 channels of its key's row. The warp turns each such block of 32 rows around in shared memory (the Q stages, which
             // the last MMAs have left; 16-byte chunks swizzled by the row), so that eight lanes write 128 consecutive bytes of a row, and the
             // block after it is on its way from tensor memory meanwhile. What is left is the stores and reductions themselves, 14 to 32 bytes per clock:
-            // 10000 -> 6800 clk for fp32 parts, 9300 -> 7700 for reductions, 6000 either way for bf16 rows.
+            // 6000 clk for fp32 parts (10000 without the turn), 8400 for reductions, 5400 for bf16 rows.
             uint8_t* turn = S.q[0] + warp * 4096;
             static_assert(sizeof(S.q) >= 8 * 4096, "a block of 32 x 32 floats per compute warp");
             const int rsub = lane >> 3, ch = lane & 7;

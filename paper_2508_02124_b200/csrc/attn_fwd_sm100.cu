@@ -1182,7 +1182,9 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
 // Query tiles per CTA: two, or one whose key tiles are dealt out to the two softmax groups where that shortens the call. Both grids
 // are estimated in steps of a CTA (two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs; the pair's
 // steps in tile mode are longer where many keys expire per tile, i.e. in short sequences. Fitted to 64 shapes of 1 to 128 heads and
-// 183 to 15889 keys, each timed with both before rows had their references from both groups, and then moved by 5 to 10 % towards two: forward, us, two
+// 183 to 15889 keys, each timed with both, and then moved by 5 to 10 % towards two for the hand-over of references and sums. Of 56 other shapes
+// (1 to 128 heads, 192 to 14712 keys, 14 chunks) 50 get the faster one or are within 3 %; the worst are 64 and 128 heads of 300 to 430 keys with few kept,
+// 17 %, and 8 heads of 12238 (w = 5098), 8 %. Forward, us, two
 // tiles / one: 16 heads of 1000 keys 37 / 19, 8 heads of 500 25 / 13, 8 heads of 4096 (w = 2048) 78 / 50, 172 rows of 26817 keys, 4 heads 109 / 71, but 64
 // heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568. The results are the same bits.
 // DMA_FLAG_BLOCK_SKIP is for two tiles: its marks are read where one group walks every entry.
