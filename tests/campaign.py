@@ -309,7 +309,8 @@ def host(T):
         try:
             got, dev = TH.host_step(case, inp), gpu_run(case, inp, backward=bwd)
             # where the library picks the token-compacted kernels (L >= 2048, 4 w <= L) and a KV head serves several query
-            # heads, dK and dV are summed over the group with floating-point atomics: equal up to the order of the adds
+            # heads, dK and dV are summed over the group with floating-point atomics: equal up to the order of the adds (of two heads
+            # the sums have one value as well; the parts cut their walks as the whole does)
             atomic = case.dtype == "bf16" and L >= 2048 and 4 * min(w, L) <= L and G > 1
             exact = ("O", "lse") + (("dK", "dV") if bwd and not atomic else ())
             bad = [k for k in exact if not torch.equal(got[k], dev[k].cpu())]
