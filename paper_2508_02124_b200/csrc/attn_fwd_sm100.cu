@@ -380,6 +380,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const bool small = __all_sync(0xffffffffu, fabsf(M) < kSmallStab);
             // Pairs of columns: one packed FMA for two arguments, one packed add for two terms of the row sum. The loop is bound by issue slots as much as by the
             // exponentials; two FMAs and two adds per pair instead: 16 heads of 4096 keys 72.2 against 69.2 us, 32 heads of 8192 keys at d = 64 189 against 179.
+            float sa[4] = {0.f, 0.f, 0.f, 0.f};
             float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
             const float2 c2 = make_float2(P.scale_log2, P.scale_log2), nM2 = make_float2(nM, nM);
             if (small) {
@@ -409,7 +410,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     for (int c = 0; c < 64; c += 2) {
                         const float2 p = make_float2(ex2(fmaf(x[half * 64 + c] - m_use, P.scale_log2, resid)),
                                                      ex2(fmaf(x[half * 64 + c + 1] - m_use, P.scale_log2, resid)));
-                        sum2[(c >> 1) & 1] = add2(sum2[(c >> 1) & 1], p);
+                        // (tile mode keeps a sum of its own here: with the packed one the compiler's other loop is 4 % slower, 155 -> 161 us at 32 heads
+                        // of 4096; token-compacted the other way round, 98 -> 103 for the last 2048 rows of 16384 keys)
+                        if constexpr (kCompact) sum2[(c >> 1) & 1] = add2(sum2[(c >> 1) & 1], p);
+                        else sa[(c >> 1) & 3] += p.x + p.y;
                         pk[c >> 1] = pack_bf16(p.x, p.y);
                     }
                     tmem_st32(tS + half * 32, pk);
@@ -421,7 +425,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     }
                 }
             }
-            const float sum = (sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y);
+            sa[0] += sum2[0].x + sum2[0].y;
+            sa[1] += sum2[1].x + sum2[1].y;
+            const float sum = (sa[0] + sa[1]) + (sa[2] + sa[3]);
             if constexpr (kSplit) s_last = sum;
             else l += sum;
             tc_wait_st();
@@ -500,13 +506,21 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const int* list = P.cidx + ((size_t)bh * npairs + lpair) * P.ccap;
             const int64_t row_stride = isK ? P.ks_l : P.vs_l;
             const __nv_bfloat16* src = (isK ? P.Kg + b * P.ks_b + hk * P.ks_h : P.Vg + b * P.vs_b + hk * P.vs_h) + (lane & 7) * 8;
-            const int rsub = lane >> 3;
-            const uint32_t sw0 = (uint32_t)(((lane & 7) ^ rsub) << 4), sw1 = (uint32_t)(((lane & 7) ^ (rsub + 4)) << 4);
-            int jrow[32];
+            // lanes 8 g .. 8 g + 7 take the rows 8 m + 2 g and 8 m + 2 g + 1
+            const int rsub = (lane >> 3) * 2;
+            const uint32_t sw0 = (uint32_t)(((lane & 7) ^ rsub) << 4), sw1 = (uint32_t)(((lane & 7) ^ (rsub + 1)) << 4) + 128;
+            int2 jrow[16];
+            list += rsub;
             if (n_iters > 0) {
 #pragma unroll
-                for (int q = 0; q < 32; ++q) jrow[q] = list[4 * q + rsub];
+                for (int m = 0; m < 16; ++m) jrow[m] = *reinterpret_cast<const int2*>(list + 8 * m);
             }
+            // Slices without padding, rows less than 4 GB apart (all but a list's last slice): three instructions per row. What the gather warps issue, the softmax
+            // warps of the same scheduler wait for: with seven, and a load per row, a slice's exponentials beside a gather took up to 470 clk more. Forward, us,
+            // before / now: 16 heads of 4096 keys 67.5 / 63.6, last 2048 rows of 16384 108.6 / 99.5, 32 heads of 16384 643 / 600, 16 of 65536 2400 / 2150.
+            const uint32_t step = (uint32_t)row_stride * 2u;
+            const int listed = P.ccnt[(size_t)bh * npairs + lpair];              // (beyond the capacity: there may be padding anywhere)
+            const int n_plain = listed <= P.ccap && row_stride > 0 && row_stride < (1ll << 31) ? listed / 128 : 0;
             bool ok = true;
             for (int it = 0; it < n_iters && ok; ++it) {
                 const int st = it % kStages;
@@ -515,18 +529,32 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 uint8_t* dst = (isK ? S.k[st] : S.v[st]) + rsub * 128;
                 if (it >= kStages) ok = mbar_wait_warp(empty, ((it / kStages) - 1) & 1, abort_flag);
                 if (!ok) break;
+                if (it < n_plain) {
+                    const uint32_t d0 = smem_u32(dst) + sw0, d1 = smem_u32(dst) + sw1;
+                    const char* base = reinterpret_cast<const char*>(src);
 #pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    const int j = jrow[q];
-                    const __nv_bfloat16* row = src + (int64_t)max(j, 0) * row_stride;
-                    uint8_t* d = dst + q * 512 + ((q & 1) ? sw1 : sw0);          // row r = 4q + rsub, chunk c ^ (r & 7)
-                    cp_async16(d, row, j >= 0 ? 16 : 0);
-                    if constexpr (kD == 128) cp_async16(d + kTileBytes / 2, row + 64, j >= 0 ? 16 : 0);
+                    for (int m = 0; m < 16; ++m) {
+                        const char* r0 = base + (uint64_t)(uint32_t)jrow[m].x * step;
+                        const char* r1 = base + (uint64_t)(uint32_t)jrow[m].y * step;
+                        cp_async16_at(d0 + m * 1024, r0);
+                        if constexpr (kD == 128) cp_async16_at(d0 + m * 1024 + kTileBytes / 2, r0 + 128);
+                        cp_async16_at(d1 + m * 1024, r1);
+                        if constexpr (kD == 128) cp_async16_at(d1 + m * 1024 + kTileBytes / 2, r1 + 128);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int q = 0; q < 32; ++q) {
+                        const int j = list[it * 128 + 8 * (q >> 1) + (q & 1)];
+                        const __nv_bfloat16* row = src + (int64_t)max(j, 0) * row_stride;
+                        uint8_t* d = dst + (q >> 1) * 1024 + ((q & 1) ? sw1 : sw0);          // row r, chunk c ^ (r & 7)
+                        cp_async16(d, row, j >= 0 ? 16 : 0);
+                        if constexpr (kD == 128) cp_async16(d + kTileBytes / 2, row + 64, j >= 0 ? 16 : 0);
+                    }
                 }
                 cp_async_arrive(full);
                 if (it + 1 < n_iters) {
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) jrow[q] = list[(it + 1) * 128 + 4 * q + rsub];
+                    for (int m = 0; m < 16; ++m) jrow[m] = *reinterpret_cast<const int2*>(list + (it + 1) * 128 + 8 * m);
                 }
             }
             for (int it = max(0, n_iters - kStages); it < n_iters && ok; ++it)

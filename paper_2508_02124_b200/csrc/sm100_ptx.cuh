@@ -74,6 +74,10 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* m, uin
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, int src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes) : "memory");
 }
+// the same of exactly 16 bytes, to a shared-memory address
+__device__ __forceinline__ void cp_async16_at(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 // one arrival on the mbarrier once every cp.async this thread has issued so far has landed (the barrier's expected
 // count must include it)
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
