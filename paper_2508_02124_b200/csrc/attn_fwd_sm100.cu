@@ -165,6 +165,56 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         S.n_iters = 0;
         fence_barrier_init();
     }
+    // Token-compacted mode: a gather warp fetches the first slice's keys beside the list's length, before the CTA's barrier. (Behind it, 16 heads of 4096 keys 64.1
+    // against 63.1 us, last 2048 rows of 16384 keys 101.0 / 99.0, 16 heads of 65536 2180 / 2080; with the rows' copies ahead of the barrier too it is no faster.)
+    const bool isK = warp == kWarpProducer;
+    int2 jrow[kCompact ? 16 : 1];
+    int listed = 0, n_plain = 0;
+    const int* list = nullptr;
+    const int rsub = (lane >> 3) * 2;              // lanes 8 g .. 8 g + 7 take the rows 8 m + 2 g and 8 m + 2 g + 1
+    // Slices without padding, rows less than 4 GB apart (all but a list's last slice): three instructions per row. What the gather warps issue, the softmax
+    // warps of the same scheduler wait for: with seven, and a load per row, a slice's exponentials beside a gather took up to 470 clk more. Forward, us,
+    // before / now: 16 heads of 4096 keys 67.5 / 63.6, last 2048 rows of 16384 108.6 / 99.5, 32 heads of 16384 643 / 600, 16 of 65536 2400 / 2150.
+    auto gather = [&](int it) {
+        const int st = it % kStages;
+        const int64_t row_stride = isK ? P.ks_l : P.vs_l;
+        const __nv_bfloat16* src = (isK ? P.Kg + b * P.ks_b + hk * P.ks_h : P.Vg + b * P.vs_b + hk * P.vs_h) + (lane & 7) * 8;
+        const uint32_t sw0 = (uint32_t)(((lane & 7) ^ rsub) << 4), sw1 = (uint32_t)(((lane & 7) ^ (rsub + 1)) << 4) + 128;
+        const uint32_t step = (uint32_t)row_stride * 2u;
+        uint8_t* dst = (isK ? S.k[st] : S.v[st]) + rsub * 128;
+        if (it < n_plain) {
+            const uint32_t d0 = smem_u32(dst) + sw0, d1 = smem_u32(dst) + sw1;
+            const char* base = reinterpret_cast<const char*>(src);
+#pragma unroll
+            for (int m = 0; m < 16; ++m) {
+                const char* r0 = base + (uint64_t)(uint32_t)jrow[kCompact ? m : 0].x * step;
+                const char* r1 = base + (uint64_t)(uint32_t)jrow[kCompact ? m : 0].y * step;
+                cp_async16_at(d0 + m * 1024, r0);
+                if constexpr (kD == 128) cp_async16_at(d0 + m * 1024 + kTileBytes / 2, r0 + 128);
+                cp_async16_at(d1 + m * 1024, r1);
+                if constexpr (kD == 128) cp_async16_at(d1 + m * 1024 + kTileBytes / 2, r1 + 128);
+            }
+        } else {
+#pragma unroll 4
+            for (int q = 0; q < 32; ++q) {
+                const int j = list[it * 128 + 8 * (q >> 1) + (q & 1)];
+                const __nv_bfloat16* row = src + (int64_t)max(j, 0) * row_stride;
+                uint8_t* d = dst + (q >> 1) * 1024 + ((q & 1) ? sw1 : sw0);          // row r, chunk c ^ (r & 7)
+                cp_async16(d, row, j >= 0 ? 16 : 0);
+                if constexpr (kD == 128) cp_async16(d + kTileBytes / 2, row + 64, j >= 0 ? 16 : 0);
+            }
+        }
+    };
+    if constexpr (kCompact) {
+        if (warp == kWarpProducer || warp == kWarpStager1) {
+            list = P.cidx + ((size_t)bh * npairs + lpair) * P.ccap + rsub;
+            listed = P.ccnt[(size_t)bh * npairs + lpair];              // (beyond the capacity: there may be padding anywhere)
+#pragma unroll
+            for (int m = 0; m < 16; ++m) jrow[m] = *reinterpret_cast<const int2*>(list + 8 * m);
+            const int64_t row_stride = isK ? P.ks_l : P.vs_l;
+            n_plain = listed <= P.ccap && row_stride > 0 && row_stride < (1ll << 31) ? listed / 128 : 0;
+        }
+    }
     if (warp == kWarpIssuer) {
         tmem_alloc(&S.tmem_base, 512);
         tmem_relinquish();
@@ -177,7 +227,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         int n = 0;
         if constexpr (kCompact) {
             // every 128-key slice of the gathered list, used by both query tiles
-            const int listed = P.ccnt[(size_t)bh * npairs + lpair];
             if (listed > P.ccap && lane == 0) atomicExch(P.status, (int32_t)DMA_ERR_MASK_OVERFLOW);
             n = min((min(listed, P.ccap) + 127) / 128, kMaxSched);
             for (int t = lane; t < n; t += 32) S.sched[t] = (uint32_t)t | (kSplit ? 1u << (30 + (t & 1)) : (1u << 30) | (has1 ? (1u << 31) : 0u));
@@ -533,61 +582,20 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // Warp 0 fetches the K rows of each 128-key slice of the gathered list, warp 3 the V rows: 16-byte
             // asynchronous copies into the 128-byte-swizzled tile layout (8 lanes per 128-byte half row, 4 rows per
             // instruction; padding entries (-1) are zero-filled). Each lane's copies report to the stage's barrier.
-            const bool isK = warp == kWarpProducer;
             if (isK && lane == 0) {
                 mbar_arrive_expect_tx(&S.q_full, has1 ? 2 * kLoadBytes : kLoadBytes);
                 for (int w = 0; w < (has1 ? 2 : 1); ++w)
                     for (int hf = 0; hf < kHalves; ++hf)
                         tma_load_4d(&S.q[w][hf * (kTileBytes / 2)], &tmQ, &S.q_full, hf * 64, (qt0 + w) * 128, h, b);
             }
-            const int* list = P.cidx + ((size_t)bh * npairs + lpair) * P.ccap;
-            const int64_t row_stride = isK ? P.ks_l : P.vs_l;
-            const __nv_bfloat16* src = (isK ? P.Kg + b * P.ks_b + hk * P.ks_h : P.Vg + b * P.vs_b + hk * P.vs_h) + (lane & 7) * 8;
-            // lanes 8 g .. 8 g + 7 take the rows 8 m + 2 g and 8 m + 2 g + 1
-            const int rsub = (lane >> 3) * 2;
-            const uint32_t sw0 = (uint32_t)(((lane & 7) ^ rsub) << 4), sw1 = (uint32_t)(((lane & 7) ^ (rsub + 1)) << 4) + 128;
-            int2 jrow[16];
-            list += rsub;
-            if (n_iters > 0) {
-#pragma unroll
-                for (int m = 0; m < 16; ++m) jrow[m] = *reinterpret_cast<const int2*>(list + 8 * m);
-            }
-            // Slices without padding, rows less than 4 GB apart (all but a list's last slice): three instructions per row. What the gather warps issue, the softmax
-            // warps of the same scheduler wait for: with seven, and a load per row, a slice's exponentials beside a gather took up to 470 clk more. Forward, us,
-            // before / now: 16 heads of 4096 keys 67.5 / 63.6, last 2048 rows of 16384 108.6 / 99.5, 32 heads of 16384 643 / 600, 16 of 65536 2400 / 2150.
-            const uint32_t step = (uint32_t)row_stride * 2u;
-            const int listed = P.ccnt[(size_t)bh * npairs + lpair];              // (beyond the capacity: there may be padding anywhere)
-            const int n_plain = listed <= P.ccap && row_stride > 0 && row_stride < (1ll << 31) ? listed / 128 : 0;
             bool ok = true;
             for (int it = 0; it < n_iters && ok; ++it) {
                 const int st = it % kStages;
                 uint64_t* empty = isK ? &S.k_empty[st] : &S.v_empty[st];
                 uint64_t* full = isK ? &S.k_full[st] : &S.v_full[st];
-                uint8_t* dst = (isK ? S.k[st] : S.v[st]) + rsub * 128;
                 if (it >= kStages) ok = mbar_wait_warp(empty, ((it / kStages) - 1) & 1, abort_flag);
                 if (!ok) break;
-                if (it < n_plain) {
-                    const uint32_t d0 = smem_u32(dst) + sw0, d1 = smem_u32(dst) + sw1;
-                    const char* base = reinterpret_cast<const char*>(src);
-#pragma unroll
-                    for (int m = 0; m < 16; ++m) {
-                        const char* r0 = base + (uint64_t)(uint32_t)jrow[m].x * step;
-                        const char* r1 = base + (uint64_t)(uint32_t)jrow[m].y * step;
-                        cp_async16_at(d0 + m * 1024, r0);
-                        if constexpr (kD == 128) cp_async16_at(d0 + m * 1024 + kTileBytes / 2, r0 + 128);
-                        cp_async16_at(d1 + m * 1024, r1);
-                        if constexpr (kD == 128) cp_async16_at(d1 + m * 1024 + kTileBytes / 2, r1 + 128);
-                    }
-                } else {
-#pragma unroll 4
-                    for (int q = 0; q < 32; ++q) {
-                        const int j = list[it * 128 + 8 * (q >> 1) + (q & 1)];
-                        const __nv_bfloat16* row = src + (int64_t)max(j, 0) * row_stride;
-                        uint8_t* d = dst + (q >> 1) * 1024 + ((q & 1) ? sw1 : sw0);          // row r, chunk c ^ (r & 7)
-                        cp_async16(d, row, j >= 0 ? 16 : 0);
-                        if constexpr (kD == 128) cp_async16(d + kTileBytes / 2, row + 64, j >= 0 ? 16 : 0);
-                    }
-                }
+                gather(it);
                 cp_async_arrive(full);
                 if (it + 1 < n_iters) {
 #pragma unroll
