@@ -5,6 +5,7 @@
 //
 // Kernels
 //   decode_select_kernel   one cluster of CTAs per (batch, head) row: exact selection and the kept indices in ascending order
+//   decode_select_stream_kernel   the same for many rows, a CTA per row that reads it once
 //   decode_attn_kernel     per (batch, head, split of the kept list): every warp gathers a batch of K and V rows with all its
 //                          loads in flight, softmax per batch, warps combined in shared memory -> partial (m, l, o). The CTA
 //                          that finishes a row last (a ticket counter, no waiting) combines the row's partials -> o, lse
@@ -63,29 +64,16 @@ struct alignas(16) SelectShared {
     int need, count, bin;
 };
 
-// list: row bh's kept indices go to list + bh * list_stride. tickets (may be NULL): one counter per row, zeroed here.
-// kState: list points at the rows of an incremental state; count and weakest kept key go to the header before it.
+// The row bh, by the cluster's nrank CTAs, from the zeroed S.hist and S.ncand on; out: its list.
+// kState: the list is that of an incremental state; count and weakest kept key go to the header before it.
 template <int kKeys, bool kState>
-__global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_select_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep, int slice,
-                                                                       int* __restrict__ list, int64_t list_stride, int* __restrict__ tickets) {
-    extern __shared__ __align__(16) uint8_t select_smem[];
-    SelectShared& S = *reinterpret_cast<SelectShared*>(select_smem);
-    cg::cluster_group cluster = cg::this_cluster();
-    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int bh = blockIdx.x / nrank, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+__device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& cluster, int nrank, int rank, const float* __restrict__ delta, int64_t ld,
+                                           int N, int keep, int slice, int bh, int* __restrict__ out) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int j0 = rank * slice, n = max(0, min(slice, N - j0));
     // this warp's part of the slice: [i0, i1), `seg` (a multiple of 32) keys per warp
     const int seg = kKeys ? 32 * kKeys : (slice + kSelectThreads - 1) / kSelectThreads * 32;
     const int i0 = warp * seg, i1 = min(n, i0 + seg), sweeps = seg / 32;
-    for (int t = tid; t < (int)sizeof(S.hist) / 4; t += kSelectThreads) (&S.hist[0][0])[t] = 0;
-    if (tid == 0) S.ncand = 0;
-    pdl_enter(delta, list, tickets);
-    int* out = list + (size_t)bh * list_stride;
-    if (tickets && rank == 0 && tid == 0) tickets[bh] = 0;
-    if (!kState && keep >= N) {                // every key is kept
-        for (int i = tid; i < n; i += kSelectThreads) out[j0 + i] = j0 + i;
-        return;
-    }
     const uint32_t* src = reinterpret_cast<const uint32_t*>(delta + (size_t)bh * ld) + j0 + i0 + lane;
     // Keys beyond the row read as 0xFFFFFFFF, which no pass counts (the sign bit of the others is masked: delta > 0, and a
     // row that breaks this still yields `keep` distinct indices).
@@ -291,6 +279,253 @@ __global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_sel
         });
     }
     if (nrank > 1) cluster.sync();             // no CTA leaves while another may still read its shared memory
+}
+
+// list: row bh's kept indices go to list + bh * list_stride. tickets (may be NULL): one counter per row, zeroed here.
+template <int kKeys, bool kState>
+__global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_select_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep, int slice,
+                                                                       int* __restrict__ list, int64_t list_stride, int* __restrict__ tickets) {
+    extern __shared__ __align__(16) uint8_t select_smem[];
+    SelectShared& S = *reinterpret_cast<SelectShared*>(select_smem);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int bh = blockIdx.x / nrank, tid = threadIdx.x;
+    for (int t = tid; t < (int)sizeof(S.hist) / 4; t += kSelectThreads) (&S.hist[0][0])[t] = 0;
+    if (tid == 0) S.ncand = 0;
+    pdl_enter(delta, list, tickets);
+    int* out = list + (size_t)bh * list_stride;
+    if (tickets && rank == 0 && tid == 0) tickets[bh] = 0;
+    if (!kState && keep >= N) {                // every key is kept
+        for (int i = rank * slice + tid; i < min(N, (rank + 1) * slice); i += kSelectThreads) out[i] = i;
+        return;
+    }
+    select_row<kKeys, kState>(S, cluster, nrank, rank, delta, ld, N, keep, slice, bh, out);
+}
+
+// The same selection, one CTA per row, two on an SM, that reads the row once: a sample brackets the threshold (4.5 standard deviations to either side), the sweep
+// leaves two bits per key (above the bracket, in it or above), and of the keys inside, a few per cent of the row, the last ones that are kept are found as above. The
+// bits are then the row's list. A word of 32 keys costs some 30 instructions in all, where the histogram of all keys and three sweeps over registers took 880 per
+// 1024 and a shared-memory add per key; both kernels are bound by them. A bracket that misses (once in 10^5 rows) or holds too many equal keys sends the
+// row to select_row, which reads it again per sweep.
+// Selection, us, kernel above / this one, w = N / 16 and N / 4: 256 rows of 65536 keys 68.7 / 32.7 and 74.0 / 40.1, 128 rows of 131072 77.3 / 38.1 and 86.2 / 44.6, 512 rows of
+// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 13.9 / 15.5 and 15.8 / 19.3 (clusters).
+constexpr int kInside = 8192;                  // most keys in the bracket (expected: 6000 of 131072 at w = N / 4; with 6656 a row of 128 did not fit, which costs 110 us)
+constexpr int kStreamMinKeys = 8192, kStreamMaxKeys = 1 << 17;        // two bits per key of a row in shared memory: 32 KB
+struct alignas(16) StreamShared {
+    int hist[2048];
+    unsigned long long list[kInside], cand[kCandidates];
+    int scan[kSelectWarps], warp_kept[kSelectWarps];
+    uint32_t warp_min[kSelectWarps], warp_max[kSelectWarps];
+    int inside, ncand, bin[2], need, count;
+    unsigned long long weakest;
+};
+constexpr size_t kStreamHead = sizeof(StreamShared) > sizeof(SelectShared) ? sizeof(StreamShared) : sizeof(SelectShared);
+static size_t stream_smem(int N) { return kStreamHead + ((size_t)(N + 31) / 32 + 1) / 2 * 16; }
+
+template <bool kState, int kSample>
+__global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep,
+                                                                              int* __restrict__ list, int64_t list_stride, int* __restrict__ tickets) {
+    extern __shared__ __align__(16) uint8_t select_smem[];
+    StreamShared& S = *reinterpret_cast<StreamShared*>(select_smem);
+    uint2* mask = reinterpret_cast<uint2*>(select_smem + kStreamHead);             // per 32 keys: above the bracket (later: kept), in it or above
+    const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    for (int t = tid; t < 2048; t += kSelectThreads) S.hist[t] = 0;
+    if (tid == 0) { S.inside = 0; S.ncand = 0; S.bin[0] = S.bin[1] = -1; }
+    pdl_enter(delta, list, tickets);
+    int* out = list + (size_t)bh * list_stride;
+    if (tickets && tid == 0) tickets[bh] = 0;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(delta + (size_t)bh * ld);
+    auto range = [&](uint32_t& umin, uint32_t& umax) {                   // of the CTA (its barrier)
+        umin = __reduce_min_sync(0xffffffffu, umin);
+        umax = __reduce_max_sync(0xffffffffu, umax);
+        if (lane == 0) { S.warp_min[warp] = umin; S.warp_max[warp] = umax; }
+        __syncthreads();
+        umin = __reduce_min_sync(0xffffffffu, S.warp_min[lane]);
+        umax = __reduce_max_sync(0xffffffffu, S.warp_max[lane]);
+    };
+    // descending running count of the histogram: this thread's bins are top + 1 and top, `excl` keys lie above them. The bins are zeroed again
+    const int top = 2046 - 2 * tid;
+    auto scan = [&](int& excl, int2& c) {
+        c = *reinterpret_cast<const int2*>(S.hist + top);
+        *reinterpret_cast<int2*>(S.hist + top) = make_int2(0, 0);
+        int incl = c.x + c.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) S.scan[warp] = incl;
+        __syncthreads();
+        excl = __reduce_add_sync(0xffffffffu, lane < warp ? S.scan[lane] : 0) + incl - c.x - c.y;
+    };
+    // the sample: one key of every N / 4096, at a scattered place
+    uint32_t lo = 0u, hi = 0x7FFFFFFFu;                                   // keys above hi are kept, keys below lo are not
+    {
+        uint32_t u[kSample / kSelectThreads], umin = 0x7FFFFFFFu, umax = 0u;
+#pragma unroll
+        for (int t = 0; t < kSample / kSelectThreads; ++t) {
+            const uint32_t i = t * kSelectThreads + tid;
+            const uint32_t j = (uint32_t)((uint64_t)i * N / kSample) + (((i * 2654435761u) >> 16) * (uint32_t)(N / kSample) >> 16);
+            u[t] = src[j] & 0x7FFFFFFFu;
+            umin = min(umin, u[t]);
+            umax = max(umax, u[t]);
+        }
+        range(umin, umax);
+        const int shift = max(0, 21 - __clz((int)(umax - umin)));
+#pragma unroll
+        for (int t = 0; t < kSample / kSelectThreads; ++t) atomicAdd(&S.hist[(u[t] - umin) >> shift], 1);
+        __syncthreads();
+        int excl;
+        int2 c;
+        scan(excl, c);
+        const float q = (float)keep / (float)N, mid = q * kSample, dev = 4.5f * sqrtf(mid * (1.0f - q)) + 4.0f;
+        const int r0 = (int)(mid - dev), r1 = (int)(mid + dev) + 1;       // ranks (from 1) of the bracket's ends
+        auto holds = [&](int r) { return excl < r && r <= excl + c.x + c.y; };
+        if (holds(r0)) S.bin[0] = r0 <= excl + c.y ? top + 1 : top;
+        if (holds(r1)) S.bin[1] = r1 <= excl + c.y ? top + 1 : top;
+        __syncthreads();
+        if (S.bin[0] >= 0) hi = min(0x7FFFFFFFu, umin + ((uint32_t)(S.bin[0] + 1) << shift) - 1u);
+        if (S.bin[1] >= 0) lo = umin + ((uint32_t)S.bin[1] << shift);
+    }
+    // the sweep: a warp takes words of 32 consecutive keys
+    const int words = (N + 31) / 32, per = (words + kSelectWarps - 1) / kSelectWarps, w0 = min(words, warp * per), w1 = min(words, w0 + per);
+    for (int wb = w0; wb < w1; wb += 8) {
+        uint32_t u[8];
+        const uint32_t* at = src + wb * 32 + lane;
+        if (wb + 8 <= w1 && wb * 32 + 256 <= N) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u[k] = at[32 * k] & 0x7FFFFFFFu;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u[k] = wb + k < w1 && (wb + k) * 32 + lane < N ? at[32 * k] & 0x7FFFFFFFu : 0xFFFFFFFFu;      // (as an int below every key)
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t ba = __ballot_sync(0xffffffffu, (int)u[k] > (int)hi), bi = __ballot_sync(0xffffffffu, (int)u[k] >= (int)lo);
+            if (lane == 0 && wb + k < w1) mask[wb + k] = make_uint2(ba, bi);
+        }
+    }
+    __syncwarp();
+    // the bracket's keys, a lane per word
+    int kept = 0;
+    uint32_t bmin = 0x7FFFFFFFu, bmax = 0u;
+    for (int wb = w0; wb < w1; wb += 32) {
+        const uint2 m = wb + lane < w1 ? mask[wb + lane] : make_uint2(0u, 0u);
+        kept += __popc(m.x);
+        uint32_t in = m.y & ~m.x;
+        while (const uint32_t some = __ballot_sync(0xffffffffu, in != 0u)) {
+            int pos = 0;
+            if (lane == 0) pos = atomicAdd(&S.inside, __popc(some));
+            pos = __shfl_sync(0xffffffffu, pos, 0);
+            if (pos >= kInside) break;                                    // (too many: the row goes to select_row)
+            pos += __popc(some & below);
+            if (in && pos < kInside) {
+                const int j = (wb + lane) * 32 + __ffs(in) - 1;
+                const uint32_t u = src[j] & 0x7FFFFFFFu;
+                S.list[pos] = key_of(__uint_as_float(u), j);
+                bmin = min(bmin, u);
+                bmax = max(bmax, u);
+                in &= in - 1u;
+            }
+        }
+    }
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane == 0) S.warp_kept[warp] = kept;
+    range(bmin, bmax);
+    const int inside = S.inside;
+    int need = keep - __reduce_add_sync(0xffffffffu, S.warp_kept[lane]);
+    bool found = need >= 1 && need <= inside && inside <= kInside;       // (the same in every thread)
+    auto each = [&](auto&& f) {                                           // the bracket's keys
+        for (int e = tid; e < inside; e += kSelectThreads) f(S.list[e]);
+    };
+    if (found) {
+        const int shift = max(0, 21 - __clz((int)(bmax - bmin)));
+        each([&](unsigned long long x) { atomicAdd(&S.hist[((uint32_t)(x >> 32) - bmin) >> shift], 1); });
+        __syncthreads();
+        int excl;
+        int2 c;
+        scan(excl, c);
+        if (excl < need && need <= excl + c.x + c.y) {
+            const bool first = need <= excl + c.y;
+            S.bin[0] = first ? top + 1 : top;
+            S.need = need - excl - (first ? 0 : c.y);
+            S.count = first ? c.y : c.x;
+        }
+        __syncthreads();
+        const uint32_t bin = (uint32_t)S.bin[0];
+        const int count = S.count;
+        need = S.need;
+        found = count <= kCandidates;
+        if (found) {
+            each([&](unsigned long long x) { if (((uint32_t)(x >> 32) - bmin) >> shift == bin) S.cand[atomicAdd(&S.ncand, 1)] = x; });
+            __syncthreads();
+            if (tid < count) {
+                const unsigned long long k = S.cand[tid];
+                int above = 0;
+                for (int i = 0; i < count; ++i) above += S.cand[i] > k;
+                if (above == need - 1) S.weakest = k;
+            }
+            __syncthreads();
+        }
+    }
+    if (!found) {                                                         // (nothing of the row has been written yet)
+        __syncthreads();
+        SelectShared& G = *reinterpret_cast<SelectShared*>(select_smem);
+        for (int t = tid; t < (int)sizeof(G.hist) / 4; t += kSelectThreads) (&G.hist[0][0])[t] = 0;
+        if (tid == 0) G.ncand = 0;
+        cg::cluster_group cluster = cg::this_cluster();
+        select_row<0, kState>(G, cluster, 1, 0, delta, ld, N, keep, (N + 31) / 32 * 32, bh, out);
+        return;
+    }
+    const unsigned long long weakest = S.weakest;
+    each([&](unsigned long long x) {
+        if (x >= weakest) {
+            const uint32_t j = 0xFFFFFFFFu - (uint32_t)x;
+            atomicOr(&mask[j >> 5].x, 1u << (j & 31));
+        }
+    });
+    __syncthreads();
+    // the bits -> indices, every warp from the position its lower words leave it
+    kept = 0;
+    for (int w = w0 + lane; w < w1; w += 32) kept += __popc(mask[w].x);
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane == 0) S.warp_kept[warp] = kept;
+    __syncthreads();
+    int at = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_kept[lane] : 0);
+    const int last = (int)(0xFFFFFFFFu - (uint32_t)weakest);              // the weakest kept key
+    constexpr int kTurn = 2 * kInside / kSelectWarps;
+    int* buf = reinterpret_cast<int*>(S.list) + warp * kTurn;             // (its keys have been read)
+    for (int wb = w0; wb < w1; wb += 32) {                                // a lane per word: a word holds a few kept keys
+        uint32_t word = wb + lane < w1 ? mask[wb + lane].x : 0u;
+        int pos = __popc(word);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        const int all = __shfl_sync(0xffffffffu, pos, 31), j0 = (wb + lane) * 32;
+        pos -= __popc(word);
+        if (kState && wb + lane < w1 && last >> 5 == wb + lane) {
+            int* hdr = out - kStateHeader;
+            hdr[0] = keep;
+            hdr[1] = at + pos + __popc(word & ((1u << (last & 31)) - 1u));
+            hdr[2] = (int)(uint32_t)weakest;
+            hdr[3] = (int)(uint32_t)(weakest >> 32);
+        }
+        const bool turn = all <= kTurn;                                   // (the lanes' short runs meet in shared memory and leave as whole lines)
+        int* to = turn ? buf : out + at;
+        while (word) {
+            to[pos++] = j0 + __ffs(word) - 1;
+            word &= word - 1u;
+        }
+        if (turn) {
+            __syncwarp();
+            for (int i = lane; i < all; i += 32) out[at + i] = buf[i];
+            __syncwarp();
+        }
+        at += all;
+    }
 }
 
 // 16 bytes of a K, V or q row, widened to fp32
@@ -786,6 +1021,17 @@ static int launch_select(const Prob& P, const float* delta, int64_t ld, int* lis
     int nrank = 1;
     // the fewest CTAs whose registers hold a row; a row that needs a cluster gets more while all rows still run at once
     while (nrank < kSelectMaxCluster && ((int64_t)nrank * kCtaKeys < P.L || (nrank > 1 && 2ll * nrank * P.B * P.Hq <= 148))) nrank *= 2;
+    // The kernel that streams a row: where the rows do not all have a wave's registers (up to 296 rows of 16384 keys only with a window of an eighth, 256 rows of 16384
+    // keys, w = N / 16 and N / 4: 14.7 / 14.2 us, but 15.2 / 16.0), or one CTA holds a row of more than 16384 keys
+    const int64_t rows = (int64_t)P.B * P.Hq;
+    if (P.w < P.L && P.L >= kStreamMinKeys && P.L <= kStreamMaxKeys &&
+        (P.L > 16384 ? nrank == 1 || rows * nrank > 148 : rows > 296 || (rows > 148 && 8ll * P.w <= P.L))) {
+        auto stream = P.L > 65536 ? (state ? decode_select_stream_kernel<true, 8192> : decode_select_stream_kernel<false, 8192>)
+                                  : (state ? decode_select_stream_kernel<true, 4096> : decode_select_stream_kernel<false, 4096>);
+        // (state of the function, which other threads' calls share: always the limit)
+        if (cudaFuncSetAttribute(stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stream_smem(kStreamMaxKeys)) != cudaSuccess) return DMA_ERR_CUDA;
+        return launch_overlapped(stream, dim3((unsigned)rows), dim3(kSelectThreads), stream_smem(P.L), st, 1, delta, ld, P.L, P.w, list, list_stride, tickets);
+    }
     const int slice = ((P.L + nrank - 1) / nrank + 31) / 32 * 32;
     auto pick = [&](auto st_tag) {
         constexpr bool kState = decltype(st_tag)::value;

@@ -108,3 +108,29 @@ def test_selection_with_infinite_weights(N, w, share):
     assert torch.equal(idx.cpu().long(), want)
     state = dma.dma_decode_state_init(p, delta.cuda(), dma.dma_decode_state(p, "cuda"))
     assert dma.decode_state_sets(state, w) == [r.tolist() for r in want[0]]
+
+
+@pytest.mark.parametrize("N", [8192, 8193, 33000, 65537, 131072])
+@pytest.mark.parametrize("kind", ["random", "tied", "few", "ramp", "outlier", "infinite"])
+def test_selection_of_many_rows(N, kind):
+    """Rows that are streamed once between a sampled bracket: the kept indices (ascending) and the carried state's sets against a stable sort, for a
+    threshold at either end of the row, brackets that hold too many keys (equal ones) and rows whose bracket lies in one place."""
+    BH = 304
+    g = torch.Generator("cuda").manual_seed(N)
+    z = torch.randn(1, BH, N, generator=g, device="cuda")
+    delta = {"random": lambda: torch.exp(torch.nn.functional.softplus(z)), "tied": lambda: torch.full_like(z, 1.5),
+             "few": lambda: 1.0 + torch.floor(z.abs() * 2) / 7.0, "ramp": lambda: torch.exp(3.0 * torch.arange(N, device="cuda") / N + 1e-4 * z),
+             "outlier": lambda: torch.where(z.abs() > 4.2, 1e38, 1.0 + 1e-3 * torch.sigmoid(z)),
+             "infinite": lambda: torch.where(z > 1.5, float("inf"), torch.exp(z))}[kind]()
+    order = torch.sort(delta, dim=-1, descending=True, stable=True)[1]
+    K = torch.zeros(1, N, 1, 64, dtype=torch.bfloat16, device="cuda")
+    q = torch.zeros(1, BH, 64, dtype=torch.bfloat16, device="cuda")
+    for w in (1, N // 16, N // 4, N - 1):
+        want = torch.sort(order[..., :w], dim=-1)[0]
+        p = dma.problem(1, BH, 1, N, 64, w)
+        _, _, idx = dma.dma_decode(p, q, K, K, delta, want_idx=True)
+        assert torch.equal(idx.long(), want), w
+        state = dma.dma_decode_state_init(p, delta, dma.dma_decode_state(p, "cuda"))
+        rows = state.view(torch.int32).view(BH, -1)
+        assert (rows[:, 0] == w).all() and torch.equal(rows[:, 8:8 + w].long(), want[0]), w
+        assert torch.equal(torch.gather(rows[:, 8:8 + w], 1, rows[:, 1:2].long())[:, 0].long(), order[0, :, w - 1]), w    # the weakest kept key
