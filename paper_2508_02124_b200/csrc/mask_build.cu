@@ -4,7 +4,7 @@
 //
 // Kernels
 //   delta_kernel        V read once (HBM-bound); z, softplus, exp in a fixed fp32 operation order
-//   tree_block_kernel, tree_merge_kernel, expiry_tree_kernel
+//   tree_block_kernel, expiry_search_kernel (longer heads: tree_merge_kernel, expiry_tree_kernel)
 //                       selection as a rank tree: the passes of a merge sort of (delta bits, ~index) keys leave one bit per key and
 //                       level, and a key's expiry (the w-th smallest index among the keys that beat it) is a walk of log2(L) steps.
 //                       Heads of up to 4096 keys: sort, walk and bitmap in the one block kernel
@@ -454,13 +454,13 @@ __device__ __forceinline__ uint32_t bitmap_word(const int* last, int kt0, int n,
 // and keep their index in the low word.
 // kMode >= 0: the head is one block (Lc = its padded length <= kBlock) and the CTA goes on from the tree in shared memory: expiry (the modes of
 // expiry_of) and, with Tr > 0 (square tiles, at most 32), the bitmap. Otherwise sorted keys and levels go to global memory.
-// 1024 keys are bound by latency, each level a chain of probes or shuffles (8.5 us); 4096 on one SM by its integer pipe (issue slots 57 %
-// busy, 24 us), which is why few heads take blocks of 1024 and two merge launches more (launch_mask_build).
+// 1024 keys are bound by latency, each level a chain of probes or shuffles (7.7 us); 4096 on one SM by its integer pipe (issue slots 57 %
+// busy, 20 us), which is why few heads take blocks of 1024 (launch_mask_build).
 template <int kBlock, int kMode>
 __global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const float* __restrict__ delta, unsigned long long* __restrict__ sorted,
                                                                    uint2* __restrict__ lev, int L, int Lc, int m, int32_t* __restrict__ expiry,
                                                                    uint32_t* __restrict__ bitmap, int w, const int32_t* __restrict__ cu, int nseq,
-                                                                   int bm, int Tr, int causal, int64_t zero_words) {
+                                                                   int bm, int Tr, int causal, int64_t zero_words, int* __restrict__ idx) {
     constexpr int kPer = kBlock > 2048 ? 8 : 4, kWarpKeys = 32 * kPer, kWarpBit = kPer == 8 ? 8 : 7;
     static_assert(kWarpKeys == 1 << kWarpBit && kPer * kBlockThreads >= kBlock, "a thread's keys, a warp's keys");
     constexpr int kWords = kBlock / 32;
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const float* 
     unsigned long long* cur = sk;
     unsigned long long* nxt = sk + padded(kBlock);
     uint2* slev = reinterpret_cast<uint2*>(sk + 2 * padded(kBlock)); // [level][kWords]
-    pdl_enter_restrict(delta, sorted, lev, expiry, bitmap, cu);
+    pdl_enter_restrict(delta, sorted, lev, expiry, bitmap, cu, idx);
     if (zero_words) zero_share(bitmap, zero_words);
     // the word of position p of the block in the level of nodes of 2 << bit keys
     auto put_word = [&](int bit, int p, uint32_t before, uint32_t bits) {
@@ -553,7 +553,15 @@ __global__ void __launch_bounds__(kBlockThreads) tree_block_kernel(const float* 
         __syncthreads();
     }
     if constexpr (kMode < 0) {
-        for (int i = tid; i < nreal; i += kBlockThreads) sorted[(size_t)bh * Lc + base + i] = cur[padded(i)];
+        for (int i = tid; i < nreal; i += kBlockThreads) {
+            const unsigned long long k = cur[padded(i)];
+            if (idx) {                                               // for expiry_search_kernel: delta bits and key numbers apart
+                reinterpret_cast<uint32_t*>(sorted)[(size_t)bh * Lc + base + i] = (uint32_t)(k >> 32);
+                idx[(size_t)bh * Lc + base + i] = (int)(0xFFFFFFFFu - (uint32_t)k);
+            } else {
+                sorted[(size_t)bh * Lc + base + i] = k;
+            }
+        }
     } else {
         int* sexp = reinterpret_cast<int*>(nxt);
         for (int r = tid; r < L; r += kBlockThreads) {
@@ -650,6 +658,180 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
     expiry[(size_t)bh * L + j] = expiry_of<kMode>([&](int l, int q) { return lv[l * W + (q >> 5)]; }, r, j, L, w, m, cu, nseq);
 }
 
+// Heads of up to kSearchKeys keys: no levels above the blocks. A key's beaters are counted block by block: in its own block they are the entries before it, in any other
+// a binary search over the block's sorted delta bits, which the CTA holds in shared memory with the whole head's. (Equal bits beat it in blocks of lower
+// indices.) The block in which the running count reaches w holds the key's expiry, found by the walk down that block's own tree. A CTA takes the keys of one block, in
+// descending order, so that a warp's 32 searches read the same few words, and since a block's keys are whole key tiles, it writes their bits of the bitmap, too.
+// This replaces a merge launch per level, the walk from the root and the bitmap kernel, each a chain of dependent loads after a launch. Bound by the latency
+// of its own chain and, from 16 blocks on, by the searches ((blocks - 1) log2(block) reads per key). Mask build, us, before / now: 16 heads of 4096 keys 23.8 / 16.4,
+// 16 of 8192 36.4 / 26.6, 32 of 16384 59.8 / 48.9, of 32768 112 / 106, 128 of 16384 211 / 196, 8 of 5000 27.3 / 16.5; packed documents 26.7 / 20.6, 40.4 / 30.5, 70.1 / 61.8, 133 / 134.
+// (With the walk in global memory, a key after the other, 17.9, 27.0, 52.3, 114, 213.)
+constexpr int kSearchKeys = 32768;
+constexpr int kSearchThreads = 1024;
+// c[u]: how many entries of the sorted (descending) block of kBlock entries at A[u] lie above than[u]
+template <int kBlock, int kPer>
+__device__ __forceinline__ void count_above(const uint32_t* (&A)[kPer], const uint32_t (&than)[kPer], int (&c)[kPer]) {
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) c[u] = 0;
+#pragma unroll
+    for (int s = kBlock / 2; s; s >>= 1)
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) c[u] += A[u][c[u] + s - 1] > than[u] ? s : 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) c[u] += A[u][c[u]] > than[u] ? 1 : 0;
+}
+
+template <int kBlock, int kMode>
+__global__ void __launch_bounds__(kSearchThreads) expiry_search_kernel(const uint32_t* __restrict__ vals, const int* __restrict__ idx, const uint2* __restrict__ lev,
+                                                                       int32_t* __restrict__ expiry, uint32_t* __restrict__ bitmap, int L, int Lc, int w, int m,
+                                                                       const int32_t* __restrict__ cu, int nseq, int bm, int T, int Wd, int causal) {
+    constexpr int kPer = kBlock / kSearchThreads, kBits = kBlock == 4096 ? 12 : 10;
+    static_assert(kBlock == 1 << kBits && kPer >= 1, "block sizes of the sort");
+    extern __shared__ __align__(16) uint32_t sv[];                   // the head's sorted blocks, [nb][kBlock], zeros beyond its keys; expiry of the CTA's block; `last`
+    const int nb = gridDim.x, a = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = a * kBlock;
+    int* sexp = reinterpret_cast<int*>(sv + nb * kBlock);
+    int* last = sexp + kBlock;                                       // [kBlock / 32]
+    pdl_enter_restrict(vals, idx, lev, expiry, bitmap, cu);
+    int key[kPer];                                                   // the keys of ranks tid, tid + 1024, ... of the block
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) key[u] = base + u * kSearchThreads + tid < Lc ? idx[(size_t)bh * Lc + base + u * kSearchThreads + tid] : L;
+    for (int i = 4 * tid; i < nb * kBlock; i += 4 * kSearchThreads)
+        *reinterpret_cast<uint4*>(sv + i) = i < Lc ? *reinterpret_cast<const uint4*>(vals + (size_t)bh * Lc + i) : make_uint4(0u, 0u, 0u, 0u);
+    const int Wl = Lc / 32, Wt = nb * kBlock / 32;
+    uint2* tree = reinterpret_cast<uint2*>(sv);                      // [kBits][Wt], once the searches are over
+    // ones of the first c entries of the node that starts at s, l levels below its block
+    auto ones_at = [&](const uint2* level, int s, int c) { return ones_of([&](int q) { return level[q >> 5]; }, s, c); };
+    int s0[kPer], s1[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        s0[u] = 0;
+        s1[u] = L;
+        if (kMode == 1 && key[u] < L) {
+            int lo = 0, hi = nseq;                                   // largest s with cu[s] <= j
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (cu[mid] <= key[u]) lo = mid; else hi = mid;
+            }
+            s0[u] = min(max(cu[lo], 0), L - 1);
+            s1[u] = min(cu[lo + 1], L);
+        }
+    }
+    __syncthreads();
+    uint32_t v[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) v[u] = sv[base + u * kSearchThreads + tid];
+    // Packed sequences: of the beaters in the block in which the key's sequence starts, those of earlier sequences, the ones along the path of s0
+    int before[kPer];
+    if constexpr (kMode == 1) {
+        int c[kPer];
+        const uint32_t* A[kPer];
+        uint32_t than[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            A[u] = sv + s0[u] / kBlock * kBlock;
+            than[u] = v[u] - (s0[u] / kBlock < a ? 1u : 0u);
+        }
+        count_above<kBlock, kPer>(A, than, c);
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            before[u] = 0;
+            if (s0[u] / kBlock == a) c[u] = u * kSearchThreads + tid;
+            if (s0[u] % kBlock == 0) c[u] = 0;
+        }
+        const uint2* level = lev + ((size_t)bh * m + (m - kBits)) * Wl;
+        for (int l = 0; l < kBits; ++l, level += Wl) {
+            const int half = kBlock >> (l + 1);
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                if (c[u] == 0) continue;
+                const int ones = ones_at(level, s0[u] & ~(2 * half - 1), c[u]);
+                if (s0[u] & half) { before[u] += c[u] - ones; c[u] = ones; } else { c[u] -= ones; }
+            }
+        }
+    }
+    int seen[kPer], s[kPer], c[kPer], k[kPer];                       // beaters in the blocks so far (of the key's sequence); the block of the w-th, its beaters there, which of them
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        seen[u] = c[u] = k[u] = 0;
+        s[u] = -1;
+    }
+    for (int b = 0; b < nb; ++b) {
+        int cb[kPer];
+        if (b == a) {
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) cb[u] = u * kSearchThreads + tid;
+        } else {
+            const uint32_t less = b < a ? 1u : 0u;                   // equal bits of a lower index count: those above v - 1
+            const uint32_t* A[kPer];
+            uint32_t than[kPer];
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                A[u] = sv + b * kBlock;
+                than[u] = v[u] - less;
+            }
+            count_above<kBlock, kPer>(A, than, cb);
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            int early = 0;
+            if (kMode == 1) early = (b + 1) * kBlock <= s0[u] ? cb[u] : b * kBlock <= s0[u] ? before[u] : 0;
+            if (key[u] < L && s[u] < 0 && seen[u] + cb[u] - early >= w) {       // (padding takes no walk: its rank may lie beyond the block's entries)
+                s[u] = b * kBlock;
+                c[u] = cb[u];
+                k[u] = w - seen[u] + early;
+            }
+            seen[u] += cb[u] - early;
+        }
+    }
+    if constexpr (kMode != 2) {
+        // the blocks' trees take the place of their keys
+        __syncthreads();
+        const uint2* lv = lev + ((size_t)bh * m + (m - kBits)) * Wl;
+        for (int i = 2 * tid; i < kBits * Wl; i += 2 * kSearchThreads) {
+            const int l = i / Wl, q = i % Wl;
+            *reinterpret_cast<uint4*>(tree + l * Wt + q) = *reinterpret_cast<const uint4*>(lv + i);
+        }
+        __syncthreads();
+        const uint2* level = tree;
+        for (int l = 0; l < kBits; ++l, level += Wt) {               // k-th smallest among the first c entries of the node starting at s
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                if (s[u] < 0) continue;
+                const int ones = ones_at(level, s[u], c[u]), zeros = c[u] - ones;
+                if (k[u] <= zeros) c[u] = zeros; else { k[u] -= zeros; c[u] = ones; s[u] += kBlock >> (l + 1); }
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int j = key[u];
+        if (j >= L) continue;
+        // (s < 0: fewer than w keys beat it inside its sequence: never dropped)
+        const int e = s[u] < 0 ? s1[u] : kMode == 2 ? 0 : (kMode == 1 && s[u] >= s1[u]) ? s1[u] : max(j, s[u]);
+        sexp[j - base] = e;
+    }
+    __syncthreads();
+    for (int j = base + tid; j < min(L, base + kBlock); j += kSearchThreads) expiry[(size_t)bh * L + j] = sexp[j - base];
+    if (bm > 0) {                                                    // square tiles, a multiple of eight of them per block
+        const int n = kBlock / bm, kt0 = base / bm;
+        for (int kt = warp; kt < n; kt += kSearchThreads / 32) {
+            int top = 0;
+            for (int j = kt * bm + lane; j < min(L - base, kt * bm + bm); j += 32) top = max(top, sexp[j] > (causal ? base + j : 0) ? sexp[j] : 0);
+            top = __reduce_max_sync(0xffffffffu, top);
+            if (lane == 0) last[kt] = top;
+        }
+        __syncthreads();
+        // (the last block's CTA writes the rest of the row's words, too)
+        const int bytes = n / 8, all = a == nb - 1 ? Wd * 4 - kt0 / 8 : min(bytes, Wd * 4 - kt0 / 8);
+        uint8_t* out = reinterpret_cast<uint8_t*>(bitmap) + (size_t)bh * T * Wd * 4 + kt0 / 8;
+        for (int i = tid; i < T * all; i += kSearchThreads) {
+            const int qt = i / all, g = i % all;
+            out[(size_t)qt * Wd * 4 + g] = g < bytes ? (uint8_t)bitmap_word(last + 8 * g, kt0 + 8 * g, 8, qt, bm, causal) : (uint8_t)0;
+        }
+    }
+}
+constexpr size_t search_smem(int nb, int block) { return ((size_t)nb * block + block + block / 32) * 4; }
+
 __global__ void fill_i32_kernel(int32_t* p, size_t n, int32_t v, uint32_t* bitmap, int64_t bitmap_words) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_enter_restrict(p, bitmap);
@@ -723,7 +905,6 @@ __global__ void __launch_bounds__(128) bitmap_kernel(const int32_t* __restrict__
 }  // namespace
 
 constexpr int kStaticChunk = kChunk;
-constexpr int kFewWhole = 3072;              // padded keys of a head that one CTA takes whole although few heads leave SMs idle
 
 // levels of the rank tree over a head of Lc (a multiple of 256) keys: the smallest m with 2^m >= Lc
 static int tree_levels(int Lc) {
@@ -811,19 +992,22 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
         rc = launch_overlapped(fill_i32_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 1, expiry, n, P.L, bitmap, zero_words);
         if (rc) return rc;
     } else {
-        // rank tree: sorted blocks, one merge pass per further level, then one walk per key; or everything in the block kernel.
-        // Blocks of 4096 keys keep few SMs busy for long where there are few; mask build, us, before (256-key chunks, blocks of 4096) / now:
-        // 8 heads of 500 keys 14.4 / 8.4, 16 of 1000 18.6 / 12.1, 8 of 2048 20.2 / 16.7, 16 of 2500 24.1 / 22.5, 16 of 4096 26.5 / 23.9 (28.8 whole),
-        // 8 of 13000 36 / 33 (38 in blocks of 4096), 128 of 4096 68 / 48, 32 of 16384 73 / 60, of 65536 292 / 229. A cluster of four CTAs per
-        // 4096 keys, which merged and walked through distributed shared memory: 26.2 at 16 heads of 4096, 37 at 8 of 13000.
+        // rank tree: sorted blocks, then a search over the blocks and a walk in one of them per key (heads beyond kSearchKeys: one merge pass per further level and a
+        // walk from the root); or everything in the block kernel. Blocks of 4096 keys keep few SMs busy for long where there are few, and blocks of 1024 take more
+        // searches. Mask build, us, blocks of 1024 / 4096: 16 heads of 4096 keys 16.4 / 30.4, 16 of 8192 26.6 / 40.8, 32 of 6000 26.0 / 38.4, 16 of 16384 38 / 42, but 48 of 8192 43.5 / 41.4,
+        // 24 of 16384 57 / 50, 32 of 16384 69 / 49; blocks of 1024 / a head whole in one CTA: 8 heads of 2000 keys 14.3 / 16.9, 16 of 3000 16.0 / 23.5, 64 of 3000 25.3 / 27.7,
+        // but 128 of 2000 24.2 / 21.3, 128 of 3000 36.8 / 32.6
         const int Lc = nchunk * kChunk, m = tree_levels(Lc);
-        const bool few = (int64_t)BH * ((Lc + kSmallBlock - 1) / kSmallBlock) <= 2 * 148, whole = Lc <= (few ? kFewWhole : kBlockKeys);
+        const int64_t small_blocks = (int64_t)BH * ((Lc + kSmallBlock - 1) / kSmallBlock);
+        const bool few = small_blocks <= 2 * 148, whole = Lc <= (!few ? kBlockKeys : small_blocks > 200 ? 2 * kSmallBlock : kSmallBlock);
         const int per_block = whole ? (Lc <= kSmallBlock ? kSmallBlock : kBlockKeys) : few ? kSmallBlock : kBlockKeys;
         const bool fused_bitmap = whole && square && P.Tr <= 32;
         const size_t keys = (size_t)BH * Lc, Wl = (size_t)Lc / 32;
         auto* buf0 = reinterpret_cast<unsigned long long*>((char*)ws + kWsHeaderBytes);
         auto* buf1 = buf0 + keys;
         uint2* lev = reinterpret_cast<uint2*>(buf1 + keys);
+        const bool search = !whole && Lc <= kSearchKeys;
+        int* idx = search ? reinterpret_cast<int*>(buf1) : nullptr;
         const int mode = !whole ? -1 : cu ? 1 : P.causal ? 0 : 2;
         auto pick = [&](auto n) {
             constexpr int kN = decltype(n)::value;
@@ -833,16 +1017,30 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
         // (state of the function, which other threads' calls share: always the limit)
         if (cudaFuncSetAttribute(block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)block_smem(kBlockKeys, true)) != cudaSuccess) return DMA_ERR_CUDA;
         rc = launch_overlapped(block, dim3((Lc + per_block - 1) / per_block, BH), dim3(kBlockThreads), block_smem(per_block, whole), st, 1, bias, buf0, lev, P.L, Lc, m,
-                               expiry, fused_bitmap || zero_words ? bitmap : nullptr, P.w, cu, nseq, P.bm, fused_bitmap ? P.Tr : 0, P.causal, zero_words);
+                               expiry, fused_bitmap || zero_words ? bitmap : nullptr, P.w, cu, nseq, P.bm, fused_bitmap ? P.Tr : 0, P.causal, zero_words, idx);
         if (rc) return rc;
         if (fused_bitmap) return DMA_OK;
+        if (search) {
+            const int nb = (Lc + per_block - 1) / per_block;
+            const bool bits = square && P.bm <= per_block / 8 && per_block % (8 * P.bm) == 0;
+            auto pick_search = [&](auto n) {
+                constexpr int kN = decltype(n)::value;
+                return cu ? expiry_search_kernel<kN, 1> : P.causal ? expiry_search_kernel<kN, 0> : expiry_search_kernel<kN, 2>;
+            };
+            auto kern = per_block == kSmallBlock ? pick_search(std::integral_constant<int, kSmallBlock>{}) : pick_search(std::integral_constant<int, kBlockKeys>{});
+            // (state of the function, which other threads' calls share: always the limit)
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)search_smem(kSearchKeys / kBlockKeys, kBlockKeys)) != cudaSuccess) return DMA_ERR_CUDA;
+            rc = launch_overlapped(kern, dim3(nb, BH), dim3(kSearchThreads), search_smem(nb, per_block), st, 1, reinterpret_cast<const uint32_t*>(buf0), (const int*)idx, lev,
+                                   expiry, bitmap, P.L, Lc, P.w, m, cu, nseq, bits ? P.bm : 0, P.Tr, P.Wd, P.causal);
+            if (rc || bits) return rc;
+        }
         int l = m - (per_block == kSmallBlock ? 11 : 13);         // level of the nodes of two blocks
-        for (int R = per_block; !whole && R < Lc; R *= 2, --l) {
+        for (int R = per_block; !whole && !search && R < Lc; R *= 2, --l) {
             rc = launch_overlapped(tree_merge_kernel, dim3((Lc + kMergeOut - 1) / kMergeOut, BH), dim3(kMergeThreads), 0, st, 1, buf0, buf1, lev + (size_t)l * Wl, Lc, R, m);
             if (rc) return rc;
             std::swap(buf0, buf1);
         }
-        if (!whole) {
+        if (!whole && !search) {
             const dim3 grid((P.L + 255) / 256, BH);
             rc = launch_overlapped(cu ? expiry_tree_kernel<1> : P.causal ? expiry_tree_kernel<0> : expiry_tree_kernel<2>, grid, dim3(256), 0, st, 1, buf0, lev,
                                    expiry, P.L, Lc, P.w, m, cu, nseq);

@@ -69,3 +69,20 @@ def test_tiles(L, tile):
     ref = oracle.select_expiry(dl, L // 6)
     assert np.array_equal(e, ref)
     assert np.array_equal(bitmap, oracle.bitmap_from_expiry(ref, *tile)), tile
+
+
+@pytest.mark.parametrize("H,L", [(2, 4097), (2, 12000), (2, 32768), (2, 32769), (80, 4097), (80, 9000)])
+def test_heads_searched_block_by_block(H, L):
+    """Equal weights across blocks, documents that begin at, one behind and inside a block, a last block of one key, windows that are never reached; up to the longest
+    head whose blocks are searched and one key beyond."""
+    for w in (3, L // 3, L - 1):
+        dl, e, bitmap = build(H, L, w, seed=L + w, levels=300)
+        ref = oracle.select_expiry(dl, w)
+        assert np.array_equal(e, ref) and np.array_equal(bitmap, oracle.bitmap_from_expiry(ref)), w
+    cu = sorted({0, 1024, 1025, 4096, L - 1, L})
+    for w in (2, 700):
+        dl, e, bitmap = build(H, L, w, seed=L, levels=300, cu=cu)
+        ref = oracle.select_expiry_varlen(dl, w, cu)
+        assert np.array_equal(e, ref) and np.array_equal(bitmap, oracle.bitmap_from_expiry(ref)), w
+    dl, e, _ = build(H, L, L // 4, seed=3, levels=300, causal=0)
+    assert np.array_equal(e, oracle.select_noncausal(dl, L // 4))
