@@ -134,3 +134,20 @@ def test_selection_of_many_rows(N, kind):
         rows = state.view(torch.int32).view(BH, -1)
         assert (rows[:, 0] == w).all() and torch.equal(rows[:, 8:8 + w].long(), want[0]), w
         assert torch.equal(torch.gather(rows[:, 8:8 + w], 1, rows[:, 1:2].long())[:, 0].long(), order[0, :, w - 1]), w    # the weakest kept key
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,dtype", [(1, 1, 64, "fp32"), (3, 3, 128, "bf16"), (6, 2, 64, "bf16"), (32, 8, 128, "bf16"), (33, 11, 128, "fp32")])
+def test_delta_of_a_few_keys(Hq, Hkv, d, dtype):
+    """Ranges of 1 to 9 keys (up to 8 take a kernel of their own) have the bits of the whole range; heads that do not fill a CTA, groups of any size."""
+    g = torch.Generator().manual_seed(d + Hq)
+    B, N, td = 2, 40, {"bf16": torch.bfloat16, "fp32": torch.float32}[dtype]
+    V = torch.randn(B, N, Hkv, d, generator=g).to(td).cuda()
+    W, A = (torch.randn(Hq, d, generator=g) / d ** 0.5).cuda(), (torch.rand(Hq, generator=g) + 0.5).cuda()
+    p = dma.problem(B, Hq, Hkv, N, d, 8, dtype=td)
+    whole, part = torch.zeros(B, Hq, N, device="cuda"), torch.full((B, Hq, N), -1.0, device="cuda")
+    dma.dma_delta_range(p, V, W, A, whole, 0, N)
+    at = 0
+    for n in (1, 2, 7, 8, 9, 1):
+        dma.dma_delta_range(p, V, W, A, part, at, at + n)
+        at += n
+    assert bits_equal(part[..., :at], whole[..., :at].cpu().numpy()) and (part[..., at:] == -1.0).all()
