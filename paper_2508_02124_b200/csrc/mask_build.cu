@@ -9,6 +9,7 @@
 //                       level, and a key's expiry (the w-th smallest index among the keys that beat it) is a walk of log2(L) steps.
 //                       Heads of up to 4096 keys: sort, walk and bitmap in the one block kernel
 //   bitmap_square_kernel, bitmap_kernel   per key tile: union of the query-tile intervals its keys are kept in
+#include <algorithm>
 #include <mutex>
 #include <utility>
 #include <type_traits>
@@ -127,14 +128,14 @@ __device__ __forceinline__ void block_reduce(float (&p)[NB], int sub) {
 // parallelism: a warp requests ALL value rows of its NEXT tile (kPass 16-byte loads per lane) before it runs the chains of
 // the current one, W is staged once per CTA, and softplus / exp of tile t (one (row, head) pair per thread, from the z
 // values in shared memory) overlap the chains of tile t + 1 (two z buffers, one barrier per tile).
-template <typename T, int D>
-__global__ void __launch_bounds__(256, sizeof(T) == 2 ? 2 : 1) delta_kernel(const T* __restrict__ V, const float* __restrict__ W,
+// Three shapes (keys per tile, CTAs per SM): launch_delta.
+template <typename T, int D, int kRows, int kCtas>
+__global__ void __launch_bounds__(256, sizeof(T) == 2 ? kCtas : 1) delta_kernel(const T* __restrict__ V, const float* __restrict__ W,
                                                     const float* __restrict__ A, float* __restrict__ delta,
                                                     int L, int Hq, int G, int64_t vs_b, int64_t vs_l, int64_t vs_h,
                                                     int j_off, int64_t ld) {
     constexpr int LPR = D / 8;            // lanes per row
     constexpr int RPW = 32 / LPR;         // rows per warp and pass
-    constexpr int kRows = 128;
     constexpr int kPass = kRows / (8 * RPW);
     using Raw = typename RawOf<T>::type;
     extern __shared__ float smem[];
@@ -966,13 +967,19 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     if (j_end - j_begin <= kFewKeys)
         return launch_overlapped(delta_few_kernel<T, D>, dim3((P.Hq * (D / 8) + 127) / 128, j_end - j_begin, P.B), dim3(128), 0, st, 1, (const T*)V, W, A, bias, P.Hq, P.G,
                                  P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
-    // two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles grid-stride; short ranges (one appended key
-    // of a decoding step) get one CTA per tile
-    const int ntiles = (j_end - j_begin + 127) / 128;
-    int per_pair = (2 * 148 + P.Hkv * P.B - 1) / (P.Hkv * P.B);
-    per_pair = per_pair < 1 ? 1 : per_pair > ntiles ? ntiles : per_pair;
-    dim3 grid(per_pair, P.Hkv, P.B);
-    return launch_overlapped(delta_kernel<T, D>, grid, dim3(256), smem, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+    // Two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles grid-stride. Tiles of 64 keys where there are few
+    // (us, tiles of 128 / 64: 16 heads of 4096 keys 4.8 / 4.1, 8 of 2500 4.6 / 3.4, but 32 of 65536 50.9 / 53.2), and where a KV head has one query head, whose tiles are short work, tiles of 32
+    // and four CTAs per SM (16 heads of 8192 keys 13.2 / 10.2, but 32 / 8 heads of 16384 16.8 / 19.0)
+    const int64_t pairs = (int64_t)P.Hkv * P.B, tiles = pairs * ((j_end - j_begin + 127) / 128);
+    auto launch = [&](auto kern, int rows, int ctas) {
+        const int ntiles = (j_end - j_begin + rows - 1) / rows;
+        const int per_pair = std::min((int)((ctas * 148 + pairs - 1) / pairs), ntiles);
+        const size_t bytes = (size_t)P.G * (D + 2 * rows) * sizeof(float);
+        return launch_overlapped(kern, dim3(per_pair, P.Hkv, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+    };
+    if (tiles <= 4 * 148) return launch(delta_kernel<T, D, 64, 2>, 64, 2);
+    if (sizeof(T) == 2 && P.G == 1) return launch(delta_kernel<T, D, 32, 4>, 32, 4);
+    return launch(delta_kernel<T, D, 128, 2>, 128, 2);
 }
 
 // delta for the keys [j_begin, j_end) only, into rows of ld entries (a decoding cache that grows)
