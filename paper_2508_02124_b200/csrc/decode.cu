@@ -757,11 +757,10 @@ constexpr int kListSplit = 256;                     // most kept keys per CTA of
 
 __device__ __forceinline__ int state_stride(int w_cap) { return kStateHeader + ((w_cap + 3) & ~3); }
 
-// what the appended key N - 1 does to a row's set: 0 nothing, 1 appended (set not full), 2 replaces the weakest
-__device__ __forceinline__ int step_mode(const int* hdr, int w_cap, unsigned long long kn) {
-    const int count = hdr[0];
-    if (count < w_cap) return 1;
-    const unsigned long long kmin = ((unsigned long long)(unsigned)hdr[3] << 32) | (unsigned)hdr[2];
+// what the appended key does to a row's set (hdr: count, position and order key of the weakest kept key): 0 nothing, 1 appended (set not full), 2 replaces the weakest
+__device__ __forceinline__ int step_mode(const int4& hdr, int w_cap, unsigned long long kn) {
+    if (hdr.x < w_cap) return 1;
+    const unsigned long long kmin = ((unsigned long long)(unsigned)hdr.w << 32) | (unsigned)hdr.z;
     return kn > kmin ? 2 : 0;
 }
 
@@ -799,21 +798,28 @@ struct alignas(16) Weakest {
     int pos, unused;
 };
 
-// brings a row's state up to date with the appended key N - 1 (every thread of the CTA takes part). weak: the weakest keys of the
+// What the update of a row's state reads, requested before the row is combined
+struct StepState {
+    int4 hdr;                  // count, position and order key of the weakest kept key
+    float delta_new;
+    uint4 weak;                // lane s < 32: the weakest key of list s (Weakest)
+    __device__ __forceinline__ void load(const float* dl, const int* row, const Weakest* w, int N, int nsplit) {
+        hdr = *reinterpret_cast<const int4*>(row);
+        delta_new = dl[N - 1];
+        weak = w && (int)threadIdx.x < min(32, nsplit) ? *reinterpret_cast<const uint4*>(w + threadIdx.x) : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
+    }
+};
+
+// brings a row's state up to date with the appended key N - 1 (every thread of the CTA takes part, and has loaded x before a barrier). weak: the weakest keys of the
 // row's nsplit lists (NULL: the kept keys are scanned)
-__device__ __forceinline__ void decode_state_update(const float* __restrict__ delta, int64_t ld, int N, int w_cap,
-                                                    int* __restrict__ state, int bh, const Weakest* __restrict__ weak, int nsplit) {
-    const float* dl = delta + (size_t)bh * ld;
-    int* hdr = state + (size_t)bh * state_stride(w_cap);
+__device__ __forceinline__ void decode_state_update(const StepState& x, const float* dl, int N, int w_cap, int* hdr, const Weakest* weak, int nsplit) {
     int* kept = hdr + kStateHeader;
-    const int newj = N - 1, count = hdr[0], weakest = hdr[1];
-    const unsigned long long kn = key_of(dl[newj], newj);
-    const int mode = step_mode(hdr, w_cap, kn);
-    __syncthreads();                                   // every thread has read the header before anyone rewrites it
+    const int newj = N - 1, count = x.hdr.x, weakest = x.hdr.y;
+    const unsigned long long kn = key_of(x.delta_new, newj), kmin = ((unsigned long long)(unsigned)x.hdr.w << 32) | (unsigned)x.hdr.z;
+    const int mode = step_mode(x.hdr, w_cap, kn);
     if (mode == 0) return;
     if (mode == 1) {                                   // the appended key has the largest index: on equal delta it is the weakest
         if (threadIdx.x == 0) {
-            const unsigned long long kmin = ((unsigned long long)(unsigned)hdr[3] << 32) | (unsigned)hdr[2];
             kept[count] = newj;
             hdr[0] = count + 1;
             if (count == 0 || kn < kmin) { hdr[1] = count; hdr[2] = (int)(uint32_t)kn; hdr[3] = (int)(uint32_t)(kn >> 32); }
@@ -822,12 +828,10 @@ __device__ __forceinline__ void decode_state_update(const float* __restrict__ de
     }
     if (weak) {
         if (threadIdx.x < 32) {
-            unsigned long long best = ~0ull;
-            int pos = -1;
-            for (int s = threadIdx.x; s < nsplit; s += 32) {
-                const Weakest x = weak[(size_t)bh * nsplit + s];
-                if (x.key < best) { best = x.key; pos = x.pos; }
-            }
+            unsigned long long best = (unsigned long long)x.weak.y << 32 | x.weak.x;
+            int pos = (int)x.weak.z;
+            for (int s = threadIdx.x + 32; s < nsplit; s += 32)
+                if (weak[s].key < best) { best = weak[s].key; pos = weak[s].pos; }
             for (int o = 16; o; o >>= 1) {
                 const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, best, o);
                 const int p2 = __shfl_xor_sync(0xffffffffu, pos, o);
@@ -864,11 +868,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const
     const float* dl = delta + (size_t)bh * ld;
     const int* hdr = state + (size_t)bh * state_stride(w_cap);
     const int* kept = hdr + kStateHeader;
-    const int newj = N - 1, count = hdr[0];
+    const int4 head = *reinterpret_cast<const int4*>(hdr);
+    const int newj = N - 1, count = head.x;
     const int e = split * kSplit + tid;
     const int held = tid < kSplit && e < w_cap ? kept[e] : 0;          // (in flight together with the header)
-    const int mode = step_mode(hdr, w_cap, key_of(dl[newj], newj));
-    const int eff = count + (mode == 1 ? 1 : 0), weakest = hdr[1];
+    const int mode = step_mode(head, w_cap, key_of(dl[newj], newj));
+    const int eff = count + (mode == 1 ? 1 : 0), weakest = head.y;
     const int mine = (e >= count || (mode == 2 && e == weakest)) ? newj : held;
     if (tid < kSplit && e < eff) list[tid] = mine;
     // When the appended key replaces the weakest one, the new weakest is found here, where the kept keys are read anyway: the combine kernel
@@ -907,14 +912,40 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
     const int bh = blockIdx.x, c = threadIdx.x % D, g = threadIdx.x / D;     // group g takes the splits s = g, g + 8, ...
     pdl_enter(partial, o, lse, delta, state, weak);
     const float* p = partial + (size_t)bh * nsplit * (D + 2);
-    float mx = -INFINITY;
-    for (int s = g; s < nsplit; s += 8) mx = fmaxf(mx, p[(size_t)s * (D + 2) + D]);
-    float l = 0.0f, acc = 0.0f;
-    for (int s = g; s < nsplit; s += 8) {
-        const float ms = p[(size_t)s * (D + 2) + D];
-        const float f = ms == -INFINITY ? 0.0f : exp2f(ms - mx);
-        l += p[(size_t)s * (D + 2) + D + 1] * f;
-        acc += p[(size_t)s * (D + 2) + c] * f;
+    const float* dl = delta + (size_t)bh * ld;
+    int* hdr = state + (size_t)bh * state_stride(w_cap);
+    const Weakest* wk = weak ? weak + (size_t)bh * nsplit : nullptr;
+    // Everything the step needs is requested at once: the group's first splits, the header, the appended key's weight and the lists' weakest keys. (The maxima,
+    // then the sums, then the state, each a round trip to L2 behind the one before: 16 captured steps of 32 rows of 2048 kept keys 147 -> 134 us, of one row 101 -> 91, of 16 rows of
+    // 4973 164 -> 141.)
+    StepState x;
+    x.load(dl, hdr, wk, N, nsplit);
+    constexpr int kBatch = 4;                                  // splits of a group that are in flight together
+    float mx = -INFINITY, l = 0.0f, acc = 0.0f;
+    for (int s0 = g; s0 < nsplit; s0 += 8 * kBatch) {
+        float ms[kBatch], ls[kBatch], as[kBatch], m = mx;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const float* ps = p + (size_t)(s0 + 8 * u) * (D + 2);
+            const bool in = s0 + 8 * u < nsplit;
+            ms[u] = in ? ps[D] : -INFINITY;
+            ls[u] = in ? ps[D + 1] : 0.0f;
+            as[u] = in ? ps[c] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) m = fmaxf(m, ms[u]);
+        if (s0 != g && mx != -INFINITY) {
+            const float f = exp2f(mx - m);
+            l *= f;
+            acc *= f;
+        }
+        mx = m;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const float f = ms[u] == -INFINITY ? 0.0f : exp2f(ms[u] - mx);
+            l += ls[u] * f;
+            acc += as[u] * f;
+        }
     }
     s_o[g][c] = acc;
     if (c == 0) { s_m[g] = mx; s_l[g] = l; }
@@ -935,7 +966,7 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
         if (c == 0) lse[bh] = lt > 0.0f ? 0.6931471805599453f * (m_all + log2f(lt)) : -INFINITY;
     }
     // incremental decoding: the attention kernel has read the row's state, which can now take in the appended key
-    decode_state_update(delta, ld, N, w_cap, state, bh, weak, nsplit);
+    decode_state_update(x, dl, N, w_cap, hdr, wk, nsplit);
 }
 
 
