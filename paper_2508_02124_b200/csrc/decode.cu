@@ -673,18 +673,37 @@ __device__ __forceinline__ void combine_row(const float* __restrict__ partial, T
     __shared__ float s_m[8], s_l[8], s_o[8][D];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const float* p = partial + (size_t)bh * nsplit * (D + 2);
-    float mx = -INFINITY;
-    for (int s = g; s < nsplit; s += 8) mx = fmaxf(mx, __ldcg(&p[(size_t)s * (D + 2) + D]));
-    float l = 0.0f, acc[CPL];
+    float mx = -INFINITY, l = 0.0f, acc[CPL];
 #pragma unroll
     for (int c = 0; c < CPL; ++c) acc[c] = 0.0f;
-    for (int s = g; s < nsplit; s += 8) {
-        const float* ps = p + (size_t)s * (D + 2);
-        const float ms = __ldcg(&ps[D]);
-        const float f = ms == -INFINITY ? 0.0f : exp2f(ms - mx);
-        l += __ldcg(&ps[D + 1]) * f;
+    constexpr int kBatch = 4;                  // splits of a warp whose loads are in flight together (the maxima first, then the sums: one more round trip to L2)
+    for (int s0 = g; s0 < nsplit; s0 += 8 * kBatch) {
+        float ms[kBatch], ls[kBatch], as[kBatch][CPL], m = mx;
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) acc[c] += __ldcg(&ps[lane * CPL + c]) * f;
+        for (int u = 0; u < kBatch; ++u) {
+            const float* ps = p + (size_t)(s0 + 8 * u) * (D + 2);
+            const bool in = s0 + 8 * u < nsplit;
+            ms[u] = in ? __ldcg(&ps[D]) : -INFINITY;
+            ls[u] = in ? __ldcg(&ps[D + 1]) : 0.0f;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) as[u][c] = in ? __ldcg(&ps[lane * CPL + c]) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) m = fmaxf(m, ms[u]);
+        if (mx != -INFINITY) {
+            const float f = exp2f(mx - m);
+            l *= f;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) acc[c] *= f;
+        }
+        mx = m;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const float f = ms[u] == -INFINITY ? 0.0f : exp2f(ms[u] - mx);
+            l += ls[u] * f;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) acc[c] += as[u][c] * f;
+        }
     }
 #pragma unroll
     for (int c = 0; c < CPL; ++c) s_o[g][lane * CPL + c] = acc[c];
