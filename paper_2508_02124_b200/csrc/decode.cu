@@ -308,9 +308,9 @@ __global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_sel
 // 1024 and a shared-memory add per key; both kernels are bound by them. A bracket that misses (once in 10^5 rows) or holds too many equal keys sends the
 // row to select_row, which reads it again per sweep.
 // Selection, us, kernel above / this one, w = N / 16 and N / 4: 256 rows of 65536 keys 68.7 / 32.7 and 74.0 / 40.1, 128 rows of 131072 77.3 / 38.1 and 86.2 / 44.6, 512 rows of
-// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 13.9 / 15.5 and 15.8 / 19.3 (clusters).
+// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7, decoding 512 rows of 5000 (w = 300) 42.0 / 37.5; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 13.9 / 15.5 and 15.8 / 19.3 (clusters).
 constexpr int kInside = 8192;                  // most keys in the bracket (expected: 6000 of 131072 at w = N / 4; with 6656 a row of 128 did not fit, which costs 110 us)
-constexpr int kStreamMinKeys = 8192, kStreamMaxKeys = 1 << 17;        // two bits per key of a row in shared memory: 32 KB
+constexpr int kStreamMinKeys = 4096, kStreamMaxKeys = 1 << 17;        // two bits per key of a row in shared memory: 32 KB
 struct alignas(16) StreamShared {
     int hist[2048];
     unsigned long long list[kInside], cand[kCandidates];
