@@ -113,11 +113,16 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
         if (nrank > 1) {
             if (tid == 0) { S.umin = umin; S.umax = umax; }
             cluster.sync();
-            for (int q = 0; q < nrank; ++q) {
-                umin = min(umin, *cluster.map_shared_rank(&S.umin, q));
-                umax = max(umax, *cluster.map_shared_rank(&S.umax, q));
+            if (warp == 0) {                   // a lane per CTA
+                const int q = min(lane, nrank - 1);
+                umin = __reduce_min_sync(0xffffffffu, *cluster.map_shared_rank(&S.umin, q));
+                umax = __reduce_max_sync(0xffffffffu, *cluster.map_shared_rank(&S.umax, q));
+                if (lane == 0) { S.warp_min[0] = umin; S.warp_max[0] = umax; }
             }
-            cluster.sync();                    // (the words may be written again)
+            __syncthreads();
+            umin = S.warp_min[0];
+            umax = S.warp_max[0];
+            if (kKeys == 0) cluster.sync();    // (a sample's range may be followed by the true one: the words are written again)
         }
     };
     bool sampled = kKeys == 0 && sweeps > 16;
@@ -143,10 +148,14 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
         const int top = 2046 - 2 * tid;
         if (nrank > 1) {
             cluster.sync();
-            for (int q = 0; q < nrank; ++q) {
-                const int2 v = *reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, q) + top);
-                c0 += v.y;
-                c1 += v.x;
+            int2 v[kSelectMaxCluster];
+#pragma unroll
+            for (int q = 0; q < kSelectMaxCluster; ++q)
+                v[q] = q < nrank ? *reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, q) + top) : make_int2(0, 0);
+#pragma unroll
+            for (int q = 0; q < kSelectMaxCluster; ++q) {
+                c0 += v[q].y;
+                c1 += v[q].x;
             }
         } else {
             __syncthreads();
@@ -196,11 +205,21 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
             const unsigned long long* cand = S.cand;
             if (nrank > 1) {
                 cluster.sync();
-                int at = 0;
-                for (int q = 0; q < nrank; ++q) {
-                    const int nq = *cluster.map_shared_rank(&S.ncand, q);
-                    if (tid < nq) S.all[at + tid] = cluster.map_shared_rank(S.cand, q)[tid];
-                    at += nq;
+                if (warp < kCandidates / 32) {
+                    const int n_here = lane < nrank ? *cluster.map_shared_rank(&S.ncand, lane) : 0;
+                    unsigned long long x[kSelectMaxCluster];
+                    int nq[kSelectMaxCluster];
+#pragma unroll
+                    for (int q = 0; q < kSelectMaxCluster; ++q) {
+                        nq[q] = __shfl_sync(0xffffffffu, n_here, q);
+                        x[q] = tid < nq[q] ? cluster.map_shared_rank(S.cand, q)[tid] : 0ull;
+                    }
+                    int at = 0;
+#pragma unroll
+                    for (int q = 0; q < kSelectMaxCluster; ++q) {
+                        if (tid < nq[q]) S.all[at + tid] = x[q];
+                        at += nq[q];
+                    }
                 }
                 cand = S.all;
             }
@@ -249,7 +268,8 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
     if (nrank > 1) {
         if (warp == kSelectWarps - 1 && lane == 0) { S.gt = gtb + cgt; S.eq = eqb + ceq; }
         cluster.sync();
-        for (int q = 0; q < rank; ++q) { gtb += *cluster.map_shared_rank(&S.gt, q); eqb += *cluster.map_shared_rank(&S.eq, q); }
+        gtb += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&S.gt, lane) : 0);
+        eqb += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&S.eq, lane) : 0);
     }
     const uint32_t below = (1u << lane) - 1u;
     if (ceq == 0) {                            // (all but a few warps)
