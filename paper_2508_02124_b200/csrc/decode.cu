@@ -38,10 +38,11 @@ __device__ __forceinline__ unsigned long long key_of(float dl, int j) {
 // What bounds it is a chain of barriers and sweeps, not the row's bytes (read once), so the sweeps run on registers: a thread
 // holds kKeys keys, key t of lane i of a warp at 32 t + i of the warp's contiguous part, which is both coalesced and in index
 // order for the compaction. Rows of up to kCtaKeys keys take one CTA; longer ones a cluster, whose CTAs read each other's
-// histograms (one cluster barrier per pass, a histogram buffer per pass); rows beyond eight CTAs' registers are read again in
+// histograms (one cluster barrier per pass, a histogram buffer per pass; two bins to a word, and the barrier before the end only
+// waited for when the list is written: 8 rows of 65536 keys 12.2 -> 10.9 us, of 131072 16.4 -> 14.2 at w = N / 4); rows beyond eight CTAs' registers are read again in
 // every sweep (kKeys = 0), and their first range comes from a sample: a threshold in one of its end bins starts over with the
 // true range. Measured, kept list written (before: threshold only, and a scan of the delta row in the attention kernel):
-// 32 rows of 16384 keys 8.1 us (7.1), 256 rows of 65536 73 us (83 in four launches), 32 rows of 65536 13.9 us, where a
+// 32 rows of 16384 keys 8.1 us (7.1), 256 rows of 65536 73 us (83 in four launches), 32 rows of 65536 11.4 us, where a
 // cluster of two takes 16.8 and one CTA that reads the row again 52. A cluster is slow to start (1024 keys: 3.8 us on one CTA,
 // 7.1 on two, 34 on eight), hence only where the registers demand it.
 constexpr int kSelectThreads = 1024, kSelectWarps = kSelectThreads / 32;
@@ -147,15 +148,33 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
         int c0 = 0, c1 = 0;
         const int top = 2046 - 2 * tid;
         if (nrank > 1) {
-            cluster.sync();
-            int2 v[kSelectMaxCluster];
+            if constexpr (kKeys > 0) {
+                // (a bin holds at most 32768 of the CTA's keys: two bins per word, half of what crosses between the SMs)
+                __syncthreads();
+                const int2 mine = *reinterpret_cast<const int2*>(hist + top);
+                __syncthreads();
+                uint32_t* packed = reinterpret_cast<uint32_t*>(hist);
+                packed[tid] = (uint32_t)mine.x | (uint32_t)mine.y << 16;
+                cluster.sync();
+                uint32_t v[kSelectMaxCluster];
 #pragma unroll
-            for (int q = 0; q < kSelectMaxCluster; ++q)
-                v[q] = q < nrank ? *reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, q) + top) : make_int2(0, 0);
+                for (int q = 0; q < kSelectMaxCluster; ++q) v[q] = q < nrank ? cluster.map_shared_rank(packed, q)[tid] : 0u;
 #pragma unroll
-            for (int q = 0; q < kSelectMaxCluster; ++q) {
-                c0 += v[q].y;
-                c1 += v[q].x;
+                for (int q = 0; q < kSelectMaxCluster; ++q) {
+                    c0 += (int)(v[q] >> 16);
+                    c1 += (int)(v[q] & 0xFFFFu);
+                }
+            } else {
+                cluster.sync();
+                int2 v[kSelectMaxCluster];
+#pragma unroll
+                for (int q = 0; q < kSelectMaxCluster; ++q)
+                    v[q] = q < nrank ? *reinterpret_cast<const int2*>(cluster.map_shared_rank(hist, q) + top) : make_int2(0, 0);
+#pragma unroll
+                for (int q = 0; q < kSelectMaxCluster; ++q) {
+                    c0 += v[q].y;
+                    c1 += v[q].x;
+                }
             }
         } else {
             __syncthreads();
@@ -270,6 +289,7 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
         cluster.sync();
         gtb += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&S.gt, lane) : 0);
         eqb += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&S.eq, lane) : 0);
+        cluster.barrier_arrive();              // (the last read of another CTA's shared memory: the list is written before the wait at the end)
     }
     const uint32_t below = (1u << lane) - 1u;
     if (ceq == 0) {                            // (all but a few warps)
@@ -298,7 +318,7 @@ __device__ __forceinline__ void select_row(SelectShared& S, cg::cluster_group& c
             eqb += __popc(be);
         });
     }
-    if (nrank > 1) cluster.sync();             // no CTA leaves while another may still read its shared memory
+    if (nrank > 1) cluster.barrier_wait();     // no CTA leaves while another may still read its shared memory
 }
 
 // list: row bh's kept indices go to list + bh * list_stride. tickets (may be NULL): one counter per row, zeroed here.
@@ -328,7 +348,7 @@ __global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_sel
 // 1024 and a shared-memory add per key; both kernels are bound by them. A bracket that misses (once in 10^5 rows) or holds too many equal keys sends the
 // row to select_row, which reads it again per sweep.
 // Selection, us, kernel above / this one, w = N / 16 and N / 4: 256 rows of 65536 keys 68.7 / 32.7 and 74.0 / 40.1, 128 rows of 131072 77.3 / 38.1 and 86.2 / 44.6, 512 rows of
-// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7, decoding 512 rows of 5000 (w = 300) 42.0 / 37.5; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 13.9 / 15.5 and 15.8 / 19.3 (clusters).
+// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7, decoding 512 rows of 5000 (w = 300) 42.0 / 37.5; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 11.4 / 15.5 and 13.2 / 19.3 (clusters).
 constexpr int kInside = 8192;                  // most keys in the bracket (expected: 6000 of 131072 at w = N / 4; with 6656 a row of 128 did not fit, which costs 110 us)
 constexpr int kStreamMinKeys = 4096, kStreamMaxKeys = 1 << 17;        // two bits per key of a row in shared memory: 32 KB
 struct alignas(16) StreamShared {
