@@ -320,13 +320,16 @@ __global__ void __launch_bounds__(512) mask_bwd_reduce_kernel(const float* __res
 
 // ---- full sampling weights: W [Hq, C], C = Hkv * D channels of the value row feed every head ----------------
 // One CTA owns R consecutive keys of one batch with their whole value rows in shared memory (fp32):
-//   1  z[h][row]: warp per RW rows, lanes stride the channels, W read once per warp from L2
-//   2  dz[row][h] = dM delta A sigmoid(z), gs[h][row] = dM delta softplus(z)
-//   3  dW partial [h][col] = sum_rows dz v: a thread owns a column and walks the rows (no cross-thread sums)
-//   4  the value tile is overwritten by sum_h dz W[h][col], then added to dV
+//   1  z, dz = dM delta A sigmoid(z) and gs = dM delta softplus(z) of a (head, row) per lane
+//   2  dW partial [h][col] = sum_rows dz v: a thread owns columns and walks the rows (no cross-thread sums)
+//   3  dV += sum_h dz W[h][col]: a thread owns columns of 16 rows
 // partial [B * blocks][Hq][C + 1]; mask_bwd_full_reduce_kernel adds them in a fixed order.
+// Bound by the loads from shared memory and by latency, not by HBM (8 MB and 0.2 G fmas for 4096 keys, 16 heads of 512 channels), so each step takes
+// as many heads by rows (columns) per load as registers hold, all warps have a task, and dM, delta and dV are requested before the sums they meet. Both
+// kernels, us, against two heads of all rows per warp, one column per thread and dV summed up in the value tile: 4096 keys, 16 heads, 512 channels 27.3 -> 16.9,
+// 8192 38.6 -> 28.1, 4096 keys, 32 heads, 1024 channels 63.6 -> 48.0, 16384 278 -> 203. Half the threads, half the rows and two CTAs per SM: 18.9, 36.5, 58.7, 265.
 constexpr size_t kFullSmem = 200 * 1024;    // the most dynamic shared memory of a CTA
-constexpr int kFullThreads = 512;     // 16 warps: the kernel is bound by instruction issue and latency, not by registers
+constexpr int kFullThreads = 512;
 
 template <typename T, int RW>
 __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __restrict__ V, const float* __restrict__ W,
@@ -359,136 +362,147 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
     for (int i = tid; i < R * HqP; i += kFullThreads) sDz[i] = 0.0f;
     __syncthreads();
 
-    // z: a warp owns HB heads at a time and all R rows; lanes stride the channels, so W is read once per CTA and each
-    // value feeds HB fmas. The per-lane sums are added across lanes by a transposing butterfly (a lane keeps half of
-    // its rows at each step), which leaves row (lane mod RL) of every head in the lane.
-    constexpr int HB = 64 / R > 1 ? 64 / R : 1;     // 64 accumulators per thread
-    constexpr int RL = R < 32 ? R : 32;            // rows reduced together
-    for (int h0 = warp * HB; h0 < Hq; h0 += (kFullThreads / 32) * HB) {
-        float acc[HB][R];
+    // z: a warp takes four heads and eight rows, lanes stride the channels: 12 loads feed 32 fmas, and the butterfly that adds the lanes'
+    // sums (a lane keeps half of its accumulators at each step) leaves one (head, row) in each lane
+    constexpr int RB = R / 8;
+    for (int task = warp; task < (Hq + 3) / 4 * RB; task += kFullThreads / 32) {
+        const int h0 = task / RB * 4, r0 = task % RB * 8;
+        const int h = h0 + (lane >> 3), row = r0 + (lane & 7), j = j0 + row;
+        const size_t at = ((size_t)b * Hq + h) * L + j;
+        const bool in = h < Hq && j < L;
+        const float gd = in ? dM[at] * delta[at] : 0.0f, ah = in ? A[h] : 0.0f;
+        float acc[32];
 #pragma unroll
-        for (int q = 0; q < HB; ++q)
+        for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+        const float* wr[4];
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[q][r] = 0.0f;
+        for (int q = 0; q < 4; ++q) wr[q] = W + (size_t)min(h0 + q, Hq - 1) * C;
+#pragma unroll 4
         for (int col = lane; col < C; col += 32) {
-            float w[HB];
+            float w[4];
 #pragma unroll
-            for (int q = 0; q < HB; ++q) w[q] = h0 + q < Hq ? __ldg(W + (size_t)(h0 + q) * C + col) : 0.0f;
+            for (int q = 0; q < 4; ++q) w[q] = __ldg(wr[q] + col);
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float v = sV[(size_t)r * C + col];
+            for (int r = 0; r < 8; ++r) {
+                const float v = sV[(size_t)(r0 + r) * C + col];
 #pragma unroll
-                for (int q = 0; q < HB; ++q) acc[q][r] = fmaf(v, w[q], acc[q][r]);
+                for (int q = 0; q < 4; ++q) acc[q * 8 + r] = fmaf(v, w[q], acc[q * 8 + r]);
             }
         }
 #pragma unroll
-        for (int q = 0; q < HB; ++q) {
+        for (int keep = 16; keep >= 1; keep >>= 1) {
+            const bool up = (lane & keep) != 0;
 #pragma unroll
-            for (int base = 0; base < R; base += RL) {
-#pragma unroll
-                for (int keep = RL >> 1; keep >= 1; keep >>= 1) {
-                    const bool up = (lane & keep) != 0;
-#pragma unroll
-                    for (int r = 0; r < keep; ++r) {
-                        const float stay = up ? acc[q][base + r + keep] : acc[q][base + r];
-                        const float give = up ? acc[q][base + r] : acc[q][base + r + keep];
-                        acc[q][base + r] = stay + __shfl_xor_sync(0xffffffffu, give, keep);
-                    }
-                }
-#pragma unroll
-                for (int m = RL; m < 32; m <<= 1) acc[q][base] += __shfl_xor_sync(0xffffffffu, acc[q][base], m);
-                if (lane < RL && h0 + q < Hq) sZ[(h0 + q) * R + base + lane] = acc[q][base];
+            for (int i = 0; i < keep; ++i) {
+                const float stay = up ? acc[i + keep] : acc[i], give = up ? acc[i] : acc[i + keep];
+                acc[i] = stay + __shfl_xor_sync(0xffffffffu, give, keep);
             }
+        }
+        if (h < Hq) {
+            const float z = acc[0], e = expf(-fabsf(z));
+            sZ[h * R + row] = in ? gd * (fmaxf(z, 0.0f) + log1pf(e)) : 0.0f;
+            sDz[row * HqP + h] = in ? gd * ah * ((z >= 0.0f ? 1.0f : e) / (1.0f + e)) : 0.0f;
         }
     }
     __syncthreads();
 
-    for (int i = tid; i < Hq * R; i += kFullThreads) {
-        const int h = i / R, row = i % R, j = j0 + row;
-        float dz = 0.0f, gs = 0.0f;
-        if (j < L) {
-            const size_t at = ((size_t)b * Hq + h) * L + j;
-            const float gd = dM[at] * delta[at];
-            const float z = sZ[i];
-            const float e = expf(-fabsf(z));
-            gs = gd * (fmaxf(z, 0.0f) + log1pf(e));
-            dz = gd * A[h] * ((z >= 0.0f ? 1.0f : e) / (1.0f + e));
-        }
-        sDz[row * HqP + h] = dz;
-        sZ[i] = gs;
-    }
-    __syncthreads();
-
+    // dW: a thread owns two columns of eight heads (half a row apart, so that loads and stores are whole lines)
     float* out = partial + ((size_t)b * gridDim.x + blockIdx.x) * Hq * (C + 1);
-    for (int col = tid; col < C; col += kFullThreads) {
-        for (int hc = 0; hc < HqP; hc += 8) {
-            float acc[8];
+    const int half = C / 2;
+    for (int i = tid; i < half * (HqP / 8); i += kFullThreads) {
+        const int hc = i / half * 8, col = i % half;
+        float acc[8][2];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-            for (int row = 0; row < R; ++row) {
-                const float v = sV[(size_t)row * C + col];
-                const float4 a = *reinterpret_cast<const float4*>(sDz + row * HqP + hc);
-                const float4 c = *reinterpret_cast<const float4*>(sDz + row * HqP + hc + 4);
-                acc[0] = fmaf(a.x, v, acc[0]); acc[1] = fmaf(a.y, v, acc[1]); acc[2] = fmaf(a.z, v, acc[2]); acc[3] = fmaf(a.w, v, acc[3]);
-                acc[4] = fmaf(c.x, v, acc[4]); acc[5] = fmaf(c.y, v, acc[5]); acc[6] = fmaf(c.z, v, acc[6]); acc[7] = fmaf(c.w, v, acc[7]);
-            }
+        for (int q = 0; q < 8; ++q) acc[q][0] = acc[q][1] = 0.0f;
+#pragma unroll 8
+        for (int row = 0; row < R; ++row) {
+            const float v0 = sV[(size_t)row * C + col], v1 = sV[(size_t)row * C + half + col];
+            float a[8];
+            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(sDz + row * HqP + hc);
+            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(sDz + row * HqP + hc + 4);
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (hc + q < Hq) out[(size_t)(hc + q) * (C + 1) + col] = acc[q];
-        }
-    }
-    if (tid < Hq) {
-        float t = 0.0f;
-        for (int row = 0; row < R; ++row) t += sZ[tid * R + row];
-        out[(size_t)tid * (C + 1) + C] = t;
-    }
-    __syncthreads();   // every thread is done with the values of its columns' neighbours: the tile may be overwritten
-
-    for (int col = tid; col < C; col += kFullThreads) {
-        for (int hc = 0; hc < HqP; hc += 8) {
-            float w[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w[q] = hc + q < Hq ? __ldg(W + (size_t)(hc + q) * C + col) : 0.0f;
-            for (int row = 0; row < R; ++row) {
-                const float4 a = *reinterpret_cast<const float4*>(sDz + row * HqP + hc);
-                const float4 c = *reinterpret_cast<const float4*>(sDz + row * HqP + hc + 4);
-                float u = a.x * w[0];
-                u = fmaf(a.y, w[1], u); u = fmaf(a.z, w[2], u); u = fmaf(a.w, w[3], u);
-                u = fmaf(c.x, w[4], u); u = fmaf(c.y, w[5], u); u = fmaf(c.z, w[6], u); u = fmaf(c.w, w[7], u);
-                float* dst = sV + (size_t)row * C + col;
-                *dst = hc == 0 ? u : *dst + u;
+            for (int q = 0; q < 8; ++q) {
+                acc[q][0] = fmaf(a[q], v0, acc[q][0]);
+                acc[q][1] = fmaf(a[q], v1, acc[q][1]);
             }
         }
-    }
-    __syncthreads();
-
-    for (int i = tid; i < R * C8; i += kFullThreads) {
-        const int row = i / C8, ch = i % C8, j = j0 + row;
-        if (j < L) {
-            T* p = dV + b * vs_b + (int64_t)j * vs_l + (ch / D8) * vs_h + (ch % D8) * 8;
-            float cur[8];
-            load8f(p, cur);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) cur[c] += sV[(size_t)row * C + ch * 8 + c];
-            store8f(p, cur);
+        for (int q = 0; q < 8; ++q)
+            if (hc + q < Hq) {
+                out[(size_t)(hc + q) * (C + 1) + col] = acc[q][0];
+                out[(size_t)(hc + q) * (C + 1) + half + col] = acc[q][1];
+            }
+    }
+    for (int h = warp; h < Hq; h += kFullThreads / 32) {
+        float s = 0.0f;
+        for (int row = lane; row < R; row += 32) s += sZ[h * R + row];
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[(size_t)h * (C + 1) + C] = s;
+    }
+
+    // dV: a thread owns two neighbouring columns of RT rows, whose values it requests before it adds up the heads
+    constexpr int RT = R < 16 ? R : 16;
+    using T2 = typename std::conditional<std::is_same<T, float>::value, float2, __nv_bfloat162>::type;
+    for (int i = tid; i < half * (R / RT); i += kFullThreads) {
+        const int r0 = i / half * RT, col = i % half * 2;
+        T* p = dV + b * vs_b + (int64_t)(j0 + r0) * vs_l + (col / D) * vs_h + col % D;
+        T2 cur[RT];
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+            if (j0 + r0 + r < L) cur[r] = *reinterpret_cast<const T2*>(p + r * vs_l);
+        float u[RT][2];
+#pragma unroll
+        for (int r = 0; r < RT; ++r) u[r][0] = u[r][1] = 0.0f;
+#pragma unroll 2
+        for (int hc = 0; hc < HqP; hc += 4) {
+            float w[4][2];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float* wp = W + (size_t)min(hc + q, Hq - 1) * C + col;        // (heads beyond Hq have dz = 0)
+                w[q][0] = __ldg(wp);
+                w[q][1] = __ldg(wp + 1);
+            }
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const float4 a = *reinterpret_cast<const float4*>(sDz + (r0 + r) * HqP + hc);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    float s = a.x * w[0][c];
+                    s = fmaf(a.y, w[1][c], s);
+                    s = fmaf(a.z, w[2][c], s);
+                    u[r][c] += fmaf(a.w, w[3][c], s);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            if (j0 + r0 + r >= L) break;
+            if constexpr (std::is_same<T, float>::value) {
+                *reinterpret_cast<float2*>(p + r * vs_l) = make_float2(cur[r].x + u[r][0], cur[r].y + u[r][1]);
+            } else {
+                const float2 f = __bfloat1622float2(cur[r]);
+                *reinterpret_cast<__nv_bfloat162*>(p + r * vs_l) = __floats2bfloat162_rn(f.x + u[r][0], f.y + u[r][1]);
+            }
         }
     }
 }
 
-// dW [Hq][C] and dA [Hq] from partial [n][Hq][C + 1]: four groups of threads each add every fourth partial in index order,
-// then the group sums are added in group order.
+// dW [Hq][C] and dA [Hq] from partial [n][Hq][C + 1]: 16 groups of threads each add every 16th partial in index order, eight requested
+// at once, then the group sums are added.
 __global__ void __launch_bounds__(512) mask_bwd_full_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dW,
                                                                    float* __restrict__ dA, int n, int Hq, int C) {
-    __shared__ float part[4][128];
+    __shared__ float part[16][32];
     pdl_enter(partial, dW, dA);
-    const int h = blockIdx.y, c = blockIdx.x * 128 + (threadIdx.x & 127), grp = threadIdx.x >> 7;
+    const int h = blockIdx.y, lane = threadIdx.x & 31, c = blockIdx.x * 32 + lane, grp = threadIdx.x >> 5;
     float s = 0.0f;
     if (c <= C)
-        for (int t = grp; t < n; t += 4) s += partial[((size_t)t * Hq + h) * (C + 1) + c];
-    part[grp][threadIdx.x & 127] = s;
+#pragma unroll 8
+        for (int t = grp; t < n; t += 16) s += partial[((size_t)t * Hq + h) * (C + 1) + c];
+    part[grp][lane] = s;
     __syncthreads();
     if (grp == 0 && c <= C) {
-        const float tot = ((part[0][threadIdx.x] + part[1][threadIdx.x]) + part[2][threadIdx.x]) + part[3][threadIdx.x];
+        const float tot = add_groups(part, lane);
         if (c < C) dW[(size_t)h * C + c] = tot; else dA[h] = tot;
     }
 }
@@ -498,9 +512,8 @@ static bool full_fits(const Prob& P, int R) {
     return (R * C + R * HqP + (size_t)P.Hq * R) * sizeof(float) <= kFullSmem;
 }
 // rows per CTA: the largest of 64, 32, 16, 8 whose tile fits 200 KiB of shared memory (0: none does); 32 instead of 64 where
-// twice the CTAs still run at once, one per SM (both kernels, us, 64 / 32 rows, 16 heads, 512 channels: 4096 keys 38 / 27, but
-// 4800 keys, 75 CTAs, 39 / 48 and 8192 keys 40 / 52: two waves of half the length cost more than one). Not 16: the partial sums
-// weigh more (training step of 4096 keys 265 us with 32 rows, 272 with 16).
+// twice the CTAs still run at once, one per SM (both kernels, us, 64 / 32 rows, 16 heads, 512 channels: 4096 keys 27.8 / 16.9, but
+// 4800 keys, 75 CTAs, 28.2 / 30.0 and 8192 keys 28.1 / 31.1: two waves of half the length cost more than one).
 static int full_rows(const Prob& P) {
     int R = 64;
     while (R >= 8 && !full_fits(P, R)) R >>= 1;
@@ -566,7 +579,7 @@ static int launch_full(const Prob& P, const void* V, const float* W, const float
     const int rc = launch_overlapped(mask_bwd_full_kernel<T, RW>, dim3(nblk, P.B), dim3(kFullThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV,
                                      (float*)ws, P.L, P.Hq, P.Hkv, P.d, P.vs[0], P.vs[1], P.vs[2]);
     if (rc) return rc;
-    return launch_overlapped(mask_bwd_full_reduce_kernel, dim3((C + 1 + 127) / 128, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
+    return launch_overlapped(mask_bwd_full_reduce_kernel, dim3(C / 32 + 1, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B * nblk, P.Hq, C);
 }
 
 template <typename T>

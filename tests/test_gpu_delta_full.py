@@ -104,6 +104,27 @@ def test_mask_bwd_config3_and_reproducible():
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(B=2, Hq=10, Hkv=2, L=2500, d=64, dtype="bf16"),       # 64 rows per CTA, heads that fill neither four nor eight
+    dict(B=1, Hq=5, Hkv=5, L=45, d=64, dtype="fp32"),          # 32 rows, 320 channels, a last CTA of 13 rows
+    dict(B=1, Hq=32, Hkv=16, L=50, d=128, dtype="bf16"),       # 16 rows
+    dict(B=1, Hq=40, Hkv=40, L=19, d=128, dtype="fp32"),       # 8 rows (weights that no mask build takes)
+])
+def test_mask_bwd_rows_per_cta_and_head_remainders(kw):
+    case = wl.small(wl.CONFIGS["2"], name="full-delta-bwd-rows", w=16, **kw)
+    inp, W = wl.make_inputs(case), wl.full_delta_weights(case)
+    _, dl = oracle.delta_full(inp["V"].float().numpy(), W.numpy(), inp["A"].numpy())
+    g = torch.Generator().manual_seed(23)
+    dM = torch.randn(case.B, case.Hq, case.L, generator=g)
+    dV = torch.zeros(case.B, case.L, case.Hkv, case.d, dtype=case.torch_dtype, device=DEV)
+    _, dW, dA = dma.dma_mask_bwd(problem_of(case, flags=FULL), inp["V"].to(DEV), W.to(DEV), inp["A"].to(DEV), torch.tensor(dl, device=DEV), dM.to(DEV), dV)
+    torch.cuda.synchronize()
+    rV, rW, rA = oracle.mask_backward_full(inp["V"].double().numpy(), W.double().numpy(), inp["A"].double().numpy(), dM.double().numpy())
+    assert_close(dV, rV, case.dtype, f"{case.name}: dV")
+    assert_close(dW, rW, "fp32", f"{case.name}: dW_delta")
+    assert_close(dA, rA, "fp32", f"{case.name}: dA")
+
+
 def test_too_many_weights_for_shared_memory_is_refused():
     case = wl.small(wl.CONFIGS["2"], B=1, Hq=64, Hkv=8, L=128, d=128, w=32, name="full-delta-big")
     p = problem_of(case, flags=FULL)
