@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(128) delta_few_kernel(const T* __restrict__ V,
 // chains of D/8 heads at a time and adds them with a transposing butterfly (at each step a lane keeps half of its
 // values and hands the other half to its partner: the same additions as the plain butterfly, a quarter of the
 // shuffles), after which lane `sub` holds the dot product of head bitrev(sub) and carries that head's running sum.
-// kFullRows keys per CTA: 64, or 32 where 64 would leave SMs without a CTA (4096 keys, 16 heads, 512 channels: 15.5 -> 14.2 us).
+// kFullRows keys per CTA: 64, or 32 where 64 would leave SMs without a CTA (4096 keys, 16 heads, 512 channels: 15.5 -> 14.2 us when it was measured, with the weights' reads in conflict).
 constexpr size_t kFullSmem = 200 * 1024;     // the most dynamic shared memory of a CTA
 
 template <typename T, int D, int kFullRows>
@@ -261,7 +261,12 @@ __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V
 #pragma unroll
     for (int m = 1, t = LPR >> 1; m < LPR; m <<= 1, t >>= 1) mine |= (sub & m) ? t : 0;
     pdl_enter_restrict(V, W, A, delta);
-    for (int i = tid; i < HqP * C; i += 256) sW[i] = i < Hq * C ? W[i] : 0.0f;
+    // (a lane's eight weights in two halves, each next to the other lanes' same half: a group's 16-byte reads meet every bank once
+    // instead of half of them twice. us: 4096 keys, 16 heads, 512 channels 9.3 -> 7.4, 16384 keys 27.2 -> 19.4, 16384 keys, 8 heads of 1024 channels 51.1 -> 35.4)
+#pragma unroll 4
+    for (int i = tid; i < HqP * C / 4; i += 256)
+        reinterpret_cast<float4*>(sW)[i / (D / 4) * (D / 4) + (i & 1) * LPR + i % (D / 4) / 2] =
+            i < Hq * C / 4 ? __ldg(reinterpret_cast<const float4*>(W) + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     __syncthreads();
     for (int r0 = 0; r0 < kFullRows; r0 += kPass) {
         int r[2];
@@ -282,8 +287,8 @@ __global__ void __launch_bounds__(256) delta_full_kernel(const T* __restrict__ V
                 float p[2][LPR];
 #pragma unroll
                 for (int q = 0; q < LPR; ++q) {
-                    const float* wp = sW + (size_t)(hb + q) * C + hk * D + sub * 8;
-                    const float4 wa = *reinterpret_cast<const float4*>(wp), wb = *reinterpret_cast<const float4*>(wp + 4);
+                    const float* wp = sW + (size_t)(hb + q) * C + hk * D + sub * 4;
+                    const float4 wa = *reinterpret_cast<const float4*>(wp), wb = *reinterpret_cast<const float4*>(wp + D / 2);
                     const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
                     for (int n = 0; n < 2; ++n) {
