@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? kCtas : 1) delta_kernel(
     };
     Raw cur[kPass], nxt[kPass];
     request(blockIdx.x, cur);
-    for (int i = tid; i < G * D; i += 256) sW[i] = W[(size_t)hk * G * D + i];
+    // (a lane's eight weights in two halves, each next to the other lanes' same half: a group's 16-byte reads meet every bank once)
+    for (int i = tid; i < G * D; i += 256) sW[i / D * D + (i >> 2 & 1) * (D / 2) + i % D / 8 * 4 + (i & 3)] = W[(size_t)hk * G * D + i];
     __syncthreads();
     int buf = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 2 ? kCtas : 1) delta_kernel(
             float w[NB][8];
 #pragma unroll
             for (int q = 0; q < NB; ++q) {
-                const float4 wa = *reinterpret_cast<const float4*>(sW + (g0 + q) * D + sub * 8), wb = *reinterpret_cast<const float4*>(sW + (g0 + q) * D + sub * 8 + 4);
+                const float4 wa = *reinterpret_cast<const float4*>(sW + (g0 + q) * D + sub * 4), wb = *reinterpret_cast<const float4*>(sW + (g0 + q) * D + D / 2 + sub * 4);
                 w[q][0] = wa.x; w[q][1] = wa.y; w[q][2] = wa.z; w[q][3] = wa.w; w[q][4] = wb.x; w[q][5] = wb.y; w[q][6] = wb.z; w[q][7] = wb.w;
             }
             int mine = 0;                 // head of the block this lane ends up with: the low bits of sub, reversed
@@ -974,7 +975,8 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
                                  P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
     // Two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles grid-stride. Tiles of 64 keys where there are few
     // (us, tiles of 128 / 64: 16 heads of 4096 keys 4.8 / 4.1, 8 of 2500 4.6 / 3.4, but 32 of 65536 50.9 / 53.2), and where a KV head has one query head, whose tiles are short work, tiles of 32
-    // and four CTAs per SM (16 heads of 8192 keys 13.2 / 10.2, but 32 / 8 heads of 16384 16.8 / 19.0)
+    // and four CTAs per SM (16 heads of 8192 keys 13.2 / 10.2, but 32 / 8 heads of 16384 16.8 / 19.0). The weights' two halves, which came later, took
+    // 4 to 7 % off each: 4.1 -> 3.9, 50.9 -> 47.4, 10.2 -> 9.8, 16.7 -> 15.7
     const int64_t pairs = (int64_t)P.Hkv * P.B, tiles = pairs * ((j_end - j_begin + 127) / 128);
     auto launch = [&](auto kern, int rows, int ctas) {
         const int ntiles = (j_end - j_begin + rows - 1) / rows;
