@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(512) mask_bwd_reduce_kernel(const float* __res
                                                               int Hkv, int G, int nblk) {
     __shared__ float part[16][32];
     pdl_enter(partial, dW, dA);
-    const int h = blockIdx.y, hk = h / G, g = h % G, lane = threadIdx.x & 31, c = blockIdx.x * 32 + lane, grp = threadIdx.x >> 5;
+    const int h = blockIdx.x, hk = h / G, g = h % G, lane = threadIdx.x & 31, c = blockIdx.y * 32 + lane, grp = threadIdx.x >> 5;
     const int total = B * nblk;
     float s = 0.0f;
     if (c <= D)
@@ -570,7 +570,7 @@ static int launch_typed(const Prob& P, const void* V, const float* W, const floa
     const int rc = launch_overlapped(kern, dim3(nblk, P.Hkv, P.B), dim3(kThreads), smem, st, 1, (const T*)V, W, A, delta, dM, (T*)dV, (float*)ws, P.L, P.Hq,
                                      P.G, P.vs[0], P.vs[1], P.vs[2]);
     if (rc) return rc;
-    return launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(D / 32 + 1, P.Hq), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G,
+    return launch_overlapped(mask_bwd_reduce_kernel<D>, dim3(P.Hq, D / 32 + 1), dim3(512), 0, st, 1, (const float*)ws, dW, dA, P.B, P.Hkv, P.G,
                              nblk);
 }
 
