@@ -332,8 +332,8 @@ __global__ void __launch_bounds__(512) mask_bwd_reduce_kernel(const float* __res
 // partial [B * blocks][Hq][C + 1]; mask_bwd_full_reduce_kernel adds them in a fixed order.
 // Bound by the loads from shared memory and by latency, not by HBM (8 MB and 0.2 G fmas for 4096 keys, 16 heads of 512 channels), so each step takes
 // as many heads by rows (columns) per load as registers hold, all warps have a task, and dM, delta and dV are requested before the sums they meet. Both
-// kernels, us, against two heads of all rows per warp, one column per thread and dV summed up in the value tile: 4096 keys, 16 heads, 512 channels 27.3 -> 16.9,
-// 8192 38.6 -> 28.1, 4096 keys, 32 heads, 1024 channels 63.6 -> 48.0, 16384 278 -> 203. Half the threads, half the rows and two CTAs per SM: 18.9, 36.5, 58.7, 265.
+// kernels, us, against two heads of all rows per warp, one column per thread and dV summed up in the value tile: 4096 keys, 16 heads, 512 channels 27.3 -> 17.0,
+// 8192 38.6 -> 28.6, 4096 keys, 32 heads, 1024 channels 63.6 -> 49.0, 16384 278 -> 209. Half the threads, half the rows and two CTAs per SM: 18.9, 36.5, 58.7, 265.
 constexpr size_t kFullSmem = 200 * 1024;    // the most dynamic shared memory of a CTA
 constexpr int kFullThreads = 512;
 
@@ -460,14 +460,19 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
         float u[RT][2];
 #pragma unroll
         for (int r = 0; r < RT; ++r) u[r][0] = u[r][1] = 0.0f;
-#pragma unroll 2
-        for (int hc = 0; hc < HqP; hc += 4) {
+#pragma unroll 1
+        for (int hc = 0; hc < HqP; hc += 4) {             // (unrolled it spills: 4096 keys 17.0 -> 18.1 us)
             float w[4][2];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float* wp = W + (size_t)min(hc + q, Hq - 1) * C + col;        // (heads beyond Hq have dz = 0)
+                const float* wp = W + (size_t)min(hc + q, Hq - 1) * C + col;
                 w[q][0] = __ldg(wp);
                 w[q][1] = __ldg(wp + 1);
+            }
+            if (hc + 4 > Hq) {             // (heads beyond Hq have dz = 0, but the last head's weights may be infinite)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (hc + q >= Hq) w[q][0] = w[q][1] = 0.0f;
             }
 #pragma unroll
             for (int r = 0; r < RT; ++r) {

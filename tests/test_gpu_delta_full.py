@@ -125,6 +125,23 @@ def test_mask_bwd_rows_per_cta_and_head_remainders(kw):
     assert_close(dA, rA, "fp32", f"{case.name}: dA")
 
 
+def test_mask_bwd_infinite_weight_in_the_last_head():
+    """The heads that pad a group of four or eight must not turn the last head's infinity into NaN: dV is inf where sigmoid(z) = 1."""
+    case = wl.small(wl.CONFIGS["2"], B=1, Hq=5, Hkv=1, L=40, d=64, dtype="fp32", w=16, name="full-delta-bwd-inf")
+    V, W, A = wl.make_inputs(case)["V"], wl.full_delta_weights(case), torch.ones(5)
+    V[..., 7] = 1.0
+    W[4, 7] = float("inf")
+    dM = torch.ones(1, 5, 40)
+    dV = torch.zeros(1, 40, 1, 64, device=DEV)
+    dma.dma_mask_bwd(problem_of(case, flags=FULL), V.to(DEV), W.to(DEV), A.to(DEV), torch.ones(1, 5, 40, device=DEV), dM.to(DEV), dV)
+    torch.cuda.synchronize()
+    assert bool(torch.isposinf(dV[..., 7]).all())
+    z = torch.einsum("lc,hc->hl", V[0, :, 0].double(), W.double())
+    ref = torch.einsum("hl,hc->lc", torch.sigmoid(z), W.double())
+    keep = torch.arange(64) != 7
+    assert_close(dV[0, :, 0][:, keep.to(DEV)], ref[:, keep].numpy(), "fp32", f"{case.name}: dV")
+
+
 def test_too_many_weights_for_shared_memory_is_refused():
     case = wl.small(wl.CONFIGS["2"], B=1, Hq=64, Hkv=8, L=128, d=128, w=32, name="full-delta-big")
     p = problem_of(case, flags=FULL)
