@@ -504,6 +504,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // (the entry before the last one first: a wait for a phase that is two ahead would not wait)
             if (ok && n_iters > 1) ok = mbar_wait_warp(&S.o_done[a ^ 1], ((n_iters - 2) >> 1) & 1, abort_flag);
             if (ok && n_iters > 0) ok = mbar_wait_warp(&S.o_done[a], ((n_iters - 1) >> 1) & 1, abort_flag);
+            // (no entry at all: nothing above has waited for the load of Q, whose buffer is written next)
+            if (ok && n_iters == 0) ok = mbar_wait_warp(&S.q_full, 0, abort_flag);
         } else if (ok && exists && n_used > 0) {
             ok = mbar_wait_warp(&S.o_done[w], (n_used - 1) & 1, abort_flag);
         }

@@ -111,3 +111,52 @@ def test_pairs_whose_tiles_use_different_key_tiles(d):
         assert float((O.float() - out["O"]).abs().max()) <= 3e-2 and float((lse - out["lse"]).abs().max()) <= 1e-3 * max(1.0, float(out["lse"].abs().max()))
         bits = out.setdefault("bits", (O[0], lse[0]))
         assert all(torch.equal(x, bits[0]) for x in O) and all(torch.equal(x, bits[1]) for x in lse), (B, flags)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,skip", [(1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (32, 0)])      # one query tile per CTA, two, two
+@pytest.mark.parametrize("path", ["tiles", "lists", "chunk", "noncausal"])
+def test_query_tiles_without_keys(path, B, skip, d):
+    """A caller's mask (padding) may leave whole query tiles, pairs of them or a head without a key: O is exactly zero there and lse -inf, whatever Q
+    holds; the other rows are as ever."""
+    L, gone = 1100, [(256, 512), (1024, 1100)]
+    case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=1, L=L, w=300, d=d, name=f"no keys {path} d{d}")
+    inp = wl.make_inputs(case)
+    inp["Q"] = inp["Q"] * 8.0
+    dl = oracle_mask(case, inp)[0]
+    if path == "noncausal":
+        e = oracle.select_noncausal(dl, case.w)
+        e[:, 1] = 0                                                        # (the second head keeps nothing)
+    else:
+        e = oracle.select_expiry_varlen(dl, case.w, [0, 256, 512, 1024, L])
+        for a, b in gone:
+            e[..., a:b] = np.arange(a, b)
+    bitmap = torch.from_numpy(oracle.bitmap_from_expiry(e).view(np.int32)).to(DEV).repeat(B, 1, 1, 1)
+    flags = {"tiles": dma.DMA_FLAG_TILE_PATH, "lists": dma.DMA_FLAG_COMPACT_KV}.get(path, 0) | skip
+    p = dma.problem(B, 2, 1, L, d, case.w, flags=flags, causal=int(path != "noncausal"))
+    Q, K, V = (inp[k].to(DEV).repeat(B, 1, 1, 1) for k in ("Q", "K", "V"))
+    bias, expiry = (torch.from_numpy(np.ascontiguousarray(x)).to(DEV).repeat(B, 1, 1) for x in (dl, e))
+    first = 256 if path == "chunk" else 0
+    empty = np.zeros(L, bool)
+    if path != "noncausal":
+        for a, b in gone:
+            empty[a:b] = True
+    rows = np.flatnonzero(~empty[first:]).astype(np.int64)
+    Or, lr = oracle.forward(*(f64(inp[k]) for k in ("Q", "K", "V")), dl.astype(np.float64), expiry=e, rows=(rows + first).astype(np.int32),
+                            causal=path != "noncausal")
+    heads = [0] if path == "noncausal" else [0, 1]
+    for _ in range(3):
+        O, lse = torch.full_like(Q[:, first:], float("nan")), torch.zeros(B, 2, L - first, device=DEV)
+        if path == "chunk":
+            dma.dma_attn_fwd_chunk(p, first, Q[:, first:].contiguous(), K, V, bias, expiry, O=O, lse=lse)
+        else:
+            dma.dma_attn_fwd(p, Q, K, V, bias, expiry, bitmap, O=O, lse=lse)
+        torch.cuda.synchronize()
+        at = torch.from_numpy(np.flatnonzero(empty[first:])).to(DEV)
+        assert bool((O[:, at] == 0).all()) and bool(torch.isneginf(lse[:, :, at]).all())
+        if path == "noncausal":
+            assert bool((O[:, :, 1] == 0).all()) and bool(torch.isneginf(lse[:, 1]).all())
+        assert all(torch.equal(x, O[0]) for x in O)
+        live = torch.from_numpy(rows).to(DEV)
+        assert_close(O[:1, live][:, :, heads], np.asarray(Or)[:, :, heads], case.dtype, f"{case.name}: O")
+        assert_close(lse[:1, heads][:, :, live], np.asarray(lr)[:, heads], case.dtype, f"{case.name}: lse", lse=True)
