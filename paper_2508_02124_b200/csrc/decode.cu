@@ -5,7 +5,7 @@
 //
 // Kernels
 //   decode_select_kernel   one cluster of CTAs per (batch, head) row: exact selection and the kept indices in ascending order
-//   decode_select_stream_kernel   the same for many rows, a CTA per row that reads it once
+//   decode_select_stream_kernel   the same for many rows and rows of one CTA's registers, a CTA per row that reads it once
 //   decode_attn_kernel     per (batch, head, split of the kept list): every warp gathers a batch of K and V rows with all its
 //                          loads in flight, softmax per batch, warps combined in shared memory -> partial (m, l, o). The CTA
 //                          that finishes a row last (a ticket counter, no waiting) combines the row's partials -> o, lse
@@ -343,35 +343,42 @@ __global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_sel
 }
 
 // The same selection, one CTA per row, two on an SM, that reads the row once: a sample brackets the threshold (4.5 standard deviations to either side), the sweep
-// leaves two bits per key (above the bracket, in it or above), and of the keys inside, a few per cent of the row, the last ones that are kept are found as above. The
-// bits are then the row's list. A word of 32 keys costs some 30 instructions in all, where the histogram of all keys and three sweeps over registers took 880 per
-// 1024 and a shared-memory add per key; both kernels are bound by them. A bracket that misses (once in 10^5 rows) or holds too many equal keys sends the
-// row to select_row, which reads it again per sweep.
-// Selection, us, kernel above / this one, w = N / 16 and N / 4: 256 rows of 65536 keys 68.7 / 32.7 and 74.0 / 40.1, 128 rows of 131072 77.3 / 38.1 and 86.2 / 44.6, 512 rows of
-// 32768 53.5 / 36.6 and 57.4 / 43.4, 32 rows of 24000 11.3 / 10.0 and 11.8 / 11.7, decoding 512 rows of 5000 (w = 300) 42.0 / 37.5; but 32 rows of 16384 7.6 / 8.0 and 7.9 / 9.2, 32 of 65536 11.4 / 15.5 and 13.2 / 19.3 (clusters).
-constexpr int kInside = 8192;                  // most keys in the bracket (expected: 6000 of 131072 at w = N / 4; with 6656 a row of 128 did not fit, which costs 110 us)
-constexpr int kStreamMinKeys = 4096, kStreamMaxKeys = 1 << 17;        // two bits per key of a row in shared memory: 32 KB
+// leaves two bits per key (above the bracket, in it or above), the keys inside, a few per cent of the row, are gathered in index order, and the last of them that
+// is kept is found as above. The bits are then the row's list. A word of 32 keys costs some 30 instructions in all, where the histogram of all keys and
+// three sweeps over registers took 880 per 1024 and a shared-memory add per key; both kernels are bound by them.
+// Weights that crowd: a bracket end whose bin holds more than kHeavy of the sample is narrowed among that bin's samples; where the bracket is one bit pattern
+// (equal weights), its first keys are kept by their bits alone, however many there are; and a bracket that misses, or holds more than kInside keys
+// of several patterns, is narrowed by a histogram of the row's keys in it and swept again. Units of 32 words go around the warps, so that a
+// bracket or a list that lies in one place of the row is not one warp's work.
+// Carried state taken up from such a row, us, kernel above / this one, at w = 64, N / 16, N / 4, N / 2, N - 1: 256 rows of 65536 keys 57 / 25, 65 / 30, 71 / 35, 79 / 39,
+// 74 / 44, all weights equal 56 / 22 .. 70 / 41, ten values 67 / 28 .. 102 / 42, weights that rise along the row 57 / 26 .. 76 / 42 (before units, narrowing and the
+// bits of equal weights: random 23 .. 160, equal 100 .. 114, ten values 26 .. 143, rising 28 .. 167); 148 rows of 131072 random 70 / 26 .. 88 / 55.
+constexpr int kInside = 8192;                  // most keys gathered from the bracket (expected: 6000 of 131072 at w = N / 4)
+constexpr int kHeavy = 128;                    // (of 4096 or 8192 samples, where an ordinary row has ten in its fullest bin)
+constexpr int kStreamMinKeys = 4097, kStreamMaxKeys = 1 << 17;        // (more keys than the sample;) two bits per key of a row in shared memory: 32 KB
+constexpr int kMaxUnits = kStreamMaxKeys / 1024;
 struct alignas(16) StreamShared {
     int hist[2048];
     unsigned long long list[kInside], cand[kCandidates];
-    int scan[kSelectWarps], warp_kept[kSelectWarps];
+    int above[kMaxUnits], inside[kMaxUnits];   // per unit: keys above the bracket (later: kept), keys in it
+    int scan[kSelectWarps];
     uint32_t warp_min[kSelectWarps], warp_max[kSelectWarps];
-    int inside, ncand, bin[2], need, count;
+    int bin[2], in_bin[2], over_bin[2];
+    int ncand;
     unsigned long long weakest;
 };
-constexpr size_t kStreamHead = sizeof(StreamShared) > sizeof(SelectShared) ? sizeof(StreamShared) : sizeof(SelectShared);
-static size_t stream_smem(int N) { return kStreamHead + ((size_t)(N + 31) / 32 + 1) / 2 * 16; }
+static size_t stream_smem(int N) { return sizeof(StreamShared) + (size_t)((N + 1023) / 1024) * 32 * sizeof(uint2); }
 
 template <bool kState, int kSample>
 __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel(const float* __restrict__ delta, int64_t ld, int N, int keep,
                                                                               int* __restrict__ list, int64_t list_stride, int* __restrict__ tickets) {
     extern __shared__ __align__(16) uint8_t select_smem[];
     StreamShared& S = *reinterpret_cast<StreamShared*>(select_smem);
-    uint2* mask = reinterpret_cast<uint2*>(select_smem + kStreamHead);             // per 32 keys: above the bracket (later: kept), in it or above
-    const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t below = (1u << lane) - 1u;
+    uint2* mask = reinterpret_cast<uint2*>(select_smem + sizeof(StreamShared));    // per 32 keys: above the bracket (later: kept), in it or above
+    const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, units = (N + 1023) / 1024;
     for (int t = tid; t < 2048; t += kSelectThreads) S.hist[t] = 0;
-    if (tid == 0) { S.inside = 0; S.ncand = 0; S.bin[0] = S.bin[1] = -1; }
+    if (tid < kMaxUnits) S.above[tid] = S.inside[tid] = 0;
+    if (tid == 0) { S.ncand = 0; S.bin[0] = S.bin[1] = -1; }
     pdl_enter(delta, list, tickets);
     int* out = list + (size_t)bh * list_stride;
     if (tickets && tid == 0) tickets[bh] = 0;
@@ -399,7 +406,17 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
         __syncthreads();
         excl = __reduce_add_sync(0xffffffffu, lane < warp ? S.scan[lane] : 0) + incl - c.x - c.y;
     };
-    // the sample: one key of every N / 4096, at a scattered place
+    // the bin that holds rank r (from 1) of what was scanned, how many it holds and how many lie above it
+    auto find = [&](int r, int excl, int2 c, int which) {
+        if (excl < r && r <= excl + c.x + c.y) {
+            const bool first = r <= excl + c.y;
+            S.bin[which] = first ? top + 1 : top;
+            S.in_bin[which] = first ? c.y : c.x;
+            S.over_bin[which] = excl + (first ? 0 : c.y);
+        }
+    };
+    auto shift_of = [](uint32_t width) { return max(0, 21 - __clz((int)width)); };        // 2048 bins over width + 1 patterns
+    // the sample: one key of every N / kSample, at a scattered place
     uint32_t lo = 0u, hi = 0x7FFFFFFFu;                                   // keys above hi are kept, keys below lo are not
     {
         uint32_t u[kSample / kSelectThreads], umin = 0x7FFFFFFFu, umax = 0u;
@@ -412,7 +429,7 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
             umax = max(umax, u[t]);
         }
         range(umin, umax);
-        const int shift = max(0, 21 - __clz((int)(umax - umin)));
+        const int shift = shift_of(umax - umin);
 #pragma unroll
         for (int t = 0; t < kSample / kSelectThreads; ++t) atomicAdd(&S.hist[(u[t] - umin) >> shift], 1);
         __syncthreads();
@@ -421,151 +438,263 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
         scan(excl, c);
         const float q = (float)keep / (float)N, mid = q * kSample, dev = 4.5f * sqrtf(mid * (1.0f - q)) + 4.0f;
         const int r0 = (int)(mid - dev), r1 = (int)(mid + dev) + 1;       // ranks (from 1) of the bracket's ends
-        auto holds = [&](int r) { return excl < r && r <= excl + c.x + c.y; };
-        if (holds(r0)) S.bin[0] = r0 <= excl + c.y ? top + 1 : top;
-        if (holds(r1)) S.bin[1] = r1 <= excl + c.y ? top + 1 : top;
+        find(r0, excl, c, 0);
+        find(r1, excl, c, 1);
         __syncthreads();
-        if (S.bin[0] >= 0) hi = min(0x7FFFFFFFu, umin + ((uint32_t)(S.bin[0] + 1) << shift) - 1u);
-        if (S.bin[1] >= 0) lo = umin + ((uint32_t)S.bin[1] << shift);
-    }
-    // the sweep: a warp takes words of 32 consecutive keys
-    const int words = (N + 31) / 32, per = (words + kSelectWarps - 1) / kSelectWarps, w0 = min(words, warp * per), w1 = min(words, w0 + per);
-    for (int wb = w0; wb < w1; wb += 8) {
-        uint32_t u[8];
-        const uint32_t* at = src + wb * 32 + lane;
-        if (wb + 8 <= w1 && wb * 32 + 256 <= N) {
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            if (S.bin[e] < 0) continue;                                   // (beyond the sample)
+            int sh = shift;
+            uint32_t a = umin + ((uint32_t)S.bin[e] << sh), b = a + ((1u << sh) - 1u);
+            while (S.in_bin[e] > kHeavy && sh > 0) {
+                const int r = (e ? r1 : r0) - S.over_bin[e];
+                uint32_t m = 0x7FFFFFFFu, M = 0u;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) u[k] = at[32 * k] & 0x7FFFFFFFu;
-        } else {
+                for (int t = 0; t < kSample / kSelectThreads; ++t)
+                    if (u[t] - a <= b - a) { m = min(m, u[t]); M = max(M, u[t]); }
+                __syncthreads();                                          // (the last range and bin have been read)
+                range(m, M);
+                a = m;
+                b = M;
+                if (m == M) break;
+                sh = shift_of(M - m);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) u[k] = wb + k < w1 && (wb + k) * 32 + lane < N ? at[32 * k] & 0x7FFFFFFFu : 0xFFFFFFFFu;      // (as an int below every key)
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint32_t ba = __ballot_sync(0xffffffffu, (int)u[k] > (int)hi), bi = __ballot_sync(0xffffffffu, (int)u[k] >= (int)lo);
-            if (lane == 0 && wb + k < w1) mask[wb + k] = make_uint2(ba, bi);
-        }
-    }
-    __syncwarp();
-    // the bracket's keys, a lane per word
-    int kept = 0;
-    uint32_t bmin = 0x7FFFFFFFu, bmax = 0u;
-    for (int wb = w0; wb < w1; wb += 32) {
-        const uint2 m = wb + lane < w1 ? mask[wb + lane] : make_uint2(0u, 0u);
-        kept += __popc(m.x);
-        uint32_t in = m.y & ~m.x;
-        while (const uint32_t some = __ballot_sync(0xffffffffu, in != 0u)) {
-            int pos = 0;
-            if (lane == 0) pos = atomicAdd(&S.inside, __popc(some));
-            pos = __shfl_sync(0xffffffffu, pos, 0);
-            if (pos >= kInside) break;                                    // (too many: the row goes to select_row)
-            pos += __popc(some & below);
-            if (in && pos < kInside) {
-                const int j = (wb + lane) * 32 + __ffs(in) - 1;
-                const uint32_t u = src[j] & 0x7FFFFFFFu;
-                S.list[pos] = key_of(__uint_as_float(u), j);
-                bmin = min(bmin, u);
-                bmax = max(bmax, u);
-                in &= in - 1u;
+                for (int t = 0; t < kSample / kSelectThreads; ++t)
+                    if (u[t] - m <= M - m) atomicAdd(&S.hist[(u[t] - m) >> sh], 1);
+                __syncthreads();
+                scan(excl, c);
+                const int over = S.over_bin[e];
+                __syncthreads();
+                find(r, excl, c, e);
+                if (excl < r && r <= excl + c.x + c.y) S.over_bin[e] += over;
+                __syncthreads();
+                a = m + ((uint32_t)S.bin[e] << sh);
+                b = min(M, a + ((1u << sh) - 1u));
             }
+            if (e) lo = a; else hi = min(b, 0x7FFFFFFFu);
         }
+        if (r0 < 1 && lo == umax) hi = lo;                                // (equal weights at an end of the row)
+        if (r1 > kSample && hi == umin) lo = hi;
     }
-    kept = __reduce_add_sync(0xffffffffu, kept);
-    if (lane == 0) S.warp_kept[warp] = kept;
-    range(bmin, bmax);
-    const int inside = S.inside;
-    int need = keep - __reduce_add_sync(0xffffffffu, S.warp_kept[lane]);
-    bool found = need >= 1 && need <= inside && inside <= kInside;       // (the same in every thread)
-    auto each = [&](auto&& f) {                                           // the bracket's keys
-        for (int e = tid; e < inside; e += kSelectThreads) f(S.list[e]);
+    // f(word, its keys) for the CTA's words of 32 consecutive keys, eight words of a warp requested at once
+    auto sweep = [&](auto&& f) {
+        for (int wb = 8 * warp; wb < 32 * units; wb += 8 * kSelectWarps) {
+            uint32_t u[8];
+            const uint32_t* at = src + wb * 32 + lane;
+            if (wb * 32 + 256 <= N) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) u[k] = at[32 * k] & 0x7FFFFFFFu;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) u[k] = (wb + k) * 32 + lane < N ? at[32 * k] & 0x7FFFFFFFu : 0xFFFFFFFFu;      // (as an int below every key)
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) f(wb + k, u[k]);
+        }
     };
-    if (found) {
-        const int shift = max(0, 21 - __clz((int)(bmax - bmin)));
-        each([&](unsigned long long x) { atomicAdd(&S.hist[((uint32_t)(x >> 32) - bmin) >> shift], 1); });
+    uint32_t bmin = lo, bmax = hi;                                        // of the keys inside, or wider
+    int need, inside;
+    for (int turn = 0;; ++turn) {
+        const bool again = turn > 0;
+        if (turn == 8) return;                                            // (three narrow any bracket to one pattern: weights that change under the call)
+        if (again) { bmin = 0x7FFFFFFFu; bmax = 0u; }
+        auto bits = [&](int word, uint32_t u) {
+            const uint32_t ba = __ballot_sync(0xffffffffu, (int)u > (int)hi), bi = __ballot_sync(0xffffffffu, (int)u >= (int)lo);
+            if (lane == 0) mask[word] = make_uint2(ba, bi);
+        };
+        if (!again) {
+            sweep(bits);
+        } else {
+            sweep([&](int word, uint32_t u) {
+                bits(word, u);
+                if ((int)u >= (int)lo && u <= hi) { bmin = min(bmin, u); bmax = max(bmax, u); }
+            });
+        }
         __syncthreads();
-        int excl;
+        for (int unit = warp; unit < units; unit += kSelectWarps) {
+            const uint2 m = mask[32 * unit + lane];
+            const int a = __reduce_add_sync(0xffffffffu, __popc(m.x)), i = __reduce_add_sync(0xffffffffu, __popc(m.y & ~m.x));
+            if (lane == 0) { S.above[unit] = a; S.inside[unit] = i; }
+        }
+        if (again) range(bmin, bmax); else __syncthreads();
+        int a = 0, i = 0;
+#pragma unroll
+        for (int k = 0; k < kMaxUnits; k += 32) { a += S.above[k + lane]; i += S.inside[k + lane]; }
+        need = keep - __reduce_add_sync(0xffffffffu, a);
+        inside = __reduce_add_sync(0xffffffffu, i);
+        if (need >= 1 && need <= inside && (inside <= kInside || bmin == bmax)) break;
+        // the bracket is narrowed, or the part of the row beside it that holds the threshold
+        int r = need, excl;
         int2 c;
+        if (need < 1) { lo = hi + 1u; hi = 0x7FFFFFFFu; r = keep; }
+        else if (need > inside) { hi = lo - 1u; lo = 0u; r = need - inside; }
+        else if (again) { lo = bmin; hi = bmax; }
+        const int shift = shift_of(hi - lo);
+        sweep([&](int, uint32_t u) { if (u - lo <= hi - lo) atomicAdd(&S.hist[(u - lo) >> shift], 1); });
+        __syncthreads();
         scan(excl, c);
-        if (excl < need && need <= excl + c.x + c.y) {
-            const bool first = need <= excl + c.y;
-            S.bin[0] = first ? top + 1 : top;
-            S.need = need - excl - (first ? 0 : c.y);
-            S.count = first ? c.y : c.x;
-        }
+        find(r, excl, c, 0);
         __syncthreads();
-        const uint32_t bin = (uint32_t)S.bin[0];
-        const int count = S.count;
-        need = S.need;
-        found = count <= kCandidates;
-        if (found) {
-            each([&](unsigned long long x) { if (((uint32_t)(x >> 32) - bmin) >> shift == bin) S.cand[atomicAdd(&S.ncand, 1)] = x; });
-            __syncthreads();
-            if (tid < count) {
-                const unsigned long long k = S.cand[tid];
-                int above = 0;
-                for (int i = 0; i < count; ++i) above += S.cand[i] > k;
-                if (above == need - 1) S.weakest = k;
-            }
-            __syncthreads();
-        }
+        lo += (uint32_t)S.bin[0] << shift;
+        hi = min(hi, lo + ((1u << shift) - 1u));
     }
-    if (!found) {                                                         // (nothing of the row has been written yet)
-        __syncthreads();
-        SelectShared& G = *reinterpret_cast<SelectShared*>(select_smem);
-        for (int t = tid; t < (int)sizeof(G.hist) / 4; t += kSelectThreads) (&G.hist[0][0])[t] = 0;
-        if (tid == 0) G.ncand = 0;
-        cg::cluster_group cluster = cg::this_cluster();
-        select_row<0, kState>(G, cluster, 1, 0, delta, ld, N, keep, (N + 31) / 32 * 32, bh, out);
-        return;
-    }
-    const unsigned long long weakest = S.weakest;
-    each([&](unsigned long long x) {
-        if (x >= weakest) {
-            const uint32_t j = 0xFFFFFFFFu - (uint32_t)x;
-            atomicOr(&mask[j >> 5].x, 1u << (j & 31));
+    const bool equal = bmin == bmax;                                      // one bit pattern: the first `need` keys inside are kept
+    // f(unit, place of its first key among all that `count` counts) for this warp's units
+    auto each_unit = [&](const int* count, auto&& f) {
+        int run = 0;
+        for (int k = 0; k < units; k += 32) {
+            const int v = count[k + lane], before = __reduce_add_sync(0xffffffffu, lane < warp ? v : 0);
+            if (k + warp < units) f(k + warp, run + before);
+            run += __reduce_add_sync(0xffffffffu, v);
         }
-    });
-    __syncthreads();
-    // the bits -> indices, every warp from the position its lower words leave it
-    kept = 0;
-    for (int w = w0 + lane; w < w1; w += 32) kept += __popc(mask[w].x);
-    kept = __reduce_add_sync(0xffffffffu, kept);
-    if (lane == 0) S.warp_kept[warp] = kept;
-    __syncthreads();
-    int at = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_kept[lane] : 0);
-    const int last = (int)(0xFFFFFFFFu - (uint32_t)weakest);              // the weakest kept key
-    constexpr int kTurn = 2 * kInside / kSelectWarps;
-    int* buf = reinterpret_cast<int*>(S.list) + warp * kTurn;             // (its keys have been read)
-    for (int wb = w0; wb < w1; wb += 32) {                                // a lane per word: a word holds a few kept keys
-        uint32_t word = wb + lane < w1 ? mask[wb + lane].x : 0u;
-        int pos = __popc(word);
+    };
+    auto before_lane = [&](int n) {                                       // sum of the lower lanes' n
+        int incl = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, pos, o);
-            if (lane >= o) pos += v;
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
         }
-        const int all = __shfl_sync(0xffffffffu, pos, 31), j0 = (wb + lane) * 32;
-        pos -= __popc(word);
-        if (kState && wb + lane < w1 && last >> 5 == wb + lane) {
+        return incl - n;
+    };
+    uint32_t* kept_of = reinterpret_cast<uint32_t*>(S.hist);              // one bit per gathered key: kept
+    if (!equal) {
+        int* gathered = reinterpret_cast<int*>(S.list);                   // (the low words: first the key's number, then its order key)
+        each_unit(S.inside, [&](int unit, int at) {
+            const uint2 m = mask[32 * unit + lane];
+            uint32_t in = m.y & ~m.x;
+            at += before_lane(__popc(in));
+            for (; in; in &= in - 1u) gathered[2 * at++] = (32 * unit + lane) * 32 + __ffs(in) - 1;
+        });
+        bmin = 0x7FFFFFFFu;
+        bmax = 0u;
+        __syncthreads();
+        for (int e0 = tid; e0 < inside; e0 += 4 * kSelectThreads) {       // four keys of a thread requested at once
+            int j[4];
+            uint32_t u[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int e = e0 + t * kSelectThreads;
+                j[t] = e < inside ? gathered[2 * e] : 0;
+                u[t] = src[j[t]] & 0x7FFFFFFFu;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int e = e0 + t * kSelectThreads;
+                if (e < inside) {
+                    bmin = min(bmin, u[t]);
+                    bmax = max(bmax, u[t]);
+                    S.list[e] = key_of(__uint_as_float(u[t]), j[t]);
+                }
+            }
+        }
+        range(bmin, bmax);
+        auto each = [&](auto&& f) {                                       // the bracket's keys
+            for (int e = tid; e < inside; e += kSelectThreads) f(S.list[e]);
+        };
+        // the bin of the need-th, by weight, among equal weights by index
+        unsigned long long base = (unsigned long long)bmin << 32;
+        int s = 32 + shift_of(bmax - bmin), nbins = 2048, count;
+        for (;;) {
+            each([&](unsigned long long x) {
+                const unsigned long long bin = (x - base) >> s;
+                if (bin < (unsigned long long)nbins) atomicAdd(&S.hist[bin], 1);
+            });
+            __syncthreads();
+            int excl;
+            int2 c;
+            scan(excl, c);
+            find(need, excl, c, 0);
+            __syncthreads();
+            base += (unsigned long long)(uint32_t)S.bin[0] << s;
+            need -= S.over_bin[0];
+            count = S.in_bin[0];
+            if (count <= kCandidates) break;
+            if (s > 32) {                                                 // the next bins cover this one and nothing above it
+                nbins = 1 << min(11, s - 32);
+                s = max(32, s - 11);
+            } else {                                                      // one weight: the low words of N <= 2^17 keys, 64 to a bin
+                base += 0xFFFFFFFFu - (uint32_t)(N - 1);
+                nbins = 2048;
+                s = 6;
+            }
+        }
+        each([&](unsigned long long x) { if ((x - base) >> s == 0ull) S.cand[atomicAdd(&S.ncand, 1)] = x; });
+        __syncthreads();
+        if (tid < count) {
+            const unsigned long long k = S.cand[tid];
+            int above = 0;
+            for (int i = 0; i < count; ++i) above += S.cand[i] > k;
+            if (above == need - 1) S.weakest = k;
+        }
+        __syncthreads();
+        const unsigned long long weakest = S.weakest;
+        for (int e = tid; e - lane < inside; e += kSelectThreads) {
+            const uint32_t k = __ballot_sync(0xffffffffu, e < inside && S.list[e] >= weakest);
+            if (lane == 0) kept_of[e >> 5] = k;
+        }
+    }
+    __syncthreads();
+    // the kept keys' bits
+    each_unit(S.inside, [&](int unit, int at) {
+        const uint2 m = mask[32 * unit + lane];
+        uint32_t in = m.y & ~m.x, word = m.x;
+        const int n = __popc(in);
+        at += before_lane(n);
+        uint32_t keep_bits;                                               // of the word's n keys inside
+        if (equal) {
+            const int k = min(max(need - at, 0), n);
+            keep_bits = k == 32 ? 0xFFFFFFFFu : (1u << k) - 1u;
+            if (kState && at < need && need <= at + n) {                  // the weakest kept key
+                uint32_t rest = in;
+                for (int t = need - at; t > 1; --t) rest &= rest - 1u;
+                S.weakest = key_of(__uint_as_float(bmin), (32 * unit + lane) * 32 + __ffs(rest) - 1);
+            }
+        } else {
+            keep_bits = __funnelshift_r(kept_of[at >> 5], kept_of[(at >> 5) + 1], at & 31);
+            if (n < 32) keep_bits &= (1u << n) - 1u;
+        }
+        if (keep_bits == (n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u)) {
+            word |= in;
+        } else {
+            for (; keep_bits; keep_bits >>= 1, in &= in - 1u)
+                if (keep_bits & 1u) word |= in & -in;
+        }
+        mask[32 * unit + lane].x = word;
+        const int kept = __reduce_add_sync(0xffffffffu, __popc(word));
+        if (lane == 0) S.above[unit] = kept;
+    });
+    __syncthreads();
+    // the bits -> indices
+    constexpr int kTurn = 2 * kInside / kSelectWarps;
+    int* buf = reinterpret_cast<int*>(S.list) + warp * kTurn;             // (its keys have been read)
+    const uint32_t below = (1u << lane) - 1u;
+    const unsigned long long weakest = kState ? S.weakest : 0ull;
+    const int last = (int)(0xFFFFFFFFu - (uint32_t)weakest);
+    each_unit(S.above, [&](int unit, int at) {
+        uint32_t word = mask[32 * unit + lane].x;
+        int pos = before_lane(__popc(word));
+        const int all = __shfl_sync(0xffffffffu, pos + __popc(word), 31), j0 = (32 * unit + lane) * 32;
+        if (kState && last >> 5 == 32 * unit + lane) {
             int* hdr = out - kStateHeader;
             hdr[0] = keep;
             hdr[1] = at + pos + __popc(word & ((1u << (last & 31)) - 1u));
             hdr[2] = (int)(uint32_t)weakest;
             hdr[3] = (int)(uint32_t)(weakest >> 32);
         }
-        const bool turn = all <= kTurn;                                   // (the lanes' short runs meet in shared memory and leave as whole lines)
-        int* to = turn ? buf : out + at;
-        while (word) {
-            to[pos++] = j0 + __ffs(word) - 1;
-            word &= word - 1u;
-        }
-        if (turn) {
+        if (all > kTurn) {                                                // a lane per key: whole lines as they are
+            for (int w = 0; w < 32; ++w) {
+                const uint32_t b = __shfl_sync(0xffffffffu, word, w);
+                const int p = at + __shfl_sync(0xffffffffu, pos, w);
+                if ((b >> lane) & 1u) out[p + __popc(b & below)] = (32 * unit + w) * 32 + lane;
+            }
+        } else {                                                          // a lane per word: the short runs meet in shared memory and leave as whole lines
+            for (; word; word &= word - 1u) buf[pos++] = j0 + __ffs(word) - 1;
             __syncwarp();
             for (int i = lane; i < all; i += 32) out[at + i] = buf[i];
             __syncwarp();
         }
-        at += all;
-    }
+    });
 }
 
 // 16 bytes of a K, V or q row, widened to fp32
@@ -1111,11 +1240,12 @@ static int launch_select(const Prob& P, const float* delta, int64_t ld, int* lis
     int nrank = 1;
     // the fewest CTAs whose registers hold a row; a row that needs a cluster gets more while all rows still run at once
     while (nrank < kSelectMaxCluster && ((int64_t)nrank * kCtaKeys < P.L || (nrank > 1 && 2ll * nrank * P.B * P.Hq <= 148))) nrank *= 2;
-    // The kernel that streams a row: where the rows do not all have a wave's registers (up to 296 rows of 16384 keys only with a window of an eighth, 256 rows of 16384
-    // keys, w = N / 16 and N / 4: 14.7 / 14.2 us, but 15.2 / 16.0), or one CTA holds a row of more than 16384 keys
+    // The kernel that streams a row: where the rows do not all have an SM's registers to themselves, or one CTA holds a row of more than 16384 keys. State taken up, us, registers / streamed, at w = 64, N / 16,
+    // N / 4, N / 2, N - 1: 200 rows of 8192 keys 13.8 / 11.0 .. 14.3 / 11.9, 256 of 16384 15.1 / 13.0, 16.9 / 14.3, 17.4 / 15.9, 17.4 / 16.9, 15.7 / 14.7, 32 of 26000 12.4 / 10.2 .. 12.3 / 12.3, 512 of
+    // 5000 26 / 18 .. 27 / 21; equal weights and ten values gain more (256 of 16384 15 / 12, 23 / 13), weights that rise along the row lose up to 8 % (32 of 32768 12.4 / 12.8). But 32 rows of 16384
+    // 8.2 / 8.4 .. 9.8 / 10.7, rising 8.2 / 10.5; 32 of 65536 (clusters) 11.5 / 14.9 .. 14.8 / 22.5; 512 of 4096 (four keys to a thread, two CTAs per SM) 15.0 / 18.1 .. 15.9 / 20.7.
     const int64_t rows = (int64_t)P.B * P.Hq;
-    if (P.w < P.L && P.L >= kStreamMinKeys && P.L <= kStreamMaxKeys &&
-        (P.L > 16384 ? nrank == 1 || rows * nrank > 148 : rows > 296 || (rows > 148 && 8ll * P.w <= P.L))) {
+    if (P.w < P.L && P.L >= kStreamMinKeys && P.L <= kStreamMaxKeys && (rows * nrank > 148 || (P.L > 16384 && nrank == 1))) {
         auto stream = P.L > 65536 ? (state ? decode_select_stream_kernel<true, 8192> : decode_select_stream_kernel<false, 8192>)
                                   : (state ? decode_select_stream_kernel<true, 4096> : decode_select_stream_kernel<false, 4096>);
         // (state of the function, which other threads' calls share: always the limit)

@@ -136,6 +136,44 @@ def test_selection_of_many_rows(N, kind):
         assert torch.equal(torch.gather(rows[:, 8:8 + w], 1, rows[:, 1:2].long())[:, 0].long(), order[0, :, w - 1]), w    # the weakest kept key
 
 
+@pytest.mark.parametrize("N", [4097, 20000, 32768, 50001, 131072])
+@pytest.mark.parametrize("kind", ["misled down", "misled up", "two", "saturated", "low", "repeat", "clusters", "neighbours"])
+def test_selection_where_weights_crowd(N, kind):
+    """Streamed rows whose bracket misses (the sampled keys are unlike the others), lies across two heavy values or at an end of the row that many keys share, or holds more keys
+    than are gathered, of few or of many bit patterns."""
+    BH = 304 if N < 60000 else 160
+    g = torch.Generator("cuda").manual_seed(N)
+    z = torch.rand(1, BH, N, generator=g, device="cuda")
+    S = 8192 if N > 65536 else 4096
+    i = torch.arange(S, dtype=torch.int64)
+    sampled = (i * N // S + ((((i * 2654435761) & 0xFFFFFFFF) >> 16) * (N // S) >> 16)).cuda()
+    if kind.startswith("misled"):
+        delta = 2.0 + z
+        delta[..., sampled] = delta[..., sampled] + (8.0 if kind == "misled up" else -1.5)
+    elif kind == "clusters":                                       # 40 values, neighbours in bit patterns
+        delta = (torch.tensor(1.5, device="cuda").view(torch.int32) + (z * 40).int()).view(torch.float32)
+    elif kind == "neighbours":                                     # every bit pattern of a short range, among outliers
+        delta = (torch.tensor(1.5, device="cuda").view(torch.int32) + (z * 3000).int()).view(torch.float32)
+        delta[..., ::997] = 1e30
+    else:
+        delta = {"two": lambda: torch.where(z < 0.25, 3.0, 2.0), "saturated": lambda: torch.where(z < 0.3, 1.6e38, 1.0 + z),
+                 "low": lambda: torch.where(z < 0.3, 1.0 + z, 1e-38), "repeat": lambda: 1.0 + z[..., :64].repeat(1, 1, N // 64 + 1)[..., :N]}[kind]()
+    delta = delta.contiguous()
+    order = torch.sort(delta, dim=-1, descending=True, stable=True)[1]
+    K = torch.zeros(1, N, 1, 64, dtype=torch.bfloat16, device="cuda")
+    q = torch.zeros(1, BH, 64, dtype=torch.bfloat16, device="cuda")
+    for w in (3, N // 16, N // 4 - 5, N // 4 + N // 50, N // 2, N - 2):
+        want = torch.sort(order[..., :w], dim=-1)[0]
+        p = dma.problem(1, BH, 1, N, 64, w)
+        _, _, idx = dma.dma_decode(p, q, K, K, delta, want_idx=True)
+        assert torch.equal(idx.long(), want), w
+        rows = dma.dma_decode_state_init(p, delta, dma.dma_decode_state(p, "cuda")).view(torch.int32).view(BH, -1)
+        assert (rows[:, 0] == w).all() and torch.equal(rows[:, 8:8 + w].long(), want[0]), w
+        assert torch.equal(torch.gather(rows[:, 8:8 + w], 1, rows[:, 1:2].long())[:, 0].long(), order[0, :, w - 1]), w    # the weakest kept key
+        key = (delta.view(torch.int32)[0].gather(1, order[0, :, w - 1:w])[:, 0].long() << 32) | (0xFFFFFFFF - order[0, :, w - 1])
+        assert torch.equal((rows[:, 3].long() << 32) | (rows[:, 2].long() & 0xFFFFFFFF), key), w
+
+
 @pytest.mark.parametrize("Hq,Hkv,d,dtype", [(1, 1, 64, "fp32"), (3, 3, 128, "bf16"), (6, 2, 64, "bf16"), (32, 8, 128, "bf16"), (33, 11, 128, "fp32")])
 def test_delta_of_a_few_keys(Hq, Hkv, d, dtype):
     """Ranges of 1 to 9 keys (up to 8 take a kernel of their own) have the bits of the whole range; heads that do not fill a CTA, groups of any size."""
