@@ -973,19 +973,23 @@ static int launch_delta(const Prob& P, const void* V, const float* W, const floa
     if (j_end - j_begin <= kFewKeys)
         return launch_overlapped(delta_few_kernel<T, D>, dim3((P.Hq * (D / 8) + 127) / 128, j_end - j_begin, P.B), dim3(128), 0, st, 1, (const T*)V, W, A, bias, P.Hq, P.G,
                                  P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
-    // Two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles grid-stride. Tiles of 64 keys where there are few
-    // (us, tiles of 128 / 64: 16 heads of 4096 keys 4.8 / 4.1, 8 of 2500 4.6 / 3.4, but 32 of 65536 50.9 / 53.2), and where a KV head has one query head, whose tiles are short work, tiles of 32
-    // and four CTAs per SM (16 heads of 8192 keys 13.2 / 10.2, but 32 / 8 heads of 16384 16.8 / 19.0). The weights' two halves, which came later, took
-    // 4 to 7 % off each: 4.1 -> 3.9, 50.9 -> 47.4, 10.2 -> 9.8, 16.7 -> 15.7
-    const int64_t pairs = (int64_t)P.Hkv * P.B, tiles = pairs * ((j_end - j_begin + 127) / 128);
+    // Two CTAs per SM in all (what the register file holds at once), each walking its (batch, KV head) pair's tiles of 128 keys grid-stride. us, tiles of 128 / the other shape:
+    // Tiles of 64 keys where a CTA then walks at most three quarters of the keys and all CTAs run at once: 8 heads of 500 keys 3.3 / 2.6, 4 of 12000 6.2 / 5.2, 32 / 8 heads of 6000 8.7 / 7.2, but 16 heads of
+    // 1500 (192 CTAs either way) 3.9 / 4.1, 32 / 8 heads of 8192 8.8 / 9.0, 8 of 16384 with 64 channels (448 keys against 512) 6.1 / 6.7.
+    // Tiles of 32 and four CTAs per SM, where a KV head has one query head, whose tiles are short work, and tiles of 128 take more than one wave of CTAs: 16 heads of 8192 keys 12.8 / 9.5, of 65536 91 / 60,
+    // 32 of 6000 18.0 / 17.3, 64 of 16384 87.9 / 85.1, but 8 heads (one wave) of 65536 30.2 / 32.3, 128 of 8192 75 / 85. With 64 channels only where they are one wave: 16 heads of 4096 keys 5.1 / 4.7, but 32
+    // of 16384 24.5 / 30.4, 128 85 / 147.
+    const int64_t pairs = (int64_t)P.Hkv * P.B;
+    const int keys = j_end - j_begin;
+    auto grid = [&](int rows, int ctas) { return (int)std::min<int64_t>((ctas * 148 + pairs - 1) / pairs, (keys + rows - 1) / rows); };      // CTAs per pair
+    auto walk = [&](int rows) { return ((keys + rows - 1) / rows + grid(rows, 2) - 1) / grid(rows, 2) * rows; };                             // keys of a CTA
     auto launch = [&](auto kern, int rows, int ctas) {
-        const int ntiles = (j_end - j_begin + rows - 1) / rows;
-        const int per_pair = std::min((int)((ctas * 148 + pairs - 1) / pairs), ntiles);
         const size_t bytes = (size_t)P.G * (D + 2 * rows) * sizeof(float);
-        return launch_overlapped(kern, dim3(per_pair, P.Hkv, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
+        return launch_overlapped(kern, dim3(grid(rows, ctas), P.Hkv, P.B), dim3(256), bytes, st, 1, (const T*)V, W, A, bias, j_end, P.Hq, P.G, P.vs[0], P.vs[1], P.vs[2], j_begin, ld);
     };
-    if (tiles <= 4 * 148) return launch(delta_kernel<T, D, 64, 2>, 64, 2);
-    if (sizeof(T) == 2 && P.G == 1) return launch(delta_kernel<T, D, 32, 4>, 32, 4);
+    if (pairs * grid(64, 2) <= 2 * 148 && 4 * walk(64) <= 3 * walk(128)) return launch(delta_kernel<T, D, 64, 2>, 64, 2);
+    if (sizeof(T) == 2 && P.G == 1 && pairs * grid(128, 2) > 2 * 148 && (D == 128 ? pairs <= 64 : pairs * grid(32, 4) <= 4 * 148))
+        return launch(delta_kernel<T, D, 32, 4>, 32, 4);
     return launch(delta_kernel<T, D, 128, 2>, 128, 2);
 }
 

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 import oracle
+from paper_2508_02124_b200 import binding as dma
 from paper_2508_02124_b200 import workloads as wl
 
 from helpers import bits_equal, gpu_mask, oracle_mask
@@ -98,3 +99,20 @@ def test_mask_full_size_configs(key):
     case = wl.CONFIGS[key]
     e, bmp = check_mask(case, wl.make_inputs(case))
     assert (e >= np.arange(case.L)).all()
+
+
+@pytest.mark.parametrize("B,Hkv,G,d,ranges", [
+    (1, 3, 1, 128, [(0, 9), (5, 2100)]), (1, 2, 4, 64, [(7, 1000)]),          # tiles of 64 keys
+    (1, 16, 1, 128, [(0, 2500), (33, 4001)]), (4, 16, 1, 128, [(1, 700)]),    # tiles of 32: several per CTA, one each
+    (1, 16, 1, 64, [(0, 4001), (31, 2600)]),
+    (2, 16, 1, 64, [(0, 2000)]), (2, 8, 2, 64, [(3, 2500)]), (8, 16, 1, 128, [(0, 700)])])      # tiles of 128
+def test_delta_by_tiles_of_32_64_and_128_keys(B, Hkv, G, d, ranges):
+    Hq, N = Hkv * G, max(e for _, e in ranges) + 3
+    g = torch.Generator().manual_seed(N)
+    V, W, A = torch.randn(B, N, Hkv, d, generator=g).to(torch.bfloat16), torch.randn(Hq, d, generator=g) / d ** 0.5, torch.rand(Hq, generator=g) + 0.5
+    _, ref = oracle.delta(V.float().numpy(), W.numpy(), A.numpy(), Hq)
+    p = dma.problem(B, Hq, Hkv, N, d, 8)
+    for a, b in ranges:
+        out = torch.full((B, Hq, N), -1.0, device="cuda")
+        dma.dma_delta_range(p, V.cuda(), W.cuda(), A.cuda(), out, a, b)
+        assert bits_equal(out[..., a:b], ref[..., a:b]) and bool((out[..., :a] == -1.0).all()) and bool((out[..., b:] == -1.0).all()), (a, b)
