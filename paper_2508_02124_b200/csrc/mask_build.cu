@@ -10,6 +10,7 @@
 //                       Heads of up to 4096 keys: sort, walk and bitmap in the one block kernel
 //   bitmap_square_kernel, bitmap_kernel   per key tile: union of the query-tile intervals its keys are kept in
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <utility>
 #include <type_traits>
@@ -693,8 +694,8 @@ __global__ void __launch_bounds__(256) expiry_tree_kernel(const unsigned long lo
 // indices.) The block in which the running count reaches w holds the key's expiry, found by the walk down that block's own tree. A CTA takes the keys of one block, in
 // descending order, so that a warp's 32 searches read the same few words, and since a block's keys are whole key tiles, it writes their bits of the bitmap, too.
 // This replaces a merge launch per level, the walk from the root and the bitmap kernel, each a chain of dependent loads after a launch. Bound by the latency
-// of its own chain and, from 16 blocks on, by the searches ((blocks - 1) log2(block) reads per key). Mask build, us, before / now: 16 heads of 4096 keys 23.8 / 16.4,
-// 16 of 8192 36.4 / 26.6, 32 of 16384 59.8 / 48.9, of 32768 112 / 106, 128 of 16384 211 / 196, 8 of 5000 27.3 / 16.5; packed documents 26.7 / 20.6, 40.4 / 30.5, 70.1 / 61.8, 133 / 134.
+// of its own chain and, from 16 blocks on, by the searches ((blocks - 1) log2(block) reads per key). Mask build, us, merged / searched (G = 4, 64 channels): 16 heads of 4096 keys 23.9 / 15.8,
+// 16 of 8192 28.7 / 18.8, 32 of 16384 55 / 43, of 32768 101 / 94, 128 of 16384 184 / 163, 8 of 6000 28.1 / 16.8; packed documents 28.3 / 19.3, 32.8 / 22.5, 65.5 / 56, 121 / 122 (launch_mask_build).
 // (With the walk in global memory, a key after the other, 17.9, 27.0, 52.3, 114, 213.)
 constexpr int kSearchKeys = 32768;
 constexpr int kSearchThreads = 1024;
@@ -1038,19 +1039,31 @@ int launch_mask_build(const Prob& P, const void* V, const float* W, const float*
     } else {
         // rank tree: sorted blocks, then a search over the blocks and a walk in one of them per key (heads beyond kSearchKeys: one merge pass per further level and a
         // walk from the root); or everything in the block kernel. Blocks of 4096 keys keep few SMs busy for long where there are few, and blocks of 1024 take more
-        // searches. Mask build, us, blocks of 1024 / 4096: 16 heads of 4096 keys 16.4 / 30.4, 16 of 8192 26.6 / 40.8, 32 of 6000 26.0 / 38.4, 16 of 16384 38 / 42, but 48 of 8192 43.5 / 41.4,
-        // 24 of 16384 57 / 50, 32 of 16384 69 / 49; blocks of 1024 / a head whole in one CTA: 8 heads of 2000 keys 14.3 / 16.9, 16 of 3000 16.0 / 23.5, 64 of 3000 25.3 / 27.7,
+        // searches: blocks of 1024 / a head whole in one CTA, mask build, us: 8 heads of 2000 keys 14.3 / 16.9, 16 of 3000 16.0 / 23.5, 64 of 3000 25.3 / 27.7,
         // but 128 of 2000 24.2 / 21.3, 128 of 3000 36.8 / 32.6
         const int Lc = nchunk * kChunk, m = tree_levels(Lc);
         const int64_t small_blocks = (int64_t)BH * ((Lc + kSmallBlock - 1) / kSmallBlock);
         const bool few = small_blocks <= 2 * 148, whole = Lc <= (!few ? kBlockKeys : small_blocks > 200 ? 2 * kSmallBlock : kSmallBlock);
-        const int per_block = whole ? (Lc <= kSmallBlock ? kSmallBlock : kBlockKeys) : few ? kSmallBlock : kBlockKeys;
+        bool small = few, search = !whole && Lc <= kSearchKeys;
+        if (search && Lc > kBlockKeys) {
+            // Estimates, us: with blocks of 1024 the SMs' share of the blocks by the searches of each; with 4096, whose trees leave an SM one CTA, waves of CTAs; packed sequences, which walk twice, also
+            // against blocks of 4096 and merge launches. Fitted to 1 to 256 heads of 4097 to 32768 keys, 73 shapes, where they choose the best within 0.2 % in the mean. Mask build, us, 1024 /
+            // 4096: 16 heads of 8192 keys 19 / 34, 32 of 9000 31 / 39, 64 of 4097 35 / 38, 64 of 9000 56 / 70, 128 of 4097 54 / 68, but 8 of 32768 54 / 48, 48 of 8192 40 / 38, 32 of 16384 63 / 43, 128 of 16384
+            // 216 / 163; packed, 1024 / 4096 / merged: 64 of 9000 67 / 91 / 86, 128 of 4097 66 / 95 / 78, 32 of 16384 75 / 57 / 65, 64 of 32768 417 / 251 / 239, 8 of 32768 64 / 62 / 54.
+            const double blocks = (Lc + kSmallBlock - 1) / kSmallBlock, large = (Lc + kBlockKeys - 1) / kBlockKeys, share = BH * blocks / 148.0;
+            const double ctas = BH * large / 148.0, waves = ctas > 3.0 ? ctas : std::ceil(ctas);       // (behind three waves their ends have drifted apart)
+            const double by_small = cu ? 12.0 + share * (9.2 + 0.6 * blocks) : P.causal ? 10.0 + share * (7.4 + 0.52 * blocks) : 9.0 + share * (6.8 + 0.45 * blocks);
+            const double by_large = waves * (cu ? 45.0 + 2.6 * large : P.causal ? 29.4 + 2.33 * large : 24.3 + 2.16 * large);
+            const double merged = 2.0 + 28.0 * std::ceil(BH * large / 296.0) + 3.4 * (m - 12) + share * (7.7 + 1.2 * (m - 12));
+            small = by_small < by_large;
+            if (cu && merged < std::min(by_small, by_large)) small = search = false;
+        }
+        const int per_block = whole ? (Lc <= kSmallBlock ? kSmallBlock : kBlockKeys) : small ? kSmallBlock : kBlockKeys;
         const bool fused_bitmap = whole && square && P.Tr <= 32;
         const size_t keys = (size_t)BH * Lc, Wl = (size_t)Lc / 32;
         auto* buf0 = reinterpret_cast<unsigned long long*>((char*)ws + kWsHeaderBytes);
         auto* buf1 = buf0 + keys;
         uint2* lev = reinterpret_cast<uint2*>(buf1 + keys);
-        const bool search = !whole && Lc <= kSearchKeys;
         int* idx = search ? reinterpret_cast<int*>(buf1) : nullptr;
         const int mode = !whole ? -1 : cu ? 1 : P.causal ? 0 : 2;
         auto pick = [&](auto n) {

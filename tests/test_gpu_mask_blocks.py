@@ -1,6 +1,6 @@
-"""Bit-exact selection on every route of the block sort: heads that one CTA takes whole (blocks of 1024 and of 4096 keys) and heads in
-blocks of either size with merge launches, at the edges of threads, warps and blocks; few and many heads, ties, packed documents, the
-non-causal mode, square tiles of other sizes and tiles that are not square."""
+"""Bit-exact selection on every route of the block sort: heads that one CTA takes whole (blocks of 1024 and of 4096 keys), heads in
+blocks of either size that are searched block by block, and those with merge launches, at the edges of threads, warps and blocks; few and many heads,
+ties, packed documents, the non-causal mode, square tiles of other sizes and tiles that are not square."""
 import numpy as np
 import pytest
 import torch
@@ -86,3 +86,14 @@ def test_heads_searched_block_by_block(H, L):
         assert np.array_equal(e, ref) and np.array_equal(bitmap, oracle.bitmap_from_expiry(ref)), w
     dl, e, _ = build(H, L, L // 4, seed=3, levels=300, causal=0)
     assert np.array_equal(e, oracle.select_noncausal(dl, L // 4))
+
+
+@pytest.mark.parametrize("H,L", [(10, 32768), (12, 28700), (20, 16385), (36, 12200), (48, 17000), (60, 8190)])
+def test_heads_searched_in_blocks_of_4096_keys(H, L):
+    """Two to eight blocks, whole and ragged, a last block of one key: all three modes (documents of 48 heads are merged), equal weights across blocks, documents that begin at, one
+    behind and inside a block."""
+    test_heads_searched_block_by_block(H, L)
+    cu = sorted({0, 4095, 4096, 4097, L // 2, L})                                # (long documents: walks that end in another block than the key's)
+    dl, e, bitmap = build(H, L, 1500, seed=L + 1, levels=2000, cu=cu)
+    ref = oracle.select_expiry_varlen(dl, 1500, cu)
+    assert np.array_equal(e, ref) and np.array_equal(bitmap, oracle.bitmap_from_expiry(ref))
