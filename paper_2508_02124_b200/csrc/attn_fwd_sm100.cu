@@ -1261,27 +1261,35 @@ size_t tc_fwd_ws_bytes(const Prob& P) {
 }
 
 // Query tiles per CTA: two, or one whose key tiles are dealt out to the two softmax groups where that shortens the call. Both grids
-// are estimated in steps of a CTA (two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs; the pair's
-// steps in tile mode are longer where many keys expire per tile, i.e. in short sequences. Fitted to 64 shapes of 1 to 128 heads and
-// 183 to 15889 keys, each timed with both, and then moved by 5 to 10 % towards two for the hand-over of references and sums. Of 56 other shapes
-// (1 to 128 heads, 192 to 14712 keys, 14 chunks) 50 get the faster one or are within 3 %; the worst are 64 and 128 heads of 300 to 430 keys with few kept,
-// 17 %, and 8 heads of 12238 (w = 5098), 8 %. Forward, us, two
-// tiles / one: 16 heads of 1000 keys 37 / 19, 8 heads of 500 25 / 13, 8 heads of 4096 (w = 2048) 78 / 50, 172 rows of 26817 keys, 4 heads 109 / 71, but 64
-// heads of 2141 keys (w = 207) 55 / 74, 32 heads of 15878 (w = 1232) 487 / 568. The results are the same bits.
+// are estimated in steps of a CTA (a key tile and two score tiles): its steps and a fixed cost, the CTAs started heaviest first on the SMs. Tile mode: the SMs' share of the work, four
+// in five key tiles before the rows taken to be active, and part of the longest CTA behind it, more of it where the caller asks for tiles because the kept keys cluster (packed documents: walks of
+// all lengths). Token-compacted, where the CTAs are of about the same length: half way between the SMs' share and whole waves. (A one-tile CTA's slices: 0.55 of the other's with all SMs
+// gathering.) Fitted to 710 shapes of 1 to 256 heads and 128 to 32768 keys, each timed with both, and held against 360 others: 0.1 % (token-compacted) and 0.4 % (tiles) from the better one in the
+// mean, where the rule of slower kernels before, without the longest CTA and the half-empty last pair, was 0.8 and 0.6 %, on documents 3 %; worst 256 heads of 1054 keys with 64 channels, 10 %,
+// and 64 of 306, 9 %. Forward, us, two tiles / one: 16 heads of 5231 keys 138 / 147, 8 of 10069 206 / 237, 128 of 170 14.8 / 17.4, 8 of 5250 (w = 1312) 49.7 / 59.0, but
+// 16 of 3880 (64 channels) 94 / 78, documents in 8 heads of 16245 keys 199 / 147, in 32 of 2144 41 / 36, the last 693 of 23017 rows, 32 heads 178 / 149. The results are the same bits.
 // DMA_FLAG_BLOCK_SKIP is for two tiles: its marks are read where one group walks every entry.
 static int fwd_tiles(const Prob& P) {
     if (P.flags & DMA_FLAG_BLOCK_SKIP) return 2;
-    constexpr double kOneSteps = 2.5, kTwoSteps = 3.0, kSms = 148.0;
-    const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2;
+    constexpr double kSms = 148.0;
+    const int Trq = (P.Lq + 127) / 128, npairs = (Trq + 1) / 2, odd = Trq & 1;
     const double heads = (double)P.B * P.Hq;
-    if (P.flags & DMA_FLAG_COMPACT_KV) {                     // lists of about the same length
-        const double n = std::min((int64_t)P.w + (P.causal ? 256 : 0), (int64_t)P.L) / 128.0;
-        return 1.1 * std::ceil(heads * Trq / kSms) * (n / 2 + kTwoSteps) < std::ceil(heads * npairs / kSms) * (n + kTwoSteps) ? 1 : 2;
+    if (P.flags & DMA_FLAG_COMPACT_KV) {
+        // a pair's list: w + 256 keys, or the keys before its last row where they are fewer (`rising` pairs; non-causal: the head's w)
+        const double full = std::min((int64_t)P.w + (P.causal ? 256 : 0), (int64_t)P.L) / 128.0, before = P.q_off / 128.0;
+        const double rising = P.causal && P.w > P.q_off ? std::min(npairs, (P.w - P.q_off) / 256) : 0;
+        const double lists = rising * before + rising * (rising + 1) + (npairs - rising) * full;
+        const double longest = rising < npairs ? full : std::min(full, before + 2.0 * npairs);
+        auto cost = [&](double ctas, double work, double cta) { return 0.5 * std::max(cta, work / kSms) + 0.5 * std::ceil(ctas / kSms) * cta; };
+        const double one = cost(heads * Trq, heads * (0.55 * (2 * lists - odd * full) + 3.5 * Trq), 0.55 * longest + 3.5);
+        return one < cost(heads * npairs, heads * (lists + 4.0 * npairs), longest + 4.0) ? 1 : 2;
     }
-    const double total = Trq * (Trq + 1) / 2.0;              // walks grow with the row: the last tile's is the longest
-    const double one = 1.05 * std::max(Trq / 2.0 + kOneSteps, heads * (total / 2 + Trq * kOneSteps) / kSms);
-    const double two = (1.0 + 2.0 / Trq) * std::max(Trq + kTwoSteps, heads * (total / 2 + npairs * kTwoSteps) / kSms);
-    return one < two ? 1 : 2;
+    const bool clustered = (P.flags & DMA_FLAG_TILE_PATH) && !(P.flags & DMA_FLAG_IGNORE_BITMAP);
+    const double tail = clustered ? 0.4 : 0.2;
+    auto cost = [&](double work, double cta) { return std::max(cta, work / kSms + tail * cta); };       // walks grow with the row: the last tile's is the longest
+    const double fixed = clustered ? 1.0 : 1.5;
+    const double one = (clustered ? 1.1 : 1.15) * cost(heads * (0.2 * Trq * (Trq + 1.0) + Trq), Trq / 2.0 + 1.0);
+    return one < cost(heads * (0.8 * (npairs * (npairs + 1.0) - odd) + fixed * npairs), Trq + fixed) ? 1 : 2;
 }
 
 int launch_tc_fwd(const Prob& P, const void* Q, const void* K, const void* V, const float* bias,

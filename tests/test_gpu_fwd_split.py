@@ -43,9 +43,10 @@ def test_one_query_tile_per_cta(L, w, rows, d):
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("L,w,rows,B,flags", [
     (1100, 64, 0, 32, 0), (1152, 1152, 0, 32, 0), (1025, 1, 0, 32, 0), (700, 200, 0, 100, 0),            # tile walk: nine and six query tiles, ragged and whole ends
+    (1100, 64, 0, 200, 0), (1152, 1152, 0, 200, 0), (1025, 1, 0, 200, 0), (1250, 90, 0, 32, 0),          # (an odd number of tiles: two per CTA for more heads)
     (2177, 40, 0, 32, dma.DMA_FLAG_TILE_PATH), (3000, 1000, 0, 32, 0), (1500, 1, 0, 64, dma.DMA_FLAG_IGNORE_BITMAP),
     (2050, 1, 0, 32, 0), (2305, 512, 0, 32, 0), (2200, 300, 0, 32, 0),                                   # token-compacted lists
-    (1000, 128, 129, 150, 0), (700, 700, 300, 150, 0), (4096, 300, 2048, 74, 0), (2500, 300, 1790, 74, 0)])   # chunks of rows
+    (1000, 128, 129, 150, 0), (700, 700, 300, 150, 0), (700, 700, 450, 150, 0), (4096, 300, 2048, 74, 0), (2500, 300, 1790, 74, 0)])   # chunks of rows
 def test_bits_do_not_depend_on_the_batch(L, w, rows, B, flags, d):
     case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=1, L=L, w=w, d=d, name=f"alone and in a batch L{L} w{w} d{d}")
     inp = wl.make_inputs(case)
@@ -91,14 +92,14 @@ def test_two_query_tiles_on_the_small_shapes(L, w, rows, d):
 
 @pytest.mark.parametrize("d", [64, 128])
 def test_pairs_whose_tiles_use_different_key_tiles(d):
-    """Documents that begin inside a pair of query tiles: one tile skips the key tiles its partner needs and enters the walk late. 64 heads take
-    two query tiles per CTA, two heads one."""
+    """Documents that begin inside a pair of query tiles: one tile skips the key tiles its partner needs and enters the walk late. 400 heads take
+    two query tiles per CTA, 64 and two heads one."""
     L, cu = 1100, torch.tensor([0, 77, 384, 520, 700, 1100], dtype=torch.int32, device=DEV)
     case = wl.small(wl.CONFIGS["2"], B=1, Hq=2, Hkv=2, L=L, w=64, d=d, name="late entry")
     inp = wl.make_inputs(case)
     W, A = inp["W_delta"].to(DEV), inp["A"].to(DEV)
     out = {}
-    for B, flags in ((1, dma.DMA_FLAG_SIMT), (1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (32, 0), (32, 0), (32, 0)):
+    for B, flags in ((1, dma.DMA_FLAG_SIMT), (1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (32, 0), (32, 0), (32, 0), (200, 0), (200, 0), (200, 0)):
         p = dma.problem(B, 2, 2, L, d, 64, flags=flags)
         Q, K, V = (inp[k].to(DEV).repeat(B, 1, 1, 1) for k in ("Q", "K", "V"))
         mask = dma.dma_mask_build_varlen(p, V, W, A, cu)
@@ -114,7 +115,7 @@ def test_pairs_whose_tiles_use_different_key_tiles(d):
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("B,skip", [(1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (32, 0)])      # one query tile per CTA, two, two
+@pytest.mark.parametrize("B,skip", [(1, 0), (1, dma.DMA_FLAG_BLOCK_SKIP), (100, 0)])     # one query tile per CTA, two, two
 @pytest.mark.parametrize("path", ["tiles", "lists", "chunk", "noncausal"])
 def test_query_tiles_without_keys(path, B, skip, d):
     """A caller's mask (padding) may leave whole query tiles, pairs of them or a head without a key: O is exactly zero there and lse -inf, whatever Q
