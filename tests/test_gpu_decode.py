@@ -52,6 +52,9 @@ def run_case(case, cap_extra=0, seed=21, tie_heads=False):
     dict(B=2, Hq=8, Hkv=2, L=3001, d=128, w=512, dtype="bf16"),       # ragged: two splits, the second partly empty
     dict(B=1, Hq=4, Hkv=4, L=5000, d=128, w=1, dtype="fp32"),         # a single key
     dict(B=1, Hq=4, Hkv=1, L=700, d=128, w=4096, dtype="bf16"),       # w >= N: dense attention over the cache
+    dict(B=1, Hq=2, Hkv=1, L=9500, d=128, w=9000, dtype="bf16"),      # 71 splits of a row: combined in three turns
+    dict(B=1, Hq=1, Hkv=1, L=13000, d=64, w=12500, dtype="fp32"),     # 98 splits
+    dict(B=2, Hq=4, Hkv=2, L=20000, d=64, w=17000, dtype="bf16"),     # 34 splits of 512 keys
 ])
 def test_small_cases(kw):
     run_case(wl.small(wl.CONFIGS["2"], name="decode-small", backward=False, **kw), cap_extra=37)

@@ -62,6 +62,8 @@ def run(case, n0, steps, seed=5, tie_head=False):
     (dict(B=2, Hq=8, Hkv=2, L=1200, d=64, w=1170, dtype="bf16"), 1140, 40),  # 160 would be more than SMs: 256 keys, ragged
     (dict(B=1, Hq=4, Hkv=4, L=300, d=128, w=1, dtype="fp32"), 200, 40),      # a single kept key
     (dict(B=1, Hq=4, Hkv=1, L=200, d=128, w=4096, dtype="bf16"), 150, 30),   # w above the cache: everything is kept
+    (dict(B=1, Hq=2, Hkv=1, L=9030, d=64, w=8900, dtype="bf16"), 9000, 25),  # 70 splits of a row: three turns of the combine kernel, two of its walk over the weakest keys
+    (dict(B=1, Hq=2, Hkv=1, L=16920, d=128, w=16500, dtype="fp32"), 16900, 12),      # 65 of 256 keys
 ])
 def test_steps_match_the_oracle(kw, n0, steps):
     run(wl.small(wl.CONFIGS["2"], name="decode-step", backward=False, **kw), n0, steps)
