@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) decode_list_attn_kernel(const
 // kernel's last CTA per row, as dma_decode does, was measured slower here, 16.5 -> 20.7 us per step: the state must then be
 // writable in the attention kernel, whose loads of the kept list no longer take the read-only path, and the update, which
 // scans the w kept keys, runs on 256 threads at the end of the row's critical path instead of 8 D.)
-template <typename T, int D>
+template <typename T, int D, int kBatch>
 __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float* __restrict__ partial, T* __restrict__ o, float* __restrict__ lse,
                                                                     int nsplit, const float* __restrict__ delta, int64_t ld,
                                                                     int N, int w_cap, int* __restrict__ state, const Weakest* __restrict__ weak) {
@@ -1103,12 +1103,11 @@ __global__ void __launch_bounds__(8 * D) decode_step_combine_kernel(const float*
     const float* dl = delta + (size_t)bh * ld;
     int* hdr = state + (size_t)bh * state_stride(w_cap);
     const Weakest* wk = weak ? weak + (size_t)bh * nsplit : nullptr;
-    // Everything the step needs is requested at once: the group's first splits, the header, the appended key's weight and the lists' weakest keys. (The maxima,
+    // Everything the step needs is requested at once: the group's first kBatch splits, the header, the appended key's weight and the lists' weakest keys. (The maxima,
     // then the sums, then the state, each a round trip to L2 behind the one before: 16 captured steps of 32 rows of 2048 kept keys 147 -> 134 us, of one row 101 -> 91, of 16 rows of
     // 4973 164 -> 141.)
     StepState x;
     x.load(dl, hdr, wk, N, nsplit);
-    constexpr int kBatch = 4;                                  // splits of a group that are in flight together
     float mx = -INFINITY, l = 0.0f, acc = 0.0f;
     for (int s0 = g; s0 < nsplit; s0 += 8 * kBatch) {
         float ms[kBatch], ls[kBatch], as[kBatch], m = mx;
@@ -1293,7 +1292,9 @@ static int launch_step_typed(const Prob& P, const void* q, const void* K, const 
                           delta, ld, (const int*)state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns, P.ks[0], P.ks[1],
                           P.ks[2], P.vs[0], P.vs[1], P.vs[2], weak);
     if (rc) return rc;
-    return launch_overlapped(decode_step_combine_kernel<T, D>, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
+    // splits of a group in flight together: more than 32 splits of a row take turns of eight instead of four (4 rows of 66141 kept keys, 259 splits, 11.5 -> 8.4 us, two of 16384, 64 splits, 3.55 -> 2.9, but 8 of 4096 2.85 -> 3.07)
+    auto combine = ns > 32 ? decode_step_combine_kernel<T, D, 8> : decode_step_combine_kernel<T, D, 4>;
+    return launch_overlapped(combine, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
                              ld, P.L, P.w_cap, state, (const Weakest*)weak);
 }
 
