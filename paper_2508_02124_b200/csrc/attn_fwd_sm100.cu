@@ -516,7 +516,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             if constexpr (kSplit) {
                 // Each group writes half of the channels. A thread holds a row: a warp turns its 32 rows around in the Q buffer, which the last S product
                 // has left (16-byte chunks swizzled by the row), so that neighbouring lanes write neighbouring 16 bytes of a row instead of 32 rows
-                // per instruction. 8 heads of 4096 keys (w = 2048) 51.5 -> 48.9 us. (With two query tiles the two groups' ends overlap, and 66.6 -> 70.4 at 16 heads of 4096.)
+                // per instruction. 8 heads of 4096 keys (w = 2048) 50.9 -> 49.3 us. (With two query tiles the two groups' ends overlap, and 66.6 -> 70.4 at 16 heads of 4096.)
                 uint8_t* turn = S.q[0] + (warp & 3) * 4096 + (kD == 128 ? w * (kTileBytes / 2) : 0);
                 constexpr int kLanes = kD == 128 ? 8 : 4, kRowsPer = 32 / kLanes;      // lanes per row, rows per instruction
                 const int ch0 = kD == 128 ? 0 : 4 * w;

@@ -7,7 +7,8 @@
 //   tree_block_kernel, expiry_search_kernel (longer heads: tree_merge_kernel, expiry_tree_kernel)
 //                       selection as a rank tree: the passes of a merge sort of (delta bits, ~index) keys leave one bit per key and
 //                       level, and a key's expiry (the w-th smallest index among the keys that beat it) is a walk of log2(L) steps.
-//                       Heads of up to 4096 keys: sort, walk and bitmap in the one block kernel
+//                       Heads of up to 1024 keys, and of up to 4096 where there are many: sort, walk and bitmap in the one block kernel
+//                       (launch_mask_build has the rules)
 //   bitmap_square_kernel, bitmap_kernel   per key tile: union of the query-tile intervals its keys are kept in
 #include <algorithm>
 #include <cmath>

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kFullThreads) mask_bwd_full_kernel(const T* __
     const int C = Hkv * D, HqP = (Hq + 7) & ~7;
     float* sV = smem;                              // [R][C]
     float* sDz = sV + (size_t)R * C;               // [R][HqP], heads beyond Hq hold 0
-    float* sZ = sDz + (size_t)R * HqP;             // [Hq][R]: z, then dM delta softplus(z)
+    float* sZ = sDz + (size_t)R * HqP;             // [Hq][R]: dM delta softplus(z)
     const int b = blockIdx.y, j0 = blockIdx.x * R;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int C8 = C / 8, D8 = D / 8;
