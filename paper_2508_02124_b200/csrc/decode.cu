@@ -343,16 +343,17 @@ __global__ void __launch_bounds__(kSelectThreads, kKeys == 0 ? 2 : 1) decode_sel
 }
 
 // The same selection, one CTA per row, two on an SM, that reads the row once: a sample brackets the threshold (4.5 standard deviations to either side), the sweep
-// leaves two bits per key (above the bracket, in it or above), the keys inside, a few per cent of the row, are gathered in index order, and the last of them that
+// leaves two bits per key (above the bracket, in it or above), the keys inside, a few per cent of the row, are gathered, and the last of them that
 // is kept is found as above. The bits are then the row's list. A word of 32 keys costs some 30 instructions in all, where the histogram of all keys and
 // three sweeps over registers took 880 per 1024 and a shared-memory add per key; both kernels are bound by them.
 // Weights that crowd: a bracket end whose bin holds more than kHeavy of the sample is narrowed among that bin's samples; where the bracket is one bit pattern
 // (equal weights), its first keys are kept by their bits alone, however many there are; and a bracket that misses, or holds more than kInside keys
-// of several patterns, is narrowed by a histogram of the row's keys in it and swept again. Units of 32 words go around the warps, so that a
-// bracket or a list that lies in one place of the row is not one warp's work.
-// Carried state taken up from such a row, us, kernel above / this one, at w = 64, N / 16, N / 4, N / 2, N - 1: 256 rows of 65536 keys 57 / 25, 65 / 30, 71 / 35, 79 / 39,
+// of several patterns, is narrowed by a histogram of the row's keys in it and swept again. A warp sweeps neighbouring words, but units of 32 words go around the warps
+// afterwards, so that a bracket or a list that lies in one place of the row is not one warp's work.
+// Carried state taken up from rows in the L2, us, kernel above / this one, at w = 64, N / 16, N / 4, N / 2, N - 1: 256 rows of 65536 keys 57 / 25, 65 / 30, 71 / 35, 79 / 39,
 // 74 / 44, all weights equal 56 / 22 .. 70 / 41, ten values 67 / 28 .. 102 / 42, weights that rise along the row 57 / 26 .. 76 / 42 (before units, narrowing and the
-// bits of equal weights: random 23 .. 160, equal 100 .. 114, ten values 26 .. 143, rising 28 .. 167); 148 rows of 131072 random 70 / 26 .. 88 / 55.
+// bits of equal weights: random 23 .. 160, equal 100 .. 114, ten values 26 .. 143, rising 28 .. 167); 148 rows of 131072 random 70 / 26 .. 88 / 55. From memory, up to N / 2: 256 rows of
+// 65536 69 / 34, 79 / 39, 84 / 44, 87 / 48; the list in the order of the keys (its place from a count of the words first) 35, 40.3, 45.7, 49.7, a warp's words 32 apart in the sweep 34.6, 39.5, 45, 48.8.
 constexpr int kInside = 8192;                  // most keys gathered from the bracket (expected: 6000 of 131072 at w = N / 4)
 constexpr int kHeavy = 128;                    // (of 4096 or 8192 samples, where an ordinary row has ten in its fullest bin)
 constexpr int kStreamMinKeys = 4097, kStreamMaxKeys = 1 << 17;        // (more keys than the sample;) two bits per key of a row in shared memory: 32 KB
@@ -360,11 +361,11 @@ constexpr int kMaxUnits = kStreamMaxKeys / 1024;
 struct alignas(16) StreamShared {
     int hist[2048];
     unsigned long long list[kInside], cand[kCandidates];
-    int above[kMaxUnits], inside[kMaxUnits];   // per unit: keys above the bracket (later: kept), keys in it
+    int above[kMaxUnits], inside[kMaxUnits], begin[kMaxUnits];         // per unit: keys above the bracket (later: kept), keys in it, where those begin in the list
     int scan[kSelectWarps];
     uint32_t warp_min[kSelectWarps], warp_max[kSelectWarps];
     int bin[2], in_bin[2], over_bin[2];
-    int ncand;
+    int ncand, listed;
     unsigned long long weakest;
 };
 static size_t stream_smem(int N) { return sizeof(StreamShared) + (size_t)((N + 1023) / 1024) * 32 * sizeof(uint2); }
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
     const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, units = (N + 1023) / 1024;
     for (int t = tid; t < 2048; t += kSelectThreads) S.hist[t] = 0;
     if (tid < kMaxUnits) S.above[tid] = S.inside[tid] = 0;
-    if (tid == 0) { S.ncand = 0; S.bin[0] = S.bin[1] = -1; }
+    if (tid == 0) { S.ncand = S.listed = 0; S.bin[0] = S.bin[1] = -1; }
     pdl_enter(delta, list, tickets);
     int* out = list + (size_t)bh * list_stride;
     if (tickets && tid == 0) tickets[bh] = 0;
@@ -478,7 +479,8 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
     }
     // f(word, its keys) for the CTA's words of 32 consecutive keys, eight words of a warp requested at once
     auto sweep = [&](auto&& f) {
-        for (int wb = 8 * warp; wb < 32 * units; wb += 8 * kSelectWarps) {
+        const int per = (32 * units + 8 * kSelectWarps - 1) / (8 * kSelectWarps) * 8, w1 = min(32 * units, (warp + 1) * per);
+        for (int wb = warp * per; wb < w1; wb += 8) {
             uint32_t u[8];
             const uint32_t* at = src + wb * 32 + lane;
             if (wb * 32 + 256 <= N) {
@@ -492,6 +494,16 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
             for (int k = 0; k < 8; ++k) f(wb + k, u[k]);
         }
     };
+    auto before_lane = [&](int n) {                                       // sum of the lower lanes' n
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        return incl - n;
+    };
+    int* gathered = reinterpret_cast<int*>(S.list);                       // (the low words: first the key's number, then its order key)
     uint32_t bmin = lo, bmax = hi;                                        // of the keys inside, or wider
     int need, inside;
     for (int turn = 0;; ++turn) {
@@ -513,8 +525,17 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
         __syncthreads();
         for (int unit = warp; unit < units; unit += kSelectWarps) {
             const uint2 m = mask[32 * unit + lane];
-            const int a = __reduce_add_sync(0xffffffffu, __popc(m.x)), i = __reduce_add_sync(0xffffffffu, __popc(m.y & ~m.x));
-            if (lane == 0) { S.above[unit] = a; S.inside[unit] = i; }
+            uint32_t in = m.y & ~m.x;
+            const int a = __reduce_add_sync(0xffffffffu, __popc(m.x)), n = __popc(in), before = before_lane(n);
+            int at = 0;
+            if (lane == 31) {
+                S.above[unit] = a;
+                S.inside[unit] = before + n;
+                S.begin[unit] = at = atomicAdd(&S.listed, before + n);
+            }
+            at = __shfl_sync(0xffffffffu, at, 31) + before;
+            if (lo != hi)
+                for (; in && at < kInside; in &= in - 1u) gathered[2 * at++] = (32 * unit + lane) * 32 + __ffs(in) - 1;
         }
         if (again) range(bmin, bmax); else __syncthreads();
         int a = 0, i = 0;
@@ -524,6 +545,7 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
         inside = __reduce_add_sync(0xffffffffu, i);
         if (need >= 1 && need <= inside && (inside <= kInside || bmin == bmax)) break;
         // the bracket is narrowed, or the part of the row beside it that holds the threshold
+        if (tid == 0) S.listed = 0;
         int r = need, excl;
         int2 c;
         if (need < 1) { lo = hi + 1u; hi = 0x7FFFFFFFu; r = keep; }
@@ -548,27 +570,10 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
             run += __reduce_add_sync(0xffffffffu, v);
         }
     };
-    auto before_lane = [&](int n) {                                       // sum of the lower lanes' n
-        int incl = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        return incl - n;
-    };
     uint32_t* kept_of = reinterpret_cast<uint32_t*>(S.hist);              // one bit per gathered key: kept
     if (!equal) {
-        int* gathered = reinterpret_cast<int*>(S.list);                   // (the low words: first the key's number, then its order key)
-        each_unit(S.inside, [&](int unit, int at) {
-            const uint2 m = mask[32 * unit + lane];
-            uint32_t in = m.y & ~m.x;
-            at += before_lane(__popc(in));
-            for (; in; in &= in - 1u) gathered[2 * at++] = (32 * unit + lane) * 32 + __ffs(in) - 1;
-        });
         bmin = 0x7FFFFFFFu;
         bmax = 0u;
-        __syncthreads();
         for (int e0 = tid; e0 < inside; e0 += 4 * kSelectThreads) {       // four keys of a thread requested at once
             int j[4];
             uint32_t u[4];
@@ -636,11 +641,12 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
     }
     __syncthreads();
     // the kept keys' bits
-    each_unit(S.inside, [&](int unit, int at) {
+    if (equal) each_unit(S.inside, [&](int unit, int at) { S.begin[unit] = at; });         // (by index)
+    __syncwarp();
+    for (int unit = warp; unit < units; unit += kSelectWarps) {
         const uint2 m = mask[32 * unit + lane];
         uint32_t in = m.y & ~m.x, word = m.x;
-        const int n = __popc(in);
-        at += before_lane(n);
+        const int n = __popc(in), at = S.begin[unit] + before_lane(n);
         uint32_t keep_bits;                                               // of the word's n keys inside
         if (equal) {
             const int k = min(max(need - at, 0), n);
@@ -663,7 +669,7 @@ __global__ void __launch_bounds__(kSelectThreads, 2) decode_select_stream_kernel
         mask[32 * unit + lane].x = word;
         const int kept = __reduce_add_sync(0xffffffffu, __popc(word));
         if (lane == 0) S.above[unit] = kept;
-    });
+    }
     __syncthreads();
     // the bits -> indices
     constexpr int kTurn = 2 * kInside / kSelectWarps;
