@@ -1298,8 +1298,9 @@ static int launch_step_typed(const Prob& P, const void* q, const void* K, const 
                           delta, ld, (const int*)state, P.w_cap, partial, P.L, P.Hq, P.G, P.scale * 1.4426950408889634f, ns, P.ks[0], P.ks[1],
                           P.ks[2], P.vs[0], P.vs[1], P.vs[2], weak);
     if (rc) return rc;
-    // splits of a group in flight together: more than 32 splits of a row take turns of eight instead of four (4 rows of 66141 kept keys, 259 splits, 11.5 -> 8.4 us, two of 16384, 64 splits, 3.55 -> 2.9, but 8 of 4096 2.85 -> 3.07)
-    auto combine = ns > 32 ? decode_step_combine_kernel<T, D, 8> : decode_step_combine_kernel<T, D, 4>;
+    // Splits of a group in flight together: one where there are no more (480 rows of 5 kept keys, a step, 7.0 -> 6.5 us, with the maxima first 6.6; 32 of 2048 8.2 -> 7.9), else four, and eight of more than 32 of a
+    // row (combine kernel: 4 rows of 66141 kept keys, 259 splits, 11.5 -> 8.4 us, two of 16384, 64 splits, 3.55 -> 2.9, but 8 of 4096 2.85 -> 3.07)
+    auto combine = ns > 32 ? decode_step_combine_kernel<T, D, 8> : ns > 8 ? decode_step_combine_kernel<T, D, 4> : decode_step_combine_kernel<T, D, 1>;
     return launch_overlapped(combine, dim3(P.B * P.Hq), dim3(8 * D), 0, st, 1, (const float*)partial, (T*)o, lse, ns, delta,
                              ld, P.L, P.w_cap, state, (const Weakest*)weak);
 }
